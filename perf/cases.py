@@ -17,9 +17,10 @@ Kinds of case:
   batch     several requests of different prefix lengths over the same weights, stepped together (spd_batch_generate);
             they go on from where they are, as `decode`
 Outputs are the logits of the last pass (of every request of a batch), which hang on every earlier choice, and the
-sampled ids (the order of two drafts of nearly the same probability is no property of a correct program).  With random weights the logits are flat, and a temperature of 0.06 makes the drafts' weights, and with them the next input,
-hang on the last bits of the logits: two correct programs drift apart within a few timesteps.  So the temperature is 1,
-and cases of several timesteps use the float32 cache (a bf16 one rounds a value in a hundred the other way).
+sampled ids (the order of two drafts of nearly the same probability is no property of a correct program).  With random
+weights the logits are flat, and a temperature of 0.06 makes the drafts' weights, and with them the next input, hang on
+the last bits of the logits: two correct programs drift apart within a few timesteps.  So the temperature is 1, and
+cases of several timesteps use the float32 cache (a bf16 one rounds a value in a hundred the other way).
 """
 from __future__ import annotations
 
