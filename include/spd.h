@@ -125,10 +125,12 @@ int spd_create(const spd_config *cfg, const spd_weights *weights, const spd_ngra
  * over the m prefix tokens (HOST int32 ids, 1 <= m < max_pos), draft i takes the i-th most probable
  * next token and its probability, no n-gram term.  out_ids / out_gamma: HOST arrays of k entries
  * (token of draft i; gamma_i of Eq. 4), either may be NULL.  Restarts the context from scratch.
- * Synchronises the stream before returning.  Prefixes of more than 32 tokens (head size 64 or 128,
- * max_pos >= 130) run all but their last 1..16 tokens through the long-prefix path (tensor-core
- * products over up to 512 tokens at a time, many small launches); its buffers are part of the
- * workspace.  The result does not depend on which path a token took beyond float rounding.
+ * Synchronises the stream before returning.  Where the context has the long-prefix path (head size 64
+ * or 128, max_pos >= 130) prefixes of more than 16 tokens, and shorter ones of a model with 16 MB of
+ * matrices per layer and more, run as its jobs (tensor-core products over up to 512 tokens at a time,
+ * 9 launches per layer; the last job ends with one launch for the LM head and the first timestep); its
+ * buffers are part of the workspace.  The result does not depend on which path a token took beyond
+ * float rounding.
  */
 int spd_prefill(spd_ctx *ctx, const int32_t *prefix_ids, int32_t m, int32_t *out_ids, float *out_gamma);
 

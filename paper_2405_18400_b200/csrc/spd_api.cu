@@ -47,8 +47,7 @@ struct Layout {
       bt_ss, bt_out, total;
 };
 
-// Tokens one long-prefix job takes at most (0: the context never runs one): prefixes of more than 64 tokens send
-// all but their last 1..16 tokens through the tensor-core path.
+// Tokens one long-prefix job takes at most (0: the context never runs one).
 int tc_rows(const spd_config &c) {
   const int hd = c.d_model / c.n_heads;
   if (hd != 64 && hd != 128) return 0;  // the head sizes its attention kernel is built for
@@ -273,26 +272,39 @@ spd::TcJob tc_job(spd_ctx *ctx) {
   return job;
 }
 
-// Runs prefix tokens [first, first + count) (positions alike), the last of which ends the prefix, through the
-// prefill kernel, kPfTokens at a time: their keys and values enter the cache, and the last launch goes on to
-// the LM head on the prefix's last token and the first timestep (Eq. 1).
+// Whether a run of up to 16 tokens is better off as a job of the long-prefix path (9 launches per layer) than in the
+// 16-token kernel (one cooperative launch whose weight stream reaches 0.44 of the copy bandwidth): from kJobLayerBytes
+// of matrices per layer on.  15 tokens, 8 layers, kernel / job: 1.6 MB per layer (no difference worth the launches;
+// the host's share is larger) 385 / 350 us, 25 MB 478 / 404, 101 MB 740 / 481, 405 MB 1263 / 901; the whole 7B shape 4.65 / 3.36 ms.
+constexpr size_t kJobLayerBytes = (size_t)16 << 20;
+bool large_layers(const spd::KParams &kp) { return 2 * (size_t)kp.d * (4 * (size_t)kp.d + 3 * (size_t)kp.f) >= kJobLayerBytes; }
+
+// Runs prefix tokens [first, first + count) (positions alike), the last of which ends the prefix: their keys and
+// values enter the cache, and the last launch goes on to the LM head on the prefix's last token and the first timestep
+// (Eq. 1).  Jobs of the long-prefix path, up to tc_rows tokens each, where the context has it and the run is longer than
+// kTcMinPrefix or the model large; else (and for the rest of such a run with a small model) the prefill kernel,
+// kPfTokens at a time.  The per-layer trace is recorded by the prefill kernel only, which then ends the prefix.
 int prefill_tokens(spd_ctx *ctx, int first, int count) {
   spd::KParams &kp = ctx->kp;
   int32_t *base = kp.prefix;
   int rc = SPD_OK;
-  // Long run of tokens: all but the last 1..16 go through the tensor-core path, in jobs of up to tc_rows tokens.
+  const int min_job = large_layers(kp) && !kp.trace ? 0 : spd::kTcMinPrefix;
+  const int jobs_end = kp.trace ? count - ((count - 1) % spd::kPfTokens + 1) : count;
   int tc_done = 0;
-  if (ctx->tc_rows > 0 && count > spd::kTcMinPrefix) {
-    const int tc_total = count - ((count - 1) % spd::kPfTokens + 1);
+  if (ctx->tc_rows > 0 && count > min_job) {
     SPD_CUDA(cudaMemsetAsync(ctx->ws + ctx->lay.state, 0, head_bytes(false), ctx->stream));
     spd::TcJob job = tc_job(ctx);
-    while (tc_done < tc_total) {
-      const int n = tc_total - tc_done < ctx->tc_rows ? tc_total - tc_done : ctx->tc_rows;
+    while (tc_done < jobs_end && (kp.trace || count - tc_done > min_job)) {
+      const int left = jobs_end - tc_done;
+      int n = left < ctx->tc_rows ? left : ctx->tc_rows;
+      // Up to two token tiles of a large model go one by one: each pass over the weights costs less than the second
+      // tile's share of the 128-token tiles' products, which need more tiles to fill the chip (7B shape, 256 tokens).
+      if (left > spd::kTcTile && left <= 2 * spd::kTcTile && large_layers(kp)) n = spd::kTcTile;
       job.ids = base + first + tc_done;
       job.pos0 = first + tc_done;
       job.n_tok = n;
       int launched = 0;
-      const cudaError_t e = spd_internal_tc_prefill(&job, ctx->stream, &launched);
+      const cudaError_t e = spd_internal_tc_prefill(&job, tc_done + n == count ? &kp : nullptr, ctx->stream, &launched);
       ctx->launches += launched;
       if (e != cudaSuccess) return cuda_fail(e, "long-prefix launch");
       tc_done += n;

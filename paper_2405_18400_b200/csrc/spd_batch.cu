@@ -339,6 +339,91 @@ __global__ void __launch_bounds__(kConsumerThreads) spd_batch_tail_kernel(const 
   }
 }
 
+// The end of a prefix on the long-prefix path: the last product's partial sums and the residual row of the prefix's last
+// token, the final norm, that row's logits, KeepTopK and the first timestep (Eq. 1), one launch.  One token row against
+// [V][d] weights is a stream of the weights (262 MB at 7B shape, 40 us at the copy bandwidth), so a block per SM takes a
+// contiguous range of the vocabulary and a warp four of its rows at a time (4 rows x 16 bytes per lane in flight, each
+// eight activations read from shared memory serve four rows), float32 multiplies; every block computes the norm itself
+// from L2 (nz + 1 rows of d floats).  The block that arrives last merges the blocks' top-k lists and takes the step.
+constexpr int kHeadRows = 4;
+__global__ void __launch_bounds__(kConsumerThreads) spd_job_head_kernel(const __grid_constant__ KParams p, const float *h, const float *y, int nz,
+                                                                        size_t zs) {
+  extern __shared__ __align__(16) float jh_x[];  // [d]: residual row times the final norm's gain
+  __shared__ float s_sum[kConsumerWarps];
+  __shared__ int s_last;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r0 = (int)((long long)p.V * blockIdx.x / gridDim.x), r1 = (int)((long long)p.V * (blockIdx.x + 1) / gridDim.x);
+  // the warp's first rows on their way to L2 while the product before this kernel still runs
+  for (int e = lane; e < kHeadRows * p.d / 64; e += 32) {
+    const int r = r0 + warp * kHeadRows + e / (p.d / 64);
+    if (r < r1) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.lm_head + (size_t)r * p.d + (e % (p.d / 64)) * 64));
+  }
+  dep_wait();
+  float sq = 0.f;
+  for (int c = threadIdx.x; c < p.d; c += kConsumerThreads) {
+    float v = h[c];
+    for (int z = 0; z < nz; ++z) v += y[z * zs + c];
+    sq = fmaf(v, v, sq);
+    jh_x[c] = v * __bfloat162float(p.final_norm[c]);
+    if (blockIdx.x == 0) p.h[c] = v;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+  if (lane == 0) s_sum[warp] = sq;
+  __syncthreads();
+  float ss = 0.f;
+#pragma unroll
+  for (int w = 0; w < kConsumerWarps; ++w) ss += s_sum[w];
+  const float rs = rsqrtf(ss / (float)p.d + p.eps);
+  for (int r = r0 + warp * kHeadRows; r < r1; r += kConsumerWarps * kHeadRows) {
+    float acc[kHeadRows];
+    const __nv_bfloat16 *w[kHeadRows];
+#pragma unroll
+    for (int i = 0; i < kHeadRows; ++i) {
+      acc[i] = 0.f;
+      w[i] = p.lm_head + (size_t)min(r + i, r1 - 1) * p.d;  // past the range: its last row again, not stored
+    }
+#pragma unroll 2
+    for (int c = lane * 8; c < p.d; c += 256) {
+      uint4 v[kHeadRows];
+#pragma unroll
+      for (int i = 0; i < kHeadRows; ++i) v[i] = __ldcs(reinterpret_cast<const uint4 *>(w[i] + c));
+      const float4 xa = *reinterpret_cast<const float4 *>(jh_x + c), xb = *reinterpret_cast<const float4 *>(jh_x + c + 4);
+#pragma unroll
+      for (int i = 0; i < kHeadRows; ++i) {
+        acc[i] = fmaf(__uint_as_float(v[i].x << 16), xa.x, acc[i]);
+        acc[i] = fmaf(__uint_as_float(v[i].x & 0xffff0000u), xa.y, acc[i]);
+        acc[i] = fmaf(__uint_as_float(v[i].y << 16), xa.z, acc[i]);
+        acc[i] = fmaf(__uint_as_float(v[i].y & 0xffff0000u), xa.w, acc[i]);
+        acc[i] = fmaf(__uint_as_float(v[i].z << 16), xb.x, acc[i]);
+        acc[i] = fmaf(__uint_as_float(v[i].z & 0xffff0000u), xb.y, acc[i]);
+        acc[i] = fmaf(__uint_as_float(v[i].w << 16), xb.z, acc[i]);
+        acc[i] = fmaf(__uint_as_float(v[i].w & 0xffff0000u), xb.w, acc[i]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kHeadRows; ++i) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+      if (lane == 0 && r + i < r1) p.logits[r + i] = acc[i] * rs;
+    }
+  }
+  __syncthreads();
+  if (warp != 0) return;
+  block_topk(p, r0, r1, blockIdx.x);
+  if (lane == 0) {
+    __threadfence();
+    s_last = atomicAdd(&p.st->bar, 1u) == gridDim.x - 1;  // zeroed by the host at the start of the call
+    __threadfence();
+  }
+  __syncwarp();
+  if (!s_last) return;
+  tail_keep_topk(p, gridDim.x);
+  tail_first(p, lane, 0);
+  __syncwarp();
+  tail_gamma(p, lane);
+}
+
 }  // namespace spd
 
 namespace {
@@ -422,4 +507,18 @@ extern "C" cudaError_t spd_internal_job_swiglu(const spd::TcJob *job, float *ss,
   const spd::TcJob &j = *job;
   return spd::launch_dep(spd::spd_batch_swiglu_kernel, dim3(j.n_tok, (j.f + 255) / 256), dim3(256), 0, s, j.y, nz, zs, ss, j.eps, j.d, j.x,
                          (size_t)j.x_term_rows * j.f, j.f);
+}
+
+extern "C" cudaError_t spd_internal_job_head(const spd::KParams *p, const float *h, const float *y, int nz, size_t zs, int sm_count, cudaStream_t s) {
+  // at most 64 KB of activations (d_model <= 16384); the attribute is per device and set on its first launch
+  static bool ready[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64 || !ready[dev]) {
+    e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_job_head_kernel), cudaFuncAttributeMaxDynamicSharedMemorySize, 65536);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) ready[dev] = true;
+  }
+  return spd::launch_dep(spd::spd_job_head_kernel, dim3(sm_count), dim3(spd::kConsumerThreads), (size_t)p->d * 4, s, *p, h, y, nz, zs);
 }

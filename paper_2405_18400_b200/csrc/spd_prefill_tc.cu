@@ -1,8 +1,9 @@
 // Long-prefix prefill (the dense pass over the prefix that precedes Eq. 1): blocks of 128..512 prefix tokens at a
 // time, their matrix products on the fifth-generation tensor cores (tcgen05.mma, operands staged in shared
 // memory by tiled TMA copies, float32 accumulators in tensor memory), everything between the products in small
-// row-wise kernels.  Only the cache is produced here: the prefix's last tokens, the LM head and the first
-// timestep stay with spd_prefill_kernel, which finds these positions in the cache like any earlier launch's.
+// row-wise kernels.  The job that ends a prefix goes on to the LM head and the first timestep of its last token
+// (7B shape, host to host: 15 / 27 / 100 / 400 / 2048 tokens 3.4 / 3.7 / 6.7 / 23 / 102 ms; with the last 1..16 tokens
+// in spd_prefill_kernel 4.7 / 9.2 / 12.2 / 24 / 108 ms).
 //
 // Product: Y[token][row] = sum_c X[token][c] W[row][c], W bf16 [rows][cols] as stored, X float32 activations
 // split exactly into three bf16 terms (x = hi + mid + lo, 8 + 8 + 8 significant bits), so that the tensor
@@ -950,12 +951,15 @@ extern "C" cudaError_t spd_internal_tc_stall(const spd::TcJob *job, cudaStream_t
 // Enqueues the decoder over j.n_tok tokens (at most j.x_term_rows) at positions j.pos0 ..: their keys and values
 // enter the cache.  The products run over whole tiles of 128 tokens: the rows past n_tok of the last tile hold
 // whatever an earlier job left, give rows of Y that nothing reads (a row of Y depends on its own token only).
+// head: the context's parameters when the job ends the prefix, else null.  Then the last layer carries on with the last
+// token's row alone once the keys and values are in the cache (nothing reads the other rows), and one more launch adds
+// the last product to the residual row, multiplies the LM head and takes the first timestep.
 // *launches receives the number of kernels enqueued.
-extern "C" cudaError_t spd_internal_tc_prefill(const spd::TcJob *job, cudaStream_t s, int *launches) {
+extern "C" cudaError_t spd_internal_tc_prefill(const spd::TcJob *job, const spd::KParams *head, cudaStream_t s, int *launches) {
   const spd::TcJob &j = *job;
   const int n = j.n_tok, d = j.d, f = j.f;
   const size_t ts_d = (size_t)j.x_term_rows * d, ts_f = (size_t)j.x_term_rows * f;
-  const uint8_t *xmap_d = j.x_tmaps, *xmap_f = j.x_tmaps + spd::kTensorMapBytes;
+  const bool small = n <= spd::kTcM;
   int count = 0;
   cudaError_t e = cudaSuccess;
   // A job of up to 128 tokens is one token tile: its products are bound by the weight stream and take the product
@@ -963,70 +967,66 @@ extern "C" cudaError_t spd_internal_tc_prefill(const spd::TcJob *job, cudaStream
   // zs floats apart, which the row-wise kernels add up).
   int nz = 1;
   size_t zs = 0;
-  auto gemm = [&](const uint8_t *xmap, int which, int N, int C) {
+  auto gemm = [&](int rows, int wide, int which, int N, int C) {
     if (e != cudaSuccess) return;
     const uint8_t *wmap = j.w_tmaps + (size_t)which * spd::kTensorMapBytes;
-    if (n <= spd::kTcM) {
-      e = spd_internal_batch_gemm(j.x_tmaps, xmap != xmap_d, wmap, j.y, j.y_floats, n, N, C, j.x_term_rows, j.st, j.sm_count, s, 1, &nz, &zs);
+    if (rows <= spd::kTcM) {
+      e = spd_internal_batch_gemm(j.x_tmaps, wide, wmap, j.y, j.y_floats, rows, N, C, j.x_term_rows, j.st, j.sm_count, s, 1, &nz, &zs);
     } else {
-      const dim3 grid((n + spd::kTcM - 1) / spd::kTcM, (N + spd::kTcN - 1) / spd::kTcN);
-      spd::spd_tc_gemm_kernel<<<grid, spd::kTcThreads, tc_gemm_smem(), s>>>(xmap, wmap, j.y, N, C, j.x_term_rows, j.st, 0);
+      const dim3 grid((rows + spd::kTcM - 1) / spd::kTcM, (N + spd::kTcN - 1) / spd::kTcN);
+      spd::spd_tc_gemm_kernel<<<grid, spd::kTcThreads, tc_gemm_smem(), s>>>(j.x_tmaps + (size_t)wide * spd::kTensorMapBytes, wmap, j.y, N, C,
+                                                                           j.x_term_rows, j.st, 0);
       e = cudaGetLastError();
+      nz = 1;
+      zs = 0;
     }
     ++count;
   };
-  if (n <= spd::kTcM) {
-    // ... and the column-parallel row-wise kernels of a batched timestep (a block per 512 columns of a token row
-    // instead of one per row; RMSNorm's 1 / rms applied behind the product from per-chunk sums of squares).
-    e = spd_internal_job_input(job, j.ss, s);
+  auto done = [&](cudaError_t r) {  // a kernel enqueued
+    if (e == cudaSuccess) e = r;
     ++count;
-    for (int l = 0; l < j.L && e == cudaSuccess; ++l) {
-      gemm(xmap_d, 4 * l, 3 * d, d);
-      if (e != cudaSuccess) break;
-      e = spd_internal_job_rope_cache(job, j.ss, nz, zs, l, s);
-      if (e != cudaSuccess) break;
-      e = j.hd == 128 ? launch_attn<128>(j, l, n, s) : launch_attn<64>(j, l, n, s);
-      count += 2;
-      gemm(xmap_d, 4 * l + 1, d, d);
-      if (e != cudaSuccess) break;
-      e = spd_internal_job_resid(job, j.ss, nz, zs, j.layers[l].ffn_norm, s);
-      ++count;
-      gemm(xmap_d, 4 * l + 2, 2 * f, d);
-      if (e != cudaSuccess) break;
-      e = spd_internal_job_swiglu(job, j.ss, nz, zs, s);
-      ++count;
-      gemm(xmap_f, 4 * l + 3, d, f);
-      if (e != cudaSuccess) break;
-      if (l + 1 < j.L) {  // the last layer's output feeds nothing here
-        e = spd_internal_job_resid(job, j.ss, nz, zs, j.layers[l + 1].attn_norm, s);
-        ++count;
-      }
-    }
-    if (launches) *launches = count;
-    return e;
-  }
+  };
+  // Row-wise kernels of few rows: the column-parallel ones of a batched timestep (a block per 512 columns of a token row
+  // instead of one per row; RMSNorm's 1 / rms applied behind the product from per-chunk sums of squares).
   auto resid = [&](const float *y, const int32_t *ids, const __nv_bfloat16 *gain) {
     if (e != cudaSuccess) return;
-    e = spd::launch_dep(spd::spd_tc_resid_norm_kernel, dim3(n), dim3(256), 0, s, j.h, y, ids, j.tok_emb, gain, j.x, ts_d, d, j.eps, nz, zs);
-    ++count;
+    done(spd::launch_dep(spd::spd_tc_resid_norm_kernel, dim3(n), dim3(256), 0, s, j.h, y, ids, j.tok_emb, gain, j.x, ts_d, d, j.eps, nz, zs));
   };
-  resid(nullptr, j.ids, j.layers[0].attn_norm);
+  if (small) done(spd_internal_job_input(job, j.ss, s));
+  else resid(nullptr, j.ids, j.layers[0].attn_norm);
   for (int l = 0; l < j.L && e == cudaSuccess; ++l) {
-    gemm(xmap_d, 4 * l, 3 * d, d);
+    gemm(n, 0, 4 * l, 3 * d, d);
     if (e != cudaSuccess) break;
-    e = spd::launch_dep(spd::spd_tc_rope_cache_kernel, dim3(n), dim3(256), 0, s, j.y, j.q, j.kcache, j.vcache, j.rope, d, j.hd, j.max_pos, l, j.pos0,
-                        j.kv_bf16, nz, zs);
+    if (small) done(spd_internal_job_rope_cache(job, j.ss, nz, zs, l, s));
+    else
+      done(spd::launch_dep(spd::spd_tc_rope_cache_kernel, dim3(n), dim3(256), 0, s, j.y, j.q, j.kcache, j.vcache, j.rope, d, j.hd, j.max_pos, l,
+                           j.pos0, j.kv_bf16, nz, zs));
     if (e != cudaSuccess) break;
-    e = j.hd == 128 ? launch_attn<128>(j, l, n, s) : launch_attn<64>(j, l, n, s);  // other head sizes never get here
-    count += 2;
-    gemm(xmap_d, 4 * l + 1, d, d);
-    resid(j.y, nullptr, j.layers[l].ffn_norm);
-    gemm(xmap_d, 4 * l + 2, 2 * f, d);
+    const bool end = head && l + 1 == j.L;
+    spd::TcJob part = j;  // the rows that carry on
+    if (end) {
+      part.h += (size_t)(n - 1) * d;
+      part.q += (size_t)(n - 1) * d;
+      part.pos0 += n - 1;
+      part.n_tok = 1;
+    }
+    const bool few = small || end;
+    done(j.hd == 128 ? launch_attn<128>(part, l, part.n_tok, s) : launch_attn<64>(part, l, part.n_tok, s));  // other head sizes never get here
+    gemm(part.n_tok, 0, 4 * l + 1, d, d);
     if (e != cudaSuccess) break;
-    e = spd::launch_dep(spd::spd_tc_swiglu_kernel, dim3(n), dim3(256), 0, s, j.y, j.x, ts_f, f, nz, zs);
-    ++count;
-    gemm(xmap_f, 4 * l + 3, d, f);
-    if (l + 1 < j.L) resid(j.y, nullptr, j.layers[l + 1].attn_norm);  // the last layer's output feeds nothing here
+    if (few) done(spd_internal_job_resid(&part, j.ss, nz, zs, j.layers[l].ffn_norm, s));
+    else resid(j.y, nullptr, j.layers[l].ffn_norm);
+    gemm(part.n_tok, 0, 4 * l + 2, 2 * f, d);
+    if (e != cudaSuccess) break;
+    if (few) done(spd_internal_job_swiglu(&part, j.ss, nz, zs, s));
+    else done(spd::launch_dep(spd::spd_tc_swiglu_kernel, dim3(n), dim3(256), 0, s, j.y, j.x, ts_f, f, nz, zs));
+    gemm(part.n_tok, 1, 4 * l + 3, d, f);
+    if (e != cudaSuccess) break;
+    if (end) done(spd_internal_job_head(head, part.h, j.y, nz, zs, j.sm_count, s));
+    else if (l + 1 < j.L) {  // without a head the last layer's output feeds nothing
+      if (few) done(spd_internal_job_resid(&part, j.ss, nz, zs, j.layers[l + 1].attn_norm, s));
+      else resid(j.y, nullptr, j.layers[l + 1].attn_norm);
+    }
   }
   if (launches) *launches = count;
   return e;

@@ -6,8 +6,7 @@ namespace spd {
 
 constexpr int kTcTile = 128;      // tokens per tile of the tensor-core products
 constexpr int kTcMaxTokens = 512; // tokens one job takes at most
-constexpr int kTcMinPrefix = 32;  // runs of more tokens than this take the path: a job of up to 128 tokens costs about 1.5 launches
-                                  // of the 16-token kernel, so two launches before the last pay for it
+constexpr int kTcMinPrefix = 16;  // runs of more tokens than this take the path with every model, shorter ones with large models
 
 struct TcJob {
   int32_t L, d, H, hd, f, max_pos, kv_bf16;
@@ -65,12 +64,14 @@ inline cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_
 
 extern "C" cudaError_t spd_internal_tc_prepare(void);
 extern "C" cudaError_t spd_internal_tc_stall(const spd::TcJob *job, cudaStream_t stream);
-extern "C" cudaError_t spd_internal_tc_prefill(const spd::TcJob *job, cudaStream_t stream, int *launches);
+extern "C" cudaError_t spd_internal_tc_prefill(const spd::TcJob *job, const spd::KParams *head, cudaStream_t stream, int *launches);
 // Row-wise kernels of a job of up to 128 tokens (column-parallel, 1 / rms applied behind the product; spd_batch.cu).
 extern "C" cudaError_t spd_internal_job_input(const spd::TcJob *job, float *ss, cudaStream_t s);
 extern "C" cudaError_t spd_internal_job_rope_cache(const spd::TcJob *job, float *ss, int nz, size_t zs, int layer, cudaStream_t s);
 extern "C" cudaError_t spd_internal_job_resid(const spd::TcJob *job, float *ss, int nz, size_t zs, const __nv_bfloat16 *gain, cudaStream_t s);
 extern "C" cudaError_t spd_internal_job_swiglu(const spd::TcJob *job, float *ss, int nz, size_t zs, cudaStream_t s);
+// The end of a prefix: last residual add, final norm, LM head, KeepTopK and first timestep of one token row (h + the sum of y).
+extern "C" cudaError_t spd_internal_job_head(const spd::KParams *p, const float *h, const float *y, int nz, size_t zs, int sm_count, cudaStream_t s);
 // The product of a batched timestep's few token rows.  dep: launch it so that it may start while the kernel before it
 // in the stream still runs (it then copies weights only, until that kernel has completed).
 extern "C" cudaError_t spd_internal_batch_gemm(const uint8_t *xmaps, int wide, const void *wmap, float *Y, size_t y_floats, int n_tok, int N, int C,

@@ -1,0 +1,72 @@
+"""Prefixes that run wholly as jobs of the long-prefix path: the last job carries the last token's row through the last
+layer alone and ends with the launch that multiplies the LM head and takes the first timestep (Eq. 1).  Models whose
+layers hold 16 MB of matrices and more send runs of any length there, smaller ones runs of more than 16 tokens."""
+import numpy as np
+import pytest
+
+import spd_inputs as si
+from tests.gpu_common import compare_first_step, compare_step, make_pair, make_tiny_pair
+
+pytestmark = pytest.mark.gpu
+
+LAM = [0.3, 0.2] + [0.0] * 6
+
+
+@pytest.fixture(scope="module")
+def wide():
+    """25 MB of matrices per layer; a vocabulary that does not divide among the blocks or by the rows a warp takes."""
+    shape = si.ModelShape("wide", 2, 1024, 16, 2752, 1501)
+    return shape, si.make_weights(shape, seed=61), si.make_ngram_tables(shape.vocab, 1.1, 50_000, (2, 3), 5000, seed=62)
+
+
+def _pair(wide, max_pos, kv_dtype, k=3):
+    shape, weights, tables = wide
+    return make_pair(shape, weights, tables, k, (2, 3), LAM, 0.4, 0.2, 0.05, max_pos, kv_dtype)
+
+
+# one token; token boxes of 16, 32, 64 and 128 rows and their last rows; a second job (128 + 1, 128 + 16, 128 + 128);
+# 257 = one job on the 128-token tiles, 513 = a job of 512 and one of a single token
+@pytest.mark.parametrize("m,jobs", [(1, 1), (2, 1), (16, 1), (17, 1), (33, 1), (65, 1), (128, 1), (129, 2), (144, 2), (256, 2), (257, 1),
+                                    (513, 2)])
+def test_whole_prefix_as_jobs(wide, m, jobs):
+    ctx, orc = _pair(wide, 768, "bf16" if m % 2 else "f32", k=5)
+    prefix = si.make_prefix("zipf", m, wide[0].vocab, 1.1, seed=800 + m)
+    compare_first_step(ctx, orc, prefix)
+    assert ctx.spd_launch_count() == 9 * wide[0].n_layers * jobs + 1
+    for _ in range(2):
+        compare_step(ctx, orc)
+    # a restart (Section 5.3) runs the three generated tokens as a job behind the cached positions
+    compare_first_step(ctx, orc, None, reset_draft=2)
+    compare_step(ctx, orc)
+    ctx.close()
+
+
+def test_end_of_a_job_leaves_what_the_prefill_kernel_leaves(wide):
+    """Residual row and logits of the last token, drafts and weights: a context of 128 positions has no long-prefix
+    buffers and sends the same prefix through the 16-token kernel; so does a traced call."""
+    a, _ = _pair(wide, 128, "f32")
+    b, _ = _pair(wide, 256, "f32")
+    c, _ = _pair(wide, 256, "f32")
+    c.spd_debug_trace(True)
+    prefix = si.make_prefix("zipf", 30, wide[0].vocab, 1.1, seed=5)
+    got = [x.spd_prefill(prefix) for x in (a, b, c)]
+    # (traced: a job of 16 tokens without an end, then the 16-token kernel)
+    assert [x.spd_launch_count() for x in (a, b, c)] == [2, 9 * wide[0].n_layers + 1, 9 * wide[0].n_layers + 1]
+    for x, (ids, g) in zip((b, c), got[1:]):
+        assert ids.tolist() == got[0][0].tolist() and np.abs(g - got[0][1]).max() < 1e-3
+        for what in ("LOGITS", "HIDDEN"):
+            assert np.abs(x.spd_debug_read(what) - a.spd_debug_read(what)).max() < 1e-4
+    assert np.abs(c.spd_debug_read("TRACE")[-1, 1] - b.spd_debug_read("HIDDEN")).max() < 1e-4
+    for x in (a, b, c):
+        x.close()
+
+
+@pytest.mark.parametrize("m,launches", [(16, 1), (17, 19), (32, 19), (513, 9 * 2 + 1)])
+def test_small_model(tiny_inputs, m, launches):
+    """The tiny model's jobs begin at 17 tokens; the one token that a job of 512 leaves over goes through the 16-token kernel."""
+    wl, _, _, _ = tiny_inputs
+    ctx, orc = make_tiny_pair(tiny_inputs, max_pos=1024)
+    compare_first_step(ctx, orc, si.make_prefix("zipf", m, wl.shape.vocab, 1.1, seed=820 + m))
+    assert ctx.spd_launch_count() == launches
+    compare_step(ctx, orc)
+    ctx.close()
