@@ -209,75 +209,117 @@ __global__ void __launch_bounds__(256) spd_batch_swiglu_kernel(const float *Y, i
   bt_put3(X, term_stride, (size_t)t * f + j, g / (1.f + __expf(-g)) * up);
 }
 
-// One (request, head) per block of four warps: softmax attention of the request's query over its own cache, a warp
-// per position with an online softmax, the warps' states merged in shared memory; output as three bf16 terms.
-__global__ void __launch_bounds__(128) spd_batch_attn_kernel(const float *Q, const KParams *kps, uint16_t *X, size_t term_stride, int d,
-                                                             int hd, int layer) {
-  dep_wait();    // the kernel before this one in the stream wrote what this one reads
-  dep_launch();  // the next one may set itself up meanwhile
-  __shared__ float s_acc[4][256];
-  __shared__ float s_m[4], s_l[4];
-  const KParams &p = kps[blockIdx.x];
-  const int head = blockIdx.y, T = bt_pos(p) + 1;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int epl = hd / 32;  // elements per lane, <= 8
-  const float scale = 1.f / sqrtf((float)hd);
-  float q[8], acc[8];
+// One (request, head) per block of eight warps: softmax attention of the request's query over its own cache.  Bound by
+// the cache rows' latency and bytes, so a position is read with one 16-byte load per lane and cache: HD * sizeof(E) / 16
+// lanes hold a position (16 for bf16 of head size 128, two positions per warp side by side), and four positions per
+// group of lanes are in flight before the first is used; they enter the running softmax together (one rescale per round).
+// A round of the block is 32 (float32, head size 128) to 128 positions (bf16, 64).  The groups' states are merged in
+// shared memory in a fixed order; output as three bf16 terms.  7B shape, bf16 cache, whole timestep of 8 / 64 requests
+// behind 150 positions each: 4.58 / 7.99 ms (a warp per position, one in flight, element-wise loads), now 3.51 / 6.14 ms.
+constexpr int kBaWarps = 8, kBaFlight = 4;
+
+template <typename E>
+__device__ __forceinline__ void ba_unpack(const uint4 &v, float (&x)[16 / sizeof(E)]) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    q[e] = e < epl ? Q[(size_t)blockIdx.x * d + head * hd + lane * epl + e] : 0.f;
+  for (int e = 0; e < 4; ++e) {
+    if constexpr (sizeof(E) == 2) {
+      x[2 * e] = __uint_as_float(w[e] << 16);
+      x[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
+    } else {
+      x[e] = __uint_as_float(w[e]);
+    }
+  }
+}
+
+template <int HD, typename E>
+__device__ void ba_head(const float *q_row, const E *kc, const E *vc, int d, int T, uint16_t *X, size_t term_stride, size_t x_at, float *s_acc,
+                        float *s_m, float *s_l) {
+  constexpr int EPL = 16 / (int)sizeof(E);           // elements per lane
+  constexpr int LP = HD / EPL;                       // lanes per position
+  constexpr int GW = 32 / LP, G = GW * kBaWarps;     // groups of lanes per warp, per block
+  const int lane = threadIdx.x & 31, group = (threadIdx.x >> 5) * GW + lane / LP, at = (lane % LP) * EPL;
+  const float scale = 1.f / sqrtf((float)HD);
+  float q[EPL], acc[EPL];
+#pragma unroll
+  for (int e = 0; e < EPL; ++e) {
+    q[e] = q_row[at + e];
     acc[e] = 0.f;
   }
   float m = -CUDART_INF_F, l = 0.f;
-  for (int t = warp; t < T; t += 4) {
-    const size_t base = ((size_t)layer * p.max_pos + t) * d + head * hd + lane * epl;
-    float dot = 0.f, vv[8];
+  for (int tb = 0; tb < T; tb += G * kBaFlight) {  // all lanes of a warp go round together (the shuffles)
+    uint4 kq[kBaFlight], vq[kBaFlight];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      vv[e] = 0.f;
-      if (e < epl) {
-        float kx;
-        if (p.kv_bf16) {
-          kx = __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(p.kcache)[base + e]);
-          vv[e] = __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(p.vcache)[base + e]);
-        } else {
-          kx = reinterpret_cast<const float *>(p.kcache)[base + e];
-          vv[e] = reinterpret_cast<const float *>(p.vcache)[base + e];
-        }
-        dot = fmaf(q[e], kx, dot);
-      }
+    for (int u = 0; u < kBaFlight; ++u) kq[u] = *reinterpret_cast<const uint4 *>(kc + (size_t)min(tb + u * G + group, T - 1) * d + at);
+#pragma unroll
+    for (int u = 0; u < kBaFlight; ++u) vq[u] = *reinterpret_cast<const uint4 *>(vc + (size_t)min(tb + u * G + group, T - 1) * d + at);
+    float sc[kBaFlight], mn = m;
+#pragma unroll
+    for (int u = 0; u < kBaFlight; ++u) {
+      float kx[EPL], dot = 0.f;
+      ba_unpack<E>(kq[u], kx);
+#pragma unroll
+      for (int e = 0; e < EPL; ++e) dot = fmaf(q[e], kx[e], dot);
+#pragma unroll
+      for (int o = LP / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+      sc[u] = tb + u * G + group < T ? dot * scale : -CUDART_INF_F;
+      mn = fmaxf(mn, sc[u]);
     }
+    if (mn > -CUDART_INF_F) {  // else no position so far belongs to this group
+      const float c = __expf(m - mn);
+      l *= c;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-    const float s = dot * scale;
-    const float mn = fmaxf(m, s);
-    const float c = __expf(m - mn), pw = __expf(s - mn);
-    l = l * c + pw;
+      for (int e = 0; e < EPL; ++e) acc[e] *= c;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = acc[e] * c + pw * vv[e];
-    m = mn;
+      for (int u = 0; u < kBaFlight; ++u) {
+        const float pw = __expf(sc[u] - mn);  // 0 past the last position
+        float vx[EPL];
+        ba_unpack<E>(vq[u], vx);
+        l += pw;
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) acc[e] = fmaf(pw, vx[e], acc[e]);
+      }
+      m = mn;
+    }
   }
 #pragma unroll
-  for (int e = 0; e < 8; ++e)
-    if (e < epl) s_acc[warp][lane * epl + e] = acc[e];
-  if (lane == 0) {
-    s_m[warp] = m;
-    s_l[warp] = l;
+  for (int e = 0; e < EPL; ++e) s_acc[group * HD + at + e] = acc[e];
+  if (lane % LP == 0) {
+    s_m[group] = m;
+    s_l[group] = l;
   }
   __syncthreads();
-  for (int c = threadIdx.x; c < hd; c += 128) {
+  if (threadIdx.x < HD) {
     float M = -CUDART_INF_F;
 #pragma unroll
-    for (int w = 0; w < 4; ++w) M = fmaxf(M, s_m[w]);
+    for (int g = 0; g < G; ++g) M = fmaxf(M, s_m[g]);
     float L = 0.f, A = 0.f;
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      const float wgt = s_m[w] == -CUDART_INF_F ? 0.f : __expf(s_m[w] - M);
-      L = fmaf(s_l[w], wgt, L);
-      A = fmaf(s_acc[w][c], wgt, A);
+#pragma unroll 8
+    for (int g = 0; g < G; ++g) {
+      const float wgt = s_m[g] == -CUDART_INF_F ? 0.f : __expf(s_m[g] - M);
+      L = fmaf(s_l[g], wgt, L);
+      A = fmaf(s_acc[g * HD + threadIdx.x], wgt, A);
     }
-    bt_put3(X, term_stride, (size_t)blockIdx.x * d + head * hd + c, A / L);
+    bt_put3(X, term_stride, x_at + threadIdx.x, A / L);
   }
+}
+
+template <int HD>
+__global__ void __launch_bounds__(kBaWarps * 32) spd_batch_attn_kernel(const float *Q, const KParams *kps, uint16_t *X, size_t term_stride, int d,
+                                                                       int layer) {
+  dep_wait();    // the kernel before this one in the stream wrote what this one reads
+  dep_launch();  // the next one may set itself up meanwhile
+  constexpr int kGroups = kBaWarps * 32 / (HD / 8);  // bf16: the larger number of groups
+  __shared__ float s_acc[kGroups * HD], s_m[kGroups], s_l[kGroups];
+  const KParams &p = kps[blockIdx.x];
+  const int T = bt_pos(p) + 1;
+  const size_t x_at = (size_t)blockIdx.x * d + blockIdx.y * HD, base = (size_t)layer * p.max_pos * d + blockIdx.y * HD;
+  if (p.kv_bf16)
+    ba_head<HD>(Q + x_at, static_cast<const __nv_bfloat16 *>(p.kcache) + base, static_cast<const __nv_bfloat16 *>(p.vcache) + base, d, T, X,
+                term_stride, x_at, s_acc, s_m, s_l);
+  else
+    ba_head<HD>(Q + x_at, static_cast<const float *>(p.kcache) + base, static_cast<const float *>(p.vcache) + base, d, T, X, term_stride, x_at,
+                s_acc, s_m, s_l);
 }
 
 // One request per block (512 threads): the request's row of logits (the LM head's partial products added, times
@@ -465,7 +507,8 @@ extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd:
     if (e != cudaSuccess) break;
     e = spd::launch_dep(spd::spd_batch_rope_cache_kernel, dim3(n, (d / 2 + 255) / 256), dim3(256), 0, s, j.y, nz, zs, ss, j.eps, j.q, kps, d, j.hd, l);
     if (e != cudaSuccess) break;
-    e = spd::launch_dep(spd::spd_batch_attn_kernel, dim3(n, j.H), dim3(128), 0, s, j.q, kps, j.x, ts_d, d, j.hd, l);
+    e = j.hd == 128 ? spd::launch_dep(spd::spd_batch_attn_kernel<128>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l)
+                    : spd::launch_dep(spd::spd_batch_attn_kernel<64>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l);
     if (e != cudaSuccess) break;
     count += 2;
     gemm(xmap_d, 4 * l + 1, j.y, y_floats, d, d);

@@ -70,3 +70,29 @@ def test_small_model(tiny_inputs, m, launches):
     assert ctx.spd_launch_count() == launches
     compare_step(ctx, orc)
     ctx.close()
+
+
+@pytest.mark.parametrize("kv_dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("d,heads", [(256, 4), (256, 2)])
+def test_batched_attention_rounds(d, heads, kv_dtype):
+    """A batch's attention takes 32 (float32, head size 128) to 128 positions (bf16, 64) per round of a block: contexts of
+    one position, around one and two rounds, and their growth across a round's end, all in one batch."""
+    import paper_2405_18400_b200 as P
+    from oracle import spd_oracle as so
+
+    shape = si.ModelShape("hd%d" % (d // heads), 2, d, heads, 512, 1000)
+    weights = si.make_weights(shape, seed=71)
+    tables = sorted(si.make_ngram_tables(shape.vocab, 1.1, 50_000, (2, 3), 5000, seed=72), key=lambda t: int(t["n"]))
+    packed, dtabs = P.pack_weights(weights, "cuda:0"), P.build_ngram_tables(tables, "cuda:0")
+    reqs = []
+    for r, m in enumerate((1, 30, 31, 62, 63, 64, 126, 127, 128, 255, 257)):
+        ctx = P.SpdContext(shape, packed, dtabs, 3, (2, 3), LAM, 0.4, 0.2, 0.05, 300, kv_dtype)
+        orc = so.Oracle(so.make_config(shape, 3, (2, 3), LAM, 0.4, 0.2, 0.05, 300, kv_dtype), weights, tables)
+        compare_first_step(ctx, orc, si.make_prefix("zipf", m, shape.vocab, 1.1, seed=840 + r))
+        reqs.append((ctx, orc))
+    for _ in range(3):
+        for (ctx, orc), got in zip(reqs, P.spd_batch_step([c for c, _ in reqs])):
+            compare_step(ctx, orc, None, stepped=got, path="prefill")
+    for ctx, orc in reqs:
+        ctx.close()
+        orc.close()
