@@ -18,8 +18,7 @@ extern "C" cudaError_t spd_internal_prefill_prepare(int *blocks_per_sm);
 extern "C" cudaError_t spd_internal_prefill_launch(const spd::KParams *p, int grid, cudaStream_t stream);
 extern "C" cudaError_t spd_internal_pack_image(const void *w, void *out, int rows, int cols, cudaStream_t stream);
 extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd::KParams *kps, int n, int V, const __nv_bfloat16 *final_norm,
-                                               float *y_logits, size_t y_floats, size_t y_logits_floats, float *ss, int32_t *results,
-                                               int sm_count, cudaStream_t s, int *launches);
+                                               float *y_logits, int32_t *results, cudaStream_t s, int *launches);
 
 namespace {
 
@@ -43,7 +42,7 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct Layout {
   size_t kcache, vcache, rope, layers, h, q, u, logits, opart, oml, pk_val, pk_id, pk_ms, state, hist_tok, hist_par, prefix,
-      trace, ns_u, pf_tmaps, pf_h, pf_q, pf_ss, pf_part, pf_ml, pf_cnt, pf_xh, pf_xo, pf_xu, tc_tmaps, tc_h, tc_q, tc_y, tc_x, bt_kp, bt_y,
+      trace, ns_u, pf_tmaps, pf_h, pf_q, pf_ss, pf_part, pf_ml, pf_cnt, pf_xh, pf_xo, pf_xu, tc_tmaps, tc_h, tc_q, tc_y, tc_parts, tc_x, bt_kp, bt_y,
       bt_ss, bt_out, total;
 };
 
@@ -116,15 +115,16 @@ Layout make_layout(const spd_config &c, int grid) {
   L.pf_xu = take(frag_bytes(c.d_ffn));
   const size_t tcr = (size_t)tc_rows(c);
   const size_t wide = (size_t)(3 * c.d_model > 2 * c.d_ffn ? 3 * c.d_model : 2 * c.d_ffn);
-  L.tc_tmaps = take(8 * sizeof(CUtensorMap));  // term buffer as [..][d] and [..][f] in boxes of 128, 16, 32 and 64 rows
+  L.tc_tmaps = take(8 * sizeof(CUtensorMap));  // term buffer as [..][d] and [..][f] in boxes of 8, 16, 32 and 64 rows
   L.tc_h = take(tcr * c.d_model * 4);
   L.tc_q = take(tcr * c.d_model * 4);
   L.tc_y = take(tcr * wide * 4);
+  L.tc_parts = take((size_t)spd::kTcMaxPairs * (tcr < spd::kTcMaxTileTok ? tcr : spd::kTcMaxTileTok) * 256 * 4);
   L.tc_x = take(3 * tcr * (size_t)(c.d_model > c.d_ffn ? c.d_model : c.d_ffn) * 2);
   // batched timesteps led by this context: the requests' parameters and their rows of logits
   L.bt_kp = take(tcr ? (size_t)spd::kTcTile * sizeof(spd::KParams) : 0);
   L.bt_y = take(tcr ? (size_t)spd::kTcTile * c.vocab * 4 : 0);
-  L.bt_ss = take(tcr ? (size_t)spd::kTcTile * 32 * 4 : 0);  // per request and 512-column chunk: sums of squares of the residual row
+  L.bt_ss = take(tcr * 32 * 4);  // per token row and 512-column chunk: sums of squares of the residual row
   L.bt_out = take(tcr ? (size_t)spd::kTcTile * spd::kBtResultWords * 4 : 0);  // per request: a timestep's results
   L.total = off;
   return L;
@@ -265,7 +265,7 @@ spd::TcJob tc_job(spd_ctx *ctx) {
   job.x_term_rows = ctx->tc_rows;
   job.st = kp.st;
   job.sm_count = ctx->grid;
-  job.y_floats = (size_t)ctx->tc_rows * (size_t)(3 * kp.d > 2 * kp.f ? 3 * kp.d : 2 * kp.f);
+  job.parts = reinterpret_cast<float *>(ctx->ws + ctx->lay.tc_parts);
   job.ss = reinterpret_cast<float *>(ctx->ws + ctx->lay.bt_ss);
   job.ids = nullptr;
   job.pos0 = job.n_tok = 0;
@@ -295,11 +295,7 @@ int prefill_tokens(spd_ctx *ctx, int first, int count) {
     SPD_CUDA(cudaMemsetAsync(ctx->ws + ctx->lay.state, 0, head_bytes(false), ctx->stream));
     spd::TcJob job = tc_job(ctx);
     while (tc_done < jobs_end && (kp.trace || count - tc_done > min_job)) {
-      const int left = jobs_end - tc_done;
-      int n = left < ctx->tc_rows ? left : ctx->tc_rows;
-      // Up to two token tiles of a large model go one by one: each pass over the weights costs less than the second
-      // tile's share of the 128-token tiles' products, which need more tiles to fill the chip (7B shape, 256 tokens).
-      if (left > spd::kTcTile && left <= 2 * spd::kTcTile && large_layers(kp)) n = spd::kTcTile;
+      const int n = jobs_end - tc_done < ctx->tc_rows ? jobs_end - tc_done : ctx->tc_rows;
       job.ids = base + first + tc_done;
       job.pos0 = first + tc_done;
       job.n_tok = n;
@@ -439,6 +435,7 @@ int spd_create(const spd_config *cfg, const spd_weights *w, const spd_ngram_tabl
   ctx->tc_rows = tc_rows(*cfg);
   if (ctx->tc_rows > 0) {
     e = spd_internal_tc_prepare();
+    if (e == cudaSuccess) e = spd_internal_job_prepare();
     if (e != cudaSuccess) return fail(cuda_fail(e, "long-prefix kernel attributes"));
   }
 
@@ -529,7 +526,7 @@ int spd_create(const spd_config *cfg, const spd_weights *w, const spd_ngram_tabl
     ok = ok && weight_map(encode, w->lm_head, cfg->vocab, d, &tmaps[(size_t)4 * cfg->n_layers]);
     if (ok && ctx->tc_rows > 0)
       for (int i = 0; i < 4 && ok; ++i) {
-        const int box_rows = i == 0 ? spd::kTcTile : 8 << i;  // 128, then 16, 32, 64 for the products of a small batch
+        const int box_rows = 8 << i;  // half the rows of a token tile of the products, at most 64
         ok = term_map(encode, ws + lay.tc_x, 3 * ctx->tc_rows, d, box_rows, &xmaps[2 * i]) &&
              term_map(encode, ws + lay.tc_x, 3 * ctx->tc_rows, f, box_rows, &xmaps[2 * i + 1]);
       }
@@ -822,11 +819,8 @@ int batch_enqueue(spd_ctx *const *ctxs, int32_t n, int32_t n_steps) {
   const spd::TcJob job = tc_job(lead);
   for (int s = 0; s < n_steps; ++s) {
     int launched = 0;
-    const int wide = 3 * c0.d_model > 2 * c0.d_ffn ? 3 * c0.d_model : 2 * c0.d_ffn;
-    const cudaError_t e = spd_internal_batch_step(&job, dkp, n, c0.vocab, lead->kp.final_norm,
-                                                  reinterpret_cast<float *>(lead->ws + lead->lay.bt_y), (size_t)lead->tc_rows * wide,
-                                                  (size_t)spd::kTcTile * c0.vocab, reinterpret_cast<float *>(lead->ws + lead->lay.bt_ss),
-                                                  reinterpret_cast<int32_t *>(lead->ws + lead->lay.bt_out), lead->grid, lead->stream, &launched);
+    const cudaError_t e = spd_internal_batch_step(&job, dkp, n, c0.vocab, lead->kp.final_norm, reinterpret_cast<float *>(lead->ws + lead->lay.bt_y),
+                                                  reinterpret_cast<int32_t *>(lead->ws + lead->lay.bt_out), lead->stream, &launched);
     lead->launches += launched;
     if (e != cudaSuccess) return cuda_fail(e, "batched timestep");
   }

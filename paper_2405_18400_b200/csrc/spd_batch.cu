@@ -23,40 +23,77 @@
 namespace spd {
 
 // v = hi + mid + lo exactly: each term takes the leading 8 significant bits of what is left, by truncation.
-__device__ __forceinline__ void bt_put3(uint16_t *X, size_t term_stride, size_t at, float v) {
-  const uint32_t hi = __float_as_uint(v) & 0xffff0000u;
-  const float r1 = v - __uint_as_float(hi);
-  const uint32_t mid = __float_as_uint(r1) & 0xffff0000u;
-  const float r2 = r1 - __uint_as_float(mid);
-  X[at] = (uint16_t)(hi >> 16);
-  X[at + term_stride] = (uint16_t)(mid >> 16);
-  X[at + 2 * term_stride] = (uint16_t)(__float_as_uint(r2) >> 16);
+__device__ __forceinline__ void bt_split3(float v, uint32_t &hi, uint32_t &mid, uint32_t &lo) {
+  hi = __float_as_uint(v) >> 16;
+  const float r1 = v - __uint_as_float(hi << 16);
+  mid = __float_as_uint(r1) >> 16;
+  lo = __float_as_uint(r1 - __uint_as_float(mid << 16)) >> 16;
 }
+__device__ __forceinline__ void bt_put3(uint16_t *X, size_t term_stride, size_t at, float v) {
+  uint32_t hi, mid, lo;
+  bt_split3(v, hi, mid, lo);
+  X[at] = (uint16_t)hi;
+  X[at + term_stride] = (uint16_t)mid;
+  X[at + 2 * term_stride] = (uint16_t)lo;
+}
+// Four neighbouring columns (at and term_stride multiples of 4).
+__device__ __forceinline__ void bt_put3x4(uint16_t *X, size_t term_stride, size_t at, const float4 &v) {
+  uint32_t h[4], m[4], l[4];
+  bt_split3(v.x, h[0], m[0], l[0]);
+  bt_split3(v.y, h[1], m[1], l[1]);
+  bt_split3(v.z, h[2], m[2], l[2]);
+  bt_split3(v.w, h[3], m[3], l[3]);
+  *reinterpret_cast<uint2 *>(X + at) = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
+  *reinterpret_cast<uint2 *>(X + at + term_stride) = make_uint2(m[0] | (m[1] << 16), m[2] | (m[3] << 16));
+  *reinterpret_cast<uint2 *>(X + at + 2 * term_stride) = make_uint2(l[0] | (l[1] << 16), l[2] | (l[3] << 16));
+}
+// Four neighbouring bf16 values (8-byte aligned).
+__device__ __forceinline__ float4 bt_load4(const __nv_bfloat16 *p) {
+  const uint2 w = *reinterpret_cast<const uint2 *>(p);
+  return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
+}
+__device__ __forceinline__ float4 bt_mul(const float4 &a, const float4 &b) { return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w); }
 
-// A batch has few token rows, so the row-wise work between the products is spread over the columns: a block takes
-// kBtCols columns of one request's row.  RMSNorm's factor 1 / rms(h) is common to a row's columns and moves behind
-// the product (as in the single-request kernel): the kernels that write a residual row h store h * gain as the next
-// product's terms and the sum of squares of their columns (ss[request][chunk]); the kernels that read that product
-// multiply its rows by rsqrt(sum of the row's chunks / d + eps).
-constexpr int kBtCols = 512;      // columns per block: two per thread
+// The row-wise work between the products, of a batch's requests or a short job's tokens, is spread over rows and columns: a
+// block takes kBtCols columns of one token row, a thread four neighbouring ones (16-byte loads; with two columns a
+// thread and 2-byte stores of the terms the SwiGLU of 100 tokens, 7B shape, took 14 us, now 8).  RMSNorm's factor 1 / rms(h)
+// is common to a row's columns and moves behind the product (as in the single-request kernel): the kernels that write a
+// residual row h store h * gain as the next product's terms and the sum of squares of their columns (ss[row][chunk]);
+// the kernels that read that product multiply its rows by rsqrt(sum of the row's chunks / d + eps).
+constexpr int kBtCols = 512;
+constexpr int kBtThreads = kBtCols / 4;
 constexpr int kBtMaxChunks = 32;  // d_model <= 16384
 static_assert(8 + 3 * kMaxK <= kBtResultWords, "a request's row of results holds the head and three lists of k");
 
-__device__ __forceinline__ float bt_block_sum(float v, float *scratch) {
+// A chunk of a residual row: stored, its terms times the gain, its sum of squares.  All threads of the block.
+__device__ __forceinline__ void bt_store_row(float *h, const __nv_bfloat16 *gain, uint16_t *X, size_t term_stride, int row, int d, int c,
+                                             const float4 &v, float *ss) {
+  __shared__ float scratch[kBtThreads / 32];
+  float sq = 0.f;
+  if (c < d) {
+    const size_t at = (size_t)row * d + c;
+    *reinterpret_cast<float4 *>(h + at) = v;
+    sq = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, v.w * v.w)));
+    bt_put3x4(X, term_stride, at, bt_mul(v, bt_load4(gain + c)));
+  }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
+  for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+  if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = sq;
   __syncthreads();
-  float s = 0.f;
+  if (threadIdx.x == 0) {
+    float s = 0.f;
 #pragma unroll
-  for (int w = 0; w < 8; ++w) s += scratch[w];
-  return s;
+    for (int w = 0; w < kBtThreads / 32; ++w) s += scratch[w];
+    ss[row * kBtMaxChunks + blockIdx.y] = s;
+  }
 }
 
-__device__ __forceinline__ float bt_rs(const float *ss, int request, int d, float eps) {
+// (ss null: the product's terms were whole RMSNorms)
+__device__ __forceinline__ float bt_rs(const float *ss, int row, int d, float eps) {
+  if (!ss) return 1.f;
   const int nch = (d + kBtCols - 1) / kBtCols;
   float s = 0.f;
-  for (int c = 0; c < nch; ++c) s += ss[request * kBtMaxChunks + c];
+  for (int c = 0; c < nch; ++c) s += ss[row * kBtMaxChunks + c];
   return rsqrtf(s / (float)d + eps);
 }
 
@@ -66,147 +103,156 @@ __device__ __forceinline__ int bt_pos(const KParams &p) { return p.pos0 + p.st->
 
 // grid (requests, column chunks): the superposed input of Eq. 3, h = sum_i gamma_i E[last token of draft i], stored as
 // the request's residual row; h * gain of the first layer's norm as three bf16 terms; the chunk's sum of squares.
-__global__ void __launch_bounds__(256) spd_batch_input_kernel(const KParams *kps, float *h, const __nv_bfloat16 *gain, uint16_t *X,
-                                                              size_t term_stride, int d, float *ss) {
-  dep_wait();    // the kernel before this one in the stream wrote what this one reads
-  dep_launch();  // the next one may set itself up meanwhile
-  __shared__ float scratch[8];
+__global__ void __launch_bounds__(kBtThreads) spd_batch_input_kernel(const KParams *kps, float *h, const __nv_bfloat16 *gain, uint16_t *X,
+                                                                     size_t term_stride, int d, float *ss) {
+  dep_launch();
+  dep_wait();
   const KParams &p = kps[blockIdx.x];
   const State *st = p.st;
-  float sq = 0.f;
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const int c = blockIdx.y * kBtCols + e * 256 + threadIdx.x;
-    if (c < d) {
-      float acc = 0.f;
-      for (int i = 0; i < p.k; ++i) acc = fmaf(st->gamma[i], __bfloat162float(p.tok_emb[(size_t)st->win[i][kWin - 1] * d + c]), acc);
-      h[(size_t)blockIdx.x * d + c] = acc;
-      sq = fmaf(acc, acc, sq);
-      bt_put3(X, term_stride, (size_t)blockIdx.x * d + c, acc * __bfloat162float(gain[c]));
+  const int c = blockIdx.y * kBtCols + threadIdx.x * 4;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (c < d)
+    for (int i = 0; i < p.k; ++i) {
+      const float g = st->gamma[i];
+      const float4 e = bt_load4(p.tok_emb + (size_t)st->win[i][kWin - 1] * d + c);
+      acc.x = fmaf(g, e.x, acc.x);
+      acc.y = fmaf(g, e.y, acc.y);
+      acc.z = fmaf(g, e.z, acc.z);
+      acc.w = fmaf(g, e.w, acc.w);
     }
-  }
-  sq = bt_block_sum(sq, scratch);
-  if (threadIdx.x == 0) ss[blockIdx.x * kBtMaxChunks + blockIdx.y] = sq;
+  bt_store_row(h, gain, X, term_stride, blockIdx.x, d, c, acc, ss);
 }
 
-// grid (requests, column chunks): residual add h += y (y = the sum of nz partial products zs floats apart), h * gain
-// of the next norm as terms, the chunk's sum of squares.
-__global__ void __launch_bounds__(256) spd_batch_resid_kernel(float *h, const float *y, int nz, size_t zs, const __nv_bfloat16 *gain, uint16_t *X,
-                                                              size_t term_stride, int d, float *ss) {
-  dep_wait();    // the kernel before this one in the stream wrote what this one reads
-  dep_launch();  // the next one may set itself up meanwhile
+// grid (tokens, column chunks): a job's residual rows start as its tokens' embeddings.
+__global__ void __launch_bounds__(kBtThreads) spd_job_input_kernel(const int32_t *ids, const __nv_bfloat16 *tok_emb, float *h,
+                                                                   const __nv_bfloat16 *gain, uint16_t *X, size_t term_stride, int d, float *ss) {
+  dep_launch();
+  dep_wait();
+  const int c = blockIdx.y * kBtCols + threadIdx.x * 4;
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (c < d) v = bt_load4(tok_emb + (size_t)ids[blockIdx.x] * d + c);
+  bt_store_row(h, gain, X, term_stride, blockIdx.x, d, c, v, ss);
+}
+
+// grid (rows, column chunks): residual add h += y, h * gain of the next norm as terms, the chunk's sum of squares.
+__global__ void __launch_bounds__(kBtThreads) spd_batch_resid_kernel(float *h, const __grid_constant__ Product y, const __nv_bfloat16 *gain,
+                                                                     uint16_t *X, size_t term_stride, int d, float *ss) {
+  dep_launch();
+  dep_wait();
+  const int c = blockIdx.y * kBtCols + threadIdx.x * 4;
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (c < d) {
+    v = *reinterpret_cast<const float4 *>(h + (size_t)blockIdx.x * d + c);
+    const float4 a = product_sum4(y, blockIdx.x, c);
+    v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
+  }
+  bt_store_row(h, gain, X, term_stride, blockIdx.x, d, c, v, ss);
+}
+
+// Long jobs (more than 128 tokens): a token row per block, the whole RMSNorm before the product.  With hundreds of rows
+// the chip is full either way; the norm stays in front of the product there so that the tensor cores see the same operands,
+// and truncate the same way, as they always have for these lengths (a bf16 cache turns a difference in the sixth digit into
+// another rounding of one value in a hundred).  The row waits in shared memory between the sum of squares, taken a column
+// per thread, and the terms, four columns per thread (8-byte stores).
+__global__ void __launch_bounds__(256) spd_job_norm_kernel(float *h, const __grid_constant__ Product y, const int32_t *ids, const __nv_bfloat16 *emb,
+                                                           const __nv_bfloat16 *gain, uint16_t *X, size_t term_stride, int d, float eps) {
+  dep_launch();
+  dep_wait();
+  extern __shared__ __align__(16) float jn_row[];  // [d]
   __shared__ float scratch[8];
-  float sq = 0.f;
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const int c = blockIdx.y * kBtCols + e * 256 + threadIdx.x;
-    if (c < d) {
-      const size_t at = (size_t)blockIdx.x * d + c;
-      float v = h[at];
-      for (int z = 0; z < nz; ++z) v += y[z * zs + at];
-      h[at] = v;
-      sq = fmaf(v, v, sq);
-      bt_put3(X, term_stride, at, v * __bfloat162float(gain[c]));
+  const int t = blockIdx.x;
+  float *hr = h + (size_t)t * d;
+  for (int c = threadIdx.x * 4; c < d; c += 1024) {
+    float4 v;
+    if (ids) v = bt_load4(emb + (size_t)ids[t] * d + c);
+    else {
+      v = *reinterpret_cast<const float4 *>(hr + c);
+      const float4 a = product_sum4(y, t, c);
+      v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
     }
+    *reinterpret_cast<float4 *>(hr + c) = v;
+    *reinterpret_cast<float4 *>(jn_row + c) = v;
   }
-  sq = bt_block_sum(sq, scratch);
-  if (threadIdx.x == 0) ss[blockIdx.x * kBtMaxChunks + blockIdx.y] = sq;
+  __syncthreads();
+  float ss = 0.f;
+  for (int c = threadIdx.x; c < d; c += 256) ss = fmaf(jn_row[c], jn_row[c], ss);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  float sum = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) sum += scratch[w];
+  const float rs = rsqrtf(sum / (float)d + eps);
+  for (int c = threadIdx.x * 4; c < d; c += 1024) {
+    const float4 v = *reinterpret_cast<const float4 *>(jn_row + c);
+    bt_put3x4(X, term_stride, (size_t)t * d + c, bt_mul(make_float4(v.x * rs, v.y * rs, v.z * rs, v.w * rs), bt_load4(gain + c)));
+  }
 }
 
-// One column pair of one token row: the QKV product's row (the sum of its nz partial sums) times 1 / rms, rotary
-// embedding of q and k (adjacent pairs) at position pos, q to Q, k and v into the cache.  Y row = [q | k | v].
-__device__ __forceinline__ void bt_rope_cache_pair(const float *Y, int nz, size_t zs, float rs, float *Q, void *kcache, void *vcache,
-                                                   const float2 *rope, int max_pos, int kv_bf16, int d, int hd, int layer, int t, int pos,
-                                                   int i) {
-  const float *yr = Y + (size_t)t * 3 * d;
-  const size_t crow = ((size_t)layer * max_pos + pos) * d;
-  const float2 cs = rope[(size_t)pos * (hd / 2) + (i % (hd / 2))];
-  float2 qq = make_float2(0.f, 0.f), kk = qq, vv = qq;
-  for (int z = 0; z < nz; ++z) {  // the product's partial sums over column ranges, in order
-    const float *yz = yr + z * zs;
-    qq.x += yz[2 * i]; qq.y += yz[2 * i + 1];
-    kk.x += yz[d + 2 * i]; kk.y += yz[d + 2 * i + 1];
-    vv.x += yz[2 * d + 2 * i]; vv.y += yz[2 * d + 2 * i + 1];
-  }
-  const float qe = qq.x * rs, qo = qq.y * rs, ke = kk.x * rs, ko = kk.y * rs;
-  Q[(size_t)t * d + 2 * i] = qe * cs.x - qo * cs.y;
-  Q[(size_t)t * d + 2 * i + 1] = qe * cs.y + qo * cs.x;
-  const float k0 = ke * cs.x - ko * cs.y, k1 = ke * cs.y + ko * cs.x;
-  const float v0 = vv.x * rs, v1 = vv.y * rs;
+// Columns c .. c+3 of one token row: the QKV product's row [q | k | v] times 1 / rms, rotary embedding of q and k
+// (adjacent pairs) at position pos, q to Q, k and v into the cache.
+__device__ __forceinline__ float4 bt_rotate(const float4 &x, const float4 &cs) {  // cs = (cos, sin) of the two pairs
+  return make_float4(x.x * cs.x - x.y * cs.y, x.x * cs.y + x.y * cs.x, x.z * cs.z - x.w * cs.w, x.z * cs.w + x.w * cs.z);
+}
+__device__ __forceinline__ void bt_store_kv(void *cache, int kv_bf16, size_t at, const float4 &v) {
   if (kv_bf16) {
-    reinterpret_cast<__nv_bfloat162 *>(kcache)[(crow >> 1) + i] = __halves2bfloat162(__float2bfloat16_rn(k0), __float2bfloat16_rn(k1));
-    reinterpret_cast<__nv_bfloat162 *>(vcache)[(crow >> 1) + i] = __halves2bfloat162(__float2bfloat16_rn(v0), __float2bfloat16_rn(v1));
+    const __nv_bfloat162 a = __halves2bfloat162(__float2bfloat16_rn(v.x), __float2bfloat16_rn(v.y));
+    const __nv_bfloat162 b = __halves2bfloat162(__float2bfloat16_rn(v.z), __float2bfloat16_rn(v.w));
+    *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(cache) + at) =
+        make_uint2(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b));
   } else {
-    reinterpret_cast<float2 *>(kcache)[(crow >> 1) + i] = make_float2(k0, k1);
-    reinterpret_cast<float2 *>(vcache)[(crow >> 1) + i] = make_float2(v0, v1);
+    *reinterpret_cast<float4 *>(static_cast<float *>(cache) + at) = v;
   }
 }
+__device__ __forceinline__ void bt_rope_cache(const Product &y, float rs, float *Q, void *kcache, void *vcache, const float2 *rope, int max_pos,
+                                              int kv_bf16, int d, int hd, int layer, int t, int pos, int c) {
+  const float4 q = product_sum4(y, t, c), k = product_sum4(y, t, d + c), v = product_sum4(y, t, 2 * d + c);
+  const float4 cs = *reinterpret_cast<const float4 *>(rope + (size_t)pos * (hd / 2) + (c % hd) / 2);
+  const size_t at = ((size_t)layer * max_pos + pos) * d + c;
+  *reinterpret_cast<float4 *>(Q + (size_t)t * d + c) = bt_rotate(make_float4(q.x * rs, q.y * rs, q.z * rs, q.w * rs), cs);
+  bt_store_kv(kcache, kv_bf16, at, bt_rotate(make_float4(k.x * rs, k.y * rs, k.z * rs, k.w * rs), cs));
+  bt_store_kv(vcache, kv_bf16, at, make_float4(v.x * rs, v.y * rs, v.z * rs, v.w * rs));
+}
 
-// grid (requests, chunks of 256 column pairs): each request at its own position, into its own cache.
-__global__ void __launch_bounds__(256) spd_batch_rope_cache_kernel(const float *Y, int nz, size_t zs, const float *ss, float eps, float *Q,
-                                                                   const KParams *kps, int d, int hd, int layer) {
-  dep_wait();    // the kernel before this one in the stream wrote what this one reads
-  dep_launch();  // the next one may set itself up meanwhile
+// grid (requests, column chunks): each request at its own position, into its own cache.
+__global__ void __launch_bounds__(kBtThreads) spd_batch_rope_cache_kernel(const __grid_constant__ Product y, const float *ss, float eps, float *Q,
+                                                                          const KParams *kps, int d, int hd, int layer) {
+  dep_wait();
+  dep_launch();
   const KParams &p = kps[blockIdx.x];
-  const int i = blockIdx.y * 256 + threadIdx.x;  // column pair
-  if (i >= d / 2) return;
-  bt_rope_cache_pair(Y, nz, zs, bt_rs(ss, blockIdx.x, d, eps), Q, p.kcache, p.vcache, p.rope, p.max_pos, p.kv_bf16, d, hd, layer, blockIdx.x,
-                     bt_pos(p), i);
+  const int c = blockIdx.y * kBtCols + threadIdx.x * 4;
+  if (c >= d) return;
+  bt_rope_cache(y, bt_rs(ss, blockIdx.x, d, eps), Q, p.kcache, p.vcache, p.rope, p.max_pos, p.kv_bf16, d, hd, layer, blockIdx.x, bt_pos(p), c);
 }
 
 // The same for a job of prefix tokens of one request (token t at position pos0 + t, one cache).
-__global__ void __launch_bounds__(256) spd_job_rope_cache_kernel(const float *Y, int nz, size_t zs, const float *ss, float eps, float *Q,
-                                                                 void *kcache, void *vcache, const float2 *rope, int max_pos, int kv_bf16, int d,
-                                                                 int hd, int layer, int pos0) {
+__global__ void __launch_bounds__(kBtThreads) spd_job_rope_cache_kernel(const __grid_constant__ Product y, const float *ss, float eps, float *Q,
+                                                                        void *kcache, void *vcache, const float2 *rope, int max_pos, int kv_bf16,
+                                                                        int d, int hd, int layer, int pos0) {
   dep_wait();
   dep_launch();
-  const int i = blockIdx.y * 256 + threadIdx.x;
-  if (i >= d / 2) return;
-  bt_rope_cache_pair(Y, nz, zs, bt_rs(ss, blockIdx.x, d, eps), Q, kcache, vcache, rope, max_pos, kv_bf16, d, hd, layer, blockIdx.x,
-                     pos0 + blockIdx.x, i);
+  const int c = blockIdx.y * kBtCols + threadIdx.x * 4;
+  if (c >= d) return;
+  bt_rope_cache(y, bt_rs(ss, blockIdx.x, d, eps), Q, kcache, vcache, rope, max_pos, kv_bf16, d, hd, layer, blockIdx.x, pos0 + blockIdx.x, c);
 }
 
-// grid (tokens, column chunks): a job's residual rows start as its tokens' embeddings; h * gain of the first layer's
-// norm as three bf16 terms; the chunk's sum of squares.
-__global__ void __launch_bounds__(256) spd_job_input_kernel(const int32_t *ids, const __nv_bfloat16 *tok_emb, float *h, const __nv_bfloat16 *gain,
-                                                            uint16_t *X, size_t term_stride, int d, float *ss) {
-  dep_wait();
-  dep_launch();
-  __shared__ float scratch[8];
-  const __nv_bfloat16 *row = tok_emb + (size_t)ids[blockIdx.x] * d;
-  float sq = 0.f;
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const int c = blockIdx.y * kBtCols + e * 256 + threadIdx.x;
-    if (c < d) {
-      const float v = __bfloat162float(row[c]);
-      h[(size_t)blockIdx.x * d + c] = v;
-      sq = fmaf(v, v, sq);
-      bt_put3(X, term_stride, (size_t)blockIdx.x * d + c, v * __bfloat162float(gain[c]));
-    }
-  }
-  sq = bt_block_sum(sq, scratch);
-  if (threadIdx.x == 0) ss[blockIdx.x * kBtMaxChunks + blockIdx.y] = sq;
-}
-
-// grid (requests, chunks of 256 rows of the FFN): u = SiLU(gate) * up from the gate / up product's row times 1 / rms
+// grid (rows, chunks of the FFN): u = SiLU(gate) * up from the gate / up product's row times 1 / rms
 // (Y row = [gate_0, up_0, gate_1, up_1, ...]), as three bf16 terms.
-__global__ void __launch_bounds__(256) spd_batch_swiglu_kernel(const float *Y, int nz, size_t zs, const float *ss, float eps, int d, uint16_t *X,
-                                                               size_t term_stride, int f) {
-  dep_wait();    // the kernel before this one in the stream wrote what this one reads
-  dep_launch();  // the next one may set itself up meanwhile
-  const int t = blockIdx.x, j = blockIdx.y * 256 + threadIdx.x;
+__device__ __forceinline__ float bt_swiglu(float gate, float up, float rs) {
+  const float g = gate * rs, u = up * rs;
+  return g / (1.f + __expf(-g)) * u;
+}
+__global__ void __launch_bounds__(kBtThreads) spd_batch_swiglu_kernel(const __grid_constant__ Product y, const float *ss, float eps, int d, uint16_t *X,
+                                                                      size_t term_stride, int f) {
+  dep_launch();
+  dep_wait();
+  const int t = blockIdx.x, j = blockIdx.y * kBtCols + threadIdx.x * 4;
   if (j >= f) return;
   const float rs = bt_rs(ss, t, d, eps);
-  const float2 *yr = reinterpret_cast<const float2 *>(Y + (size_t)t * 2 * f);
-  float2 gu = make_float2(0.f, 0.f);
-  for (int z = 0; z < nz; ++z) {
-    const float2 more = yr[z * (zs / 2) + j];
-    gu.x += more.x;
-    gu.y += more.y;
-  }
-  const float g = gu.x * rs, up = gu.y * rs;
-  bt_put3(X, term_stride, (size_t)t * f + j, g / (1.f + __expf(-g)) * up);
+  const float4 a = product_sum4(y, t, 2 * j), b = product_sum4(y, t, 2 * j + 4);
+  bt_put3x4(X, term_stride, (size_t)t * f + j,
+            make_float4(bt_swiglu(a.x, a.y, rs), bt_swiglu(a.z, a.w, rs), bt_swiglu(b.x, b.y, rs), bt_swiglu(b.z, b.w, rs)));
 }
 
 // One (request, head) per block of eight warps: softmax attention of the request's query over its own cache.  Bound by
@@ -307,8 +353,8 @@ __device__ void ba_head(const float *q_row, const E *kc, const E *vc, int d, int
 template <int HD>
 __global__ void __launch_bounds__(kBaWarps * 32) spd_batch_attn_kernel(const float *Q, const KParams *kps, uint16_t *X, size_t term_stride, int d,
                                                                        int layer) {
-  dep_wait();    // the kernel before this one in the stream wrote what this one reads
-  dep_launch();  // the next one may set itself up meanwhile
+  dep_launch();
+  dep_wait();
   constexpr int kGroups = kBaWarps * 32 / (HD / 8);  // bf16: the larger number of groups
   __shared__ float s_acc[kGroups * HD], s_m[kGroups], s_l[kGroups];
   const KParams &p = kps[blockIdx.x];
@@ -326,19 +372,32 @@ __global__ void __launch_bounds__(kBaWarps * 32) spd_batch_attn_kernel(const flo
 // 1 / rms of the final norm) goes to its own buffer; every warp ranks a sixteenth of the vocabulary, warp 0 merges
 // the sixteen lists (KeepTopK with log-probabilities under temperature tau, Algorithm 1); then Eq. 5-7, Eq. 2 and
 // Eq. 4 on the request's own draft state, as block 0 of the single-request kernel does.
-__global__ void __launch_bounds__(kConsumerThreads) spd_batch_tail_kernel(const KParams *kps, const float *Y, int nz, size_t zs, const float *ss,
+__global__ void __launch_bounds__(kConsumerThreads) spd_batch_tail_kernel(const KParams *kps, const __grid_constant__ Product y, const float *ss,
                                                                           float eps, int V, int32_t *results) {
-  dep_wait();    // the kernel before this one in the stream wrote what this one reads
-  dep_launch();  // the next one may set itself up meanwhile
+  dep_wait();
+  dep_launch();
   extern __shared__ __align__(16) uint8_t bt_smem[];
   __shared__ int s_dead, s_quit;
   const KParams &p = kps[blockIdx.x];
   const float rs = bt_rs(ss, blockIdx.x, p.d, eps);
-  const float *row = Y + (size_t)blockIdx.x * V;
-  for (int c = threadIdx.x; c < V; c += kConsumerThreads) {
-    float z = row[c];
-    for (int i = 1; i < nz; ++i) z += row[i * zs + c];
-    p.logits[c] = z * rs;
+  const float *row = y.y + (size_t)blockIdx.x * V;
+  // a warp takes row tiles of the product (256 logits, alike in their parts) in turn
+  for (int rt = threadIdx.x >> 5; rt * 256 < V; rt += kConsumerWarps) {
+    const TileParts tp = product_parts(y, blockIdx.x, rt);
+    float z[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int c = rt * 256 + e * 32 + (threadIdx.x & 31);
+      z[e] = c < V ? row[c] : 0.f;
+    }
+    for (int q = tp.first; q < tp.last; ++q)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) z[e] += y.parts[q * tp.step + tp.at + e * 32 + (threadIdx.x & 31)];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int c = rt * 256 + e * 32 + (threadIdx.x & 31);
+      if (c < V) p.logits[c] = z[e] * rs;
+    }
   }
   if (threadIdx.x == 0) s_dead = s_quit = 0;
   __syncthreads();
@@ -386,10 +445,10 @@ __global__ void __launch_bounds__(kConsumerThreads) spd_batch_tail_kernel(const 
 // [V][d] weights is a stream of the weights (262 MB at 7B shape, 40 us at the copy bandwidth), so a block per SM takes a
 // contiguous range of the vocabulary and a warp four of its rows at a time (4 rows x 16 bytes per lane in flight, each
 // eight activations read from shared memory serve four rows), float32 multiplies; every block computes the norm itself
-// from L2 (nz + 1 rows of d floats).  The block that arrives last merges the blocks' top-k lists and takes the step.
+// from L2.  The block that arrives last merges the blocks' top-k lists and takes the step.
 constexpr int kHeadRows = 4;
-__global__ void __launch_bounds__(kConsumerThreads) spd_job_head_kernel(const __grid_constant__ KParams p, const float *h, const float *y, int nz,
-                                                                        size_t zs) {
+__global__ void __launch_bounds__(kConsumerThreads) spd_job_head_kernel(const __grid_constant__ KParams p, const float *h,
+                                                                        const __grid_constant__ Product y) {
   extern __shared__ __align__(16) float jh_x[];  // [d]: residual row times the final norm's gain
   __shared__ float s_sum[kConsumerWarps];
   __shared__ int s_last;
@@ -402,12 +461,13 @@ __global__ void __launch_bounds__(kConsumerThreads) spd_job_head_kernel(const __
   }
   dep_wait();
   float sq = 0.f;
-  for (int c = threadIdx.x; c < p.d; c += kConsumerThreads) {
-    float v = h[c];
-    for (int z = 0; z < nz; ++z) v += y[z * zs + c];
-    sq = fmaf(v, v, sq);
-    jh_x[c] = v * __bfloat162float(p.final_norm[c]);
-    if (blockIdx.x == 0) p.h[c] = v;
+  for (int c = threadIdx.x * 4; c < p.d; c += kConsumerThreads * 4) {
+    float4 v = *reinterpret_cast<const float4 *>(h + c);
+    const float4 a = product_sum4(y, 0, c);
+    v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
+    sq = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, sq))));
+    *reinterpret_cast<float4 *>(jh_x + c) = bt_mul(v, bt_load4(p.final_norm + c));
+    if (blockIdx.x == 0) *reinterpret_cast<float4 *>(p.h + c) = v;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
@@ -473,95 +533,82 @@ constexpr size_t kBatchTailSmem = 20480;
 }
 
 // Enqueues one batched timestep of n requests (kps: their parameters in device memory, in row order) on stream s.
-// job: the buffers of the context that lends its long-prefix workspace (h, y, q, x, tensor maps); y_logits: [128][V]
-// floats; lm_tmap: the LM head's tensor map.  *launches receives the number of kernels enqueued.
+// job: the buffers of the context that lends its long-prefix workspace; y_logits: [128][V] floats.  *launches receives
+// the number of kernels enqueued.
 extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd::KParams *kps, int n, int V, const __nv_bfloat16 *final_norm,
-                                               float *y_logits, size_t y_floats, size_t y_logits_floats, float *ss, int32_t *results,
-                                               int sm_count, cudaStream_t s, int *launches) {
+                                               float *y_logits, int32_t *results, cudaStream_t s, int *launches) {
   const spd::TcJob &j = *job;
   const int d = j.d, f = j.f;
   const size_t ts_d = (size_t)j.x_term_rows * d, ts_f = (size_t)j.x_term_rows * f;
-  const uint8_t *xmap_d = j.x_tmaps, *xmap_f = j.x_tmaps + spd::kTensorMapBytes;
+  const int nch = (d + spd::kBtCols - 1) / spd::kBtCols, nch_f = (f + spd::kBtCols - 1) / spd::kBtCols;
+  const dim3 threads(spd::kBtThreads);
   int count = 0;
   cudaError_t e = cudaSuccess;
-  // The product built for few token rows (weights as the wide operand, columns split among blocks): its output is nz
-  // partial sums zs floats apart.
-  int nz = 1;
-  size_t zs = 0;
-  auto gemm = [&](const uint8_t *xmap, int which, float *Y, size_t room, int N, int C) {
-    if (e != cudaSuccess) return;
-    const uint8_t *wmap = j.w_tmaps + (size_t)which * spd::kTensorMapBytes;
-    e = spd_internal_batch_gemm(j.x_tmaps, xmap != xmap_d, wmap, Y, room, n, N, C, j.x_term_rows, j.st, sm_count, s, 1, &nz, &zs);
+  spd::Product pr;  // where the last product's sums are
+  auto done = [&](cudaError_t r) {  // a kernel enqueued
+    e = r;
     ++count;
   };
-  const int nch = (d + spd::kBtCols - 1) / spd::kBtCols;
+  auto product = [&](int wide, int which, float *Y, int N) {
+    if (e == cudaSuccess) done(spd_internal_product(job, n, wide, which, Y, N, &pr, s));
+  };
   auto resid = [&](const __nv_bfloat16 *gain) {
-    if (e != cudaSuccess) return;
-    e = spd::launch_dep(spd::spd_batch_resid_kernel, dim3(n, nch), dim3(256), 0, s, j.h, j.y, nz, zs, gain, j.x, ts_d, d, ss);
-    ++count;
+    if (e == cudaSuccess) done(spd::launch_dep(spd::spd_batch_resid_kernel, dim3(n, nch), threads, 0, s, j.h, pr, gain, j.x, ts_d, d, j.ss));
   };
-  e = spd::launch_dep(spd::spd_batch_input_kernel, dim3(n, nch), dim3(256), 0, s, kps, j.h, j.layers[0].attn_norm, j.x, ts_d, d, ss);
-  ++count;
+  done(spd::launch_dep(spd::spd_batch_input_kernel, dim3(n, nch), threads, 0, s, kps, j.h, j.layers[0].attn_norm, j.x, ts_d, d, j.ss));
   for (int l = 0; l < j.L && e == cudaSuccess; ++l) {
-    gemm(xmap_d, 4 * l, j.y, y_floats, 3 * d, d);
-    if (e != cudaSuccess) break;
-    e = spd::launch_dep(spd::spd_batch_rope_cache_kernel, dim3(n, (d / 2 + 255) / 256), dim3(256), 0, s, j.y, nz, zs, ss, j.eps, j.q, kps, d, j.hd, l);
-    if (e != cudaSuccess) break;
-    e = j.hd == 128 ? spd::launch_dep(spd::spd_batch_attn_kernel<128>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l)
-                    : spd::launch_dep(spd::spd_batch_attn_kernel<64>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l);
-    if (e != cudaSuccess) break;
-    count += 2;
-    gemm(xmap_d, 4 * l + 1, j.y, y_floats, d, d);
+    product(0, 4 * l, j.y, 3 * d);
+    if (e == cudaSuccess)
+      done(spd::launch_dep(spd::spd_batch_rope_cache_kernel, dim3(n, nch), threads, 0, s, pr, j.ss, j.eps, j.q, kps, d, j.hd, l));
+    if (e == cudaSuccess)
+      done(j.hd == 128 ? spd::launch_dep(spd::spd_batch_attn_kernel<128>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l)
+                       : spd::launch_dep(spd::spd_batch_attn_kernel<64>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l));
+    product(0, 4 * l + 1, j.y, d);
     resid(j.layers[l].ffn_norm);
-    gemm(xmap_d, 4 * l + 2, j.y, y_floats, 2 * f, d);
-    if (e != cudaSuccess) break;
-    e = spd::launch_dep(spd::spd_batch_swiglu_kernel, dim3(n, (f + 255) / 256), dim3(256), 0, s, j.y, nz, zs, ss, j.eps, d, j.x, ts_f, f);
-    ++count;
-    gemm(xmap_f, 4 * l + 3, j.y, y_floats, d, f);
+    product(0, 4 * l + 2, j.y, 2 * f);
+    if (e == cudaSuccess) done(spd::launch_dep(spd::spd_batch_swiglu_kernel, dim3(n, nch_f), threads, 0, s, pr, j.ss, j.eps, d, j.x, ts_f, f));
+    product(1, 4 * l + 3, j.y, d);
     resid(l + 1 < j.L ? j.layers[l + 1].attn_norm : final_norm);
   }
-  gemm(xmap_d, 4 * j.L, y_logits, y_logits_floats, V, d);
-  if (e == cudaSuccess) {
-    e = spd::launch_dep(spd::spd_batch_tail_kernel, dim3(n), dim3(spd::kConsumerThreads), kBatchTailSmem, s, kps, y_logits, nz, zs, ss, j.eps, V, results);
-    ++count;
-  }
+  product(0, 4 * j.L, y_logits, V);
+  if (e == cudaSuccess)
+    done(spd::launch_dep(spd::spd_batch_tail_kernel, dim3(n), dim3(spd::kConsumerThreads), kBatchTailSmem, s, kps, pr, j.ss, j.eps, V, results));
   if (launches) *launches = count;
   return e;
 }
 
-// The row-wise kernels of a job of up to 128 prefix tokens of one request (the long-prefix path's small jobs): the same
-// column-parallel kernels as a batched timestep's, token t at position job.pos0 + t.  ss: [128][32] floats.
-extern "C" cudaError_t spd_internal_job_input(const spd::TcJob *job, float *ss, cudaStream_t s) {
+// The row-wise kernels of a job of prefix tokens of one request (the long-prefix path), token t at position job.pos0 + t.
+extern "C" cudaError_t spd_internal_job_resid(const spd::TcJob *job, const spd::Product *y, const __nv_bfloat16 *gain, cudaStream_t s) {
   const spd::TcJob &j = *job;
-  return spd::launch_dep(spd::spd_job_input_kernel, dim3(j.n_tok, (j.d + spd::kBtCols - 1) / spd::kBtCols), dim3(256), 0, s, j.ids, j.tok_emb, j.h,
-                         j.layers[0].attn_norm, j.x, (size_t)j.x_term_rows * j.d, j.d, ss);
+  const dim3 grid(j.n_tok, (j.d + spd::kBtCols - 1) / spd::kBtCols);
+  const size_t ts = (size_t)j.x_term_rows * j.d;
+  if (!y) return spd::launch_dep(spd::spd_job_input_kernel, grid, dim3(spd::kBtThreads), 0, s, j.ids, j.tok_emb, j.h, gain, j.x, ts, j.d, j.ss);
+  return spd::launch_dep(spd::spd_batch_resid_kernel, grid, dim3(spd::kBtThreads), 0, s, j.h, *y, gain, j.x, ts, j.d, j.ss);
 }
-extern "C" cudaError_t spd_internal_job_rope_cache(const spd::TcJob *job, float *ss, int nz, size_t zs, int layer, cudaStream_t s) {
+extern "C" cudaError_t spd_internal_job_norm(const spd::TcJob *job, const spd::Product *y, const __nv_bfloat16 *gain, cudaStream_t s) {
   const spd::TcJob &j = *job;
-  return spd::launch_dep(spd::spd_job_rope_cache_kernel, dim3(j.n_tok, (j.d / 2 + 255) / 256), dim3(256), 0, s, j.y, nz, zs, ss, j.eps, j.q, j.kcache,
-                         j.vcache, j.rope, j.max_pos, j.kv_bf16, j.d, j.hd, layer, j.pos0);
+  const spd::Product none = {};
+  return spd::launch_dep(spd::spd_job_norm_kernel, dim3(j.n_tok), dim3(256), (size_t)j.d * 4, s, j.h, y ? *y : none, y ? nullptr : j.ids, j.tok_emb, gain,
+                         j.x, (size_t)j.x_term_rows * j.d, j.d, j.eps);
 }
-extern "C" cudaError_t spd_internal_job_resid(const spd::TcJob *job, float *ss, int nz, size_t zs, const __nv_bfloat16 *gain, cudaStream_t s) {
+extern "C" cudaError_t spd_internal_job_rope_cache(const spd::TcJob *job, const spd::Product *y, int normed, int layer, cudaStream_t s) {
   const spd::TcJob &j = *job;
-  return spd::launch_dep(spd::spd_batch_resid_kernel, dim3(j.n_tok, (j.d + spd::kBtCols - 1) / spd::kBtCols), dim3(256), 0, s, j.h, j.y, nz, zs, gain,
-                         j.x, (size_t)j.x_term_rows * j.d, j.d, ss);
+  return spd::launch_dep(spd::spd_job_rope_cache_kernel, dim3(j.n_tok, (j.d + spd::kBtCols - 1) / spd::kBtCols), dim3(spd::kBtThreads), 0, s, *y,
+                         normed ? nullptr : j.ss, j.eps, j.q, j.kcache, j.vcache, j.rope, j.max_pos, j.kv_bf16, j.d, j.hd, layer, j.pos0);
 }
-extern "C" cudaError_t spd_internal_job_swiglu(const spd::TcJob *job, float *ss, int nz, size_t zs, cudaStream_t s) {
+extern "C" cudaError_t spd_internal_job_swiglu(const spd::TcJob *job, const spd::Product *y, int normed, cudaStream_t s) {
   const spd::TcJob &j = *job;
-  return spd::launch_dep(spd::spd_batch_swiglu_kernel, dim3(j.n_tok, (j.f + 255) / 256), dim3(256), 0, s, j.y, nz, zs, ss, j.eps, j.d, j.x,
-                         (size_t)j.x_term_rows * j.f, j.f);
+  return spd::launch_dep(spd::spd_batch_swiglu_kernel, dim3(j.n_tok, (j.f + spd::kBtCols - 1) / spd::kBtCols), dim3(spd::kBtThreads), 0, s, *y,
+                         normed ? nullptr : j.ss, j.eps, j.d, j.x, (size_t)j.x_term_rows * j.f, j.f);
 }
 
-extern "C" cudaError_t spd_internal_job_head(const spd::KParams *p, const float *h, const float *y, int nz, size_t zs, int sm_count, cudaStream_t s) {
-  // at most 64 KB of activations (d_model <= 16384); the attribute is per device and set on its first launch
-  static bool ready[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+extern "C" cudaError_t spd_internal_job_head(const spd::KParams *p, const float *h, const spd::Product *y, int sm_count, cudaStream_t s) {
+  return spd::launch_dep(spd::spd_job_head_kernel, dim3(sm_count), dim3(spd::kConsumerThreads), (size_t)p->d * 4, s, *p, h, *y);
+}
+
+// Kernel attributes of the current device: a row of up to 16384 float32 values in shared memory.
+extern "C" cudaError_t spd_internal_job_prepare(void) {
+  const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_job_norm_kernel), cudaFuncAttributeMaxDynamicSharedMemorySize, 65536);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64 || !ready[dev]) {
-    e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_job_head_kernel), cudaFuncAttributeMaxDynamicSharedMemorySize, 65536);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) ready[dev] = true;
-  }
-  return spd::launch_dep(spd::spd_job_head_kernel, dim3(sm_count), dim3(spd::kConsumerThreads), (size_t)p->d * 4, s, *p, h, y, nz, zs);
+  return cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_job_head_kernel), cudaFuncAttributeMaxDynamicSharedMemorySize, 65536);
 }

@@ -7,13 +7,8 @@
 //
 // Product: Y[token][row] = sum_c X[token][c] W[row][c], W bf16 [rows][cols] as stored, X float32 activations
 // split exactly into three bf16 terms (x = hi + mid + lo, 8 + 8 + 8 significant bits), so that the tensor
-// cores see exact operands and the float32 accumulator receives what a float32 product would.  One block
-// computes a tile of 128 tokens x 128 rows: a producer thread fills a ring of stages (three term tiles of
-// 128 tokens x 64 columns and one weight tile of 128 rows x 64 columns, all in the 128-byte-swizzled K-major
-// layout the tensor cores read), one thread issues the 12 instructions of a stage (3 terms x 4 k-steps of 16
-// columns) and hands the stage back with tcgen05.commit; four accumulators take turns, each the sum of 8 stages,
-// and four warps add those sums in registers (round-to-nearest) and write the tile to global memory.  Every wait is bounded; a wait that runs out records SPD_ETIMEOUT in the
-// context's state, the block waits for its copies in flight, frees its tensor memory and returns.
+// cores see exact operands and the float32 accumulator receives what a float32 product would.  One persistent kernel
+// for every number of token rows (a batch of requests, a short prefix, a job of 512 tokens): see spd_tc_product_kernel.
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
@@ -23,35 +18,18 @@
 
 namespace spd {
 
-constexpr int kTcM = 128;                      // tokens of a tile = lanes of tensor memory
-constexpr int kTcN = 128;                      // weight rows of a tile = float32 columns of tensor memory
+constexpr int kTcRows = 128;                   // weight rows of a tile in one block = lanes of tensor memory
 constexpr int kTcKB = 64;                      // columns per stage: one 128-byte swizzle row of bf16
-constexpr int kTcTermBytes = kTcM * kTcKB * 2; // one term tile
-constexpr int kTcWBytes = kTcN * kTcKB * 2;
-constexpr int kTcStageBytes = 3 * kTcTermBytes + kTcWBytes;  // 64 KB
-constexpr int kTcStages = 3;
-constexpr int kTcThreads = 192;                // producer warp, issuing warp, four warps for the accumulator
+constexpr int kTcWBytes = kTcRows * kTcKB * 2;
+constexpr int kTcThreads = 320;                // producer warp, issuing warp, eight warps for the accumulator
+constexpr int kTcMaxStages = 10;
 constexpr int kTcWBoxRows = 32;                // the weights' tensor maps describe boxes of 32 rows x 64 columns
-constexpr int kTcSegSteps = 8;                 // stages summed inside tensor memory before the sum moves to registers
-constexpr int kTcAccs = 4;                     // accumulators in rotation: 4 x 128 columns = all of tensor memory
+constexpr int kTcMaxAccs = 4;                   // accumulator sets in rotation
 constexpr unsigned long long kTcWaitNs = 1500ull * 1000ull * 1000ull;
 
 // ---------------------------------------------------------------- PTX: tensor memory and tcgen05
-__device__ __forceinline__ void tc_box_load(uint32_t dst, const void *tmap, int x, int y, uint64_t *bar) {
-  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-               "l"(tmap), "r"(x), "r"(y), "r"(smem_u32(bar))
-               : "memory");
-}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// Whole warp: allocates `cols` columns (a power of two >= 32) of tensor memory, base address into *slot (shared).
-__device__ __forceinline__ void tc_alloc(uint32_t *slot, uint32_t cols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(cols) : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tc_dealloc(uint32_t base, uint32_t cols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols) : "memory");
-}
 // Shared-memory operand descriptor: K-major tile whose rows are 128 bytes (64 bf16) in the 128-byte swizzle,
 // groups of 8 rows 1024 bytes apart.
 __device__ __forceinline__ uint64_t tc_desc(uint32_t saddr) {
@@ -66,58 +44,84 @@ __device__ __forceinline__ uint64_t tc_desc(uint32_t saddr) {
 __device__ __forceinline__ constexpr uint32_t tc_idesc(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-__device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
-      : "memory");
+// 8 or 16 consecutive float32 columns of this thread's lane of tensor memory (tc_ld_wait before their use).
+__device__ __forceinline__ void tc_ld(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
 }
-// The mbarrier receives one arrival once every tcgen05.mma issued so far by this thread has completed.
-__device__ __forceinline__ void tc_commit(uint64_t *bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// 32 consecutive float32 columns of this thread's lane of tensor memory.
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-        "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// 16 consecutive float32 columns of this thread's lane of tensor memory.
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+__device__ __forceinline__ void tc_ld(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
         "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tc_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// ---- block pairs (cta_group::2): the two blocks of a cluster multiply one tile of 256 rows; the even one ("leader") issues.
+// One thread of a converged warp.  The compiler knows that it is one, which `lane == 0` does not say: tensor and copy
+// instructions take their operands from the warp's uniform registers, and with `lane == 0` around them a stage of four
+// instructions and seven copies cost the issuing threads about twice the cycles (QKV product of 15 tokens, 7B shape: 25.7 us
+// against 22.7).
+__device__ __forceinline__ bool tc_elect() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ uint32_t tc_cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// Address, in the cluster's shared-memory window, of the leader's object at this block's address.
+__device__ __forceinline__ uint32_t tc_leader_addr(const void *p) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(smem_u32(p)));
+  return r;
+}
+__device__ __forceinline__ void tc_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// A copy into this block's shared memory whose bytes are counted on the leader's barrier (`bar` from tc_leader_addr).
+__device__ __forceinline__ void tc_pair_box_load(uint32_t dst, const void *tmap, int x, int y, uint32_t bar) {
+  asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+               "l"(tmap), "r"(x), "r"(y), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void tc_pair_alloc(uint32_t *slot, uint32_t cols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(cols) : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tc_pair_dealloc(uint32_t base, uint32_t cols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols) : "memory");
+}
+__device__ __forceinline__ void tc_pair_mma(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// The mbarrier at this address in both blocks receives one arrival once every mma issued so far by this thread has completed.
+__device__ __forceinline__ void tc_pair_commit(uint64_t *bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),
+               "h"((uint16_t)3)
+               : "memory");
+}
+__device__ __forceinline__ void tc_cluster_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 struct TcShared {
-  uint64_t full[kTcStages], empty[kTcStages], acc_full[kTcAccs], acc_empty[kTcAccs];
-  uint32_t tmem_base;
-  int dead;
-};
-
-// The same for the small-batch product, whose ring has up to kBgMaxStages stages.
-constexpr int kBgMaxStages = 8;
-struct BgShared {
-  uint64_t full[kBgMaxStages], empty[kBgMaxStages], acc_full[kTcAccs], acc_empty[kTcAccs];
+  uint64_t full[kTcMaxStages], empty[kTcMaxStages], acc_full[kTcMaxAccs], acc_empty[kTcMaxAccs];
   uint32_t tmem_base;
   int dead;
 };
 
 // Bounded wait on an mbarrier phase; false when the block gave up (here or elsewhere).
-template <typename Shared>
-__device__ __forceinline__ bool tc_wait(Shared &sh, State *st, uint64_t *bar, uint32_t parity, int info) {
+__device__ __forceinline__ bool tc_wait(TcShared &sh, State *st, uint64_t *bar, uint32_t parity, int info) {
   if (mbar_try_wait(bar, parity)) return true;
   volatile int *dead = &sh.dead;
   unsigned long long t0 = globaltimer();
@@ -135,188 +139,73 @@ __device__ __forceinline__ bool tc_wait(Shared &sh, State *st, uint64_t *bar, ui
   return true;
 }
 
-// Y[m0 .. m0+127][n0 .. n0+127] of Y = X W^T.  tmap_x: the term tiles, a [3 * x_term_rows][C] bf16 matrix in boxes
-// of 128 rows x 64 columns (term j's tokens start at row j * x_term_rows); tmap_w: W [N][C] in boxes of 32 rows x
-// 64 columns.  Rows and columns past either matrix arrive as zeros.  grid = (ceil(tokens / 128), ceil(N / 128)).
-// stall (test hook): the producer announces its first stage but issues no copies for it, so the wait for that
-// stage runs out.
-__global__ void __launch_bounds__(kTcThreads, 1)
-    spd_tc_gemm_kernel(const void *tmap_x, const void *tmap_w, float *Y, int N, int C, int x_term_rows, State *st, int stall) {
+// Y = X W^T for up to 512 token rows, by one pair of blocks per two SMs that stay for the whole product.
+//
+// Tile: 256 weight rows (tcgen05.mma.cta_group::2, M = 256, 128 rows in each block's shared and tensor memory) x the token
+// rows of a tile.  The weights are the wide operand whatever the number of tokens, the terms the narrow one:
+//   F = 16, 32, 64 (up to that many token rows): the three term tiles lie behind one another, so one instruction of
+//     N = 3 x rows per 16 columns multiplies all three (N = 64 for 16 rows: a multiple of 32 is wanted; the 16 columns
+//     left over hold nothing that is read); each term has its own accumulator columns, added in the epilogue's registers.
+//   128, 256 (that many rows at most, N = the tile's rows rounded up to 32): one instruction per term and 16 columns, all
+//     into the same columns.
+// Each block brings its 128 weight rows and half of the tile's tokens.
+//
+// What bounds it: with up to about 64 tokens the weight stream; beyond, the tensor pipe (N = 128: 89 cycles an
+// instruction of 64, N = 256: 136 of 128, measured with the copies left out), whose operands come from shared memory.
+// Work is dealt in stages (64 columns of one tile): the product's stages, tile by tile and in a tile column by column, are
+// cut into as many equal runs as there are pairs, so no pair idles in a last wave; a pair's ring of stages and its
+// accumulators run on across tiles, so that a tile's epilogue overlaps the next one's stages.  A tile that the cuts divide
+// is summed by the reader: the part with the tile's first column is written to Y, a later part to its pair's own buffer (a
+// pair has at most one: the start of its run).
+// Measured (7B shape, gate / up product, ncu): 512 tokens 172 us = 1.61 PFLOP/s counting the three terms, 0.97 of the bf16
+// burst peak (128 x 128 tiles of single blocks: 250 us); 100 tokens 57 us; 15 tokens 34.5 us where the bytes need 27.6 (the
+// four products of a layer 91 us for 62; about 8 us of each are start and end, which the dependent launches hide in part).
+// Tried: asking the weights behind the first ring into L2 before dep_wait (8 to 32 stages): 2 to 5 % slower.
+//
+// Accumulation: an accumulator takes the sums of a segment of stages (96 additions), then moves to registers, where the
+// segments are added with round-to-nearest: the tensor cores add into their accumulator with truncation, whose error grows
+// with the length of the chain.
+//
+// tmap_x: the term tiles, a [3 * x_term_rows][C] bf16 matrix in boxes of kBoxRows rows x 64 columns (term j's tokens start
+// at row j * x_term_rows); tmap_w: W [N][C] in boxes of 32 rows x 64 columns; rows and columns past either matrix arrive as
+// zeros.  Barriers: a stage's copies by both blocks are counted on the leader's `full`; a commit signals `empty` and
+// `acc_full` in both blocks; the epilogue warps of both arrive at the leader's `acc_empty`.  Every wait is bounded.
+// Launched as a programmatic dependent: a block is set up and copies the weights of its whole first ring while the kernel
+// before it still runs; the terms, which that kernel writes, are asked for after dep_wait.
+// stall (test hook): the leader announces its first stage but no copies are issued for it, so the wait for it runs out.
+template <int NT>
+struct TcShape {
+  static constexpr bool kFused = NT <= 64;
+  static constexpr int kTermRows = NT / 2;                              // token rows that a block brings per term
+  static constexpr int kBoxRows = kTermRows < 64 ? kTermRows : 64;
+  static constexpr int kTermBytes = kTermRows * kTcKB * 2;
+  static constexpr int kCols = kFused ? (NT == 16 ? 64 : 3 * NT) : NT;  // accumulator columns (not fused: at most)
+  static constexpr int kCopyBytes = kTcWBytes + 3 * kTermBytes;
+  static constexpr int kStageBytes = NT == 16 ? kTcWBytes + 4096 : kCopyBytes;  // 16 rows: room for the 32 rows that N = 64 reads
+  static constexpr int kStages = NT == 16 ? 10 : (NT == 32 ? 9 : (NT == 64 ? 7 : (NT == 128 ? 5 : 3)));  // 192 - 200 KB
+  static constexpr int kAccs = NT == 64 || NT == 256 ? 2 : 4;
+  static constexpr int kAccStride = 512 / kAccs;                        // columns from one accumulator set to the next
+  static constexpr int kSegSteps = kFused ? 24 : 8;
+  static constexpr int kHalf = NT / 2;                                  // tokens whose sums one epilogue thread holds
+  static constexpr int kLd = kFused && NT == 16 ? 8 : 16;               // columns per tensor-memory load
+  static constexpr size_t kSmem = (size_t)kStages * kStageBytes + 1024;
+  static_assert(kStages <= kTcMaxStages && kAccs <= kTcMaxAccs && kCols <= kAccStride && kSmem <= 227 * 1024, "ring, accumulators and barriers fit");
+};
+
+template <int NT>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
+    spd_tc_product_kernel(const void *tmap_x, const void *tmap_w, float *Y, float *parts, const __grid_constant__ Product pr, int n_tok,
+                          int x_term_rows, State *st, int stall) {
+  using S = TcShape<NT>;
   extern __shared__ __align__(16) uint8_t tc_smem_raw[];
   uint8_t *smem = tc_smem_raw + ((1024u - (smem_u32(tc_smem_raw) & 1023u)) & 1023u);
   __shared__ TcShared sh;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nk = (C + kTcKB - 1) / kTcKB;
-  const int m0 = blockIdx.x * kTcM, n0 = blockIdx.y * kTcN;  // token tiles vary fastest: blocks that share weight rows run together
-  if (threadIdx.x == 0) {
-    sh.dead = 0;
-    for (int s = 0; s < kTcStages; ++s) {
-      mbar_init(&sh.full[s], 1);
-      mbar_init(&sh.empty[s], 1);
-    }
-    for (int a = 0; a < kTcAccs; ++a) {
-      mbar_init(&sh.acc_full[a], 1);
-      mbar_init(&sh.acc_empty[a], 4);  // one arrival per warp that reads the accumulator
-    }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) tc_alloc(&sh.tmem_base, kTcAccs * kTcN);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = sh.tmem_base;
-  const uint32_t ring = smem_u32(smem);
-
-  if (warp == 0) {
-    if (lane == 0) {
-      // producer: the activations were written by ordinary stores of earlier kernels on the stream
-      uint32_t stage = 0, phase = 0, issued = 0;
-      bool ok = true;
-      for (int ks = 0; ks < nk; ++ks) {
-        if (!tc_wait(sh, st, &sh.empty[stage], phase ^ 1u, 400)) { ok = false; break; }
-        mbar_expect_tx(&sh.full[stage], (uint32_t)kTcStageBytes);
-        const uint32_t base = ring + stage * (uint32_t)kTcStageBytes;
-        if (stall && ks == 0) {
-          if (++stage == (uint32_t)kTcStages) { stage = 0; phase ^= 1u; }
-          continue;  // nothing in flight for this stage
-        }
-#pragma unroll
-        for (int j = 0; j < 3; ++j) tc_box_load(base + j * kTcTermBytes, tmap_x, ks * kTcKB, j * x_term_rows + m0, &sh.full[stage]);
-#pragma unroll
-        for (int j = 0; j < kTcN / kTcWBoxRows; ++j)
-          tc_box_load(base + 3 * kTcTermBytes + j * (kTcWBoxRows * kTcKB * 2), tmap_w, ks * kTcKB, n0 + j * kTcWBoxRows, &sh.full[stage]);
-        if (issued < (uint32_t)kTcStages) ++issued;
-        if (++stage == (uint32_t)kTcStages) { stage = 0; phase ^= 1u; }
-      }
-      if (!ok) {
-        // giving up: wait (bounded) for the copies already issued, so that none lands after the block has gone
-        uint32_t s = stage, ph = phase;
-        for (uint32_t i = 0; i < issued; ++i) {
-          if (s == 0) { s = (uint32_t)kTcStages; ph ^= 1u; }
-          --s;
-          unsigned long long t0 = globaltimer();
-          while (!mbar_try_wait(&sh.full[s], ph) && globaltimer() - t0 < kTcWaitNs) {}
-        }
-      }
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = tc_idesc(kTcM, kTcN);
-      uint32_t stage = 0, phase = 0;
-      for (int ks = 0; ks < nk; ++ks) {
-        const int seg = ks / kTcSegSteps, in_seg = ks - seg * kTcSegSteps, a = seg % kTcAccs;
-        if (in_seg == 0 && !tc_wait(sh, st, &sh.acc_empty[a], (uint32_t)((seg / kTcAccs) & 1) ^ 1u, 430)) break;  // its last sum has been read
-        if (!tc_wait(sh, st, &sh.full[stage], phase, 410)) break;
-        tc_fence_after();
-        const uint32_t base = ring + stage * (uint32_t)kTcStageBytes;
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-#pragma unroll
-          for (int kk = 0; kk < kTcKB / 16; ++kk)  // 16 columns = 32 bytes further into the swizzled rows
-            tc_mma(tmem + (uint32_t)(a * kTcN), tc_desc(base + j * kTcTermBytes + kk * 32), tc_desc(base + 3 * kTcTermBytes + kk * 32),
-                   idesc, (uint32_t)((in_seg | j | kk) != 0));
-        tc_commit(&sh.empty[stage]);  // the stage is free once these have read it
-        if (in_seg == kTcSegSteps - 1 || ks == nk - 1) tc_commit(&sh.acc_full[a]);  // the segment's sum is complete
-        if (++stage == (uint32_t)kTcStages) { stage = 0; phase ^= 1u; }
-      }
-    }
-    __syncwarp();
-  } else {
-    // The sums of kTcSegSteps stages each move from tensor memory to registers, where they are added with
-    // round-to-nearest: the tensor cores add into their accumulator with truncation, whose error grows with the
-    // length of the chain.  Warp w may read lanes 32 (w % 4) .. 32 (w % 4) + 31, a token per thread.
-    const int quarter = warp & 3;
-    float sum[kTcN];
-#pragma unroll
-    for (int j = 0; j < kTcN; ++j) sum[j] = 0.f;
-    const int nseg = (nk + kTcSegSteps - 1) / kTcSegSteps;
-    bool ok = true;
-    for (int seg = 0; seg < nseg; ++seg) {
-      const int a = seg % kTcAccs;
-      if (!tc_wait(sh, st, &sh.acc_full[a], (uint32_t)((seg / kTcAccs) & 1), 420)) { ok = false; break; }
-      tc_fence_after();
-#pragma unroll
-      for (int c0 = 0; c0 < kTcN; c0 += 32) {
-        uint32_t r[32];
-        tc_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * kTcN + c0), r);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) sum[c0 + j] += __uint_as_float(r[j]);
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sh.acc_empty[a]);
-    }
-    if (ok) {
-      float *row = Y + (size_t)(m0 + quarter * 32 + lane) * N + n0;
-#pragma unroll
-      for (int j = 0; j < kTcN; j += 4)
-        if (n0 + j < N) *reinterpret_cast<float4 *>(row + j) = make_float4(sum[j], sum[j + 1], sum[j + 2], sum[j + 3]);
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    tc_dealloc(tmem, kTcAccs * kTcN);
-  }
-}
-
-// ---------------------------------------------------------------- products of a small batch
-// Y[token][row] = sum_c X[token][c] W[row][c] for up to NP <= 64 token rows (the requests of a batched timestep).
-// With so few tokens the product is bound by the weight stream, so the tile is turned round: the 128 weight rows
-// are the wide operand of tcgen05.mma (M = 128) and the requests' terms the narrow one (N = NP), a stage holds
-// 16 KB of weights and only 3 x NP x 128 bytes of terms (spd_tc_gemm_kernel, built for 128 tokens per tile, brings
-// 48 KB of terms per 16 KB of weights), and the columns are split among blockIdx.y so that every product fills
-// the GPU: block (x, y) adds columns [64 kb_lo, 64 kb_hi) of rows 128 x .. 128 x + 127 into its own copy of Y
-// (Y + y * split_stride), which the kernels that read Y add up in a fixed order.  Accumulators as in
-// spd_tc_gemm_kernel: sets of tensor-memory columns in rotation, each the sum of a segment of stages (96 additions),
-// fetched by the epilogue warps and added in registers with round-to-nearest (BgShape says how many sets and
-// stages for each box).  Every wait is bounded.
-// Launched as a programmatic dependent (a batched timestep), a block is set up and copies the weights of its first
-// stages while the kernel before it still runs; the terms, which that kernel writes, are asked for after dep_wait.
-template <int NP>
-struct BgShape {
-  static constexpr int kTermBytes = NP * kTcKB * 2;                 // one term tile: NP token rows x 64 columns
-  static constexpr int kStageBytes = kTcWBytes + 3 * kTermBytes;    // 128 weight rows x 64 columns, then the three term tiles
-  // Two blocks per SM wherever they fit (91, 87 and 83 KB for NP = 16, 32, 64; NP = 128: one block of 197 KB): one
-  // block's set-up and epilogue run beside the other's stages.  64 token rows with one block of five stages took
-  // 6.9 ms per 7B timestep, with two blocks of two stages 5.5 ms; three blocks of fewer stages for NP <= 32 were
-  // slower than two (4.4 against 4.0 ms for 8 requests).
-  static constexpr int kStages = NP <= 16 ? 4 : (NP <= 32 ? 3 : (NP <= 64 ? 2 : 3));
-  // Boxes of 16 and 32 rows: the three term tiles lie behind one another in a stage, 3 NP rows of one K-major operand,
-  // so one instruction of N = 3 NP per 16 columns multiplies all three (a third of the instructions; an instruction
-  // of N = 16 costs about as much as one of N = 48: 8 requests 3.63 -> 3.35 ms per 7B timestep).  Each term then has
-  // its own NP accumulator columns, added up in the epilogue's registers, and an accumulator may take three times
-  // as many stages for the same number of additions (96) before it is fetched.  Two blocks per SM share the 512
-  // columns of tensor memory, so a block has 256: four accumulator sets of 48 columns, two of 96, or one of 192
-  // (the product then waits while its sum is fetched, once or twice per block; the SM's other block does not).
-  // Boxes of 128 rows keep one instruction per term.
-  static constexpr bool kFused = NP <= 64;
-  static constexpr int kAccCols = kFused ? 3 * NP : NP;  // columns of one accumulator set
-  static constexpr int kAccs = NP == 32 ? 2 : (NP == 64 ? 1 : kTcAccs);  // accumulator sets in rotation
-  static constexpr int kSegSteps = kFused ? 3 * kTcSegSteps : kTcSegSteps;  // stages summed in one accumulator
-  static constexpr int kTmemCols = kFused ? 256 : 4 * NP;  // a power of two
-  static_assert(kAccs * kAccCols <= kTmemCols && kAccs <= kTcAccs, "the accumulator sets fit the allocation and the barrier arrays");
-};
-
-template <int NP>
-__global__ void __launch_bounds__(kTcThreads)
-    spd_batch_gemm_kernel(const void *tmap_x, const void *tmap_w, float *Y, size_t split_stride, int n_tok, int N, int C, int x_term_rows,
-                          State *st) {
-  using S = BgShape<NP>;
-  static_assert(S::kStages <= kBgMaxStages, "the block's mbarrier arrays hold kBgMaxStages stages");
-  extern __shared__ __align__(16) uint8_t tc_smem_raw[];
-  uint8_t *smem = tc_smem_raw + ((1024u - (smem_u32(tc_smem_raw) & 1023u)) & 1023u);
-  __shared__ BgShared sh;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nk_all = (C + kTcKB - 1) / kTcKB;
-  const int kb_lo = (int)((long long)nk_all * blockIdx.y / gridDim.y), kb_hi = (int)((long long)nk_all * (blockIdx.y + 1) / gridDim.y);
-  const int nk = kb_hi - kb_lo;
-  const int n0 = blockIdx.x * kTcN;
+  const int rank = (int)tc_cluster_rank(), pair = (int)(blockIdx.x >> 1);
+  const int u0 = product_cut(pr, pair), u1 = product_cut(pr, pair + 1);  // this pair's run of stages
+  const int tile_tok = pr.tile_tok;                                      // tokens of a tile
   dep_launch();
   if (threadIdx.x == 0) {
-    // the two descriptors on their way before the first copies ask for them
     asm volatile("prefetch.tensormap [%0];" ::"l"(tmap_w) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(tmap_x) : "memory");
     sh.dead = 0;
@@ -324,135 +213,188 @@ __global__ void __launch_bounds__(kTcThreads)
       mbar_init(&sh.full[s], 1);
       mbar_init(&sh.empty[s], 1);
     }
-    for (int a = 0; a < kTcAccs; ++a) {
+    for (int a = 0; a < S::kAccs; ++a) {
       mbar_init(&sh.acc_full[a], 1);
-      mbar_init(&sh.acc_empty[a], 4);
+      mbar_init(&sh.acc_empty[a], 16);  // one arrival per warp that reads the accumulator, eight in each block
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) tc_alloc(&sh.tmem_base, S::kTmemCols);
-  tc_fence_before();
   __syncthreads();
+  if (warp == 1) tc_pair_alloc(&sh.tmem_base, 512);
+  tc_fence_before();
+  tc_cluster_sync();
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
   const uint32_t ring = smem_u32(smem);
 
   if (warp == 0) {
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0, issued = 0;
+    if (tc_elect()) {
       bool ok = true;
-      // the first round of the ring: every stage is free; the weights go first, the terms once they are written
-      const int first = nk < S::kStages ? nk : S::kStages;
-      for (int ks = 0; ks < first; ++ks) {
-        mbar_expect_tx(&sh.full[ks], (uint32_t)S::kStageBytes);
-        const uint32_t base = ring + (uint32_t)ks * (uint32_t)S::kStageBytes;
+      int issued = 0;
+      const int tile0 = u0 / pr.nk;
+      int kb = u0 - tile0 * pr.nk, rt = tile0 / pr.tok_tiles, tt = tile0 - rt * pr.tok_tiles;
+      auto next = [&]() {
+        if (++kb == pr.nk) {
+          kb = 0;
+          if (++tt == pr.tok_tiles) { tt = 0; ++rt; }
+        }
+      };
+      const uint32_t bar0 = tc_leader_addr(&sh.full[0]);
+      auto weights = [&](uint32_t stage) {
+        const uint32_t base = ring + stage * (uint32_t)S::kStageBytes, bar = bar0 + stage * 8u;
+        const int row = rt * (2 * kTcRows) + rank * kTcRows;
 #pragma unroll
-        for (int j = 0; j < kTcN / kTcWBoxRows; ++j)
-          tc_box_load(base + j * (kTcWBoxRows * kTcKB * 2), tmap_w, (kb_lo + ks) * kTcKB, n0 + j * kTcWBoxRows, &sh.full[ks]);
+        for (int j = 0; j < kTcRows / kTcWBoxRows; ++j)
+          tc_pair_box_load(base + j * (kTcWBoxRows * kTcKB * 2), tmap_w, kb * kTcKB, row + j * kTcWBoxRows, bar);
+      };
+      auto terms = [&](uint32_t stage) {
+        const uint32_t base = ring + stage * (uint32_t)S::kStageBytes + kTcWBytes, bar = bar0 + stage * 8u;
+        const int t0 = tt * tile_tok + rank * (tile_tok / 2);
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+          for (int b = 0; b < S::kTermRows / S::kBoxRows; ++b)
+            tc_pair_box_load(base + j * S::kTermBytes + b * (S::kBoxRows * kTcKB * 2), tmap_x, kb * kTcKB, j * x_term_rows + t0 + b * S::kBoxRows, bar);
+      };
+      // the first round of the ring: every stage is free; the weights go first, the terms once they are written
+      const int first = min(u1 - u0, S::kStages);
+      const int kb0 = kb, rt0 = rt, tt0 = tt;
+      for (int i = 0; i < first; ++i, next()) {
+        if (rank == 0) mbar_expect_tx(&sh.full[i], (uint32_t)(2 * S::kCopyBytes));
+        if (!(stall && i == 0)) weights(i);
       }
       dep_wait();
       asm volatile("fence.proxy.async;" ::: "memory");  // the terms were written with ordinary stores
-      for (int ks = 0; ks < first; ++ks) {
-        const uint32_t base = ring + (uint32_t)ks * (uint32_t)S::kStageBytes;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) tc_box_load(base + kTcWBytes + j * S::kTermBytes, tmap_x, (kb_lo + ks) * kTcKB, j * x_term_rows, &sh.full[ks]);
-      }
-      issued = (uint32_t)first;
-      if (first == S::kStages) phase = 1u;
-      else stage = (uint32_t)first;
-      for (int ks = first; ks < nk; ++ks) {
-        if (!tc_wait(sh, st, &sh.empty[stage], phase ^ 1u, 500)) { ok = false; break; }
-        mbar_expect_tx(&sh.full[stage], (uint32_t)S::kStageBytes);
-        const uint32_t base = ring + stage * (uint32_t)S::kStageBytes;
-        const int col = (kb_lo + ks) * kTcKB;
-#pragma unroll
-        for (int j = 0; j < kTcN / kTcWBoxRows; ++j)
-          tc_box_load(base + j * (kTcWBoxRows * kTcKB * 2), tmap_w, col, n0 + j * kTcWBoxRows, &sh.full[stage]);
-#pragma unroll
-        for (int j = 0; j < 3; ++j) tc_box_load(base + kTcWBytes + j * S::kTermBytes, tmap_x, col, j * x_term_rows, &sh.full[stage]);
+      kb = kb0; rt = rt0; tt = tt0;
+      for (int i = 0; i < first; ++i, next())
+        if (!(stall && i == 0)) terms(i);
+      issued = first;
+      uint32_t stage = 0, phase = 0;
+      for (int u = u0 + first; u < u1; ++u, next()) {
+        if (!tc_wait(sh, st, &sh.empty[stage], phase, 400)) { ok = false; break; }
+        if (rank == 0) mbar_expect_tx(&sh.full[stage], (uint32_t)(2 * S::kCopyBytes));
+        weights(stage);
+        terms(stage);
+        ++issued;
         if (++stage == (uint32_t)S::kStages) { stage = 0; phase ^= 1u; }
       }
       if (!ok) {
-        uint32_t s = stage, ph = phase;
-        for (uint32_t i = 0; i < issued; ++i) {
-          if (s == 0) { s = (uint32_t)S::kStages; ph ^= 1u; }
-          --s;
-          unsigned long long t0 = globaltimer();
-          while (!mbar_try_wait(&sh.full[s], ph) && globaltimer() - t0 < kTcWaitNs) {}
+        // giving up: wait (bounded) for the copies already issued, so that none lands after the blocks have gone.  The
+        // leader sees its own and the other block's on its barriers; the other block, whose shared memory stays until both
+        // reach the cluster barrier below, gives copies that the leader never announced 10 ms.
+        const unsigned long long t = globaltimer();
+        if (rank == 0) {
+          for (int i = issued - 1; i >= 0 && i >= issued - S::kStages; --i) {
+            if (stall && i == 0) break;  // nothing was copied for it
+            while (!mbar_try_wait(&sh.full[i % S::kStages], (uint32_t)(i / S::kStages) & 1u) && globaltimer() - t < kTcWaitNs) {}
+          }
+        } else {
+          while (globaltimer() - t < 10ull * 1000ull * 1000ull) {}
         }
       }
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = tc_idesc(kTcN, S::kAccCols);  // M = 128 weight rows, N = NP token rows (x 3 terms when fused)
+    if (rank == 0 && tc_elect()) {
+      const uint32_t idesc = tc_idesc(2 * kTcRows, S::kFused ? S::kCols : tile_tok);
       uint32_t stage = 0, phase = 0;
-      for (int ks = 0; ks < nk; ++ks) {
-        const int seg = ks / S::kSegSteps, in_seg = ks - seg * S::kSegSteps, a = seg % S::kAccs;
-        if (in_seg == 0 && !tc_wait(sh, st, &sh.acc_empty[a], (uint32_t)((seg / S::kAccs) & 1) ^ 1u, 530)) break;
-        if (!tc_wait(sh, st, &sh.full[stage], phase, 510)) break;
+      int seg = 0, in_seg = 0, kb = u0 % pr.nk;
+      for (int u = u0; u < u1; ++u) {
+        const int a = seg % S::kAccs;
+        if (in_seg == 0 && !tc_wait(sh, st, &sh.acc_empty[a], (uint32_t)((seg / S::kAccs) & 1) ^ 1u, 430)) break;  // its last sum has been read
+        if (!tc_wait(sh, st, &sh.full[stage], phase, 410)) break;
         tc_fence_after();
-        const uint32_t base = ring + stage * (uint32_t)S::kStageBytes;
-        if constexpr (S::kFused) {
+        const uint32_t base = ring + stage * (uint32_t)S::kStageBytes, acc = tmem + (uint32_t)(a * S::kAccStride);
 #pragma unroll
-          for (int kk = 0; kk < kTcKB / 16; ++kk)
-            tc_mma(tmem + (uint32_t)(a * S::kAccCols), tc_desc(base + kk * 32), tc_desc(base + kTcWBytes + kk * 32), idesc,
-                   (uint32_t)((in_seg | kk) != 0));
-        } else {
+        for (int j = 0; j < (S::kFused ? 1 : 3); ++j)
 #pragma unroll
-          for (int j = 0; j < 3; ++j)
-#pragma unroll
-            for (int kk = 0; kk < kTcKB / 16; ++kk)
-              tc_mma(tmem + (uint32_t)(a * S::kAccCols), tc_desc(base + kk * 32), tc_desc(base + kTcWBytes + j * S::kTermBytes + kk * 32), idesc,
-                     (uint32_t)((in_seg | j | kk) != 0));
-        }
-        tc_commit(&sh.empty[stage]);
-        if (in_seg == S::kSegSteps - 1 || ks == nk - 1) tc_commit(&sh.acc_full[a]);
+          for (int kk = 0; kk < kTcKB / 16; ++kk)  // 16 columns = 32 bytes further into the swizzled rows
+            tc_pair_mma(acc, tc_desc(base + kk * 32), tc_desc(base + kTcWBytes + j * S::kTermBytes + kk * 32), idesc,
+                        (uint32_t)((in_seg | j | kk) != 0));
+        tc_pair_commit(&sh.empty[stage]);  // the stage is free in both blocks once these have read it
         if (++stage == (uint32_t)S::kStages) { stage = 0; phase ^= 1u; }
+        ++kb;
+        if (++in_seg == S::kSegSteps || kb == pr.nk || u + 1 == u1) {
+          tc_pair_commit(&sh.acc_full[a]);  // the segment's sum is complete
+          ++seg;
+          in_seg = 0;
+        }
+        if (kb == pr.nk) kb = 0;
       }
     }
     __syncwarp();
   } else {
-    // lane l of warp w reads tensor-memory lane 32 (w % 4) + l: weight row n0 + that, a token per column
-    const int quarter = warp & 3;
-    float sum[NP];
-#pragma unroll
-    for (int j = 0; j < NP; ++j) sum[j] = 0.f;
-    const int nseg = (nk + S::kSegSteps - 1) / S::kSegSteps;
+    // Warp w may read lanes 32 (w % 4) .. 32 (w % 4) + 31 of tensor memory: a weight row per thread, a token per column;
+    // warps 2..5 take the first half of the tile's tokens, 6..9 the second.
+    const int quarter = warp & 3, half = (warp - 2) >> 2, half_tok = tile_tok / 2;
+    const uint32_t lanes = tmem + ((uint32_t)(quarter * 32) << 16);
+    int seg = 0;
     bool ok = true;
-    for (int seg = 0; seg < nseg; ++seg) {
-      const int a = seg % S::kAccs;
-      if (!tc_wait(sh, st, &sh.acc_full[a], (uint32_t)((seg / S::kAccs) & 1), 520)) { ok = false; break; }
-      tc_fence_after();
+    dep_wait();  // Y and the pairs' buffers are written below (the kernel before this one may still be reading them)
+    for (int u = u0; u < u1 && ok;) {
+      const int tile = u / pr.nk, kb = u - tile * pr.nk, stages = min(pr.nk - kb, u1 - u);
+      float sum[S::kHalf];
 #pragma unroll
-      for (int c0 = 0; c0 < S::kAccCols; c0 += 16) {  // (fused: the columns of term c0 / NP, added to the same tokens' sums)
-        uint32_t r[16];
-        tc_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * S::kAccCols + c0), r);
+      for (int j = 0; j < S::kHalf; ++j) sum[j] = 0.f;
+      for (int done = 0; done < stages; done += S::kSegSteps, ++seg) {
+        const int a = seg % S::kAccs;
+        if (!tc_wait(sh, st, &sh.acc_full[a], (uint32_t)((seg / S::kAccs) & 1), 420)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t acc = lanes + (uint32_t)(a * S::kAccStride);
+        if constexpr (S::kFused) {
+          // a half's columns: its tokens' first terms, second terms, third terms
+          const uint32_t from = acc + (uint32_t)(half * (S::kCols / 2));
 #pragma unroll
-        for (int j = 0; j < 16; ++j) sum[c0 % NP + j] += __uint_as_float(r[j]);
+          for (int c0 = 0; c0 < 3 * S::kHalf; c0 += S::kLd) {
+            uint32_t r[S::kLd];
+            tc_ld(from + (uint32_t)c0, r);
+            tc_ld_wait();
+#pragma unroll
+            for (int j = 0; j < S::kLd; ++j) sum[(c0 + j) % S::kHalf] += __uint_as_float(r[j]);
+          }
+        } else {
+          const uint32_t from = acc + (uint32_t)(half * half_tok);
+#pragma unroll
+          for (int c0 = 0; c0 < S::kHalf; c0 += 32)
+            if (c0 < half_tok) {  // (half_tok is a multiple of 16)
+              uint32_t r[16], q[16];
+              tc_ld(from + (uint32_t)c0, r);
+              if (c0 + 16 < half_tok) tc_ld(from + (uint32_t)(c0 + 16), q);
+              tc_ld_wait();
+#pragma unroll
+              for (int j = 0; j < 16; ++j) sum[c0 + j] += __uint_as_float(r[j]);
+              if (c0 + 16 < half_tok) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) sum[c0 + 16 + j] += __uint_as_float(q[j]);
+              }
+            }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) tc_cluster_arrive(tc_leader_addr(&sh.acc_empty[a]));
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sh.acc_empty[a]);
-    }
-    const int row = n0 + quarter * 32 + lane;
-    dep_wait();  // (long since true: the sums came from terms copied after the producer's dep_wait)
-    if (ok && row < N) {
-      float *out = Y + (size_t)blockIdx.y * split_stride + row;
+      const int in_tile = rank * kTcRows + quarter * 32 + lane, row = tile / pr.tok_tiles * (2 * kTcRows) + in_tile;
+      const int t_lo = half * half_tok, t0 = tile % pr.tok_tiles * tile_tok + t_lo;  // first token of this half in the tile, overall
+      if (ok && row < pr.N) {
+        // the lanes of a warp write 32 consecutive floats of a token's row
+        float *out = kb == 0 ? Y + (size_t)t0 * pr.N + row : parts + ((size_t)pair * tile_tok + t_lo) * (2 * kTcRows) + in_tile;
+        const size_t step = kb == 0 ? (size_t)pr.N : (size_t)(2 * kTcRows);
 #pragma unroll
-      for (int j = 0; j < NP; ++j)
-        if (j < n_tok) out[(size_t)j * N] = sum[j];  // the lanes of a warp write 32 consecutive floats of token j's row
+        for (int j = 0; j < S::kHalf; ++j)
+          if (j < half_tok && t0 + j < n_tok) out[j * step] = sum[j];
+      }
+      u += stages;
     }
   }
   tc_fence_before();
-  __syncthreads();
+  tc_cluster_sync();  // neither block leaves while the other may still signal or read its shared memory
   if (warp == 1) {
     tc_fence_after();
-    tc_dealloc(tmem, S::kTmemCols);
+    tc_pair_dealloc(tmem, 512);
   }
 }
 
-// ---------------------------------------------------------------- row-wise kernels between the products
+// ---------------------------------------------------------------- attention of a job
 // v = hi + mid + lo exactly: each term takes the leading 8 significant bits of what is left, by truncation.
 __device__ __forceinline__ void tc_put3(uint16_t *X, size_t term_stride, size_t at, float v) {
   const uint32_t hi = __float_as_uint(v) & 0xffff0000u;
@@ -464,94 +406,6 @@ __device__ __forceinline__ void tc_put3(uint16_t *X, size_t term_stride, size_t 
   X[at + 2 * term_stride] = (uint16_t)(__float_as_uint(r2) >> 16);
 }
 
-// Block sum in a fixed order (256 threads).
-__device__ __forceinline__ float tc_block_sum(float v, float *scratch) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
-  __syncthreads();
-  float s = 0.f;
-#pragma unroll
-  for (int w = 0; w < 8; ++w) s += scratch[w];
-  __syncthreads();
-  return s;
-}
-
-// One token per block: the residual row (the embedding of ids[t] when `ids`, else h + y when `y`; y, like every
-// product's output read below, is the sum of nz partial products zs floats apart), stored, and
-// when `gain`: its RMSNorm (x * rsqrt(mean x^2 + eps) * gain) as three bf16 terms for the next product.
-__global__ void __launch_bounds__(256) spd_tc_resid_norm_kernel(float *h, const float *y, const int32_t *ids, const __nv_bfloat16 *emb,
-                                                                const __nv_bfloat16 *gain, uint16_t *X, size_t term_stride, int d, float eps,
-                                                                int nz, size_t zs) {
-  dep_wait();    // the kernel before this one in the stream wrote what this one reads
-  dep_launch();  // the next one may set itself up meanwhile
-  __shared__ float scratch[8];
-  const int t = blockIdx.x;
-  float *hr = h + (size_t)t * d;
-  float ss = 0.f;
-  for (int c = threadIdx.x; c < d; c += 256) {
-    float v;
-    if (ids) v = __bfloat162float(emb[(size_t)ids[t] * d + c]);
-    else {
-      v = hr[c];
-      for (int z = 0; z < nz; ++z) v += y[z * zs + (size_t)t * d + c];
-    }
-    hr[c] = v;
-    ss = fmaf(v, v, ss);
-  }
-  if (!gain) return;
-  const float rs = rsqrtf(tc_block_sum(ss, scratch) / (float)d + eps);
-  for (int c = threadIdx.x; c < d; c += 256) tc_put3(X, term_stride, (size_t)t * d + c, hr[c] * rs * __bfloat162float(gain[c]));
-}
-
-// One token per block: rotary embedding of q and k (adjacent pairs), q to Q, k and v into the cache at the
-// token's position.  Y row = [q | k | v].
-__global__ void __launch_bounds__(256) spd_tc_rope_cache_kernel(const float *Y, float *Q, void *kcache, void *vcache, const float2 *rope,
-                                                                int d, int hd, int max_pos, int layer, int pos0, int kv_bf16, int nz, size_t zs) {
-  dep_wait();    // the kernel before this one in the stream wrote what this one reads
-  dep_launch();  // the next one may set itself up meanwhile
-  const int t = blockIdx.x, pos = pos0 + t;
-  const float *yr = Y + (size_t)t * 3 * d;
-  const size_t crow = ((size_t)layer * max_pos + pos) * d;
-  for (int i = threadIdx.x; i < d / 2; i += 256) {
-    const float2 cs = rope[(size_t)pos * (hd / 2) + (i % (hd / 2))];
-    float qe = 0.f, qo = 0.f, ke = 0.f, ko = 0.f, v0 = 0.f, v1 = 0.f;
-    for (int z = 0; z < nz; ++z) {
-      const float *yz = yr + z * zs;
-      qe += yz[2 * i]; qo += yz[2 * i + 1];
-      ke += yz[d + 2 * i]; ko += yz[d + 2 * i + 1];
-      v0 += yz[2 * d + 2 * i]; v1 += yz[2 * d + 2 * i + 1];
-    }
-    Q[(size_t)t * d + 2 * i] = qe * cs.x - qo * cs.y;
-    Q[(size_t)t * d + 2 * i + 1] = qe * cs.y + qo * cs.x;
-    const float k0 = ke * cs.x - ko * cs.y, k1 = ke * cs.y + ko * cs.x;
-    if (kv_bf16) {
-      reinterpret_cast<__nv_bfloat162 *>(kcache)[(crow >> 1) + i] = __halves2bfloat162(__float2bfloat16_rn(k0), __float2bfloat16_rn(k1));
-      reinterpret_cast<__nv_bfloat162 *>(vcache)[(crow >> 1) + i] = __halves2bfloat162(__float2bfloat16_rn(v0), __float2bfloat16_rn(v1));
-    } else {
-      reinterpret_cast<float2 *>(kcache)[(crow >> 1) + i] = make_float2(k0, k1);
-      reinterpret_cast<float2 *>(vcache)[(crow >> 1) + i] = make_float2(v0, v1);
-    }
-  }
-}
-
-// One token per block: u = SiLU(gate) * up from Y row = [gate_0, up_0, gate_1, up_1, ...], as three bf16 terms.
-__global__ void __launch_bounds__(256) spd_tc_swiglu_kernel(const float *Y, uint16_t *X, size_t term_stride, int f, int nz, size_t zs) {
-  dep_wait();    // the kernel before this one in the stream wrote what this one reads
-  dep_launch();  // the next one may set itself up meanwhile
-  const int t = blockIdx.x;
-  const float2 *yr = reinterpret_cast<const float2 *>(Y + (size_t)t * 2 * f);
-  for (int j = threadIdx.x; j < f; j += 256) {
-    float2 gu = yr[j];
-    for (int z = 1; z < nz; ++z) {
-      const float2 more = yr[z * (zs / 2) + j];
-      gu.x += more.x;
-      gu.y += more.y;
-    }
-    tc_put3(X, term_stride, (size_t)t * f + j, gu.x / (1.f + __expf(-gu.x)) * gu.y);
-  }
-}
-
 // Causal attention over a float32 cache (a bf16 cache takes spd_tc_attn_mma_kernel below): 16 consecutive tokens
 // of one head.  The block brings 32 cached positions at
 // a time into shared memory as float32 (keys with padded rows, so that a lane per position reads its row without
@@ -561,8 +415,8 @@ __global__ void __launch_bounds__(256) spd_tc_swiglu_kernel(const float *Y, uint
 template <int HD>
 __global__ void __launch_bounds__(256) spd_tc_attn_kernel(const float *Q, const float *kcache, const float *vcache, uint16_t *X,
                                                           size_t term_stride, int d, int max_pos, int layer, int pos0, int n_tok) {
-  dep_wait();    // the kernel before this one in the stream wrote what this one reads
-  dep_launch();  // the next one may set itself up meanwhile
+  dep_launch();
+  dep_wait();
   constexpr int kTok = 16, kPos = 32;
   constexpr int KS = HD + 4;    // key row stride in floats: 16-byte aligned, rows 4 banks apart
   constexpr int DPL = HD / 32;  // value dimensions per lane
@@ -706,8 +560,8 @@ __device__ __forceinline__ void tc_split3(float v, uint32_t &hi, uint32_t &mid, 
 template <int HD>
 __global__ void __launch_bounds__(128) spd_tc_attn_mma_kernel(const float *Q, const uint16_t *kcache, const uint16_t *vcache, uint16_t *X,
                                                               size_t term_stride, int d, int max_pos, int layer, int pos0, int n_tok) {
-  dep_wait();    // the kernel before this one in the stream wrote what this one reads
-  dep_launch();  // the next one may set itself up meanwhile
+  dep_launch();
+  dep_wait();
   constexpr int kTok = 64, kPos = 64;
   constexpr int RS = HD * 2 + 16;  // bytes per tile row
   constexpr int KS = HD / 16;      // k-steps over the head's dimensions
@@ -865,13 +719,29 @@ cudaError_t launch_attn(const spd::TcJob &j, int layer, int n_tok, cudaStream_t 
                          static_cast<const float *>(j.vcache), j.x, ts, j.d, j.max_pos, layer, j.pos0, n_tok);
 }
 
-size_t tc_gemm_smem() { return (size_t)spd::kTcStages * spd::kTcStageBytes + 1024; }
+template <int NT>
+cudaError_t launch_product(const spd::TcJob &j, int wide, const void *wmap, float *Y, const spd::Product &pr, int n_tok, cudaStream_t s, int stall) {
+  using S = spd::TcShape<NT>;
+  // the term buffer's tensor maps, two each (d_model and d_ffn columns): boxes of 8, 16, 32 and 64 rows
+  const int slot = (S::kBoxRows == 8 ? 0 : (S::kBoxRows == 16 ? 1 : (S::kBoxRows == 32 ? 2 : 3))) * 2 + (wide ? 1 : 0);
+  return spd::launch_dep(spd::spd_tc_product_kernel<NT>, dim3(2 * pr.pairs), dim3(spd::kTcThreads), S::kSmem, s,
+                         j.x_tmaps + (size_t)slot * spd::kTensorMapBytes, wmap, Y, j.parts, pr, n_tok, j.x_term_rows, j.st, stall);
+}
+
+template <int NT>
+cudaError_t allow_product_smem() {
+  return cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_tc_product_kernel<NT>), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)spd::TcShape<NT>::kSmem);
+}
 
 }  // namespace
 
 extern "C" cudaError_t spd_internal_tc_prepare(void) {
-  cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_tc_gemm_kernel), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)tc_gemm_smem());
+  cudaError_t e = allow_product_smem<16>();
+  if (e == cudaSuccess) e = allow_product_smem<32>();
+  if (e == cudaSuccess) e = allow_product_smem<64>();
+  if (e == cudaSuccess) e = allow_product_smem<128>();
+  if (e == cudaSuccess) e = allow_product_smem<256>();
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_tc_attn_mma_kernel<64>), cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)attn_mma_smem<64>());
@@ -881,76 +751,31 @@ extern "C" cudaError_t spd_internal_tc_prepare(void) {
   return e;
 }
 
-namespace {
-template <int NP>
-cudaError_t launch_batch_gemm(const void *xmap, const void *wmap, float *Y, size_t zs, int nz, int n_tok, int N, int C, int x_term_rows,
-                              spd::State *st, cudaStream_t s, int dep) {
-  using S = spd::BgShape<NP>;
-  const size_t smem = (size_t)S::kStages * S::kStageBytes + 1024;
-  // the shared-memory attribute is per device: set on a device's first launch of this instance
-  static bool ready[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64 || !ready[dev]) {
-    e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_batch_gemm_kernel<NP>), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) ready[dev] = true;
+// Product of n_tok token rows (<= x_term_rows) with matrix `which` of the layers' tensor maps: `wide` terms have d_ffn
+// columns, else d_model.  *out tells the readers of Y where its sums are (product_sum).
+extern "C" cudaError_t spd_internal_product(const spd::TcJob *job, int n_tok, int wide, int which, float *Y, int N, spd::Product *out, cudaStream_t s) {
+  const spd::TcJob &j = *job;
+  const void *wmap = j.w_tmaps + (size_t)which * spd::kTensorMapBytes;
+  const spd::Product pr = spd::plan_product(n_tok, N, wide ? j.f : j.d, j.sm_count, Y, j.parts);
+  *out = pr;
+  switch (pr.shape) {
+    case 16: return launch_product<16>(j, wide, wmap, Y, pr, n_tok, s, 0);
+    case 32: return launch_product<32>(j, wide, wmap, Y, pr, n_tok, s, 0);
+    case 64: return launch_product<64>(j, wide, wmap, Y, pr, n_tok, s, 0);
+    case 128: return launch_product<128>(j, wide, wmap, Y, pr, n_tok, s, 0);
+    default: return launch_product<256>(j, wide, wmap, Y, pr, n_tok, s, 0);
   }
-  const dim3 grid((N + spd::kTcN - 1) / spd::kTcN, nz);
-  if (dep) return spd::launch_dep(spd::spd_batch_gemm_kernel<NP>, grid, dim3(spd::kTcThreads), smem, s, xmap, wmap, Y, zs, n_tok, N, C, x_term_rows, st);
-  spd::spd_batch_gemm_kernel<NP><<<grid, spd::kTcThreads, smem, s>>>(xmap, wmap, Y, zs, n_tok, N, C, x_term_rows, st);
-  return cudaGetLastError();
-}
-}  // namespace
-
-// Product of a batch (n_tok <= 128 token rows): xmaps = the term buffer's tensor maps with boxes of 128, 16, 32 and 64
-// rows (two each: d_model and d_ffn columns; `wide` picks the second).  The columns are split nz ways (chosen here
-// for the fewest waves of blocks, within y_floats of room for the partial sums); *out_nz and
-// *out_zs tell the reader of Y how many partial sums there are and how far apart.
-extern "C" cudaError_t spd_internal_batch_gemm(const uint8_t *xmaps, int wide, const void *wmap, float *Y, size_t y_floats, int n_tok, int N, int C,
-                                               int x_term_rows, spd::State *st, int sm_count, cudaStream_t s, int dep, int *out_nz, size_t *out_zs) {
-  const int np = n_tok <= 16 ? 16 : (n_tok <= 32 ? 32 : (n_tok <= 64 ? 64 : 128));
-  // the term buffer's tensor maps: boxes of 128 rows first, then 16, 32 and 64 (two each: d_model and d_ffn columns)
-  const int slot = (np == 128 ? 0 : (np == 16 ? 1 : (np == 32 ? 2 : 3))) * 2 + (wide ? 1 : 0);
-  const void *xmap = xmaps + (size_t)slot * spd::kTensorMapBytes;
-  const int tiles = (N + spd::kTcN - 1) / spd::kTcN, nk = (C + spd::kTcKB - 1) / spd::kTcKB;
-  const size_t zs = (size_t)n_tok * N;
-  // The split that needs the fewest stage times: the blocks run in waves of as many as fit the GPU (two per SM, one
-  // with boxes of 128 rows), a block costs its stages plus about eight stages' worth of set-up, ring fill and epilogue,
-  // and a last wave that is nearly empty costs as much as a full one (the 7B gate / up product, 172 row tiles: two
-  // ways = 344 blocks = two waves of 32 stages, three ways = 516 blocks = two waves of 22).  At least 8 stages of
-  // work per block, and room for the partial sums.
-  const int slots = (np == 128 ? 1 : 2) * (sm_count > 0 ? sm_count : 1);
-  int nz_max = nk / 8;
-  if ((size_t)nz_max * zs > y_floats) nz_max = (int)(y_floats / zs);
-  if (nz_max < 1) nz_max = 1;
-  int nz = 1;
-  long best = -1;
-  for (int z = 1; z <= nz_max; ++z) {
-    const long waves = ((long)tiles * z + slots - 1) / slots;
-    const long cost = waves * ((nk + z - 1) / z + 8);
-    if (best < 0 || cost < best) { best = cost; nz = z; }
-  }
-  *out_nz = nz;
-  *out_zs = zs;
-  if (np == 16) return launch_batch_gemm<16>(xmap, wmap, Y, zs, nz, n_tok, N, C, x_term_rows, st, s, dep);
-  if (np == 32) return launch_batch_gemm<32>(xmap, wmap, Y, zs, nz, n_tok, N, C, x_term_rows, st, s, dep);
-  if (np == 64) return launch_batch_gemm<64>(xmap, wmap, Y, zs, nz, n_tok, N, C, x_term_rows, st, s, dep);
-  return launch_batch_gemm<128>(xmap, wmap, Y, zs, nz, n_tok, N, C, x_term_rows, st, s, dep);
 }
 
-// Test hook: one tile of the first layer's QKV product whose first stage never arrives (see the kernel's `stall`).
+// Test hook: the first layer's QKV product by one pair whose first stage never arrives (see the kernel's `stall`).
 extern "C" cudaError_t spd_internal_tc_stall(const spd::TcJob *job, cudaStream_t s) {
   const spd::TcJob &j = *job;
-  spd::spd_tc_gemm_kernel<<<dim3(1, 1), spd::kTcThreads, tc_gemm_smem(), s>>>(j.x_tmaps, j.w_tmaps, j.y, 3 * j.d, j.d, j.x_term_rows, j.st, 1);
-  return cudaGetLastError();
+  return launch_product<16>(j, 0, j.w_tmaps, j.y, spd::plan_product(1, 3 * j.d, j.d, 2, j.y, j.parts), 1, s, 1);
 }
 
 // Enqueues the decoder over j.n_tok tokens (at most j.x_term_rows) at positions j.pos0 ..: their keys and values
-// enter the cache.  The products run over whole tiles of 128 tokens: the rows past n_tok of the last tile hold
-// whatever an earlier job left, give rows of Y that nothing reads (a row of Y depends on its own token only).
+// enter the cache.  The term rows past n_tok hold whatever an earlier job left and give rows of Y that nothing reads
+// (a row of Y depends on its own token only).
 // head: the context's parameters when the job ends the prefix, else null.  Then the last layer carries on with the last
 // token's row alone once the keys and values are in the cache (nothing reads the other rows), and one more launch adds
 // the last product to the residual row, multiplies the LM head and takes the first timestep.
@@ -958,50 +783,24 @@ extern "C" cudaError_t spd_internal_tc_stall(const spd::TcJob *job, cudaStream_t
 extern "C" cudaError_t spd_internal_tc_prefill(const spd::TcJob *job, const spd::KParams *head, cudaStream_t s, int *launches) {
   const spd::TcJob &j = *job;
   const int n = j.n_tok, d = j.d, f = j.f;
-  const size_t ts_d = (size_t)j.x_term_rows * d, ts_f = (size_t)j.x_term_rows * f;
-  const bool small = n <= spd::kTcM;
   int count = 0;
   cudaError_t e = cudaSuccess;
-  // A job of up to 128 tokens is one token tile: its products are bound by the weight stream and take the product
-  // made for few token rows (weights as the wide operand, columns split among blocks; its output is nz partial sums
-  // zs floats apart, which the row-wise kernels add up).
-  int nz = 1;
-  size_t zs = 0;
-  auto gemm = [&](int rows, int wide, int which, int N, int C) {
-    if (e != cudaSuccess) return;
-    const uint8_t *wmap = j.w_tmaps + (size_t)which * spd::kTensorMapBytes;
-    if (rows <= spd::kTcM) {
-      e = spd_internal_batch_gemm(j.x_tmaps, wide, wmap, j.y, j.y_floats, rows, N, C, j.x_term_rows, j.st, j.sm_count, s, 1, &nz, &zs);
-    } else {
-      const dim3 grid((rows + spd::kTcM - 1) / spd::kTcM, (N + spd::kTcN - 1) / spd::kTcN);
-      spd::spd_tc_gemm_kernel<<<grid, spd::kTcThreads, tc_gemm_smem(), s>>>(j.x_tmaps + (size_t)wide * spd::kTensorMapBytes, wmap, j.y, N, C,
-                                                                           j.x_term_rows, j.st, 0);
-      e = cudaGetLastError();
-      nz = 1;
-      zs = 0;
-    }
+  spd::Product pr;  // where the last product's sums are
+  auto done = [&](cudaError_t r) {  // a kernel enqueued (after an error: not)
+    e = r;
     ++count;
   };
-  auto done = [&](cudaError_t r) {  // a kernel enqueued
-    if (e == cudaSuccess) e = r;
-    ++count;
+  auto product = [&](int rows, int wide, int which, int N) {
+    if (e == cudaSuccess) done(spd_internal_product(job, rows, wide, which, j.y, N, &pr, s));
   };
-  // Row-wise kernels of few rows: the column-parallel ones of a batched timestep (a block per 512 columns of a token row
-  // instead of one per row; RMSNorm's 1 / rms applied behind the product from per-chunk sums of squares).
-  auto resid = [&](const float *y, const int32_t *ids, const __nv_bfloat16 *gain) {
-    if (e != cudaSuccess) return;
-    done(spd::launch_dep(spd::spd_tc_resid_norm_kernel, dim3(n), dim3(256), 0, s, j.h, y, ids, j.tok_emb, gain, j.x, ts_d, d, j.eps, nz, zs));
+  const bool normed = n > spd::kTcTile;  // long jobs: the norm before the product
+  auto resid = [&](const spd::TcJob &part, const spd::Product *y, const __nv_bfloat16 *gain) {
+    if (e == cudaSuccess) done(normed && part.n_tok == n ? spd_internal_job_norm(&part, y, gain, s) : spd_internal_job_resid(&part, y, gain, s));
   };
-  if (small) done(spd_internal_job_input(job, j.ss, s));
-  else resid(nullptr, j.ids, j.layers[0].attn_norm);
+  resid(j, nullptr, j.layers[0].attn_norm);
   for (int l = 0; l < j.L && e == cudaSuccess; ++l) {
-    gemm(n, 0, 4 * l, 3 * d, d);
-    if (e != cudaSuccess) break;
-    if (small) done(spd_internal_job_rope_cache(job, j.ss, nz, zs, l, s));
-    else
-      done(spd::launch_dep(spd::spd_tc_rope_cache_kernel, dim3(n), dim3(256), 0, s, j.y, j.q, j.kcache, j.vcache, j.rope, d, j.hd, j.max_pos, l,
-                           j.pos0, j.kv_bf16, nz, zs));
-    if (e != cudaSuccess) break;
+    product(n, 0, 4 * l, 3 * d);
+    if (e == cudaSuccess) done(spd_internal_job_rope_cache(job, &pr, normed, l, s));
     const bool end = head && l + 1 == j.L;
     spd::TcJob part = j;  // the rows that carry on
     if (end) {
@@ -1010,23 +809,15 @@ extern "C" cudaError_t spd_internal_tc_prefill(const spd::TcJob *job, const spd:
       part.pos0 += n - 1;
       part.n_tok = 1;
     }
-    const bool few = small || end;
-    done(j.hd == 128 ? launch_attn<128>(part, l, part.n_tok, s) : launch_attn<64>(part, l, part.n_tok, s));  // other head sizes never get here
-    gemm(part.n_tok, 0, 4 * l + 1, d, d);
-    if (e != cudaSuccess) break;
-    if (few) done(spd_internal_job_resid(&part, j.ss, nz, zs, j.layers[l].ffn_norm, s));
-    else resid(j.y, nullptr, j.layers[l].ffn_norm);
-    gemm(part.n_tok, 0, 4 * l + 2, 2 * f, d);
-    if (e != cudaSuccess) break;
-    if (few) done(spd_internal_job_swiglu(&part, j.ss, nz, zs, s));
-    else done(spd::launch_dep(spd::spd_tc_swiglu_kernel, dim3(n), dim3(256), 0, s, j.y, j.x, ts_f, f, nz, zs));
-    gemm(part.n_tok, 1, 4 * l + 3, d, f);
-    if (e != cudaSuccess) break;
-    if (end) done(spd_internal_job_head(head, part.h, j.y, nz, zs, j.sm_count, s));
-    else if (l + 1 < j.L) {  // without a head the last layer's output feeds nothing
-      if (few) done(spd_internal_job_resid(&part, j.ss, nz, zs, j.layers[l + 1].attn_norm, s));
-      else resid(j.y, nullptr, j.layers[l + 1].attn_norm);
-    }
+    if (e == cudaSuccess)
+      done(j.hd == 128 ? launch_attn<128>(part, l, part.n_tok, s) : launch_attn<64>(part, l, part.n_tok, s));  // other head sizes never get here
+    product(part.n_tok, 0, 4 * l + 1, d);
+    resid(part, &pr, j.layers[l].ffn_norm);
+    product(part.n_tok, 0, 4 * l + 2, 2 * f);
+    if (e == cudaSuccess) done(spd_internal_job_swiglu(&part, &pr, normed && !end, s));
+    product(part.n_tok, 1, 4 * l + 3, d);
+    if (end && e == cudaSuccess) done(spd_internal_job_head(head, part.h, &pr, j.sm_count, s));
+    else if (l + 1 < j.L) resid(part, &pr, j.layers[l + 1].attn_norm);  // without a head the last layer's output feeds nothing
   }
   if (launches) *launches = count;
   return e;

@@ -8,25 +8,94 @@ constexpr int kTcTile = 128;      // tokens per tile of the tensor-core products
 constexpr int kTcMaxTokens = 512; // tokens one job takes at most
 constexpr int kTcMinPrefix = 16;  // runs of more tokens than this take the path with every model, shorter ones with large models
 
+// A product Y = X W^T as it is dealt out among pairs of blocks, and where its sums are (spd_tc_product_kernel).  Tiles of
+// 256 weight rows x tile_tok token rows, token tiles fastest; a tile has nk stages of 64 columns; the stages of all tiles,
+// one after the other, are cut into `pairs` equal runs.  Of a tile that is cut, the part with its first column is in y
+// [token][N], each later part in the buffer [tile_tok][256] of its pair.
+constexpr int kTcMaxPairs = 80;  // pairs of blocks used at most (74 on 148 SMs)
+constexpr int kTcMaxTileTok = 256;
+struct Product {
+  const float *y, *parts;
+  int32_t N, nk, tile_tok, tok_tiles, total, pairs, shape;  // shape: 16, 32, 64, 128 or 256, the kernel's instance
+  int32_t align;  // a cut lies a multiple of so many stages behind its tile's first (rounded down)
+};
+
+inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *y, const float *parts) {
+  Product pr;
+  pr.y = y;
+  pr.parts = parts;
+  pr.N = N;
+  pr.nk = (C + 63) / 64;
+  // Up to 64 token rows the three terms share an instruction; up to 256 rows are one tile (fewer bytes per
+  // instruction with more rows), more are as many equal tiles as are needed, in steps of 32 rows.
+  pr.shape = n_tok <= 16 ? 16 : (n_tok <= 32 ? 32 : (n_tok <= 64 ? 64 : (n_tok <= 128 ? 128 : 256)));
+  pr.tok_tiles = (n_tok + kTcMaxTileTok - 1) / kTcMaxTileTok;
+  pr.tile_tok = pr.shape <= 64 ? pr.shape : ((n_tok + pr.tok_tiles - 1) / pr.tok_tiles + 31) / 32 * 32;
+  pr.total = (N + 255) / 256 * pr.tok_tiles * pr.nk;
+  // Long jobs are cut where an accumulator's segment ends, so that a tile's segment sums do not depend on the cuts.
+  pr.align = pr.shape == 256 ? 8 : 1;
+  // a pair takes four stages at least, or two segments (small matrices: fewer parts to add)
+  const int most = sm_count / 2 < kTcMaxPairs ? sm_count / 2 : kTcMaxPairs, worth = pr.total / (pr.align > 1 ? 2 * pr.align : 4);
+  pr.pairs = most < worth ? most : worth;
+  if (pr.pairs < 1) pr.pairs = 1;
+  return pr;
+}
+
+#ifdef __CUDACC__
+// First stage of a pair's run.
+__device__ __forceinline__ int product_cut(const Product &pr, int pair) {
+  const int raw = (int)((unsigned)pr.total * (unsigned)pair / (unsigned)pr.pairs);
+  return raw - raw % pr.nk % pr.align;
+}
+// The last pair whose cut, before the rounding, is not behind a stage.
+__device__ __forceinline__ int product_pair(const Product &pr, int stage) {
+  return (int)(((unsigned)(stage + 1) * (unsigned)pr.pairs - 1u) / (unsigned)pr.total);
+}
+// The later parts of row tile `rt`'s sums for token t: parts [first, last) and the offset of row 0 of the tile in part 0.
+struct TileParts {
+  int first, last;
+  size_t at, step;
+};
+__device__ __forceinline__ TileParts product_parts(const Product &pr, int t, int rt) {
+  const int tt = t / pr.tile_tok, u = (rt * pr.tok_tiles + tt) * pr.nk;
+  TileParts tp;
+  tp.first = product_pair(pr, u + min(pr.align, pr.nk) - 1) + 1;  // (cuts that were rounded down to the tile's first stage)
+  tp.last = product_pair(pr, u + pr.nk - 1) + 1;
+  tp.step = (size_t)pr.tile_tok * 256;
+  tp.at = (size_t)(t - tt * pr.tile_tok) * 256;
+  return tp;
+}
+// Y[t][r .. r+3]; r and N multiples of 4.
+__device__ __forceinline__ float4 product_sum4(const Product &pr, int t, int r) {
+  const TileParts tp = product_parts(pr, t, r >> 8);
+  float4 v = *reinterpret_cast<const float4 *>(pr.y + (size_t)t * pr.N + r);
+  for (int p = tp.first; p < tp.last; ++p) {
+    const float4 w = *reinterpret_cast<const float4 *>(pr.parts + p * tp.step + tp.at + (r & 255));
+    v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+  }
+  return v;
+}
+#endif
+
 struct TcJob {
   int32_t L, d, H, hd, f, max_pos, kv_bf16;
   float eps;
   const LayerW *layers;              // HOST copy of the layer table [L]
   const __nv_bfloat16 *tok_emb;
-  const uint8_t *w_tmaps;            // device: tensor maps of the layers' matrices, four per layer
-  const uint8_t *x_tmaps;            // device: tensor maps of the term buffer seen as [3 * x_term_rows][d] and [..][f], boxes of 128 rows;
-                                     // then three more pairs with boxes of 16, 32 and 64 rows (products of a small batch)
+  const uint8_t *w_tmaps;            // device: tensor maps of the layers' matrices, four per layer, then the LM head's
+  const uint8_t *x_tmaps;            // device: tensor maps of the term buffer seen as [3 * x_term_rows][d] and [..][f], in boxes of 8, 16, 32
+                                     // and 64 rows (two each)
   void *kcache, *vcache;
   const float2 *rope;
   float *h, *y, *q;                  // [x_term_rows][d], [x_term_rows][max(3d, 2f)], [x_term_rows][d]
+  float *parts;                      // [kTcMaxPairs][min(x_term_rows, kTcMaxTileTok)][256]: parts of a product's cut tiles
   uint16_t *x;                       // [3][x_term_rows][max(d, f)] bf16 terms
   int32_t x_term_rows;
   const int32_t *ids;                // device: the job's token ids
   int32_t pos0, n_tok;               // first position; tokens (<= x_term_rows)
   State *st;
   int32_t sm_count;                  // SMs of the device
-  size_t y_floats;                   // room of y in floats (partial sums of a column-split product)
-  float *ss;                         // [128][32]: sums of squares of the residual rows per 512-column chunk (jobs of up to 128 tokens)
+  float *ss;                         // [x_term_rows][32]: sums of squares of the residual rows per 512-column chunk
 };
 
 // Words of a request's row in a batched timestep's results (written by the tail kernel, fetched by the host in one copy).
@@ -41,10 +110,14 @@ __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 #endif
 
-// Launch with programmatic stream serialization: the kernel may be brought onto the SMs while the one before it in the
-// stream still runs, and waits there (dep_wait) until that one has completed.  The kernels launched this way start
-// with dep_wait (the small-batch product: before its first read of the terms), so that the launch latency, the
-// set-up of a block and the product's first weight copies overlap the tail of the kernel before.
+// Launch with programmatic stream serialization: the kernel may be brought onto the SMs once every block of the one
+// before it in the stream has said so (dep_launch) or has ended, and waits there (dep_wait) until that one has completed.
+// Every block passes dep_wait before it ends, so a kernel that has completed stands for all before it and the kernels of a
+// chain may be set up several deep; before its dep_wait a block touches only weights and its own shared and tensor memory.
+// No kernel waits for one that cannot start: a block comes onto an SM only when all blocks of the kernel before it have.
+// All kernels say so first thing, so that the next product's first weight copies are under way while the one before
+// drains (8 / 64 requests 3.29 / 4.38 -> 3.19 / 4.30 ms per 7B timestep), but for the rotary embedding: the attention's
+// blocks would be placed while the product still holds most SMs, unevenly (3.49 -> 3.51 ms when it was tried).
 template <typename... P, typename... A>
 inline cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
   cudaLaunchConfig_t cfg = {};
@@ -63,16 +136,16 @@ inline cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_
 }  // namespace spd
 
 extern "C" cudaError_t spd_internal_tc_prepare(void);
+extern "C" cudaError_t spd_internal_job_prepare(void);
 extern "C" cudaError_t spd_internal_tc_stall(const spd::TcJob *job, cudaStream_t stream);
 extern "C" cudaError_t spd_internal_tc_prefill(const spd::TcJob *job, const spd::KParams *head, cudaStream_t stream, int *launches);
-// Row-wise kernels of a job of up to 128 tokens (column-parallel, 1 / rms applied behind the product; spd_batch.cu).
-extern "C" cudaError_t spd_internal_job_input(const spd::TcJob *job, float *ss, cudaStream_t s);
-extern "C" cudaError_t spd_internal_job_rope_cache(const spd::TcJob *job, float *ss, int nz, size_t zs, int layer, cudaStream_t s);
-extern "C" cudaError_t spd_internal_job_resid(const spd::TcJob *job, float *ss, int nz, size_t zs, const __nv_bfloat16 *gain, cudaStream_t s);
-extern "C" cudaError_t spd_internal_job_swiglu(const spd::TcJob *job, float *ss, int nz, size_t zs, cudaStream_t s);
-// The end of a prefix: last residual add, final norm, LM head, KeepTopK and first timestep of one token row (h + the sum of y).
-extern "C" cudaError_t spd_internal_job_head(const spd::KParams *p, const float *h, const float *y, int nz, size_t zs, int sm_count, cudaStream_t s);
-// The product of a batched timestep's few token rows.  dep: launch it so that it may start while the kernel before it
-// in the stream still runs (it then copies weights only, until that kernel has completed).
-extern "C" cudaError_t spd_internal_batch_gemm(const uint8_t *xmaps, int wide, const void *wmap, float *Y, size_t y_floats, int n_tok, int N, int C,
-                                               int x_term_rows, spd::State *st, int sm_count, cudaStream_t s, int dep, int *out_nz, size_t *out_zs);
+// A product of n_tok token rows with matrix `which` of the weights' tensor maps; `wide`: the terms have d_ffn columns.
+extern "C" cudaError_t spd_internal_product(const spd::TcJob *job, int n_tok, int wide, int which, float *Y, int N, spd::Product *out, cudaStream_t s);
+// Row-wise kernels of a job (spd_batch.cu).
+// y null: the rows start as the embeddings of the job's tokens.  normed: the product's terms were whole RMSNorms (spd_internal_job_norm).
+extern "C" cudaError_t spd_internal_job_resid(const spd::TcJob *job, const spd::Product *y, const __nv_bfloat16 *gain, cudaStream_t s);
+extern "C" cudaError_t spd_internal_job_norm(const spd::TcJob *job, const spd::Product *y, const __nv_bfloat16 *gain, cudaStream_t s);
+extern "C" cudaError_t spd_internal_job_rope_cache(const spd::TcJob *job, const spd::Product *y, int normed, int layer, cudaStream_t s);
+extern "C" cudaError_t spd_internal_job_swiglu(const spd::TcJob *job, const spd::Product *y, int normed, cudaStream_t s);
+// The end of a prefix: last residual add, final norm, LM head, KeepTopK and first timestep of one token row (h + y).
+extern "C" cudaError_t spd_internal_job_head(const spd::KParams *p, const float *h, const spd::Product *y, int sm_count, cudaStream_t s);
