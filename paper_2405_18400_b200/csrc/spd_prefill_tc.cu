@@ -549,142 +549,172 @@ __device__ __forceinline__ void tc_split3(float v, uint32_t &hi, uint32_t &mid, 
   lo = __float_as_uint(r1 - __uint_as_float(mid)) & 0xffff0000u;
 }
 
-// Causal attention of 64 consecutive tokens of one head over a bf16 cache, on tensor cores (mma.sync m16n8k16:
+__device__ __forceinline__ void tc_cp16(uint32_t dst, const void *src, uint32_t bytes) {  // 16 bytes, zeros past `bytes` (0 or 16)
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
+// Causal attention of 16 x WARPS consecutive tokens of one head over a bf16 cache, on tensor cores (mma.sync m16n8k16:
 // the attention's share of the arithmetic is small, so the warp-level instructions serve).  Keys and values
 // are bf16 already and therefore exact operands; the scaled queries and the softmax weights are float32 and go
 // in as three bf16 terms each, as the activations of the products do.  A warp owns 16 tokens: scores of a tile of
-// 64 cached positions (tokens x positions, keys read from padded shared-memory rows), online softmax on the
-// accumulator fragments, the weights' terms repacked in registers as the next product's left operand, values
-// through transposing matrix loads.  Rows of every shared-memory tile are 16 bytes longer than their data: eight
-// consecutive rows then start in different bank groups.
-template <int HD>
-__global__ void __launch_bounds__(128) spd_tc_attn_mma_kernel(const float *Q, const uint16_t *kcache, const uint16_t *vcache, uint16_t *X,
-                                                              size_t term_stride, int d, int max_pos, int layer, int pos0, int n_tok) {
+// 64 cached positions (tokens x positions), online softmax on the accumulator fragments, the weights' terms repacked in
+// registers as the next product's left operand, values through transposing matrix loads.  Rows of every shared-memory
+// tile are 16 bytes longer than their data: eight consecutive rows then start in different bank groups.
+// What bounds it: the 384 instructions of a tile and warp; so the next tile's rows travel (cp.async, two buffers) while
+// a tile is multiplied, consecutive instructions go to different accumulators, and tiles wholly behind a warp's tokens
+// skip the mask.  One block per SM: eight warps when 64-token blocks would outnumber the SMs, else four.
+// spd_prefill of 400 / 2048 tokens, 7B shape: 18.9 / 81.4 -> 18.3 / 78.9 ms (before: one tile buffer, two blocks of four
+// warps per SM, three dependent instructions in a row).
+template <int HD, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, 1)
+    spd_tc_attn_mma_kernel(const float *Q, const uint16_t *kcache, const uint16_t *vcache, uint16_t *X, size_t term_stride, int d, int max_pos,
+                           int layer, int pos0, int n_tok) {
   dep_launch();
   dep_wait();
-  constexpr int kTok = 64, kPos = 64;
+  constexpr int kTok = 16 * WARPS, kPos = 64, kThr = WARPS * 32;
   constexpr int RS = HD * 2 + 16;  // bytes per tile row
   constexpr int KS = HD / 16;      // k-steps over the head's dimensions
   constexpr int DT = HD / 8;       // output tiles of 8 dimensions
+  constexpr int kBuf = 2 * kPos * RS;
   extern __shared__ __align__(16) uint8_t at_smem[];
-  uint8_t *sq = at_smem;                // [3 terms][64 tokens][RS]
-  uint8_t *sk = sq + 3 * kTok * RS;     // [64 positions][RS]
-  uint8_t *sv = sk + kPos * RS;
+  const uint32_t sq_u = smem_u32(at_smem);            // [3 terms][tokens][RS]
+  const uint32_t kv_u = sq_u + 3 * kTok * RS;         // two buffers of [64 positions][RS] keys, then values
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q = lane & 3;
   const int head = blockIdx.y, t0 = blockIdx.x * kTok;
-  const float scale = 1.f / sqrtf((float)HD);
-  for (int i = tid; i < kTok * HD; i += 128) {
-    const int tt = i / HD, c = i - tt * HD;
-    const float v = t0 + tt < n_tok ? Q[(size_t)(t0 + tt) * d + head * HD + c] * scale : 0.f;
-    uint32_t hi, mid, lo;
-    tc_split3(v, hi, mid, lo);
-    uint16_t *dst = reinterpret_cast<uint16_t *>(sq + tt * RS) + c;
-    dst[0] = (uint16_t)(hi >> 16);
-    dst[kTok * RS / 2] = (uint16_t)(mid >> 16);
-    dst[2 * kTok * RS / 2] = (uint16_t)(lo >> 16);
-  }
   const int last_pos = pos0 + min(t0 + kTok - 1, n_tok - 1);  // the last position a token of this block sees
+  auto fetch = [&](int tile0, int buf) {
+    const uint32_t dst = kv_u + (uint32_t)(buf * kBuf);
+    for (int i = tid; i < kPos * HD / 8; i += kThr) {
+      const int r = i / (HD / 8), c8 = i - r * (HD / 8), pos = tile0 + r;
+      const size_t at = ((size_t)layer * max_pos + min(pos, last_pos)) * d + head * HD + c8 * 8;
+      const uint32_t bytes = pos <= last_pos ? 16u : 0u, off = (uint32_t)(r * RS + c8 * 16);
+      tc_cp16(dst + off, kcache + at, bytes);
+      tc_cp16(dst + kPos * RS + off, vcache + at, bytes);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  fetch(0, 0);
+  const float scale = 1.f / sqrtf((float)HD);
+  for (int i = tid; i < kTok * HD / 4; i += kThr) {
+    const int tt = i / (HD / 4), c = (i - tt * (HD / 4)) * 4;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (t0 + tt < n_tok) v = *reinterpret_cast<const float4 *>(Q + (size_t)(t0 + tt) * d + head * HD + c);
+    uint32_t h[4], m[4], l[4];
+    tc_split3(v.x * scale, h[0], m[0], l[0]);
+    tc_split3(v.y * scale, h[1], m[1], l[1]);
+    tc_split3(v.z * scale, h[2], m[2], l[2]);
+    tc_split3(v.w * scale, h[3], m[3], l[3]);
+    uint8_t *dst = at_smem + tt * RS + c * 2;
+    *reinterpret_cast<uint2 *>(dst) = make_uint2(h[1] | (h[0] >> 16), h[3] | (h[2] >> 16));
+    *reinterpret_cast<uint2 *>(dst + kTok * RS) = make_uint2(m[1] | (m[0] >> 16), m[3] | (m[2] >> 16));
+    *reinterpret_cast<uint2 *>(dst + 2 * kTok * RS) = make_uint2(l[1] | (l[0] >> 16), l[3] | (l[2] >> 16));
+  }
   const int tw = t0 + warp * 16;
-  const int p_lo = pos0 + tw + g, p_hi = p_lo + 8, warp_last = pos0 + tw + 15;
+  const int p_first = pos0 + tw, p_lo = p_first + g, p_hi = p_lo + 8, warp_last = p_first + 15;
   float m[2] = {-CUDART_INF_F, -CUDART_INF_F}, l[2] = {0.f, 0.f};
   float o[DT][4];
 #pragma unroll
   for (int i = 0; i < DT; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
-  const uint32_t sq_u = smem_u32(sq), sk_u = smem_u32(sk), sv_u = smem_u32(sv);
-  // per-lane offsets: left operand (tokens x dimensions), keys (32-bit words), values (transposed matrices)
-  const uint32_t a_off = (uint32_t)((warp * 16 + (lane & 7) + ((lane >> 3) & 1) * 8) * RS + (lane >> 4) * 16);
-  const uint32_t k_off = (uint32_t)(g * RS + q * 4);
-  const uint32_t v_off = (uint32_t)((((lane >> 3) & 1) * 8 + (lane & 7)) * RS + (lane >> 4) * 16);
-  for (int tile0 = 0; tile0 <= last_pos; tile0 += kPos) {
-    __syncthreads();  // the previous tile has been used; first round: the queries are in place after the next barrier
-    for (int i = tid; i < kPos * HD / 8; i += 128) {
-      const int r = i / (HD / 8), c8 = i - r * (HD / 8);
-      const int pos = tile0 + r;
-      uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
-      if (pos <= last_pos) {
-        const size_t at = ((size_t)layer * max_pos + pos) * d + head * HD + c8 * 8;
-        a = *reinterpret_cast<const uint4 *>(kcache + at);
-        b = *reinterpret_cast<const uint4 *>(vcache + at);
-      }
-      *reinterpret_cast<uint4 *>(sk + r * RS + c8 * 16) = a;
-      *reinterpret_cast<uint4 *>(sv + r * RS + c8 * 16) = b;
+  // per-lane offsets: left operand (tokens x dimensions), keys (two tiles of 8 positions x 16 dimensions), values (transposed)
+  const uint32_t a_off = sq_u + (uint32_t)((warp * 16 + (lane & 7) + ((lane >> 3) & 1) * 8) * RS + (lane >> 4) * 16);
+  const uint32_t k_off = (uint32_t)(((lane >> 4) * 8 + (lane & 7)) * RS + ((lane >> 3) & 1) * 16);
+  const uint32_t v_off = (uint32_t)((((lane >> 3) & 1) * 8 + (lane & 7)) * RS + (lane >> 4) * 16 + kPos * RS);
+  int buf = 0;
+  for (int tile0 = 0; tile0 <= last_pos; tile0 += kPos, buf ^= 1) {
+    if (tile0 + kPos <= last_pos) {
+      fetch(tile0 + kPos, buf ^ 1);  // (every warp has left that buffer: the barrier at the end of the round)
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
-    __syncthreads();
-    if (tile0 > warp_last) continue;  // nothing of this tile is visible to the warp's tokens (the barriers are above)
-    float s[kPos / 8][4];
+    __syncthreads();  // the tile (first round: and the queries) is in place for all
+    if (tile0 <= warp_last) {  // else nothing of this tile is visible to the warp's tokens
+      const uint32_t sk_u = kv_u + (uint32_t)(buf * kBuf);
+      float s[kPos / 8][4];
 #pragma unroll
-    for (int i = 0; i < kPos / 8; ++i) s[i][0] = s[i][1] = s[i][2] = s[i][3] = 0.f;
+      for (int i = 0; i < kPos / 8; ++i) s[i][0] = s[i][1] = s[i][2] = s[i][3] = 0.f;
 #pragma unroll
-    for (int ks = 0; ks < KS; ++ks) {
-      uint32_t a[3][4];
+      for (int ks = 0; ks < KS; ++ks) {
+        uint32_t kb[kPos / 16][4];
 #pragma unroll
-      for (int j = 0; j < 3; ++j) tc_ldsm_x4(sq_u + (uint32_t)(j * kTok * RS) + a_off + (uint32_t)(ks * 32), a[j]);
-#pragma unroll
-      for (int nt = 0; nt < kPos / 8; ++nt) {
-        uint32_t b0, b1;
-        const uint32_t addr = sk_u + k_off + (uint32_t)(nt * 8 * RS + ks * 32);
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b0) : "r"(addr));
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b1) : "r"(addr + 16));
-#pragma unroll
-        for (int j = 0; j < 3; ++j) tc_mma_sync(s[nt], a[j], b0, b1);
-      }
-    }
-    // causal mask, row maxima (rows g and g + 8 of the warp's 16 tokens; a row lives in the four lanes of a quad)
-    float mx[2] = {-CUDART_INF_F, -CUDART_INF_F};
-#pragma unroll
-    for (int nt = 0; nt < kPos / 8; ++nt)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int pos = tile0 + nt * 8 + 2 * q + (e & 1);
-        if (pos > (e < 2 ? p_lo : p_hi)) s[nt][e] = -CUDART_INF_F;
-        mx[e >> 1] = fmaxf(mx[e >> 1], s[nt][e]);
-      }
-    float c[2];
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
-      mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
-      const float mn = fmaxf(m[r], mx[r]);  // finite: position 0 is visible to every token in the first tile
-      c[r] = __expf(m[r] - mn);
-      m[r] = mn;
-      l[r] *= c[r];
-    }
-#pragma unroll
-    for (int i = 0; i < DT; ++i) {
-      o[i][0] *= c[0]; o[i][1] *= c[0]; o[i][2] *= c[1]; o[i][3] *= c[1];
-    }
-    // the weights and their terms, repacked as left operands: positions 16 kk .. 16 kk + 15 are score tiles 2 kk, 2 kk + 1
-    uint32_t pt[kPos / 16][3][4];
-#pragma unroll
-    for (int nt = 0; nt < kPos / 8; ++nt) {
-      float pw[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) pw[e] = __expf(s[nt][e] - m[e >> 1]);
-      l[0] += pw[0] + pw[1];
-      l[1] += pw[2] + pw[3];
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        uint32_t h0, m0, l0, h1, m1, l1;
-        tc_split3(pw[2 * r], h0, m0, l0);
-        tc_split3(pw[2 * r + 1], h1, m1, l1);
-        const int reg = (nt & 1) * 2 + r;
-        pt[nt >> 1][0][reg] = h1 | (h0 >> 16);
-        pt[nt >> 1][1][reg] = m1 | (m0 >> 16);
-        pt[nt >> 1][2][reg] = l1 | (l0 >> 16);
-      }
-    }
-#pragma unroll
-    for (int kk = 0; kk < kPos / 16; ++kk)
-#pragma unroll
-      for (int dp = 0; dp < DT / 2; ++dp) {
-        uint32_t b[4];
-        tc_ldsm_x4_trans(sv_u + v_off + (uint32_t)(kk * 16 * RS + dp * 32), b);
+        for (int np = 0; np < kPos / 16; ++np) tc_ldsm_x4(sk_u + k_off + (uint32_t)(np * 16 * RS + ks * 32), kb[np]);
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-          tc_mma_sync(o[2 * dp], pt[kk][j], b[0], b[1]);
-          tc_mma_sync(o[2 * dp + 1], pt[kk][j], b[2], b[3]);
+          uint32_t a[4];
+          tc_ldsm_x4(a_off + (uint32_t)(j * kTok * RS + ks * 32), a);
+#pragma unroll
+          for (int np = 0; np < kPos / 16; ++np) {
+            tc_mma_sync(s[2 * np], a, kb[np][0], kb[np][1]);
+            tc_mma_sync(s[2 * np + 1], a, kb[np][2], kb[np][3]);
+          }
         }
       }
+      // causal mask, row maxima (rows g and g + 8 of the warp's 16 tokens; a row lives in the four lanes of a quad)
+      if (tile0 + kPos - 1 > p_first) {
+#pragma unroll
+        for (int nt = 0; nt < kPos / 8; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int pos = tile0 + nt * 8 + 2 * q + (e & 1);
+            if (pos > (e < 2 ? p_lo : p_hi)) s[nt][e] = -CUDART_INF_F;
+          }
+      }
+      float mx[2] = {-CUDART_INF_F, -CUDART_INF_F};
+#pragma unroll
+      for (int nt = 0; nt < kPos / 8; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) mx[e >> 1] = fmaxf(mx[e >> 1], s[nt][e]);
+      float c[2];
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
+        mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
+        const float mn = fmaxf(m[r], mx[r]);  // finite: position 0 is visible to every token in the first tile
+        c[r] = __expf(m[r] - mn);
+        m[r] = mn;
+        l[r] *= c[r];
+      }
+#pragma unroll
+      for (int i = 0; i < DT; ++i) {
+        o[i][0] *= c[0]; o[i][1] *= c[0]; o[i][2] *= c[1]; o[i][3] *= c[1];
+      }
+      // per 16 positions: the weights and their terms, repacked as the left operand, times the values
+#pragma unroll
+      for (int kk = 0; kk < kPos / 16; ++kk) {
+        uint32_t pt[3][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float pw[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) pw[e] = __expf(s[2 * kk + h][e] - m[e >> 1]);
+          l[0] += pw[0] + pw[1];
+          l[1] += pw[2] + pw[3];
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            uint32_t h0, m0, l0, h1, m1, l1;
+            tc_split3(pw[2 * r], h0, m0, l0);
+            tc_split3(pw[2 * r + 1], h1, m1, l1);
+            pt[0][h * 2 + r] = h1 | (h0 >> 16);
+            pt[1][h * 2 + r] = m1 | (m0 >> 16);
+            pt[2][h * 2 + r] = l1 | (l0 >> 16);
+          }
+        }
+#pragma unroll
+        for (int dq = 0; dq < DT / 2; dq += 4) {
+          uint32_t vb[4][4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) tc_ldsm_x4_trans(sk_u + v_off + (uint32_t)(kk * 16 * RS + (dq + i) * 32), vb[i]);
+#pragma unroll
+          for (int j = 0; j < 3; ++j)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              tc_mma_sync(o[2 * (dq + i)], pt[j], vb[i][0], vb[i][1]);
+              tc_mma_sync(o[2 * (dq + i) + 1], pt[j], vb[i][2], vb[i][3]);
+            }
+        }
+      }
+    }
+    __syncthreads();  // the tile's buffer may be filled again
   }
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
@@ -695,9 +725,17 @@ __global__ void __launch_bounds__(128) spd_tc_attn_mma_kernel(const float *Q, co
 #pragma unroll
   for (int i = 0; i < DT; ++i)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int t = tw + g + (e >> 1) * 8;
-      if (t < n_tok) tc_put3(X, term_stride, (size_t)t * d + head * HD + i * 8 + 2 * q + (e & 1), o[i][e] * inv[e >> 1]);
+    for (int r = 0; r < 2; ++r) {
+      const int t = tw + g + r * 8;
+      if (t < n_tok) {
+        uint32_t h0, m0, l0, h1, m1, l1;
+        tc_split3(o[i][2 * r] * inv[r], h0, m0, l0);
+        tc_split3(o[i][2 * r + 1] * inv[r], h1, m1, l1);
+        uint16_t *dst = X + (size_t)t * d + head * HD + i * 8 + 2 * q;
+        *reinterpret_cast<uint32_t *>(dst) = h1 | (h0 >> 16);
+        *reinterpret_cast<uint32_t *>(dst + term_stride) = m1 | (m0 >> 16);
+        *reinterpret_cast<uint32_t *>(dst + 2 * term_stride) = l1 | (l0 >> 16);
+      }
     }
 }
 
@@ -705,18 +743,27 @@ __global__ void __launch_bounds__(128) spd_tc_attn_mma_kernel(const float *Q, co
 
 namespace {
 
-template <int HD>
-constexpr size_t attn_mma_smem() { return (size_t)5 * 64 * (HD * 2 + 16); }  // three query terms, keys, values: 64 padded rows each
+template <int HD, int WARPS>
+constexpr size_t attn_mma_smem() { return (size_t)(3 * 16 * WARPS + 4 * 64) * (HD * 2 + 16); }  // query terms; two buffers of keys and values
+
+template <int HD, int WARPS>
+cudaError_t launch_attn_mma(const spd::TcJob &j, int layer, int n_tok, cudaStream_t s) {
+  return spd::launch_dep(spd::spd_tc_attn_mma_kernel<HD, WARPS>, dim3((n_tok + 16 * WARPS - 1) / (16 * WARPS), j.H), dim3(WARPS * 32),
+                         attn_mma_smem<HD, WARPS>(), s, j.q, static_cast<const uint16_t *>(j.kcache), static_cast<const uint16_t *>(j.vcache), j.x,
+                         (size_t)j.x_term_rows * j.d, j.d, j.max_pos, layer, j.pos0, n_tok);
+}
 
 template <int HD>
 cudaError_t launch_attn(const spd::TcJob &j, int layer, int n_tok, cudaStream_t s) {
-  const size_t ts = (size_t)j.x_term_rows * j.d;
-  if (j.kv_bf16)
-    return spd::launch_dep(spd::spd_tc_attn_mma_kernel<HD>, dim3((n_tok + 63) / 64, j.H), dim3(128), attn_mma_smem<HD>(), s, j.q,
-                           static_cast<const uint16_t *>(j.kcache), static_cast<const uint16_t *>(j.vcache), j.x, ts, j.d, j.max_pos, layer, j.pos0,
-                           n_tok);
+  if (j.kv_bf16) return (n_tok + 63) / 64 * j.H > j.sm_count ? launch_attn_mma<HD, 8>(j, layer, n_tok, s) : launch_attn_mma<HD, 4>(j, layer, n_tok, s);
   return spd::launch_dep(spd::spd_tc_attn_kernel<HD>, dim3((n_tok + 15) / 16, j.H), dim3(256), 0, s, j.q, static_cast<const float *>(j.kcache),
-                         static_cast<const float *>(j.vcache), j.x, ts, j.d, j.max_pos, layer, j.pos0, n_tok);
+                         static_cast<const float *>(j.vcache), j.x, (size_t)j.x_term_rows * j.d, j.d, j.max_pos, layer, j.pos0, n_tok);
+}
+
+template <int HD, int WARPS>
+cudaError_t allow_attn_smem() {
+  return cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_tc_attn_mma_kernel<HD, WARPS>), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)attn_mma_smem<HD, WARPS>());
 }
 
 template <int NT>
@@ -742,12 +789,10 @@ extern "C" cudaError_t spd_internal_tc_prepare(void) {
   if (e == cudaSuccess) e = allow_product_smem<64>();
   if (e == cudaSuccess) e = allow_product_smem<128>();
   if (e == cudaSuccess) e = allow_product_smem<256>();
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_tc_attn_mma_kernel<64>), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)attn_mma_smem<64>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_tc_attn_mma_kernel<128>), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)attn_mma_smem<128>());
+  if (e == cudaSuccess) e = allow_attn_smem<64, 4>();
+  if (e == cudaSuccess) e = allow_attn_smem<64, 8>();
+  if (e == cudaSuccess) e = allow_attn_smem<128, 4>();
+  if (e == cudaSuccess) e = allow_attn_smem<128, 8>();
   return e;
 }
 
