@@ -234,7 +234,7 @@ def run_batched(args, wl, P, dev, rank, world, packed, dtabs, k, K, W):
            "ms_per_step": ms / K, "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "bf16", "data": "synthetic",
            "config": cfg,
            "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "traffic": None,
-                        "peak_kind": peak_kind, "bytes_per_step": bytes_step, "kernel": "spd_batch_gemm_kernel",
+                        "peak_kind": peak_kind, "bytes_per_step": bytes_step, "kernel": "spd_tc_product_kernel",
                         "note": "weights once per timestep + per request its KV cache, embedding rows and table probes; the time is "
                                 "the whole timestep's (the products are about 70 % of it)"},
            "e2e": e2e, "gpu_launches": int(launches), "clocks": clocks, "batch": B}
@@ -341,8 +341,8 @@ def run_ours(args, wl):
         e2e_s = max_over_ranks(e2e_s, dev, world)
     e2e = {"value": world * k * gen / e2e_s if e2e_s else None, "unit": UNIT, "h2d_bytes_per_step": 4.0 * wl.prefix_len / gen,
            "d2h_bytes_per_step": 12.0 * k, "what": "spd_prefill(host ids) + %d spd_step calls returning ids, parents and gamma "
-           "to the host, per request of %d tokens per draft; prefill = one launch of the batched kernel per 16 prefix tokens, the last one ending with the LM head and the first timestep; "
-           "prefixes over 32 tokens send all but their last 1..16 tokens through the tcgen05 long-prefix path" % (gen - 1, gen),
+           "to the host, per request of %d tokens per draft; prefill = jobs of up to 512 tokens on tcgen05 products, the last one ending with the LM head and the first timestep "
+           "(up to 16 tokens of a small model: one launch of the 16-token kernel)" % (gen - 1, gen),
            "ms_per_request": e2e_s * 1e3 if e2e_s else None,
            "ms_to_first_drafts": min(first_t) * 1e3 if first_t else None}
 
@@ -359,7 +359,7 @@ def run_ours(args, wl):
             torch.cuda.synchronize()
             ts.append(e0.elapsed_time(e1))
         pf_ms = max_over_ranks(float(np.median(ts)), dev, world)
-        n_tc = wl.prefix_len - ((wl.prefix_len - 1) % 16 + 1)
+        n_tc = wl.prefix_len
         sh = wl.shape
         layer_params = sh.n_layers * (4 * sh.d_model * sh.d_model + 3 * sh.d_model * sh.d_ffn)
         tflop = n_tc * layer_params * 2 / 1e12           # the method's own arithmetic: tokens x weights x 2
@@ -367,8 +367,7 @@ def run_ours(args, wl):
         prefill_rec = {"ms": pf_ms, "tokens": wl.prefix_len, "tokens_through_tcgen05_products": n_tc, "bound": "tensor",
                        "achieved": tflop / (pf_ms * 1e-3), "peak": tpeak, "unit": "TFLOP/s", "frac": tflop / (pf_ms * 1e-3) / tpeak,
                        "peak_kind": tkind, "issued_tflops": 3 * tflop / (pf_ms * 1e-3), "issued_frac": 3 * tflop / (pf_ms * 1e-3) / tpeak,
-                       "note": "whole spd_prefill call (products, attention, row-wise kernels, the last tokens' launch of the 16-token "
-                               "kernel with LM head and first timestep); achieved / frac count the method's arithmetic (tokens x layer "
+                       "note": "whole spd_prefill call (products, attention, row-wise kernels, LM head and first timestep); achieved / frac count the method's arithmetic (tokens x layer "
                                "weights x 2); issued_* count what the tensor cores execute, three bf16 terms per float32 activation"}
 
     # ---- the same number of drafts from k separate single-draft passes through the same kernels
