@@ -193,7 +193,8 @@ __global__ void __launch_bounds__(256) spd_job_norm_kernel(float *h, const __gri
 // Columns c .. c+3 of one token row: the QKV product's row [q | k | v] times 1 / rms, rotary embedding of q and k
 // (adjacent pairs) at position pos, q to Q, k and v into the cache.
 __device__ __forceinline__ float4 bt_rotate(const float4 &x, const float4 &cs) {  // cs = (cos, sin) of the two pairs
-  return make_float4(x.x * cs.x - x.y * cs.y, x.x * cs.y + x.y * cs.x, x.z * cs.z - x.w * cs.w, x.z * cs.w + x.w * cs.z);
+  return make_float4(__fmaf_rn(x.x, cs.x, -__fmul_rn(x.y, cs.y)), __fmaf_rn(x.x, cs.y, __fmul_rn(x.y, cs.x)),
+                     __fmaf_rn(x.z, cs.z, -__fmul_rn(x.w, cs.w)), __fmaf_rn(x.z, cs.w, __fmul_rn(x.w, cs.z)));
 }
 __device__ __forceinline__ void bt_store_kv(void *cache, int kv_bf16, size_t at, const float4 &v) {
   if (kv_bf16) {

@@ -26,16 +26,18 @@ inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *
   pr.parts = parts;
   pr.N = N;
   pr.nk = (C + 63) / 64;
-  // Up to 64 token rows the three terms share an instruction; up to 256 rows are one tile (fewer bytes per
-  // instruction with more rows), more are as many equal tiles as are needed, in steps of 32 rows.
-  pr.shape = n_tok <= 16 ? 16 : (n_tok <= 32 ? 32 : (n_tok <= 64 ? 64 : (n_tok <= 128 ? 128 : 256)));
-  pr.tok_tiles = (n_tok + kTcMaxTileTok - 1) / kTcMaxTileTok;
+  // Up to 64 token rows the three terms share an instruction; up to 256 rows are one tile; more rows make enough tiles of
+  // up to 128 (in steps of 32 rows, all alike) to fill the pairs without cutting one: then every sum is one pair's.
+  // Between 129 and 256 rows tiles are cut, where an accumulator's segment ends.
+  const bool whole = n_tok > kTcMaxTileTok;
+  pr.shape = n_tok <= 16 ? 16 : (n_tok <= 32 ? 32 : (n_tok <= 64 ? 64 : (n_tok <= 128 || whole ? 128 : 256)));
+  pr.tok_tiles = whole ? (n_tok + 127) / 128 : 1;
   pr.tile_tok = pr.shape <= 64 ? pr.shape : ((n_tok + pr.tok_tiles - 1) / pr.tok_tiles + 31) / 32 * 32;
   pr.total = (N + 255) / 256 * pr.tok_tiles * pr.nk;
-  // Long jobs are cut where an accumulator's segment ends, so that a tile's segment sums do not depend on the cuts.
-  pr.align = pr.shape == 256 ? 8 : 1;
-  // a pair takes four stages at least, or two segments (small matrices: fewer parts to add)
-  const int most = sm_count / 2 < kTcMaxPairs ? sm_count / 2 : kTcMaxPairs, worth = pr.total / (pr.align > 1 ? 2 * pr.align : 4);
+  pr.align = whole ? pr.nk : (pr.shape == 256 ? 8 : 1);
+  // a pair takes a tile, two segments or four stages at least (small matrices: fewer parts to add)
+  const int least = whole ? pr.nk : (pr.align > 1 ? 2 * pr.align : 4);
+  const int most = sm_count / 2 < kTcMaxPairs ? sm_count / 2 : kTcMaxPairs, worth = pr.total / least;
   pr.pairs = most < worth ? most : worth;
   if (pr.pairs < 1) pr.pairs = 1;
   return pr;
