@@ -110,8 +110,11 @@ __device__ __forceinline__ void tc_pair_commit(uint64_t *bar) {
                "h"((uint16_t)3)
                : "memory");
 }
+// Arrival of a warp that has read an accumulator (tcgen05.wait::ld, tcgen05.fence::before_thread_sync): nothing written
+// to memory hangs on it, so it is relaxed.  As a release it waits for the warp's stores to memory, about half a microsecond of the
+// issuing thread's time per segment: 15 tokens, 7B shape, segments of 4 stages, 3.65 ms against 3.32.
 __device__ __forceinline__ void tc_cluster_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 struct TcShared {
@@ -162,9 +165,11 @@ __device__ __forceinline__ bool tc_wait(TcShared &sh, State *st, uint64_t *bar, 
 // four products of a layer 91 us for 62; about 8 us of each are start and end, which the dependent launches hide in part).
 // Tried: asking the weights behind the first ring into L2 before dep_wait (8 to 32 stages): 2 to 5 % slower.
 //
-// Accumulation: an accumulator takes the sums of a segment of stages (96 additions), then moves to registers, where the
+// Accumulation: an accumulator takes the sums of a segment of stages (pr.seg), then moves to registers, where the
 // segments are added with round-to-nearest: the tensor cores add into their accumulator with truncation, whose error grows
-// with the length of the chain.
+// with the length of the chain.  First timestep's largest logit error, 7B shape, float32 cache, against 64 bits: 15 / 64 / 100 /
+// 200 tokens 2.0e-5 / 2.4e-5 / 5.1e-5 / 5.2e-5 (segments of 24 stages, 8 from 65 rows on: 8.0e-5 / 9.6e-5 / 1.2e-4 / 1.4e-4; the
+// 16-token kernel 1.3e-4), in the same time.
 //
 // tmap_x: the term tiles, a [3 * x_term_rows][C] bf16 matrix in boxes of kBoxRows rows x 64 columns (term j's tokens start
 // at row j * x_term_rows); tmap_w: W [N][C] in boxes of 32 rows x 64 columns; rows and columns past either matrix arrive as
@@ -185,7 +190,6 @@ struct TcShape {
   static constexpr int kStages = NT == 16 ? 10 : (NT == 32 ? 9 : (NT == 64 ? 7 : (NT == 128 ? 5 : 3)));  // 192 - 200 KB
   static constexpr int kAccs = NT == 64 || NT == 256 ? 2 : 4;
   static constexpr int kAccStride = 512 / kAccs;                        // columns from one accumulator set to the next
-  static constexpr int kSegSteps = kFused ? 24 : 8;
   static constexpr int kHalf = NT / 2;                                  // tokens whose sums one epilogue thread holds
   static constexpr int kLd = kFused && NT == 16 ? 8 : 16;               // columns per tensor-memory load
   static constexpr size_t kSmem = (size_t)kStages * kStageBytes + 1024;
@@ -305,16 +309,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
         if (!tc_wait(sh, st, &sh.full[stage], phase, 410)) break;
         tc_fence_after();
         const uint32_t base = ring + stage * (uint32_t)S::kStageBytes, acc = tmem + (uint32_t)(a * S::kAccStride);
+        const uint32_t term0 = base + kTcWBytes + (!S::kFused && pr.small_first ? 2 * S::kTermBytes : 0);
+        const int term_step = pr.small_first ? -S::kTermBytes : S::kTermBytes;
 #pragma unroll
         for (int j = 0; j < (S::kFused ? 1 : 3); ++j)
 #pragma unroll
           for (int kk = 0; kk < kTcKB / 16; ++kk)  // 16 columns = 32 bytes further into the swizzled rows
-            tc_pair_mma(acc, tc_desc(base + kk * 32), tc_desc(base + kTcWBytes + j * S::kTermBytes + kk * 32), idesc,
-                        (uint32_t)((in_seg | j | kk) != 0));
+            tc_pair_mma(acc, tc_desc(base + kk * 32), tc_desc(term0 + j * term_step + kk * 32), idesc, (uint32_t)((in_seg | j | kk) != 0));
         tc_pair_commit(&sh.empty[stage]);  // the stage is free in both blocks once these have read it
         if (++stage == (uint32_t)S::kStages) { stage = 0; phase ^= 1u; }
         ++kb;
-        if (++in_seg == S::kSegSteps || kb == pr.nk || u + 1 == u1) {
+        if (++in_seg == pr.seg || kb == pr.nk || u + 1 == u1) {
           tc_pair_commit(&sh.acc_full[a]);  // the segment's sum is complete
           ++seg;
           in_seg = 0;
@@ -336,16 +341,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
       float sum[S::kHalf];
 #pragma unroll
       for (int j = 0; j < S::kHalf; ++j) sum[j] = 0.f;
-      for (int done = 0; done < stages; done += S::kSegSteps, ++seg) {
+      for (int done = 0; done < stages; done += pr.seg, ++seg) {
         const int a = seg % S::kAccs;
         if (!tc_wait(sh, st, &sh.acc_full[a], (uint32_t)((seg / S::kAccs) & 1), 420)) { ok = false; break; }
         tc_fence_after();
         const uint32_t acc = lanes + (uint32_t)(a * S::kAccStride);
         if constexpr (S::kFused) {
-          // a half's columns: its tokens' first terms, second terms, third terms
+          // a half's columns: its tokens' first terms, second terms, third terms; the small ones are added first (one load
+          // in flight: with three of 16 columns 64 tokens took 4.29 ms instead of 4.15)
           const uint32_t from = acc + (uint32_t)(half * (S::kCols / 2));
 #pragma unroll
-          for (int c0 = 0; c0 < 3 * S::kHalf; c0 += S::kLd) {
+          for (int c0 = 3 * S::kHalf - S::kLd; c0 >= 0; c0 -= S::kLd) {
             uint32_t r[S::kLd];
             tc_ld(from + (uint32_t)c0, r);
             tc_ld_wait();

@@ -18,6 +18,8 @@ struct Product {
   const float *y, *parts;
   int32_t N, nk, tile_tok, tok_tiles, total, pairs, shape;  // shape: 16, 32, 64, 128 or 256, the kernel's instance
   int32_t align;  // a cut lies a multiple of so many stages behind its tile's first (rounded down)
+  int32_t seg;    // stages whose sums an accumulator takes before they move to registers
+  int32_t small_first;  // one instruction per term: a stage's small terms before the large one
 };
 
 inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *y, const float *parts) {
@@ -35,6 +37,14 @@ inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *
   pr.tile_tok = pr.shape <= 64 ? pr.shape : ((n_tok + pr.tok_tiles - 1) / pr.tok_tiles + 31) / 32 * 32;
   pr.total = (N + 255) / 256 * pr.tok_tiles * pr.nk;
   pr.align = whole ? pr.nk : (pr.shape == 256 ? 8 : 1);
+  // The accumulators add with truncation, so the error grows with the additions between two moves to registers: 4 per stage
+  // and accumulator where every term has its own (up to 64 rows), 12 where the terms share one (small ones first: 4 at the
+  // sum's own size).  4 stages cost nothing (2: 1 % at 15 tokens, 3 % at 64; 1: 2 % and 10 %), and where the terms share one
+  // never more than the 3 C / 128 additions that a warp of the 16-token kernel chains.  Uncut tiles of wide matrices keep up to
+  // 8 stages, the terms in order: behind long prefixes a bf16 cache then holds the bits that it always has.
+  const int most_seg = whole ? 8 : 4;
+  pr.seg = pr.shape <= 64 ? 4 : (C < 512 ? 1 : (C / 512 < most_seg ? C / 512 : most_seg));
+  pr.small_first = pr.seg < 8;
   // a pair takes a tile, two segments or four stages at least (small matrices: fewer parts to add)
   const int least = whole ? pr.nk : (pr.align > 1 ? 2 * pr.align : 4);
   const int most = sm_count / 2 < kTcMaxPairs ? sm_count / 2 : kTcMaxPairs, worth = pr.total / least;
