@@ -135,7 +135,7 @@ static __device__ void tail_score_select(Blk &b, bool first, int step) {
           if (bi < 0 || ranks_before(z, c, bv, bi)) { bv = z; bi = c; }
         }
         warp_best(bv, bi);
-        if (lane == r) { my_sel = bi; my_score = bv; }
+        if (lane == r) { my_sel = max(bi, 0); my_score = bv; }  // NaN scores can leave a round without a winner: keep the option valid
         pv = bv;
         pi = bi;
       }

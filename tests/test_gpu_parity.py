@@ -518,3 +518,14 @@ def test_image_and_row_major_paths_agree_at_7b_width():
     assert np.array_equal(out[0][0], out[1][0])
     assert np.abs(out[0][3] - out[1][3]).max() < 1e-4
     assert np.abs(out[0][2] - out[1][2]).max() < 1e-4
+
+
+@pytest.mark.parametrize("k", [2, 16])
+def test_scores_that_are_not_numbers_still_choose_existing_options(tiny_inputs, k):
+    """With NaN scores no option ranks before another after the first round; every draft still continues an existing one."""
+    ctx, _ = make_tiny_pair(tiny_inputs, k=k)
+    hist = np.zeros((k, 4), np.int32)
+    ctx.spd_debug_score(hist, np.full(k, np.nan, np.float32), np.arange(k, dtype=np.int32), np.zeros(k, np.float32))
+    sel = ctx.spd_debug_read("SEL")
+    assert sel.min() >= 0 and sel.max() < k * k
+    ctx.close()
