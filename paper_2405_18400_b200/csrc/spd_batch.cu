@@ -301,6 +301,7 @@ __device__ void ba_head(const float *q_row, const E *kc, const E *vc, int d, int
 #pragma unroll
     for (int u = 0; u < kBaFlight; ++u) vq[u] = *reinterpret_cast<const uint4 *>(vc + (size_t)min(tb + u * G + group, T - 1) * d + at);
     float sc[kBaFlight], mn = m;
+    bool any = false;
 #pragma unroll
     for (int u = 0; u < kBaFlight; ++u) {
       float kx[EPL], dot = 0.f;
@@ -311,8 +312,9 @@ __device__ void ba_head(const float *q_row, const E *kc, const E *vc, int d, int
       for (int o = LP / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
       sc[u] = tb + u * G + group < T ? dot * scale : -CUDART_INF_F;
       mn = fmaxf(mn, sc[u]);
+      any |= sc[u] != -CUDART_INF_F;
     }
-    if (mn > -CUDART_INF_F) {  // else no position so far belongs to this group
+    if (any) {  // else no position of this round belongs to the group (a NaN score, which fmaxf passes over, has to reach the sums)
       const float c = __expf(m - mn);
       l *= c;
 #pragma unroll

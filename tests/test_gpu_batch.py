@@ -125,3 +125,38 @@ def test_batch_argument_checks(tiny_inputs):
     assert a.spd_debug_read("CAND_TOK").tolist() == small.spd_debug_read("CAND_TOK").tolist()
     for c in (a, b, small, stopper):
         c.close()
+
+
+@pytest.mark.parametrize("kv_dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("heads,k", [(4, 3), (2, 16)])
+def test_a_nan_in_the_cache_reaches_the_logits(heads, k, kv_dtype):
+    """A damaged cache row is not left out of the softmax: behind a NaN key, at whichever position and so in whichever group
+    of lanes, a request's logits are NaN, and only that request's.  (19 positions: most groups hold one.)"""
+    import paper_2405_18400_b200 as P
+
+    shape = si.ModelShape("hd%d" % (256 // heads), 2, 256, heads, 512, 1000)
+    packed = P.pack_weights(si.make_weights(shape, seed=73), "cuda:0")
+    args = (k, (2, 3), [0.0] * 8, 0.4, 0.2, 0.05, 256, kv_dtype)
+    ctxs = [P.SpdContext(shape, packed, [], *args) for _ in range(2)]
+    prefixes = [si.make_prefix("zipf", 18, shape.vocab, 1.1, seed=74 + r) for r in range(2)]
+    dtype, size = (torch.bfloat16, 2) if kv_dtype == "bf16" else (torch.float32, 4)
+    sound = None
+    for position in (None, 0, 1, 9, 17):
+        for ctx, prefix in zip(ctxs, prefixes):
+            ctx.spd_prefill(prefix)
+        if position is not None:
+            # keys of the first layer, the workspace's first bytes: [max_pos][d_model]; the last head's first dimension
+            keys = ctxs[1].workspace[: 256 * 256 * size].view(dtype).view(256, 256)
+            keys[position, 256 - 256 // heads] = float("nan")
+        P.spd_batch_step(ctxs)
+        z = [ctx.spd_debug_read("LOGITS") for ctx in ctxs]
+        if position is None:
+            sound = z[0]
+            assert np.isfinite(z[1]).all()
+        else:
+            assert np.isnan(z[1]).all(), position
+        assert np.array_equal(z[0], sound)
+        for ids, par, _ in P.spd_batch_step(ctxs):     # and the drafts stay ones that can be carried on
+            assert ids.min() >= 0 and ids.max() < shape.vocab and par.min() >= 0 and par.max() < k
+    for ctx in ctxs:
+        ctx.close()
