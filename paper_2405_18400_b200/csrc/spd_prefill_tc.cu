@@ -177,7 +177,8 @@ __device__ __forceinline__ bool tc_wait(TcShared &sh, State *st, uint64_t *bar, 
 // `acc_full` in both blocks; the epilogue warps of both arrive at the leader's `acc_empty`.  Every wait is bounded.
 // Launched as a programmatic dependent: a block is set up and copies the weights of its whole first ring while the kernel
 // before it still runs; the terms, which that kernel writes, are asked for after dep_wait.
-// stall (test hook): the leader announces its first stage but no copies are issued for it, so the wait for it runs out.
+// stall (test hook): the leader announces its first stage but no copies are issued for it, so the wait for it runs out.  In
+// a run longer than the ring the producers give up too, in a shorter one they are done by then.
 template <int NT>
 struct TcShape {
   static constexpr bool kFused = NT <= 64;
@@ -282,19 +283,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
         ++issued;
         if (++stage == (uint32_t)S::kStages) { stage = 0; phase ^= 1u; }
       }
-      if (!ok) {
-        // giving up: wait (bounded) for the copies already issued, so that none lands after the blocks have gone.  The
-        // leader sees its own and the other block's on its barriers; the other block, whose shared memory stays until both
-        // reach the cluster barrier below, gives copies that the leader never announced 10 ms.
-        const unsigned long long t = globaltimer();
-        if (rank == 0) {
-          for (int i = issued - 1; i >= 0 && i >= issued - S::kStages; --i) {
-            if (stall && i == 0) break;  // nothing was copied for it
-            while (!mbar_try_wait(&sh.full[i % S::kStages], (uint32_t)(i / S::kStages) & 1u) && globaltimer() - t < kTcWaitNs) {}
-          }
-        } else {
-          while (globaltimer() - t < 10ull * 1000ull * 1000ull) {}
-        }
+      // No copy may land, and no instruction read a stage, after the blocks have gone, also when the issuing thread or the
+      // epilogue gives up behind a producer that is done (a run no longer than the ring).  So before the cluster barrier
+      // below the leader waits for the bytes of its last stages, its own and the other block's, which are counted on its
+      // barriers; the other block waits until its last stages have been multiplied.  Both are over by themselves in a run
+      // that succeeds (the epilogue waits as long) and bounded; a producer that gave up itself leaves 10 ms, for copies that
+      // the leader never announced.
+      const unsigned long long t = globaltimer(), limit = ok || rank == 0 ? kTcWaitNs : 10ull * 1000ull * 1000ull;
+      for (int i = max(0, issued - S::kStages); i < issued; ++i) {
+        if (stall && i == 0) continue;  // nothing was copied for it
+        uint64_t *bar = rank == 0 ? &sh.full[i % S::kStages] : &sh.empty[i % S::kStages];
+        while (!mbar_try_wait(bar, (uint32_t)(i / S::kStages) & 1u) && globaltimer() - t < limit) {}
       }
     }
     __syncwarp();
@@ -818,10 +817,12 @@ extern "C" cudaError_t spd_internal_product(const spd::TcJob *job, int n_tok, in
   }
 }
 
-// Test hook: the first layer's QKV product by one pair whose first stage never arrives (see the kernel's `stall`).
-extern "C" cudaError_t spd_internal_tc_stall(const spd::TcJob *job, cudaStream_t s) {
+// Test hook: one pair whose first stage never arrives (see the kernel's `stall`), on the first layer's QKV product or, `few`,
+// on four stages of it at most (256 rows, 256 columns).
+extern "C" cudaError_t spd_internal_tc_stall(const spd::TcJob *job, int few, cudaStream_t s) {
   const spd::TcJob &j = *job;
-  return launch_product<16>(j, 0, j.w_tmaps, j.y, spd::plan_product(1, 3 * j.d, j.d, 2, j.y, j.parts), 1, s, 1);
+  const spd::Product pr = spd::plan_product(1, few ? 256 : 3 * j.d, few && j.d > 256 ? 256 : j.d, 2, j.y, j.parts);
+  return launch_product<16>(j, 0, j.w_tmaps, j.y, pr, 1, s, 1);
 }
 
 // Enqueues the decoder over j.n_tok tokens (at most j.x_term_rows) at positions j.pos0 ..: their keys and values

@@ -149,7 +149,7 @@ inline cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_
 
 extern "C" cudaError_t spd_internal_tc_prepare(void);
 extern "C" cudaError_t spd_internal_job_prepare(void);
-extern "C" cudaError_t spd_internal_tc_stall(const spd::TcJob *job, cudaStream_t stream);
+extern "C" cudaError_t spd_internal_tc_stall(const spd::TcJob *job, int few, cudaStream_t stream);
 extern "C" cudaError_t spd_internal_tc_prefill(const spd::TcJob *job, const spd::KParams *head, cudaStream_t stream, int *launches);
 // A product of n_tok token rows with matrix `which` of the weights' tensor maps; `wide`: the terms have d_ffn columns.
 extern "C" cudaError_t spd_internal_product(const spd::TcJob *job, int n_tok, int wide, int which, float *Y, int N, spd::Product *out, cudaStream_t s);

@@ -98,6 +98,27 @@ def test_expired_wait_in_the_products_is_reported_and_the_context_stays_usable(t
     ctx.close(); ref.close(); small.close()
 
 
+def test_expired_wait_in_runs_longer_and_shorter_than_the_ring(tiny_inputs):
+    """The hook launches two runs of stages whose first never arrives: one longer than the ring of stages, whose producers
+    give up as well, and one of four stages, whose producers are done by then and have to wait for their copies before the
+    blocks leave.  Both end by themselves with the expired wait on record, and short and long prefixes afterwards run as on a
+    fresh context."""
+    import time
+    wl, _, _, _ = tiny_inputs
+    ctx, _ = make_tiny_pair(tiny_inputs, max_pos=512)
+    ref, _ = make_tiny_pair(tiny_inputs, max_pos=512)
+    for m in (17, 70, 300):
+        before = ctx.spd_launch_count()
+        t0 = time.perf_counter()
+        assert ctx.spd_debug_expire_products() == -7
+        assert 2.5 < time.perf_counter() - t0 < 12.0 and ctx.spd_launch_count() - before == 2
+        prefix = si.make_prefix("zipf", m, wl.shape.vocab, 1.1, seed=78 + m)
+        (ids, g), (ids0, g0) = ctx.spd_prefill(prefix), ref.spd_prefill(prefix)
+        assert ids.tolist() == ids0.tolist() and np.array_equal(g, g0)
+        assert np.array_equal(ctx.spd_debug_read("LOGITS"), ref.spd_debug_read("LOGITS"))
+    ctx.close(); ref.close()
+
+
 def test_long_prefix_13b_width():
     """Two layers at the 13B shape's width (d_model 5120, 40 heads of 128, d_ffn 13824): 80 and 216 stages per
     row (10 and 27 accumulator segments, so the four accumulators are reused several times), 120 / 40 / 216 / 40
