@@ -74,6 +74,17 @@ bool valid_config(const spd_config *c) {
 // Bytes of a prefill fragment buffer for C columns: per 16 columns, 2 token tiles x 3 terms x 32 lanes x 8 bytes.
 size_t frag_bytes(int C) { return (size_t)((C + 15) / 16) * 2 * 3 * 32 * 8; }
 
+// Floats that the parts of cut tiles take at most in a product of up to `rows` token rows with a matrix [N][C].
+size_t part_floats(int rows, int N, int C) {
+  size_t most = 0;
+  for (int n = 16; n <= rows; n += n < 32 ? 16 : 32) {  // every number of rows that a tile can have
+    const spd::Product pr = spd::plan_product(n, N, C, 2 * spd::kTcMaxPairs, nullptr, nullptr);
+    const size_t floats = (size_t)pr.pairs * pr.tile_tok * 256;
+    if (floats > most) most = floats;
+  }
+  return most;
+}
+
 Layout make_layout(const spd_config &c, int grid) {
   Layout L{};
   size_t off = 0;
@@ -118,13 +129,30 @@ Layout make_layout(const spd_config &c, int grid) {
   L.tc_tmaps = take(8 * sizeof(CUtensorMap));  // term buffer as [..][d] and [..][f] in boxes of 8, 16, 32 and 64 rows
   L.tc_h = take(tcr * c.d_model * 4);
   L.tc_q = take(tcr * c.d_model * 4);
-  L.tc_y = take(tcr * wide * 4);
-  L.tc_parts = take((size_t)spd::kTcMaxPairs * (tcr < spd::kTcMaxTileTok ? tcr : spd::kTcMaxTileTok) * 256 * 4);
+  // The products' output, the parts of cut tiles and a batch's rows of logits share one area.  Only products of up to 256
+  // rows cut tiles, so a layer's parts begin behind that many rows of output and may reach into the rows of logits; the
+  // LM head's product writes these and puts its own parts where a layer's output was.
+  {
+    const size_t rows = tcr < (size_t)spd::kTcMaxTileTok ? tcr : (size_t)spd::kTcMaxTileTok;
+    const size_t shapes[4][2] = {{3 * (size_t)c.d_model, (size_t)c.d_model}, {(size_t)c.d_model, (size_t)c.d_model},
+                                 {2 * (size_t)c.d_ffn, (size_t)c.d_model}, {(size_t)c.d_model, (size_t)c.d_ffn}};
+    size_t layer_parts = 0;
+    for (const auto &sh : shapes) {
+      const size_t n = part_floats((int)rows, (int)sh[0], (int)sh[1]);
+      if (n > layer_parts) layer_parts = n;
+    }
+    const size_t head_parts = tcr ? part_floats(spd::kTcTile, c.vocab, c.d_model) : 0;
+    const size_t parts_at = align_up(rows * wide * 4, 256);
+    const size_t logits_at = align_up((tcr * wide > head_parts ? tcr * wide : head_parts) * 4, 256);
+    const size_t parts_end = parts_at + layer_parts * 4, logits_end = logits_at + (tcr ? (size_t)spd::kTcTile * c.vocab * 4 : 0);
+    L.tc_y = take(parts_end > logits_end ? parts_end : logits_end);
+    L.tc_parts = L.tc_y + parts_at;
+    L.bt_y = L.tc_y + logits_at;
+  }
   L.tc_x = take(3 * tcr * (size_t)(c.d_model > c.d_ffn ? c.d_model : c.d_ffn) * 2);
-  // batched timesteps led by this context: the requests' parameters and their rows of logits
+  // batched timesteps led by this context: the requests' parameters
   L.bt_kp = take(tcr ? (size_t)spd::kTcTile * sizeof(spd::KParams) : 0);
-  L.bt_y = take(tcr ? (size_t)spd::kTcTile * c.vocab * 4 : 0);
-  L.bt_ss = take(tcr * 32 * 4);  // per token row and 512-column chunk: sums of squares of the residual row
+  L.bt_ss = take(tcr ? (size_t)spd::kTcTile * 32 * 4 : 0);  // per token row (of up to 128) and 512-column chunk: sums of squares of the residual row
   L.bt_out = take(tcr ? (size_t)spd::kTcTile * spd::kBtResultWords * 4 : 0);  // per request: a timestep's results
   L.total = off;
   return L;
@@ -266,6 +294,7 @@ spd::TcJob tc_job(spd_ctx *ctx) {
   job.st = kp.st;
   job.sm_count = ctx->grid;
   job.parts = reinterpret_cast<float *>(ctx->ws + ctx->lay.tc_parts);
+  job.head_parts = job.y;
   job.ss = reinterpret_cast<float *>(ctx->ws + ctx->lay.bt_ss);
   job.ids = nullptr;
   job.pos0 = job.n_tok = 0;

@@ -552,28 +552,30 @@ extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd:
     e = r;
     ++count;
   };
-  auto product = [&](int wide, int which, float *Y, int N) {
-    if (e == cudaSuccess) done(spd_internal_product(job, n, wide, which, Y, N, &pr, s));
+  auto product = [&](int wide, int which, int N) {
+    if (e == cudaSuccess) done(spd_internal_product(job, n, wide, which, j.y, N, &pr, s));
   };
   auto resid = [&](const __nv_bfloat16 *gain) {
     if (e == cudaSuccess) done(spd::launch_dep(spd::spd_batch_resid_kernel, dim3(n, nch), threads, 0, s, j.h, pr, gain, j.x, ts_d, d, j.ss));
   };
   done(spd::launch_dep(spd::spd_batch_input_kernel, dim3(n, nch), threads, 0, s, kps, j.h, j.layers[0].attn_norm, j.x, ts_d, d, j.ss));
   for (int l = 0; l < j.L && e == cudaSuccess; ++l) {
-    product(0, 4 * l, j.y, 3 * d);
+    product(0, 4 * l, 3 * d);
     if (e == cudaSuccess)
       done(spd::launch_dep(spd::spd_batch_rope_cache_kernel, dim3(n, nch), threads, 0, s, pr, j.ss, j.eps, j.q, kps, d, j.hd, l));
     if (e == cudaSuccess)
       done(j.hd == 128 ? spd::launch_dep(spd::spd_batch_attn_kernel<128>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l)
                        : spd::launch_dep(spd::spd_batch_attn_kernel<64>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l));
-    product(0, 4 * l + 1, j.y, d);
+    product(0, 4 * l + 1, d);
     resid(j.layers[l].ffn_norm);
-    product(0, 4 * l + 2, j.y, 2 * f);
+    product(0, 4 * l + 2, 2 * f);
     if (e == cudaSuccess) done(spd::launch_dep(spd::spd_batch_swiglu_kernel, dim3(n, nch_f), threads, 0, s, pr, j.ss, j.eps, d, j.x, ts_f, f));
-    product(1, 4 * l + 3, j.y, d);
+    product(1, 4 * l + 3, d);
     resid(l + 1 < j.L ? j.layers[l + 1].attn_norm : final_norm);
   }
-  product(0, 4 * j.L, y_logits, V);
+  spd::TcJob head = j;
+  head.parts = j.head_parts;
+  if (e == cudaSuccess) done(spd_internal_product(&head, n, 0, 4 * j.L, y_logits, V, &pr, s));
   if (e == cudaSuccess)
     done(spd::launch_dep(spd::spd_batch_tail_kernel, dim3(n), dim3(spd::kConsumerThreads), kBatchTailSmem, s, kps, pr, j.ss, j.eps, V, results));
   if (launches) *launches = count;

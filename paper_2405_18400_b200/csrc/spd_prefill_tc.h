@@ -100,14 +100,15 @@ struct TcJob {
   void *kcache, *vcache;
   const float2 *rope;
   float *h, *y, *q;                  // [x_term_rows][d], [x_term_rows][max(3d, 2f)], [x_term_rows][d]
-  float *parts;                      // [kTcMaxPairs][min(x_term_rows, kTcMaxTileTok)][256]: parts of a product's cut tiles
+  float *parts;                      // [pairs][rows of a tile][256]: parts of a product's cut tiles
+  float *head_parts;                 // the same for the LM head's product of a batch, whose output overlaps `parts`
   uint16_t *x;                       // [3][x_term_rows][max(d, f)] bf16 terms
   int32_t x_term_rows;
   const int32_t *ids;                // device: the job's token ids
   int32_t pos0, n_tok;               // first position; tokens (<= x_term_rows)
   State *st;
   int32_t sm_count;                  // SMs of the device
-  float *ss;                         // [x_term_rows][32]: sums of squares of the residual rows per 512-column chunk
+  float *ss;                         // [128][32]: sums of squares of the residual rows per 512-column chunk
 };
 
 // Words of a request's row in a batched timestep's results (written by the tail kernel, fetched by the host in one copy).

@@ -53,6 +53,20 @@ def test_workspace_bytes_and_config_checks(lib):
     assert lib.spd_strerror(-7) == b"bounded device wait expired" and lib.spd_strerror(0) == b"ok"
 
 
+@pytest.mark.parametrize("max_pos,extra_mb", [(192, 0), (258, 5), (300, 5), (386, 0), (514, 0), (2304, 0)])
+def test_workspace_of_the_long_prefix_path(lib, max_pos, extra_mb):
+    """Its buffers at 7B shape, per token row of a job (up to 512): residual and query row, the widest product's row, three
+    bf16 terms of the widest operand; and a batch's 128 rows of logits.  The parts of cut tiles (up to 80 pairs x 256 rows x 256
+    floats, 21 MB) lie in these; only jobs of exactly 256 rows at most need a little more."""
+    n = C.c_size_t()
+    d, f, v, layers = 4096, 11008, 32000, 32
+    cfg = _cfg(n_layers=layers, d_model=d, n_heads=32, d_ffn=f, vocab=v, max_pos=max_pos, kv_dtype=1)
+    assert lib.spd_workspace_bytes(C.byref(cfg), C.byref(n)) == 0
+    rows = min(512, (max_pos - 2) // 128 * 128)
+    want = 2 * layers * max_pos * d * 2 + rows * (2 * d * 4 + 2 * f * 4 + 3 * f * 2) + 128 * v * 4
+    assert want < n.value < want + ((8 + extra_mb) << 20)   # 8 MB: the buffers of the other paths
+
+
 def _unpack(img):
     a = img.numpy().view(np.uint32).reshape(-1, 4)
     used = a[a[:, 3] > 0]
