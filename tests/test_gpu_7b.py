@@ -75,9 +75,8 @@ def test_7b_steps_match_oracle(big):
 
 
 def test_7b_long_prefix_on_tensor_cores(big):
-    """A 150-token prefix at full size: 144 tokens through the tcgen05 products and the tensor-core attention (two
-    jobs, since this context's 192 positions cap a job at 128 tokens: a full tile, then a tile with 16 tokens in
-    it), the last 6 tokens and the first timestep through the 16-token kernel."""
+    """A 150-token prefix at full size through the tcgen05 products and the tensor-core attention: two jobs, since this
+    context's 192 positions cap a job at 128 tokens, one of 128 and one of 22 that ends with the LM head."""
     wl, ctx, orc, tables, _ = big
     prefix = si.make_prefix(wl.prefix_kind, 150, wl.shape.vocab, wl.zipf_s, seed=41)
     stats = []

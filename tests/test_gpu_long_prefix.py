@@ -1,7 +1,7 @@
-"""Prefixes of more than 32 tokens: all but the last 1..16 tokens go through the tensor-core path (tcgen05
-products over tiles of 128 tokens, up to 512 tokens per job), the rest through the 16-token prefill kernel,
-which ends with the first timestep (Eq. 1).  Both fill the same cache; the first timestep and the steps after
-it are compared with the oracle as for short prefixes."""
+"""Prefixes of more than 16 tokens: jobs of the long-prefix path (tcgen05 products, up to 512 tokens per job), the last of
+which ends with the LM head and the first timestep (Eq. 1).  With the small models here a rest of 1..16 tokens behind a full
+job goes through the 16-token kernel instead.  Both fill the same cache; the first timestep and the steps after it are compared
+with the oracle as for short prefixes."""
 import numpy as np
 import pytest
 
@@ -12,19 +12,21 @@ pytestmark = pytest.mark.gpu
 
 
 def _expected_launches(m, layers, job_tokens):
-    tc = m - ((m - 1) % 16 + 1) if m > 32 else 0
-    jobs = -(-tc // job_tokens) if tc else 0
-    return jobs * 9 * layers + (m - tc + 15) // 16
+    """9 launches per layer and job; one more for the end of the last job or, with a small model, for a rest of 1..16 tokens
+    in the 16-token kernel (no length here leaves one to a large model)."""
+    jobs = 0
+    while m > 16:
+        m -= min(m, job_tokens)
+        jobs += 1
+    return jobs * 9 * layers + 1
 
 
 @pytest.mark.parametrize("kv_dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("m", [33, 64, 65, 129, 145, 293, 700])
 def test_long_prefix_tiny(tiny_inputs, m, kv_dtype):
-    """Tiny shape: d_ffn = 688 leaves a ragged last 64-column stage and 2 d_ffn = 1376 a ragged last row tile;
-    33 = the shortest prefix that takes the path (a job of 17 tokens: jobs of up to 128 tokens take the product made
-    for few token rows, with token boxes of 16, 32, 64 or 128 rows), 64 and 65 = jobs of 48 and 64 tokens, 129 = 128
-    tokens, 145 = 129 tokens (the shortest job on the 128-token tiles), 293 = one job of 288 tokens (a last tile of
-    32), 700 = a job of 512 tokens and one of 176."""
+    """Tiny shape: d_ffn = 688 leaves a ragged last 64-column stage and 2 d_ffn = 1376 a ragged last row tile; 33, 64 and
+    65 = around the step from three terms in one instruction to one, 129 and 145 = one tile that may be cut, 293 = three
+    uncut tiles of 128 rows, the last with 37 tokens, 700 = a job of 512 tokens and one of 188."""
     wl, _, _, _ = tiny_inputs
     prefix = si.make_prefix("zipf", m, wl.shape.vocab, 1.1, seed=500 + m)
     ctx, orc = make_tiny_pair(tiny_inputs, max_pos=1024, kv_dtype=kv_dtype)
@@ -121,7 +123,7 @@ def test_expired_wait_in_runs_longer_and_shorter_than_the_ring(tiny_inputs):
 
 def test_long_prefix_13b_width():
     """Two layers at the 13B shape's width (d_model 5120, 40 heads of 128, d_ffn 13824): 80 and 216 stages per
-    row (10 and 27 accumulator segments, so the four accumulators are reused several times), 120 / 40 / 216 / 40
+    row (10 and 27 accumulator segments, so the four accumulators are reused several times), 60 / 20 / 108 / 20
     row tiles, a job of 512 tokens and a partial one."""
     import torch
     import paper_2405_18400_b200 as P
@@ -174,9 +176,9 @@ def test_both_prefill_paths_agree(tiny_inputs):
 def test_long_context_decode_7b_width():
     """The long-prefix workload's regime at the 7B shape's width (d_model 4096, 32 heads of 128, d_ffn 11008; two
     layers keep the CPU oracle's dense pass over 2048 tokens to half a minute): a 2048-token prefix through four
-    jobs of the long-prefix path and one launch of the 16-token kernel, then decode steps over more than 2048
-    cached positions, where every head's positions are split over four blocks (bf16 cache, 16-byte loads, eight
-    positions in flight per warp) and the partial results merged."""
+    jobs of the long-prefix path, then decode steps over more than 2048 cached positions, where every head's positions
+    are split over four blocks (bf16 cache, 16-byte loads, eight positions in flight per warp) and the partial results
+    merged."""
     import torch
     import paper_2405_18400_b200 as P
     from oracle import spd_oracle as so
@@ -209,8 +211,8 @@ def test_long_context_decode_7b_width():
 
 
 def test_prefix_of_64_tokens_13b_width():
-    """A 64-token prefix at the 13B shape's width (the fifth workload's prefix): a long-prefix job of 48 tokens on the
-    product made for few token rows, then one launch of the 16-token kernel; five drafts, then decode steps."""
+    """A 64-token prefix at the 13B shape's width (the fifth workload's prefix): one job, the most token rows that share an
+    instruction for the three terms; five drafts, then decode steps."""
     import torch
     import paper_2405_18400_b200 as P
     from oracle import spd_oracle as so
@@ -236,3 +238,17 @@ def test_prefix_of_64_tokens_13b_width():
     assert max(s["eps_z"] for s in stats if "eps_z" in s) < 2e-3
     ctx.close()
     orc.close()
+
+
+@pytest.mark.parametrize("m", [300, 512])
+def test_attention_blocks_of_128_tokens_head_size_64(m):
+    """Head size 64 with 32 heads: more (64-token block, head) pairs than the chip has SMs, so the attention takes 128 tokens
+    and eight warps per block; 300 leaves a last block of 44."""
+    shape = si.ModelShape("h32", 1, 2048, 32, 512, 1000)
+    weights = si.make_weights(shape, seed=81)
+    tables = si.make_ngram_tables(shape.vocab, 1.1, 50_000, (2, 3), 5000, seed=82)
+    ctx, orc = make_pair(shape, weights, tables, 3, (2, 3), [0.3, 0.2] + [0.0] * 6, 0.4, 0.2, 0.05, 640, "bf16")
+    compare_first_step(ctx, orc, si.make_prefix("zipf", m, shape.vocab, 1.1, seed=83 + m))
+    assert ctx.spd_launch_count() == _expected_launches(m, 1, 512)
+    compare_step(ctx, orc)
+    ctx.close()

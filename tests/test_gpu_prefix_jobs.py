@@ -24,11 +24,14 @@ def _pair(wide, max_pos, kv_dtype, k=3):
     return make_pair(shape, weights, tables, k, (2, 3), LAM, 0.4, 0.2, 0.05, max_pos, kv_dtype)
 
 
-# one token; the products' instances for up to 16, 32, 64, 128 and 256 token rows at both ends of their ranges (96 and 97:
-# the step in the rows of a tile); two token tiles (257: of 160 rows, 320 and 321, 512); 513 = a job of 512 and one of one
-# token.  A layer's products have 192, 64, 352 and 172 stages, cut into 48, 16, 74 and 43 runs: tiles of two to four parts
+# One token; the products' instances for up to 16, 32, 64, 128 and 256 token rows at both ends of their ranges (96 and 97, 160
+# and 161: a step in the rows of a tile).  Up to 256 rows a tile may be cut: a layer's products have 192, 64, 352 and 172 stages
+# there, cut into 48, 16, 74 and 43 runs, so tiles of two to four parts (129 rows on: two segments of a run at least).  More
+# rows make uncut tiles of up to 128 rows, all alike: three of 96 (257, 288), three of 128 (289, 384), four of 128 (385, 512).
+# 513 = a job of 512 and one of one token.
 @pytest.mark.parametrize("m,jobs", [(1, 1), (2, 1), (16, 1), (17, 1), (32, 1), (33, 1), (64, 1), (65, 1), (96, 1), (97, 1), (128, 1), (129, 1),
-                                    (160, 1), (161, 1), (256, 1), (257, 1), (320, 1), (321, 1), (512, 1), (513, 2)])
+                                    (160, 1), (161, 1), (256, 1), (257, 1), (288, 1), (289, 1), (320, 1), (321, 1), (384, 1), (385, 1), (512, 1),
+                                    (513, 2)])
 def test_whole_prefix_as_jobs(wide, m, jobs):
     ctx, orc = _pair(wide, 768, "bf16" if m % 2 else "f32", k=5)
     prefix = si.make_prefix("zipf", m, wide[0].vocab, 1.1, seed=800 + m)
