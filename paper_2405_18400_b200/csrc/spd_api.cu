@@ -301,10 +301,11 @@ spd::TcJob tc_job(spd_ctx *ctx) {
   return job;
 }
 
-// Whether a run of up to 16 tokens is better off as a job of the long-prefix path (9 launches per layer) than in the
-// 16-token kernel (one cooperative launch whose weight stream reaches 0.44 of the copy bandwidth): from kJobLayerBytes
-// of matrices per layer on.  15 tokens, 8 layers, kernel / job: 1.6 MB per layer (no difference worth the launches;
-// the host's share is larger) 385 / 350 us, 25 MB 478 / 404, 101 MB 740 / 481, 405 MB 1263 / 901; the whole 7B shape 4.65 / 3.36 ms.
+// Whether a run of up to 16 tokens goes as a job of the long-prefix path (9 launches per layer) instead of the 16-token
+// kernel (one cooperative launch whose weight stream reaches 0.44 of the copy bandwidth): from kJobLayerBytes of matrices
+// per layer on.  15 tokens, 8 layers, kernel / job: 1.6 MB per layer 379 / 313 us, 5.9 MB 391 / 339, 11 MB 453 / 370, 15 MB
+// 452 / 380, 25 MB 478 / 396, 101 MB 740 / 481, 405 MB 1263 / 901; the whole 7B shape 4.65 / 3.33 ms.  So a job is the faster
+// one at every size; small models, where it wins 0.03 to 0.08 ms, keep the kernel for its single launch.
 constexpr size_t kJobLayerBytes = (size_t)16 << 20;
 bool large_layers(const spd::KParams &kp) { return 2 * (size_t)kp.d * (4 * (size_t)kp.d + 3 * (size_t)kp.f) >= kJobLayerBytes; }
 

@@ -2,15 +2,16 @@
 // remark: batching is complementary to the method, since each request still needs one pass for its k drafts).
 //
 // A request is a context of its own (prefix, KV cache, draft state); the requests of a batch share the weights and
-// the n-gram tables.  Their superposed inputs (Eq. 3) are the token rows of a tensor-core product made for few rows
-// (spd_batch_gemm_kernel in spd_prefill_tc.cu: the 128 weight rows of a tile are the wide tcgen05.mma operand, the
-// requests' activations, as three exact bf16 terms, the narrow one, TMEM accumulators, columns split among blocks),
+// the n-gram tables.  Their superposed inputs (Eq. 3) are the token rows of the tensor-core products
+// (spd_tc_product_kernel in spd_prefill_tc.cu: the 256 weight rows of a tile are the wide tcgen05.mma operand, the
+// requests' activations, as three exact bf16 terms, the narrow one, TMEM accumulators, stages dealt among pairs of blocks),
 // so the weights are streamed once per timestep whatever the number of requests.  Between the products run
 // element-wise kernels spread over requests and columns: the superposed embedding, the rotary embedding and the
 // append to the request's own cache at its own position, attention over that cache (a block per request and head),
 // residual add and SwiGLU; RMSNorm's 1 / rms is applied behind the product that follows it.  After the LM head (one
 // more product, a row of logits per request) a block per request runs the method's tail on the request's own draft
-// state: KeepTopK, Eq. 5-7 with the n-gram probes, Eq. 2, Eq. 4.
+// state: KeepTopK, Eq. 5-7 with the n-gram probes, Eq. 2, Eq. 4.  The row-wise kernels serve the jobs of the long-prefix path
+// as well, whose norm for long jobs and whose last launch are here too.
 #include <cuda_runtime.h>
 #include <math_constants.h>
 

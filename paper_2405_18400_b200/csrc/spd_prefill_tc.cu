@@ -1,9 +1,9 @@
-// Long-prefix prefill (the dense pass over the prefix that precedes Eq. 1): blocks of 128..512 prefix tokens at a
+// Long-prefix prefill (the dense pass over the prefix that precedes Eq. 1): jobs of up to 512 prefix tokens at a
 // time, their matrix products on the fifth-generation tensor cores (tcgen05.mma, operands staged in shared
 // memory by tiled TMA copies, float32 accumulators in tensor memory), everything between the products in small
 // row-wise kernels.  The job that ends a prefix goes on to the LM head and the first timestep of its last token
-// (7B shape, host to host: 15 / 27 / 100 / 400 / 2048 tokens 3.4 / 3.7 / 6.7 / 23 / 102 ms; with the last 1..16 tokens
-// in spd_prefill_kernel 4.7 / 9.2 / 12.2 / 24 / 108 ms).
+// (7B shape, host to host: 15 / 27 / 100 / 400 / 2048 tokens 3.3 / 3.5 / 5.8 / 19 / 84 ms; with 128 x 128 tiles of single
+// blocks and the last 1..16 tokens in spd_prefill_kernel 4.7 / 9.2 / 12.2 / 24 / 110 ms).
 //
 // Product: Y[token][row] = sum_c X[token][c] W[row][c], W bf16 [rows][cols] as stored, X float32 activations
 // split exactly into three bf16 terms (x = hi + mid + lo, 8 + 8 + 8 significant bits), so that the tensor
@@ -156,14 +156,17 @@ __device__ __forceinline__ bool tc_wait(TcShared &sh, State *st, uint64_t *bar, 
 // What bounds it: with up to about 64 tokens the weight stream; beyond, the tensor pipe (N = 128: 89 cycles an
 // instruction of 64, N = 256: 136 of 128, measured with the copies left out), whose operands come from shared memory.
 // Work is dealt in stages (64 columns of one tile): the product's stages, tile by tile and in a tile column by column, are
-// cut into as many equal runs as there are pairs, so no pair idles in a last wave; a pair's ring of stages and its
-// accumulators run on across tiles, so that a tile's epilogue overlaps the next one's stages.  A tile that the cuts divide
-// is summed by the reader: the part with the tile's first column is written to Y, a later part to its pair's own buffer (a
-// pair has at most one: the start of its run).
-// Measured (7B shape, gate / up product, ncu): 512 tokens 172 us = 1.61 PFLOP/s counting the three terms, 0.97 of the bf16
-// burst peak (128 x 128 tiles of single blocks: 250 us); 100 tokens 57 us; 15 tokens 34.5 us where the bytes need 27.6 (the
-// four products of a layer 91 us for 62; about 8 us of each are start and end, which the dependent launches hide in part).
-// Tried: asking the weights behind the first ring into L2 before dep_wait (8 to 32 stages): 2 to 5 % slower.
+// cut into as many runs as there are pairs; a pair's ring of stages and its accumulators run on across tiles, so that a tile's
+// epilogue overlaps the next one's stages.  Up to 256 token rows the runs are equal, so no pair idles in a last wave, and a
+// tile that the cuts divide is summed by the reader: the part with the tile's first column is written to Y, a later part to its
+// pair's own buffer (a pair has at most one: the start of its run).  More rows make uncut tiles of up to 128 rows: then pairs
+// idle (7B shape, 512 tokens: 64 tiles on 74 pairs in the attention-output and down products, two or three a pair in QKV's
+// 192), but every sum is one pair's, as in the earlier kernels, whose bits a bf16 cache behind a long prefix keeps.
+// Measured (7B shape, gate / up product, ncu, one launch at a time): 512 tokens 168 us = 1.65 PFLOP/s counting the three terms,
+// 0.98 of the bf16 burst peak (128 x 128 tiles of single blocks: 250 us); 200 tokens 75 us; 100 tokens 46 us; 64 tokens 37 us;
+// 15 tokens 35 us where the bytes need 27.6 (the four products of a layer 93 us for 62; about 8 us of each are start and end,
+// which the dependent launches hide in part).  Tried: asking the weights behind the first ring into L2 before dep_wait (8 to
+// 32 stages): 2 to 5 % slower.
 //
 // Accumulation: an accumulator takes the sums of a segment of stages (pr.seg), then moves to registers, where the
 // segments are added with round-to-nearest: the tensor cores add into their accumulator with truncation, whose error grows
@@ -568,8 +571,8 @@ __device__ __forceinline__ void tc_cp16(uint32_t dst, const void *src, uint32_t 
 // What bounds it: the 384 instructions of a tile and warp; so the next tile's rows travel (cp.async, two buffers) while
 // a tile is multiplied, consecutive instructions go to different accumulators, and tiles wholly behind a warp's tokens
 // skip the mask.  One block per SM: eight warps when 64-token blocks would outnumber the SMs, else four.
-// spd_prefill of 400 / 2048 tokens, 7B shape: 18.9 / 81.4 -> 18.3 / 78.9 ms (before: one tile buffer, two blocks of four
-// warps per SM, three dependent instructions in a row).
+// spd_prefill of 400 / 2048 tokens, 7B shape, 0.6 / 2.5 ms shorter than with one tile buffer, two blocks of four warps per SM
+// and three dependent instructions in a row; a job of 512 tokens at position 0 takes 49 us a layer (ncu).
 template <int HD, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 1)
     spd_tc_attn_mma_kernel(const float *Q, const uint16_t *kcache, const uint16_t *vcache, uint16_t *X, size_t term_stride, int d, int max_pos,
@@ -802,7 +805,7 @@ extern "C" cudaError_t spd_internal_tc_prepare(void) {
 }
 
 // Product of n_tok token rows (<= x_term_rows) with matrix `which` of the layers' tensor maps: `wide` terms have d_ffn
-// columns, else d_model.  *out tells the readers of Y where its sums are (product_sum).
+// columns, else d_model.  *out tells the readers of Y where its sums are (product_sum4).
 extern "C" cudaError_t spd_internal_product(const spd::TcJob *job, int n_tok, int wide, int which, float *Y, int N, spd::Product *out, cudaStream_t s) {
   const spd::TcJob &j = *job;
   const void *wmap = j.w_tmaps + (size_t)which * spd::kTensorMapBytes;

@@ -4,9 +4,13 @@
 
 namespace spd {
 
-constexpr int kTcTile = 128;      // tokens per tile of the tensor-core products
+// Requests of a batch at most; jobs of up to so many tokens apply 1 / rms behind the product; the most tokens of a context's
+// jobs are a multiple of it.
+constexpr int kTcTile = 128;
 constexpr int kTcMaxTokens = 512; // tokens one job takes at most
-constexpr int kTcMinPrefix = 16;  // runs of more tokens than this take the path with every model, shorter ones with large models
+// Runs of more tokens than this take the path with every model, shorter ones with large models: beyond, the 16-token kernel needs
+// two launches (27 tokens, 7B shape: 9.2 ms, the job 3.5; 17 tokens, 8 layers of 1.6 MB: the job 0.32 where one launch takes 0.38).
+constexpr int kTcMinPrefix = 16;
 
 // A product Y = X W^T as it is dealt out among pairs of blocks, and where its sums are (spd_tc_product_kernel).  Tiles of
 // 256 weight rows x tile_tok token rows, token tiles fastest; a tile has nk stages of 64 columns; the stages of all tiles,
