@@ -43,11 +43,13 @@ inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *
   pr.align = whole ? pr.nk : (pr.shape == 256 ? 8 : 1);
   // The accumulators add with truncation, so the error grows with the additions between two moves to registers: 4 per stage
   // and accumulator where every term has its own (up to 64 rows), 12 where the terms share one (small ones first: 4 at the
-  // sum's own size).  4 stages cost nothing (2: 1 % at 15 tokens, 3 % at 64; 1: 2 % and 10 %), and where the terms share one
-  // never more than the 3 C / 128 additions that a warp of the 16-token kernel chains.  Uncut tiles of wide matrices keep up to
-  // 8 stages, the terms in order: behind long prefixes a bf16 cache then holds the bits that it always has.
-  const int most_seg = whole ? 8 : 4;
-  pr.seg = pr.shape <= 64 ? 4 : (C < 512 ? 1 : (C / 512 < most_seg ? C / 512 : most_seg));
+  // sum's own size).  4 stages cost nothing (2: 1 % at 15 tokens, 3 % at 64; 1: 2 % and 10 %).  Where the terms share one, C / 512
+  // stages, as many additions as the 3 C / 128 that a warp of the 16-token kernel chains; two at least beyond 128 rows, where
+  // the epilogue of one stage takes longer than its instructions (8 layers of 256 columns, 200 tokens: one stage 0.85 ms, two
+  // 0.77; error of the first timestep 4.0e-7 and 5.9e-7, the 16-token kernel's path 1.9e-6).  Uncut tiles of wide matrices keep
+  // up to 8 stages, the terms in order: behind long prefixes a bf16 cache then holds the bits that it always has.
+  const int least_seg = whole || pr.shape == 256 ? 2 : 1, most_seg = whole ? 8 : 4, wide = C / 512;
+  pr.seg = pr.shape <= 64 ? 4 : (wide < least_seg ? least_seg : (wide < most_seg ? wide : most_seg));
   pr.small_first = pr.seg < 8;
   // a pair takes a tile, two segments or four stages at least (small matrices: fewer parts to add)
   const int least = whole ? pr.nk : (pr.align > 1 ? 2 * pr.align : 4);
