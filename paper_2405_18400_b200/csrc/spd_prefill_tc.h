@@ -34,7 +34,7 @@ inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *
   pr.nk = (C + 63) / 64;
   // Up to 64 token rows the three terms share an instruction; up to 256 rows are one tile; more rows make enough tiles of
   // up to 128 (in steps of 32 rows, all alike) to fill the pairs without cutting one: then every sum is one pair's.
-  // Between 129 and 256 rows tiles are cut, where an accumulator's segment ends.
+  // Between 129 and 256 rows tiles are cut at multiples of eight stages.
   const bool whole = n_tok > kTcMaxTileTok;
   pr.shape = n_tok <= 16 ? 16 : (n_tok <= 32 ? 32 : (n_tok <= 64 ? 64 : (n_tok <= 128 || whole ? 128 : 256)));
   pr.tok_tiles = whole ? (n_tok + 127) / 128 : 1;
