@@ -189,6 +189,7 @@ bool term_map(TensorMapEncode encode, const void *x, int rows, int cols, int box
 static_assert(sizeof(CUtensorMap) == spd::kTensorMapBytes, "the prefill kernel steps through the tensor maps by this size");
 
 constexpr int kLayoutGrid = 1024;  // workspace is sized for up to this many blocks
+static_assert(spd::kMaxLists <= kLayoutGrid, "a launch's blocks fit the workspace");
 
 }  // namespace
 
@@ -440,7 +441,7 @@ int spd_create(const spd_config *cfg, const spd_weights *w, const spd_ngram_tabl
   e = cudaGetDeviceProperties(&prop, ctx->device);
   if (e != cudaSuccess) return fail(cuda_fail(e, "cudaGetDeviceProperties"));
   if (!prop.cooperativeLaunch) return fail(SPD_EINVAL);
-  ctx->grid = prop.multiProcessorCount < kLayoutGrid ? prop.multiProcessorCount : kLayoutGrid;
+  ctx->grid = prop.multiProcessorCount < spd::kMaxLists ? prop.multiProcessorCount : spd::kMaxLists;
 
   spd::KParams &kp = ctx->kp;
   std::memset(&kp, 0, sizeof kp);

@@ -18,6 +18,7 @@ constexpr int kMaxRowsPerChunk = 8;
 constexpr int kMaxStages = 16;
 constexpr int kMaxVec = 4;          // 16-byte column vectors per thread: columns <= 4 * 512 * 8
 constexpr int kMaxSplit = 8;        // attention splits per head
+constexpr int kMaxLists = 160;      // lists that KeepTopK merges, so the blocks of a launch at most (148 on a B200); a multiple of 32
 constexpr int kTensorMapBytes = 128; // size of one tensor map object (CUtensorMap)
 constexpr int kPfTokens = 16;       // prefix tokens one prefill launch takes
 constexpr int kUnitRows = 8;        // rows of a unit of a matrix in fragment order (the granularity of the blocks' shares; 4 was

@@ -23,19 +23,32 @@ __device__ __forceinline__ void warp_best(float &v, int &i) {
 }
 
 // One warp: the k best logits among rows [r0, r1) and (max, sum exp) of z / tau over them, into list `slot` of the
-// partial lists (the decode and prefill kernels: warp 0 of each block, slot = the block).
+// partial lists (the decode and prefill kernels: warp 0 of each block, slot = the block), best first.  A lane asks for eight
+// rows at a time, and keeps them for all rounds when that is all there is (up to 256 rows: a block's share of the LM head).
+constexpr int kTopkFlight = 8;
 static __device__ void block_topk(const KParams &p, int r0, int r1, int slot) {
   const int lane = threadIdx.x & 31;
+  const bool once = r1 - r0 <= 32 * kTopkFlight;
+  float z[kTopkFlight];
+  auto fetch = [&](int r) {
+#pragma unroll
+    for (int e = 0; e < kTopkFlight; ++e) z[e] = r + 32 * e < r1 ? p.logits[r + 32 * e] : 0.f;
+  };
+  fetch(r0 + lane);
   float pv = 0.f;
   int pi = -1;
   float mx = -CUDART_INF_F;
   for (int j = 0; j < p.k; ++j) {
     float bv = 0.f;
     int bi = -1;
-    for (int r = r0 + lane; r < r1; r += 32) {
-      const float z = p.logits[r];
-      if (j > 0 && !ranks_before(pv, pi, z, r)) continue;  // already taken (or is the previous winner)
-      if (bi < 0 || ranks_before(z, r, bv, bi)) { bv = z; bi = r; }
+    for (int r = r0 + lane; r < r1; r += 32 * kTopkFlight) {
+      if (!once) fetch(r);
+#pragma unroll
+      for (int e = 0; e < kTopkFlight; ++e) {
+        const int id = r + 32 * e;
+        // (rows already taken, the previous winner among them, are passed over)
+        if (id < r1 && (j == 0 || ranks_before(pv, pi, z[e], id)) && (bi < 0 || ranks_before(z[e], id, bv, bi))) { bv = z[e]; bi = id; }
+      }
     }
     warp_best(bv, bi);
     if (lane == 0) {
@@ -55,50 +68,72 @@ static __device__ void block_topk(const KParams &p, int r0, int r1, int slot) {
     }
   }
   float s = 0.f;
-  for (int r = r0 + lane; r < r1; r += 32) s += __expf(p.logits[r] * p.inv_tau - mx);
+  for (int r = r0 + lane; r < r1; r += 32 * kTopkFlight) {
+    if (!once) fetch(r);
+#pragma unroll
+    for (int e = 0; e < kTopkFlight; ++e)
+      if (r + 32 * e < r1) s += __expf(z[e] * p.inv_tau - mx);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) p.pk_ms[slot] = make_float2(mx, s);
 }
 
-// KeepTopK over the whole vocabulary from the n_lists partial lists (Algorithm 1), with
-// log-probabilities under temperature tau.  Warp 0.
+// KeepTopK over the whole vocabulary from the n_lists (<= kMaxLists) partial lists (Algorithm 1), with log-probabilities
+// under temperature tau.  Warp 0.  The lists are in rank order, so a lane keeps the heads of its lists in registers and a
+// round is a vote over the heads and one load, of the winning list's next entry: the warp stands alone between two grid
+// barriers here, and a trip to L2 per candidate and round (148 lists: 14 of them for k = 3, 37 for k = 8) was most of a
+// timestep's tail (with the other two places where loads stood in a row, block_topk and the input's embedding: tiny model, 150 steps
+// in one launch, 11.4 -> 8.6 ms; 7B shape, k = 8, 2.76 -> 2.64 ms per timestep).
 static __device__ void tail_keep_topk(const KParams &p, int n_lists) {
   const int lane = threadIdx.x & 31;
+  constexpr int kMine = kMaxLists / 32;
   State *st = p.st;
-  const int ncand = n_lists * p.k;
+  float2 ms[kMine];
+  float hv[kMine];
+  int hid[kMine], next[kMine];
+#pragma unroll
+  for (int i = 0; i < kMine; ++i) {
+    const int g = lane + 32 * i;
+    const bool in = g < n_lists;
+    ms[i] = in ? __ldcg(&p.pk_ms[g]) : make_float2(-CUDART_INF_F, 0.f);
+    hv[i] = in ? __ldcg(&p.pk_val[(size_t)g * p.k]) : 0.f;
+    hid[i] = in ? __ldcg(&p.pk_id[(size_t)g * p.k]) : -1;
+    next[i] = 1;
+  }
   float M = -CUDART_INF_F;
-  for (int g = lane; g < n_lists; g += 32) M = fmaxf(M, __ldcg(&p.pk_ms[g]).x);
+#pragma unroll
+  for (int i = 0; i < kMine; ++i) M = fmaxf(M, ms[i].x);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
   float S = 0.f;
-  for (int g = lane; g < n_lists; g += 32) {
-    const float2 ms = __ldcg(&p.pk_ms[g]);
-    if (ms.x > -CUDART_INF_F) S = fmaf(ms.y, __expf(ms.x - M), S);
-  }
+#pragma unroll
+  for (int i = 0; i < kMine; ++i)
+    if (lane + 32 * i < n_lists && ms[i].x > -CUDART_INF_F) S = fmaf(ms[i].y, __expf(ms[i].x - M), S);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) S += __shfl_xor_sync(0xffffffffu, S, o);
   const float lse = M + __logf(S);
-  float pv = 0.f;
-  int pi = -1;
   for (int j = 0; j < p.k; ++j) {
     float bv = 0.f;
     int bi = -1;
-    for (int c = lane; c < ncand; c += 32) {
-      const int id = __ldcg(&p.pk_id[c]);
-      if (id < 0) continue;
-      const float z = __ldcg(&p.pk_val[c]);
-      if (j > 0 && !ranks_before(pv, pi, z, id)) continue;
-      if (bi < 0 || ranks_before(z, id, bv, bi)) { bv = z; bi = id; }
-    }
+#pragma unroll
+    for (int i = 0; i < kMine; ++i)
+      if (hid[i] >= 0 && (bi < 0 || ranks_before(hv[i], hid[i], bv, bi))) { bv = hv[i]; bi = hid[i]; }
     warp_best(bv, bi);
     if (lane == 0) {
       // non-finite logits can leave a round without a winner: keep the token id valid
       st->cand_tok[j] = bi < 0 ? 0 : bi;
       st->cand_lp[j] = bv * p.inv_tau - lse;
     }
-    pv = bv;
-    pi = bi;
+#pragma unroll
+    for (int i = 0; i < kMine; ++i)
+      if (bi >= 0 && hid[i] == bi) {  // this list's head was taken (an id is in one list only)
+        const size_t at = (size_t)(lane + 32 * i) * p.k + next[i];
+        const bool more = next[i] < p.k;
+        hid[i] = more ? __ldcg(&p.pk_id[at]) : -1;
+        hv[i] = more ? __ldcg(&p.pk_val[at]) : 0.f;
+        ++next[i];
+      }
   }
   __syncwarp();
 }

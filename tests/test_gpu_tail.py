@@ -1,0 +1,29 @@
+"""The serial end of a timestep: per-block lists of the best logits (a lane keeps up to eight rows of its block in registers,
+more are read again each round) and their merge (a lane walks the heads of its lists)."""
+import pytest
+
+import spd_inputs as si
+from tests.gpu_common import compare_first_step, compare_step, make_pair
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("vocab,k,hot", [
+    (96, 16, None),        # fewer rows than blocks: empty lists and lists of one, all shorter than k
+    (1504, 16, (40, 56)),  # the k best rows in two or three neighbouring blocks: a list is used up
+    (37888, 8, (4, 8)),    # 256 rows a block: the most that stay in registers; some of the best in one lane's stride
+    (40000, 5, None),      # more than that
+])
+def test_keep_topk_lists(vocab, k, hot):
+    shape = si.ModelShape("tail", 1, 128, 2, 128, vocab)
+    weights = si.make_weights(shape, seed=91)
+    if hot:
+        weights["lm_head"][hot[0]:hot[1]] *= 8   # exact in bf16; these rows' logits are the largest and the smallest
+    tables = si.make_ngram_tables(vocab, 1.1, 20_000, (2, 3), 2000, seed=92)
+    ctx, orc = make_pair(shape, weights, tables, k, (2, 3), [0.3, 0.2] + [0.0] * 6, 0.4, 0.2, 0.05, 256, "f32")
+    compare_first_step(ctx, orc, si.make_prefix("zipf", 9, vocab, 1.1, seed=93))   # the 16-token kernel's end
+    for _ in range(2):
+        compare_step(ctx, orc)
+    compare_first_step(ctx, orc, si.make_prefix("zipf", 20, vocab, 1.1, seed=94))  # the end of a job
+    compare_step(ctx, orc)
+    ctx.close()
