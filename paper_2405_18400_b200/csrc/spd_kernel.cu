@@ -416,15 +416,18 @@ __device__ __forceinline__ void consume_matrix(Blk &b, int R, int C, int gran, c
 }
 
 // ---------------------------------------------------------------- consumer: matrices in fragment order on the tensor cores
-// D (16 x 8) += A (16 x 16) * B (16 x 8): mma.sync m16n8k16, bf16 in, float32 accumulate.  A = a unit's weight rows x 16
-// columns in its first rows (the others are zero: a1 = a3 = 0), B = the three terms of 16 values of x in columns 0..2, so
-// that a lane's B registers are all in use and stay in registers for a whole phase.  d[0], d[1] of lane 4 g + t: weight
-// row g times terms 2t and 2t + 1; d[2], d[3] stay zero.
-__device__ __forceinline__ void mma_terms(float (&d)[4], uint32_t a0, uint32_t a2, uint32_t b0, uint32_t b1) {
+// D (16 x 8) += A (16 x 16) * B (16 x 8): mma.sync m16n8k16, bf16 in, float32 accumulate.  A's rows 0..7 are a unit's
+// weight rows x 16 columns, its rows 8..15 the same weight rows x the next 16 columns; B has the three terms of the first
+// 16 values of x in columns 0..2 and those of the next 16 in columns 3..5.  Wanted of the product are rows 0..7 of columns
+// 0..2 and rows 8..15 of columns 3..5 (the rest pairs columns with the wrong values of x and is not read), so one
+// instruction does the work of two with half-empty operands (A's rows 8..15 zero): the multiply loop from shared memory,
+// without waiting for HBM, 2.30 -> 2.10 ms per 7B timestep.  d[0], d[1] of lane 4 g + t: weight row g, columns 2t and
+// 2t + 1; d[2], d[3]: the same of row 8 + g.
+__device__ __forceinline__ void mma_terms(float (&d)[4], const uint4 &w, const uint2 &x) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
+      : "r"(w.x), "r"(w.z), "r"(w.y), "r"(w.w), "r"(x.x), "r"(x.y));
 }
 
 // Term g (0, 1, 2) of v = hi + mid + lo, each the leading 8 significant bits of what is left (by truncation), so that
@@ -438,9 +441,9 @@ __device__ __forceinline__ uint32_t term_of(float v, int g) {
   return pick >> 16;
 }
 
-// The activation vector as B fragments in shared memory, behind the scratch area: per pair of 16-column blocks 12
-// vectors of 16 bytes, vector 4 g + t = term g of columns 2t, 2t+1 | 2t+8, 2t+9 of the first block and the same of
-// the second (what lane 4 g + t feeds to the two instructions of the pair; lanes 12..31 feed zeros).
+// The activation vector as B fragments in shared memory, behind the scratch area: per 32 columns 24 vectors of 8 bytes,
+// vector 4 g + t (g = 0..2: term g of the first 16 columns, g = 3..5: term g - 3 of the other 16) = columns 2t, 2t+1 | 2t+8,
+// 2t+9 of its block: what lane 4 g + t feeds to the instruction (lanes 24..31 feed columns that nothing reads).
 __device__ __forceinline__ uint32_t *xfrag_base(const KParams &p) {
   return reinterpret_cast<uint32_t *>(smem + (size_t)p.n_stages * p.stage_bytes + kScratchBytes);
 }
@@ -453,29 +456,28 @@ __device__ __forceinline__ void store_frags(const KParams &p, int C, const float
   for (int i = 0; i < kMaxVec; ++i) {
     const int v = (int)threadIdx.x + i * kConsumerThreads;
     if (v < nv) {
-      // columns 8 v .. 8 v + 7: pair v / 4, word (v & 3) of each vector = block (v / 2) & 1, half v & 1
-      uint32_t *dst = xf + (size_t)(v >> 2) * 48 + (v & 3);
+      // columns 8 v .. 8 v + 7: the 32 columns v / 4, of these block (v / 2) & 1, half v & 1
+      uint32_t *dst = xf + (size_t)(v >> 2) * 48 + ((v >> 1) & 1) * 24 + (v & 1);
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
         const float x0 = xr[i][2 * t], x1 = xr[i][2 * t + 1];
 #pragma unroll
-        for (int g = 0; g < 3; ++g) dst[g * 16 + t * 4] = term_of(x0, g) | (term_of(x1, g) << 16);
+        for (int g = 0; g < 3; ++g) dst[g * 8 + t * 2] = term_of(x0, g) | (term_of(x1, g) << 16);
       }
     }
   }
 }
 
-// Streams this block's units of one matrix in fragment order through the ring: per unit and pair of column blocks one
-// 16-byte load of weights (lanes of the unit's rows; the others feed zero rows) and one of x (the fragments of two
-// instructions) and two instructions, the pairs of a stage dealt to the warps in turn; a row's sum is the sum of its
-// three terms' columns of the accumulator.
+// Streams this block's units of one matrix in fragment order through the ring: per unit and 32 columns one 16-byte load of
+// weights, one 8-byte load of x and one instruction, the pairs of column blocks of a stage dealt to the warps in turn; a
+// row's sum is the sum of its six wanted columns of the accumulator.
 __device__ __forceinline__ void consume_image(Blk &b, int R, int C, int kind, const EpiArgs &ea) {
   const KParams &p = *b.p;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int r0, r1;
   cta_rows(R, kUnitRows, r0, r1);
   const int n_pairs = C / 32;
-  const uint4 *xf = reinterpret_cast<const uint4 *>(xfrag_base(p)) + lane;  // lanes < 12 only
+  const uint2 *xf = reinterpret_cast<const uint2 *>(xfrag_base(p)) + min(lane, 23);
   float h_pre = 0.f;
   if (kind == kEpiAddH && r0 + (int)threadIdx.x < min(r0 + kTile, r1)) h_pre = __ldcg(p.h + r0 + threadIdx.x);
   float rs = 1.f;
@@ -484,29 +486,24 @@ __device__ __forceinline__ void consume_image(Blk &b, int R, int C, int kind, co
     const int t1 = min(t0 + kTile, r1);
     float *part = scratch_base(p) + (size_t)buf * kTile * kConsumerWarps;
     for (int r = t0; r < t1; r += kUnitRows) {
-      float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
       const int per_stage = (int)(img_chunk(p, C) / kPairBytes);
       for (int pr0 = 0; pr0 < n_pairs; pr0 += per_stage) {  // one stage
         wait_mbar(b, &s_full[b.c_stage], b.c_phase, 300);
         const uint8_t *stage = smem + (size_t)b.c_stage * p.stage_bytes;
         const int n = min(per_stage, n_pairs - pr0);
 #pragma unroll 1  // unrolled, the loop costs more registers than the kernel has
-        for (int j = warp; j < n; j += kConsumerWarps) {
-          uint4 w = make_uint4(0u, 0u, 0u, 0u);
-          if (lane < 4 * kUnitRows) w = lds128(stage + ((size_t)j * (4 * kUnitRows) + lane) * 16);
-          uint4 x = make_uint4(0u, 0u, 0u, 0u);
-          if (lane < 12) x = xf[(size_t)(pr0 + j) * 12];
-          mma_terms(c0, w.x, w.y, x.x, x.y);
-          mma_terms(c1, w.z, w.w, x.z, x.w);
-        }
+        for (int j = warp; j < n; j += kConsumerWarps)
+          mma_terms(c, lds128(stage + ((size_t)j * (4 * kUnitRows) + lane) * 16), xf[(size_t)(pr0 + j) * 24]);
         __syncwarp();
         if (lane == 0) mbar_arrive(&s_empty[b.c_stage]);
         if (++b.c_stage == (uint32_t)p.n_stages) { b.c_stage = 0; b.c_phase ^= 1u; }
       }
-      // row g: terms 0 and 1 in lane 4 g, term 2 in lane 4 g + 1 (whose d[1] is a sum of zeros)
-      const float s01 = (c0[0] + c1[0]) + (c0[1] + c1[1]);
-      const float s2 = __shfl_down_sync(0xffffffffu, s01, 1);
-      if ((lane & 3) == 0 && lane < 4 * kUnitRows) part[(size_t)(r - t0 + (lane >> 2)) * kConsumerWarps + warp] = s01 + s2;
+      // row g: columns 0 and 1 in lane 4 g; 2 and, of row 8 + g, 3 in lane 4 g + 1; 4 and 5 of row 8 + g in lane 4 g + 2
+      const int t = lane & 3;
+      const float sum = (t == 2 ? c[2] : c[0]) + (t == 0 ? c[1] : c[3]);
+      const float s1 = __shfl_down_sync(0xffffffffu, sum, 1), s2 = __shfl_down_sync(0xffffffffu, sum, 2);
+      if (t == 0) part[(size_t)(r - t0 + (lane >> 2)) * kConsumerWarps + warp] = sum + s1 + s2;
     }
     named_sync(1, kConsumerThreads);
     if (kind != kEpiAddH && t0 == r0) {
@@ -685,98 +682,108 @@ __device__ __forceinline__ void prefetch_kv(const KParams &p, int layer, int pos
   }
 }
 
-// Fast path of the attention phase for a bf16 cache and head_dim 128 (a cache row of a head is 256 bytes):
-// half a warp takes one position with 16-byte loads, and each warp keeps eight positions in flight, so a
-// long context costs a few dependent memory round trips instead of one per position.  Each half-warp runs
-// its own online softmax; halves, then warps, are merged at the end exactly like the general path.
-__device__ void attention_phase_bf16_hd128(Blk &b, int layer, int pos) {
+// The values of a 16-byte vector.
+template <typename E>
+__device__ __forceinline__ void unpack16(const uint4 &v, float (&x)[16 / sizeof(E)]) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    if constexpr (sizeof(E) == 2) {
+      x[2 * e] = __uint_as_float(w[e] << 16);
+      x[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
+    } else {
+      x[e] = __uint_as_float(w[e]);
+    }
+  }
+}
+// The attention phase for head sizes 64 and 128: HD * sizeof(E) / 16 lanes take one position with 16-byte loads (a whole
+// warp for float32 of head size 128, half of one for bf16, a quarter for bf16 of 64), and each such group keeps four positions
+// in flight, which enter its running softmax together (one rescale per round instead of four dependent ones): the phase stands
+// between two grid barriers with the ring full, and a trip to L2 per position and warp was 6.8 us of it with a float32 cache
+// behind 20 positions (now 2.5).  Groups, then warps, are merged at the end exactly like in the general path.
+template <int HD, typename E>
+__device__ void attention_rows(Blk &b, int layer, int pos) {
   const KParams &p = *b.p;
+  constexpr int EPL = 16 / (int)sizeof(E), LP = HD / EPL, GW = 32 / LP, F = 4;
   const int T = pos + 1, ns = attn_splits(p, T), items = p.H * ns;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, half = lane >> 4, l16 = lane & 15;
-  const float scale = 1.f / sqrtf(128.f);
-  float *s_acc = scratch_base(p);                           // [warps][128]
-  float *s_m = scratch_base(p) + kConsumerWarps * 256;      // [warps]
-  float *s_l = s_m + kConsumerWarps;               // [warps]
-  const __nv_bfloat16 *kc = reinterpret_cast<const __nv_bfloat16 *>(p.kcache);
-  const __nv_bfloat16 *vc = reinterpret_cast<const __nv_bfloat16 *>(p.vcache);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / LP, at = (lane % LP) * EPL;
+  const float scale = 1.f / sqrtf((float)HD);
+  float *s_acc = scratch_base(p), *s_m = scratch_base(p) + kConsumerWarps * 256, *s_l = s_m + kConsumerWarps;
+  const E *kc = reinterpret_cast<const E *>(p.kcache), *vc = reinterpret_cast<const E *>(p.vcache);
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
     const int head = item / ns, sp = item - head * ns;
     const int t0 = (int)((long long)T * sp / ns), t1 = (int)((long long)T * (sp + 1) / ns);
-    float q[8], acc[8];
-    load8(p.q + head * 128 + l16 * 8, q);
+    float q[EPL], acc[EPL];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+    for (int e = 0; e < EPL; e += 4) {
+      const float4 a = __ldcg(reinterpret_cast<const float4 *>(p.q + head * HD + at + e));
+      q[e] = a.x; q[e + 1] = a.y; q[e + 2] = a.z; q[e + 3] = a.w;
+    }
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
     float m = -CUDART_INF_F, l = 0.f;
-    const size_t col = (size_t)head * 128 + l16 * 8;
-    // A round = four positions per half-warp; they enter the running softmax together (one rescale per round instead
-    // of four dependent ones).
-    constexpr int kStep = kConsumerWarps * 8;
-    uint4 kq[4], vq[4];
-    auto fetch = [&](int tb, const __nv_bfloat16 *cache, uint4 (&dst)[4]) {
+    const size_t col = (size_t)head * HD + at;
+    uint4 kq[F], vq[F];
+    auto fetch = [&](int tb, const E *cache, uint4 (&dst)[F]) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int t = max(min(tb + 2 * u + half, t1 - 1), 0);  // clamped: the extra loads are discarded below
+      for (int u = 0; u < F; ++u) {
+        const int t = max(min(tb + GW * u + grp, t1 - 1), 0);
         dst[u] = __ldcg(reinterpret_cast<const uint4 *>(cache + ((size_t)layer * p.max_pos + t) * p.d + col));
       }
     };
-    for (int tb = t0 + warp * 8; tb < t1; tb += kStep) {
+    for (int tb = t0 + warp * (F * GW); tb < t1; tb += kConsumerWarps * F * GW) {
       fetch(tb, kc, kq);
       fetch(tb, vc, vq);
-      float sc[4];
+      float sc[F];
       float mn = m;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const uint32_t kw[4] = {kq[u].x, kq[u].y, kq[u].z, kq[u].w};
-        float dot = 0.f;
+      for (int u = 0; u < F; ++u) {
+        float kx[EPL], dot = 0.f;
+        unpack16<E>(kq[u], kx);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          dot = fmaf(q[2 * e], __uint_as_float(kw[e] << 16), dot);
-          dot = fmaf(q[2 * e + 1], __uint_as_float(kw[e] & 0xffff0000u), dot);
-        }
+        for (int e = 0; e < EPL; ++e) dot = fmaf(q[e], kx[e], dot);
 #pragma unroll
-        for (int o = 8; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-        sc[u] = tb + 2 * u + half < t1 ? dot * scale : -CUDART_INF_F;  // uniform within the half-warp
+        for (int o = LP / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+        sc[u] = tb + GW * u + grp < t1 ? dot * scale : -CUDART_INF_F;
         mn = fmaxf(mn, sc[u]);
       }
-      if (mn > -CUDART_INF_F) {  // else nothing of this round (nor of an earlier one) belongs to the half-warp
+      if (tb + grp < t1) {  // else no position of this round belongs to the group (a NaN score, which fmaxf passes over, has to reach the sums)
         const float c = __expf(m - mn);
         l *= c;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] *= c;
+        for (int e = 0; e < EPL; ++e) acc[e] *= c;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const float pw = __expf(sc[u] - mn);  // 0 for a position past the range
+        for (int u = 0; u < F; ++u) {
+          const float pw = __expf(sc[u] - mn);
           l += pw;
-          const uint32_t vw[4] = {vq[u].x, vq[u].y, vq[u].z, vq[u].w};
+          float vx[EPL];
+          unpack16<E>(vq[u], vx);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            acc[2 * e] = fmaf(pw, __uint_as_float(vw[e] << 16), acc[2 * e]);
-            acc[2 * e + 1] = fmaf(pw, __uint_as_float(vw[e] & 0xffff0000u), acc[2 * e + 1]);
-          }
+          for (int e = 0; e < EPL; ++e) acc[e] = fmaf(pw, vx[e], acc[e]);
         }
         m = mn;
       }
     }
-    // merge the two half-warps
-    {
-      const float mo = __shfl_xor_sync(0xffffffffu, m, 16), lo = __shfl_xor_sync(0xffffffffu, l, 16);
+#pragma unroll
+    for (int o = LP; o < 32; o <<= 1) {
+      const float mo = __shfl_xor_sync(0xffffffffu, m, o), lo = __shfl_xor_sync(0xffffffffu, l, o);
       const float M = fmaxf(m, mo);
       const float w_self = m == -CUDART_INF_F ? 0.f : __expf(m - M), w_oth = mo == -CUDART_INF_F ? 0.f : __expf(mo - M);
       l = l * w_self + lo * w_oth;
 #pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] = acc[e] * w_self + __shfl_xor_sync(0xffffffffu, acc[e], 16) * w_oth;
+      for (int e = 0; e < EPL; ++e) acc[e] = acc[e] * w_self + __shfl_xor_sync(0xffffffffu, acc[e], o) * w_oth;
       m = M;
     }
-    if (half == 0) {
+    if (grp == 0) {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) s_acc[warp * 256 + l16 * 8 + e] = acc[e];
+      for (int e = 0; e < EPL; ++e) s_acc[warp * 256 + at + e] = acc[e];
     }
     if (lane == 0) {
       s_m[warp] = m;
       s_l[warp] = l;
     }
     named_sync(1, kConsumerThreads);
-    if (threadIdx.x < 128) {
+    if (threadIdx.x < HD) {
       float M = -CUDART_INF_F;
 #pragma unroll
       for (int w = 0; w < kConsumerWarps; ++w) M = fmaxf(M, s_m[w]);
@@ -787,7 +794,7 @@ __device__ void attention_phase_bf16_hd128(Blk &b, int layer, int pos) {
         L = fmaf(s_l[w], wgt, L);
         A = fmaf(s_acc[w * 256 + threadIdx.x], wgt, A);
       }
-      p.opart[(size_t)item * 128 + threadIdx.x] = A;
+      p.opart[(size_t)item * HD + threadIdx.x] = A;
       if (threadIdx.x == 0) p.oml[item] = make_float2(M, L);
     }
     named_sync(1, kConsumerThreads);
@@ -796,8 +803,14 @@ __device__ void attention_phase_bf16_hd128(Blk &b, int layer, int pos) {
 
 __device__ void attention_phase(Blk &b, int layer, int pos) {
   const KParams &p = *b.p;
-  if (p.kv_bf16 && p.hd == 128) {
-    attention_phase_bf16_hd128(b, layer, pos);
+  if (p.hd == 128) {
+    if (p.kv_bf16) attention_rows<128, __nv_bfloat16>(b, layer, pos);
+    else attention_rows<128, float>(b, layer, pos);
+    return;
+  }
+  if (p.hd == 64) {
+    if (p.kv_bf16) attention_rows<64, __nv_bfloat16>(b, layer, pos);
+    else attention_rows<64, float>(b, layer, pos);
     return;
   }
   const int T = pos + 1, ns = attn_splits(p, T), items = p.H * ns;
@@ -865,20 +878,6 @@ __device__ void attention_phase(Blk &b, int layer, int pos) {
   }
 }
 
-// The values of a 16-byte vector.
-template <typename E>
-__device__ __forceinline__ void unpack16(const uint4 &v, float (&x)[16 / sizeof(E)]) {
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    if constexpr (sizeof(E) == 2) {
-      x[2 * e] = __uint_as_float(w[e] << 16);
-      x[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
-    } else {
-      x[e] = __uint_as_float(w[e]);
-    }
-  }
-}
 // Next LM input (block 0): the token embedding in prefill and sampling, the superposed embedding of Eq. 3 in
 // decode.  Eight columns per thread: the rows come from device memory, and with two-byte loads in a loop over the columns their
 // latency was paid eight times at d_model 4096, all other blocks waiting.
