@@ -96,6 +96,7 @@ __device__ __forceinline__ int rows_per_chunk(const KParams &p, int C) {
 struct Producer {
   uint32_t stage, phase;
   uint32_t issued;  // chunks issued so far (saturating at n_stages for the drain)
+  uint64_t policy;  // the weights' L2 policy
 };
 
 __device__ __forceinline__ void produce_matrix(Blk &b, Producer &pr, const __nv_bfloat16 *W, int R, int C, int gran) {
@@ -112,8 +113,8 @@ __device__ __forceinline__ void produce_matrix(Blk &b, Producer &pr, const __nv_
       if (s_dead) return;
       const uint32_t bytes = (uint32_t)n * rowbytes;
       mbar_expect_tx(&s_full[pr.stage], bytes);
-      bulk_load(smem + (size_t)pr.stage * p.stage_bytes, (const uint8_t *)W + (size_t)r * rowbytes, bytes,
-                &s_full[pr.stage]);
+      bulk_load_policy(smem + (size_t)pr.stage * p.stage_bytes, (const uint8_t *)W + (size_t)r * rowbytes, bytes, &s_full[pr.stage],
+                       pr.policy);
       if (pr.issued < (uint32_t)p.n_stages) ++pr.issued;
       if (++pr.stage == (uint32_t)p.n_stages) { pr.stage = 0; pr.phase ^= 1u; }
     }
@@ -145,7 +146,7 @@ __device__ __forceinline__ void produce_image(Blk &b, Producer &pr, const __nv_b
       wait_mbar(b, &s_empty[pr.stage], pr.phase ^ 1u, 200);
       if (s_dead) return;
       mbar_expect_tx(&s_full[pr.stage], bytes);
-      bulk_load(smem + (size_t)pr.stage * p.stage_bytes, src + off, bytes, &s_full[pr.stage]);
+      bulk_load_policy(smem + (size_t)pr.stage * p.stage_bytes, src + off, bytes, &s_full[pr.stage], pr.policy);
       if (pr.issued < (uint32_t)p.n_stages) ++pr.issued;
       if (++pr.stage == (uint32_t)p.n_stages) { pr.stage = 0; pr.phase ^= 1u; }
     }
@@ -155,7 +156,7 @@ __device__ __forceinline__ void produce_image(Blk &b, Producer &pr, const __nv_b
 template <bool kSampler, bool kImg>
 __device__ void producer_main(Blk &b) {
   const KParams &p = *b.p;
-  Producer pr{0u, 0u, 0u};
+  Producer pr{0u, 0u, 0u, evict_first_policy()};
   // The layers' pointers sit in device memory that the weight stream has long pushed out of L2 when their turn
   // comes: each layer's are fetched while the layer before is streamed.
   LayerW lw = p.layers[0];

@@ -91,6 +91,12 @@ __device__ __forceinline__ void tc_pair_box_load(uint32_t dst, const void *tmap,
                "l"(tmap), "r"(x), "r"(y), "r"(bar)
                : "memory");
 }
+__device__ __forceinline__ void tc_pair_box_load_policy(uint32_t dst, const void *tmap, int x, int y, uint32_t bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
+      "l"(tmap), "r"(x), "r"(y), "r"(bar), "l"(policy)
+      : "memory");
+}
 __device__ __forceinline__ void tc_pair_alloc(uint32_t *slot, uint32_t cols) {
   asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(cols) : "memory");
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
@@ -248,12 +254,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
         }
       };
       const uint32_t bar0 = tc_leader_addr(&sh.full[0]);
+      const uint64_t policy = evict_first_policy();
       auto weights = [&](uint32_t stage) {
         const uint32_t base = ring + stage * (uint32_t)S::kStageBytes, bar = bar0 + stage * 8u;
         const int row = rt * (2 * kTcRows) + rank * kTcRows;
 #pragma unroll
         for (int j = 0; j < kTcRows / kTcWBoxRows; ++j)
-          tc_pair_box_load(base + j * (kTcWBoxRows * kTcKB * 2), tmap_w, kb * kTcKB, row + j * kTcWBoxRows, bar);
+          tc_pair_box_load_policy(base + j * (kTcWBoxRows * kTcKB * 2), tmap_w, kb * kTcKB, row + j * kTcWBoxRows, bar, policy);
       };
       auto terms = [&](uint32_t stage) {
         const uint32_t base = ring + stage * (uint32_t)S::kStageBytes + kTcWBytes, bar = bar0 + stage * 8u;

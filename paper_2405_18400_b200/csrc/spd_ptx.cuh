@@ -30,12 +30,28 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Bulk asynchronous copy global -> shared of `bytes` (multiple of 16, both addresses 16-byte aligned);
-// completion is counted on `bar` in bytes.
+// The weights' way through L2: evicted first.  A pass streams 13 GB of them (7B shape) through 126 MB of L2, and without the
+// hint they push out what is small and comes back every layer or pass (activation vectors, norm gains, cache rows, rotary
+// table, draft state), whose next readers then wait for device memory behind the stream.  7B shape, without / with: a
+// decode timestep 2.608 / 2.530 ms, behind 2048 positions 3.05 / 2.94; spd_prefill of 27 tokens 3.46 / 3.29 ms; a timestep of
+// 8 requests 3.24 / 3.13 ms.
+__device__ __forceinline__ uint64_t evict_first_policy() {
+  uint64_t pol;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+  return pol;
+}
+// Bulk asynchronous copy global -> shared of `bytes` (multiple of 16, both addresses 16-byte aligned); completion is counted
+// on `bar` in bytes.
 __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                    smem_u32(dst)),
                "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+__device__ __forceinline__ void bulk_load_policy(void *dst, const void *src, uint32_t bytes, uint64_t *bar, uint64_t policy) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
+                   smem_u32(dst)),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
                : "memory");
 }
 __device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
