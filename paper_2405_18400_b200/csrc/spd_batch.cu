@@ -66,8 +66,11 @@ constexpr int kBtThreads = kBtCols / 4;
 constexpr int kBtMaxChunks = 32;  // d_model <= 16384
 static_assert(8 + 3 * kMaxK <= kBtResultWords, "a request's row of results holds the head and three lists of k");
 
+// The gains of the thread's columns: weights, asked for before dep_wait.
+__device__ __forceinline__ float4 bt_gain(const __nv_bfloat16 *gain, int c, int d) { return c < d ? bt_load4(gain + c) : make_float4(0.f, 0.f, 0.f, 0.f); }
+
 // A chunk of a residual row: stored, its terms times the gain, its sum of squares.  All threads of the block.
-__device__ __forceinline__ void bt_store_row(float *h, const __nv_bfloat16 *gain, uint16_t *X, size_t term_stride, int row, int d, int c,
+__device__ __forceinline__ void bt_store_row(float *h, const float4 &gain, uint16_t *X, size_t term_stride, int row, int d, int c,
                                              const float4 &v, float *ss) {
   __shared__ float scratch[kBtThreads / 32];
   float sq = 0.f;
@@ -75,7 +78,7 @@ __device__ __forceinline__ void bt_store_row(float *h, const __nv_bfloat16 *gain
     const size_t at = (size_t)row * d + c;
     *reinterpret_cast<float4 *>(h + at) = v;
     sq = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, v.w * v.w)));
-    bt_put3x4(X, term_stride, at, bt_mul(v, bt_load4(gain + c)));
+    bt_put3x4(X, term_stride, at, bt_mul(v, gain));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
@@ -94,7 +97,13 @@ __device__ __forceinline__ float bt_rs(const float *ss, int row, int d, float ep
   if (!ss) return 1.f;
   const int nch = (d + kBtCols - 1) / kBtCols;
   float s = 0.f;
-  for (int c = 0; c < nch; ++c) s += ss[row * kBtMaxChunks + c];
+  for (int c = 0; c < nch; c += 8) {  // (asked for together, added in order)
+    float a[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) a[u] = c + u < nch ? ss[row * kBtMaxChunks + c + u] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += a[u];
+  }
   return rsqrtf(s / (float)d + eps);
 }
 
@@ -107,10 +116,11 @@ __device__ __forceinline__ int bt_pos(const KParams &p) { return p.pos0 + p.st->
 __global__ void __launch_bounds__(kBtThreads) spd_batch_input_kernel(const KParams *kps, float *h, const __nv_bfloat16 *gain, uint16_t *X,
                                                                      size_t term_stride, int d, float *ss) {
   dep_launch();
+  const int c = blockIdx.y * kBtCols + threadIdx.x * 4;
+  const float4 gq = bt_gain(gain, c, d);
   dep_wait();
   const KParams &p = kps[blockIdx.x];
   const State *st = p.st;
-  const int c = blockIdx.y * kBtCols + threadIdx.x * 4;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   if (c < d)
     for (int i = 0; i < p.k; ++i) {
@@ -121,33 +131,35 @@ __global__ void __launch_bounds__(kBtThreads) spd_batch_input_kernel(const KPara
       acc.z = fmaf(g, e.z, acc.z);
       acc.w = fmaf(g, e.w, acc.w);
     }
-  bt_store_row(h, gain, X, term_stride, blockIdx.x, d, c, acc, ss);
+  bt_store_row(h, gq, X, term_stride, blockIdx.x, d, c, acc, ss);
 }
 
 // grid (tokens, column chunks): a job's residual rows start as its tokens' embeddings.
 __global__ void __launch_bounds__(kBtThreads) spd_job_input_kernel(const int32_t *ids, const __nv_bfloat16 *tok_emb, float *h,
                                                                    const __nv_bfloat16 *gain, uint16_t *X, size_t term_stride, int d, float *ss) {
   dep_launch();
-  dep_wait();
   const int c = blockIdx.y * kBtCols + threadIdx.x * 4;
+  const float4 gq = bt_gain(gain, c, d);
+  dep_wait();
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
   if (c < d) v = bt_load4(tok_emb + (size_t)ids[blockIdx.x] * d + c);
-  bt_store_row(h, gain, X, term_stride, blockIdx.x, d, c, v, ss);
+  bt_store_row(h, gq, X, term_stride, blockIdx.x, d, c, v, ss);
 }
 
 // grid (rows, column chunks): residual add h += y, h * gain of the next norm as terms, the chunk's sum of squares.
 __global__ void __launch_bounds__(kBtThreads) spd_batch_resid_kernel(float *h, const __grid_constant__ Product y, const __nv_bfloat16 *gain,
                                                                      uint16_t *X, size_t term_stride, int d, float *ss) {
   dep_launch();
-  dep_wait();
   const int c = blockIdx.y * kBtCols + threadIdx.x * 4;
+  const float4 gq = bt_gain(gain, c, d);
+  dep_wait();
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
   if (c < d) {
     v = *reinterpret_cast<const float4 *>(h + (size_t)blockIdx.x * d + c);
     const float4 a = product_sum4(y, blockIdx.x, c);
     v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
   }
-  bt_store_row(h, gain, X, term_stride, blockIdx.x, d, c, v, ss);
+  bt_store_row(h, gq, X, term_stride, blockIdx.x, d, c, v, ss);
 }
 
 // Long jobs (more than 128 tokens): a token row per block, the whole RMSNorm before the product.  With hundreds of rows
@@ -207,10 +219,12 @@ __device__ __forceinline__ void bt_store_kv(void *cache, int kv_bf16, size_t at,
     *reinterpret_cast<float4 *>(static_cast<float *>(cache) + at) = v;
   }
 }
-__device__ __forceinline__ void bt_rope_cache(const Product &y, float rs, float *Q, void *kcache, void *vcache, const float2 *rope, int max_pos,
-                                              int kv_bf16, int d, int hd, int layer, int t, int pos, int c) {
+__device__ __forceinline__ float4 bt_angles(const float2 *rope, int hd, int pos, int c) {
+  return *reinterpret_cast<const float4 *>(rope + (size_t)pos * (hd / 2) + (c % hd) / 2);
+}
+__device__ __forceinline__ void bt_rope_cache(const Product &y, float rs, float *Q, void *kcache, void *vcache, const float4 &cs, int max_pos,
+                                              int kv_bf16, int d, int layer, int t, int pos, int c) {
   const float4 q = product_sum4(y, t, c), k = product_sum4(y, t, d + c), v = product_sum4(y, t, 2 * d + c);
-  const float4 cs = *reinterpret_cast<const float4 *>(rope + (size_t)pos * (hd / 2) + (c % hd) / 2);
   const size_t at = ((size_t)layer * max_pos + pos) * d + c;
   *reinterpret_cast<float4 *>(Q + (size_t)t * d + c) = bt_rotate(make_float4(q.x * rs, q.y * rs, q.z * rs, q.w * rs), cs);
   bt_store_kv(kcache, kv_bf16, at, bt_rotate(make_float4(k.x * rs, k.y * rs, k.z * rs, k.w * rs), cs));
@@ -225,18 +239,21 @@ __global__ void __launch_bounds__(kBtThreads) spd_batch_rope_cache_kernel(const 
   const KParams &p = kps[blockIdx.x];
   const int c = blockIdx.y * kBtCols + threadIdx.x * 4;
   if (c >= d) return;
-  bt_rope_cache(y, bt_rs(ss, blockIdx.x, d, eps), Q, p.kcache, p.vcache, p.rope, p.max_pos, p.kv_bf16, d, hd, layer, blockIdx.x, bt_pos(p), c);
+  const int pos = bt_pos(p);
+  bt_rope_cache(y, bt_rs(ss, blockIdx.x, d, eps), Q, p.kcache, p.vcache, bt_angles(p.rope, hd, pos, c), p.max_pos, p.kv_bf16, d, layer, blockIdx.x,
+                pos, c);
 }
 
 // The same for a job of prefix tokens of one request (token t at position pos0 + t, one cache).
 __global__ void __launch_bounds__(kBtThreads) spd_job_rope_cache_kernel(const __grid_constant__ Product y, const float *ss, float eps, float *Q,
                                                                         void *kcache, void *vcache, const float2 *rope, int max_pos, int kv_bf16,
                                                                         int d, int hd, int layer, int pos0) {
+  const int c = blockIdx.y * kBtCols + threadIdx.x * 4, pos = pos0 + blockIdx.x;
+  const float4 cs = c < d ? bt_angles(rope, hd, pos, c) : make_float4(0.f, 0.f, 0.f, 0.f);  // (a table as old as the context)
   dep_wait();
   dep_launch();
-  const int c = blockIdx.y * kBtCols + threadIdx.x * 4;
   if (c >= d) return;
-  bt_rope_cache(y, bt_rs(ss, blockIdx.x, d, eps), Q, kcache, vcache, rope, max_pos, kv_bf16, d, hd, layer, blockIdx.x, pos0 + blockIdx.x, c);
+  bt_rope_cache(y, bt_rs(ss, blockIdx.x, d, eps), Q, kcache, vcache, cs, max_pos, kv_bf16, d, layer, blockIdx.x, pos, c);
 }
 
 // grid (rows, chunks of the FFN): u = SiLU(gate) * up from the gate / up product's row times 1 / rms
@@ -463,6 +480,7 @@ __global__ void __launch_bounds__(kConsumerThreads) spd_job_head_kernel(const __
     const int r = r0 + warp * kHeadRows + e / (p.d / 64);
     if (r < r1) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.lm_head + (size_t)r * p.d + (e % (p.d / 64)) * 64));
   }
+  for (int c = threadIdx.x * 64; c < p.d; c += kConsumerThreads * 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.final_norm + c));
   dep_wait();
   float sq = 0.f;
   for (int c = threadIdx.x * 4; c < p.d; c += kConsumerThreads * 4) {
