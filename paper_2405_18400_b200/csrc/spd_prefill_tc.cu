@@ -155,7 +155,7 @@ __device__ __forceinline__ bool tc_wait(TcShared &sh, State *st, uint64_t *bar, 
 //   F = 16, 32, 64 (up to that many token rows): the three term tiles lie behind one another, so one instruction of
 //     N = 3 x rows per 16 columns multiplies all three (N = 64 for 16 rows: a multiple of 32 is wanted; the 16 columns
 //     left over hold nothing that is read); each term has its own accumulator columns, added in the epilogue's registers.
-//   128, 256 (that many rows at most, N = the tile's rows rounded up to 32): one instruction per term and 16 columns, all
+//   128, 256 (that many rows at most, N = the tile's rows rounded up to 16): one instruction per term and 16 columns, all
 //     into the same columns.
 // Each block brings its 128 weight rows and half of the tile's tokens.
 //
@@ -318,13 +318,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
         if (!tc_wait(sh, st, &sh.full[stage], phase, 410)) break;
         tc_fence_after();
         const uint32_t base = ring + stage * (uint32_t)S::kStageBytes, acc = tmem + (uint32_t)(a * S::kAccStride);
-        const uint32_t term0 = base + kTcWBytes + (!S::kFused && pr.small_first ? 2 * S::kTermBytes : 0);
-        const int term_step = pr.small_first ? -S::kTermBytes : S::kTermBytes;
+        const uint32_t term0 = base + kTcWBytes + (S::kFused ? 0 : 2 * S::kTermBytes);  // (a stage's small terms before the large one)
 #pragma unroll
         for (int j = 0; j < (S::kFused ? 1 : 3); ++j)
 #pragma unroll
           for (int kk = 0; kk < kTcKB / 16; ++kk)  // 16 columns = 32 bytes further into the swizzled rows
-            tc_pair_mma(acc, tc_desc(base + kk * 32), tc_desc(term0 + j * term_step + kk * 32), idesc, (uint32_t)((in_seg | j | kk) != 0));
+            tc_pair_mma(acc, tc_desc(base + kk * 32), tc_desc(term0 - j * S::kTermBytes + kk * 32), idesc, (uint32_t)((in_seg | j | kk) != 0));
         tc_pair_commit(&sh.empty[stage]);  // the stage is free in both blocks once these have read it
         if (++stage == (uint32_t)S::kStages) { stage = 0; phase ^= 1u; }
         ++kb;
@@ -371,7 +370,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
           const uint32_t from = acc + (uint32_t)(half * half_tok);
 #pragma unroll
           for (int c0 = 0; c0 < S::kHalf; c0 += 32)
-            if (c0 < half_tok) {  // (half_tok is a multiple of 16)
+            if (c0 < half_tok) {  // (a multiple of 8: the last load may bring columns behind the half, whose sums go nowhere)
               uint32_t r[16], q[16];
               tc_ld(from + (uint32_t)c0, r);
               if (c0 + 16 < half_tok) tc_ld(from + (uint32_t)(c0 + 16), q);

@@ -23,7 +23,6 @@ struct Product {
   int32_t N, nk, tile_tok, tok_tiles, total, pairs, shape;  // shape: 16, 32, 64, 128 or 256, the kernel's instance
   int32_t align;  // a cut lies a multiple of so many stages behind its tile's first (rounded down)
   int32_t seg;    // stages whose sums an accumulator takes before they move to registers
-  int32_t small_first;  // one instruction per term: a stage's small terms before the large one
 };
 
 inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *y, const float *parts) {
@@ -33,24 +32,26 @@ inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *
   pr.N = N;
   pr.nk = (C + 63) / 64;
   // Up to 64 token rows the three terms share an instruction; up to 256 rows are one tile; more rows make enough tiles of
-  // up to 128 (in steps of 32 rows, all alike) to fill the pairs without cutting one: then every sum is one pair's.
-  // Between 129 and 256 rows tiles are cut at multiples of eight stages.
+  // up to 128 (all alike) to fill the pairs without cutting one: then every sum is one pair's.  From 65 rows on a tile's rows
+  // are rounded up to 16, which is what an instruction's N allows (to 32: 100 tokens, 7B shape, 5.5 ms instead of 5.1; 400
+  // tokens 18.6 instead of 17.0).  Between 129 and 256 rows tiles are cut at multiples of eight stages.
   const bool whole = n_tok > kTcMaxTileTok;
   pr.shape = n_tok <= 16 ? 16 : (n_tok <= 32 ? 32 : (n_tok <= 64 ? 64 : (n_tok <= 128 || whole ? 128 : 256)));
   pr.tok_tiles = whole ? (n_tok + 127) / 128 : 1;
-  pr.tile_tok = pr.shape <= 64 ? pr.shape : ((n_tok + pr.tok_tiles - 1) / pr.tok_tiles + 31) / 32 * 32;
+  pr.tile_tok = pr.shape <= 64 ? pr.shape : ((n_tok + pr.tok_tiles - 1) / pr.tok_tiles + 15) / 16 * 16;
   pr.total = (N + 255) / 256 * pr.tok_tiles * pr.nk;
   pr.align = whole ? pr.nk : (pr.shape == 256 ? 8 : 1);
   // The accumulators add with truncation, so the error grows with the additions between two moves to registers: 4 per stage
   // and accumulator where every term has its own (up to 64 rows), 12 where the terms share one (small ones first: 4 at the
   // sum's own size).  4 stages cost nothing (2: 1 % at 15 tokens, 3 % at 64; 1: 2 % and 10 %).  Where the terms share one, C / 512
-  // stages, as many additions as the 3 C / 128 that a warp of the 16-token kernel chains; two at least beyond 128 rows, where
-  // the epilogue of one stage takes longer than its instructions (8 layers of 256 columns, 200 tokens: one stage 0.85 ms, two
-  // 0.77; error of the first timestep 4.0e-7 and 5.9e-7, the 16-token kernel's path 1.9e-6).  Uncut tiles of wide matrices keep
-  // up to 8 stages, the terms in order: behind long prefixes a bf16 cache then holds the bits that it always has.
-  const int least_seg = whole || pr.shape == 256 ? 2 : 1, most_seg = whole ? 8 : 4, wide = C / 512;
+  // stages at most, as many additions as the 3 C / 128 that a warp of the 16-token kernel chains; two at least beyond 128 rows,
+  // where the epilogue of one stage takes longer than its instructions (8 layers of 256 columns, 200 tokens: one stage 0.85 ms,
+  // two 0.77; error of the first timestep 4.0e-7 and 5.9e-7, the 16-token kernel's path 1.9e-6).  129 to 384 rows take no more
+  // than those two, so that a prefix of that length is no further from 64 bits in one job than in two shorter ones (7B shape,
+  // first timestep's logits, relative 2-norm: 200 tokens 5.5e-6, with four stages 1.1e-5; 300 tokens 6.8e-6, four 1.3e-5, 256 and
+  // 44 tokens apart 9.8e-6), for 1 % of the time; beyond, four (512 tokens 1.1e-5; with eight and the terms in order 2.9e-5).
+  const int least_seg = n_tok > 128 ? 2 : 1, most_seg = n_tok > 128 && n_tok <= 384 ? 2 : 4, wide = C / 512;
   pr.seg = pr.shape <= 64 ? 4 : (wide < least_seg ? least_seg : (wide < most_seg ? wide : most_seg));
-  pr.small_first = pr.seg < 8;
   // a pair takes a tile, two segments or four stages at least (small matrices: fewer parts to add)
   const int least = whole ? pr.nk : (pr.align > 1 ? 2 * pr.align : 4);
   const int most = sm_count / 2 < kTcMaxPairs ? sm_count / 2 : kTcMaxPairs, worth = pr.total / least;
