@@ -17,7 +17,7 @@ extern "C" cudaError_t spd_internal_prepare(size_t dyn_smem, int *blocks_per_sm)
 extern "C" cudaError_t spd_internal_prefill_prepare(int *blocks_per_sm);
 extern "C" cudaError_t spd_internal_prefill_launch(const spd::KParams *p, int grid, cudaStream_t stream);
 extern "C" cudaError_t spd_internal_pack_image(const void *w, void *out, int rows, int cols, cudaStream_t stream);
-extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd::KParams *kps, int n, int V, const __nv_bfloat16 *final_norm,
+extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd::KParams *kps, int n, int begin, int V, const __nv_bfloat16 *final_norm,
                                                float *y_logits, int32_t *results, cudaStream_t s, int *launches);
 
 namespace {
@@ -248,19 +248,59 @@ int pick_ring(const spd_config &c, int32_t stage_bytes, int32_t n_stages, size_t
   return SPD_OK;
 }
 
-// Waits for the stream and returns what the device recorded; with a stop token configured, also takes over the
-// device's count of generated tokens and its stop flag (a launch may have ended before its last step).
-int check_device_error(spd_ctx *ctx) {
-  int32_t head[6] = {0, 0, 0, 0, 0, 0};  // stop, abort flag, err, err_info, win_len, n_gen
-  static_assert(offsetof(spd::State, n_gen) - offsetof(spd::State, stop) == 5 * sizeof(int32_t), "the fields read here are adjacent");
-  SPD_CUDA(cudaMemcpyAsync(head, ctx->ws + ctx->lay.state + offsetof(spd::State, stop), sizeof head, cudaMemcpyDeviceToHost,
-                           ctx->stream));
+// What a call tells its caller about the last step, as it lies in the state: one copy.  (A copy into pageable memory is a round
+// trip of its own: with four of them a step of the tiny model took 114 us, of which the device worked 54; now 82.)
+struct StepResult {
+  int32_t stop, abort_flag, err, err_info, win_len, n_gen;
+  int32_t win[spd::kMaxK][spd::kWin];
+  float logP[spd::kMaxK], gamma[spd::kMaxK];
+  int32_t cand_tok[spd::kMaxK], sel[spd::kMaxK];
+};
+static_assert(offsetof(StepResult, n_gen) == offsetof(spd::State, n_gen) - offsetof(spd::State, stop) &&
+                  offsetof(StepResult, gamma) == offsetof(spd::State, gamma) - offsetof(spd::State, stop) &&
+                  offsetof(StepResult, sel) == offsetof(spd::State, sel) - offsetof(spd::State, stop),
+              "the state's fields lie in this order");
+
+// Enqueues the copy; await_result then waits for the stream and returns what the device recorded; with a stop token configured,
+// it also takes over the device's count of generated tokens and its stop flag (a launch may have ended before its last step).
+int fetch_result(spd_ctx *ctx, StepResult &r) {
+  SPD_CUDA(cudaMemcpyAsync(&r, ctx->ws + ctx->lay.state + offsetof(spd::State, stop), sizeof r, cudaMemcpyDeviceToHost, ctx->stream));
+  return SPD_OK;
+}
+int await_result(spd_ctx *ctx, const StepResult &r) {
   SPD_CUDA(cudaStreamSynchronize(ctx->stream));
-  if (head[2] == 0 && ctx->cfg.eos_id >= 0 && ctx->decoding) {
-    ctx->n_gen = head[5];
-    if (head[0]) ctx->stopped = true;
+  if (r.err == 0 && ctx->cfg.eos_id >= 0 && ctx->decoding) {
+    ctx->n_gen = r.n_gen;
+    if (r.stop) ctx->stopped = true;
   }
-  return head[2];
+  return r.err;
+}
+int check_device_error(spd_ctx *ctx) {
+  StepResult r;
+  const int rc = fetch_result(ctx, r);
+  return rc ? rc : await_result(ctx, r);
+}
+
+// The way out of a call that fails: the copies from the caller's memory and from this call's have been made.
+int give_back(spd_ctx *ctx, int rc) {
+  cudaStreamSynchronize(ctx->stream);
+  return rc;
+}
+
+// The first timestep's drafts behind a prefix: waits, then token and weight of each draft.
+int first_drafts(spd_ctx *ctx, int32_t *out_ids, float *out_gamma) {
+  StepResult r;
+  int rc = fetch_result(ctx, r);
+  if (rc) return rc;
+  if ((rc = await_result(ctx, r))) return rc;
+  ctx->prefilled = true;
+  ctx->n_gen = 1;
+  ctx->stopped = ctx->cfg.eos_id >= 0 && r.cand_tok[0] == ctx->cfg.eos_id;
+  for (int i = 0; i < ctx->cfg.k; ++i) {
+    if (out_ids) out_ids[i] = r.cand_tok[i];
+    if (out_gamma) out_gamma[i] = r.gamma[i];
+  }
+  return SPD_OK;
 }
 
 // Bytes of the state's head that every launch zeroes: with `keep_err` (later launches of a multi-launch call)
@@ -625,24 +665,13 @@ int spd_prefill(spd_ctx *ctx, const int32_t *prefix_ids, int32_t m, int32_t *out
     for (int j = 0; j < st.win_len; ++j) st.win[i][spd::kWin - st.win_len + j] = prefix_ids[m - st.win_len + j];
   SPD_CUDA(cudaMemcpyAsync(ctx->ws + ctx->lay.state, &st, sizeof st, cudaMemcpyHostToDevice, ctx->stream));
   SPD_CUDA(cudaMemcpyAsync(ctx->ws + ctx->lay.prefix, prefix_ids, (size_t)m * 4, cudaMemcpyHostToDevice, ctx->stream));
-  SPD_CUDA(cudaStreamSynchronize(ctx->stream));  // st and the caller's ids may go out of scope
   ctx->prefilled = false;
   ctx->decoding = false;
-  if ((rc = prefill_tokens(ctx, 0, m))) return rc;
-  int32_t ids[SPD_MAX_K];
-  float gamma[SPD_MAX_K];
-  if ((rc = read_state(ctx, offsetof(spd::State, cand_tok), ids, sizeof ids))) return rc;
-  if ((rc = read_state(ctx, offsetof(spd::State, gamma), gamma, sizeof gamma))) return rc;
-  if ((rc = check_device_error(ctx))) return rc;
-  ctx->prefilled = true;
+  rc = prefill_tokens(ctx, 0, m);
+  if (!rc) rc = first_drafts(ctx, out_ids, out_gamma);
+  if (rc) return give_back(ctx, rc);
   ctx->m = m;
-  ctx->n_gen = 1;
-  ctx->stopped = c.eos_id >= 0 && ids[0] == c.eos_id;
   ctx->prefix.assign(prefix_ids, prefix_ids + m);
-  for (int i = 0; i < c.k; ++i) {
-    if (out_ids) out_ids[i] = ids[i];
-    if (out_gamma) out_gamma[i] = gamma[i];
-  }
   return SPD_OK;
 }
 
@@ -675,23 +704,12 @@ int spd_reset(spd_ctx *ctx, int32_t draft, int32_t *out_ids, float *out_gamma) {
     for (int j = 0; j < st.win_len; ++j) st.win[i][spd::kWin - st.win_len + j] = ctx->prefix[m2 - st.win_len + j];
   SPD_CUDA(cudaMemcpyAsync(ctx->ws + ctx->lay.state, &st, sizeof st, cudaMemcpyHostToDevice, ctx->stream));
   SPD_CUDA(cudaMemcpyAsync(ctx->ws + ctx->lay.prefix + (size_t)m * 4, seq.data(), (size_t)n * 4, cudaMemcpyHostToDevice, ctx->stream));
-  SPD_CUDA(cudaStreamSynchronize(ctx->stream));
   ctx->prefilled = false;
   ctx->decoding = false;
-  if ((rc = prefill_tokens(ctx, m, n))) return rc;
-  int32_t ids[SPD_MAX_K];
-  float gamma[SPD_MAX_K];
-  if ((rc = read_state(ctx, offsetof(spd::State, cand_tok), ids, sizeof ids))) return rc;
-  if ((rc = read_state(ctx, offsetof(spd::State, gamma), gamma, sizeof gamma))) return rc;
-  if ((rc = check_device_error(ctx))) return rc;
-  ctx->prefilled = true;
+  rc = prefill_tokens(ctx, m, n);
+  if (!rc) rc = first_drafts(ctx, out_ids, out_gamma);
+  if (rc) return give_back(ctx, rc);
   ctx->m = m2;
-  ctx->n_gen = 1;
-  ctx->stopped = c.eos_id >= 0 && ids[0] == c.eos_id;
-  for (int i = 0; i < k; ++i) {
-    if (out_ids) out_ids[i] = ids[i];
-    if (out_gamma) out_gamma[i] = gamma[i];
-  }
   return SPD_OK;
 }
 
@@ -708,7 +726,6 @@ int spd_sample(spd_ctx *ctx, int32_t n_new, float top_p, float temperature, cons
   int rc = set_device(ctx);
   if (rc) return rc;
   SPD_CUDA(cudaMemcpyAsync(ctx->ws + ctx->lay.ns_u, uniforms, (size_t)n_new * 4, cudaMemcpyHostToDevice, ctx->stream));
-  SPD_CUDA(cudaStreamSynchronize(ctx->stream));  // the caller's array may go out of scope
   ctx->prefilled = false;
   ctx->decoding = false;
   // pass i draws token m + i from the logits of the pass before (the first from those the prefill left),
@@ -720,26 +737,15 @@ int spd_sample(spd_ctx *ctx, int32_t n_new, float top_p, float temperature, cons
   kp.ns_inv_temp = 1.0f / temperature;
   rc = launch(ctx, spd::kModeSample, n_new, m, 0);
   kp.prefix = base;
-  if (rc) return rc;
+  if (rc) return give_back(ctx, rc);
   std::vector<int32_t> fresh(n_new);
-  int32_t ids[SPD_MAX_K];
-  float gamma[SPD_MAX_K];
   SPD_CUDA(cudaMemcpyAsync(fresh.data(), ctx->ws + ctx->lay.prefix + (size_t)m * 4, (size_t)n_new * 4, cudaMemcpyDeviceToHost,
                            ctx->stream));
-  if ((rc = read_state(ctx, offsetof(spd::State, cand_tok), ids, sizeof ids))) return rc;
-  if ((rc = read_state(ctx, offsetof(spd::State, gamma), gamma, sizeof gamma))) return rc;
-  if ((rc = check_device_error(ctx))) return rc;
+  if ((rc = first_drafts(ctx, out_ids, out_gamma))) return give_back(ctx, rc);
   ctx->prefix.insert(ctx->prefix.end(), fresh.begin(), fresh.end());
-  ctx->prefilled = true;
   ctx->m = m + n_new;
-  ctx->n_gen = 1;
-  ctx->stopped = c.eos_id >= 0 && ids[0] == c.eos_id;
   for (int i = 0; i < n_new; ++i)
     if (out_new) out_new[i] = fresh[i];
-  for (int i = 0; i < c.k; ++i) {
-    if (out_ids) out_ids[i] = ids[i];
-    if (out_gamma) out_gamma[i] = gamma[i];
-  }
   return SPD_OK;
 }
 
@@ -769,18 +775,17 @@ int spd_sync(spd_ctx *ctx) {
 int spd_step(spd_ctx *ctx, int32_t *out_ids, int32_t *out_parent, float *out_gamma) {
   int rc = spd_generate_async(ctx, 1);
   if (rc) return rc;
+  StepResult r;
+  if ((rc = fetch_result(ctx, r))) return rc;
+  if ((rc = await_result(ctx, r))) {
+    ctx->prefilled = false;
+    return rc;
+  }
   const int k = ctx->cfg.k;
-  int32_t ids[SPD_MAX_K], par[SPD_MAX_K];
-  float gamma[SPD_MAX_K];
-  const size_t row = (size_t)(ctx->n_gen - 1) * k * 4;  // a launch always completes its first step
-  SPD_CUDA(cudaMemcpyAsync(ids, ctx->ws + ctx->lay.hist_tok + row, (size_t)k * 4, cudaMemcpyDeviceToHost, ctx->stream));
-  SPD_CUDA(cudaMemcpyAsync(par, ctx->ws + ctx->lay.hist_par + row, (size_t)k * 4, cudaMemcpyDeviceToHost, ctx->stream));
-  if ((rc = read_state(ctx, offsetof(spd::State, gamma), gamma, sizeof gamma))) return rc;
-  if ((rc = spd_sync(ctx))) return rc;
-  for (int i = 0; i < k; ++i) {
-    if (out_ids) out_ids[i] = ids[i];
-    if (out_parent) out_parent[i] = par[i];
-    if (out_gamma) out_gamma[i] = gamma[i];
+  for (int i = 0; i < k; ++i) {  // option i * k + j: draft i continued with kept token j
+    if (out_ids) out_ids[i] = r.cand_tok[r.sel[i] % k];
+    if (out_parent) out_parent[i] = r.sel[i] / k;
+    if (out_gamma) out_gamma[i] = r.gamma[i];
   }
   return SPD_OK;
 }
@@ -788,29 +793,31 @@ int spd_step(spd_ctx *ctx, int32_t *out_ids, int32_t *out_parent, float *out_gam
 int spd_generate(spd_ctx *ctx, int32_t n_steps, int32_t *out_tokens, int32_t *out_len, float *out_logp, float *out_gamma) {
   int rc = spd_generate_async(ctx, n_steps);
   if (rc) return rc;
-  if ((rc = spd_sync(ctx))) return rc;  // with a stop token the run may have ended early: n_gen is the device's from here on
+  StepResult r;
+  if ((rc = fetch_result(ctx, r))) return rc;
+  if ((rc = await_result(ctx, r))) {  // with a stop token the run may have ended early: n_gen is the device's from here on
+    ctx->prefilled = false;
+    return rc;
+  }
   const int k = ctx->cfg.k, len = ctx->n_gen;
   std::vector<int32_t> tok((size_t)len * k), par((size_t)len * k);
-  float logp[SPD_MAX_K], gamma[SPD_MAX_K];
   SPD_CUDA(cudaMemcpyAsync(tok.data(), ctx->ws + ctx->lay.hist_tok, tok.size() * 4, cudaMemcpyDeviceToHost, ctx->stream));
   SPD_CUDA(cudaMemcpyAsync(par.data(), ctx->ws + ctx->lay.hist_par, par.size() * 4, cudaMemcpyDeviceToHost, ctx->stream));
-  if ((rc = read_state(ctx, offsetof(spd::State, logP), logp, sizeof logp))) return rc;
-  if ((rc = read_state(ctx, offsetof(spd::State, gamma), gamma, sizeof gamma))) return rc;
   SPD_CUDA(cudaStreamSynchronize(ctx->stream));
   if (out_tokens) {
     // follow each surviving draft's parent links back to the first timestep
-    for (int r = 0; r < k; ++r) {
-      int cur = r;
+    for (int d = 0; d < k; ++d) {
+      int cur = d;
       for (int s = len - 1; s >= 0; --s) {
-        out_tokens[(size_t)r * len + s] = tok[(size_t)s * k + cur];
+        out_tokens[(size_t)d * len + s] = tok[(size_t)s * k + cur];
         cur = par[(size_t)s * k + cur];
       }
     }
   }
   if (out_len) *out_len = len;
   for (int i = 0; i < k; ++i) {
-    if (out_logp) out_logp[i] = logp[i];
-    if (out_gamma) out_gamma[i] = gamma[i];
+    if (out_logp) out_logp[i] = r.logP[i];
+    if (out_gamma) out_gamma[i] = r.gamma[i];
   }
   return SPD_OK;
 }
@@ -846,15 +853,13 @@ int batch_enqueue(spd_ctx *const *ctxs, int32_t n, int32_t n_steps) {
   for (int r = 0; r < n; ++r) {
     kps[r] = ctxs[r]->kp;
     kps[r].pos0 = ctxs[r]->m - 1;
-    SPD_CUDA(cudaMemsetAsync(ctxs[r]->ws + ctxs[r]->lay.state, 0, head_bytes(false), lead->stream));
   }
   spd::KParams *dkp = reinterpret_cast<spd::KParams *>(lead->ws + lead->lay.bt_kp);
-  SPD_CUDA(cudaMemcpyAsync(dkp, kps.data(), kps.size() * sizeof(spd::KParams), cudaMemcpyHostToDevice, lead->stream));
-  SPD_CUDA(cudaStreamSynchronize(lead->stream));  // `kps` leaves scope
+  SPD_CUDA(cudaMemcpyAsync(dkp, kps.data(), kps.size() * sizeof(spd::KParams), cudaMemcpyHostToDevice, lead->stream));  // (pageable: read on return)
   const spd::TcJob job = tc_job(lead);
   for (int s = 0; s < n_steps; ++s) {
     int launched = 0;
-    const cudaError_t e = spd_internal_batch_step(&job, dkp, n, c0.vocab, lead->kp.final_norm, reinterpret_cast<float *>(lead->ws + lead->lay.bt_y),
+    const cudaError_t e = spd_internal_batch_step(&job, dkp, n, s == 0, c0.vocab, lead->kp.final_norm, reinterpret_cast<float *>(lead->ws + lead->lay.bt_y),
                                                   reinterpret_cast<int32_t *>(lead->ws + lead->lay.bt_out), lead->stream, &launched);
     lead->launches += launched;
     if (e != cudaSuccess) return cuda_fail(e, "batched timestep");
@@ -866,13 +871,20 @@ int batch_enqueue(spd_ctx *const *ctxs, int32_t n, int32_t n_steps) {
   return SPD_OK;
 }
 
-int batch_wait(spd_ctx *const *ctxs, int32_t n) {
+// One copy and one wait for the whole batch: the tail kernel left every request's state words and new tokens of the last
+// timestep in its row of the leading context's results.  (The products record a wait that ran out in the leading context's
+// state, which is row 0's.)
+int batch_wait(spd_ctx *const *ctxs, int32_t n, std::vector<int32_t> &rows) {
+  spd_ctx *lead = ctxs[0];
+  rows.resize((size_t)n * spd::kBtResultWords);
+  SPD_CUDA(cudaMemcpyAsync(rows.data(), lead->ws + lead->lay.bt_out, rows.size() * 4, cudaMemcpyDeviceToHost, lead->stream));
+  SPD_CUDA(cudaStreamSynchronize(lead->stream));
   int first = SPD_OK;
   for (int r = 0; r < n; ++r) {
-    const int rc = check_device_error(ctxs[r]);
-    if (rc) {
+    const int32_t err = rows[(size_t)r * spd::kBtResultWords + 2];
+    if (err) {
       ctxs[r]->prefilled = false;
-      if (!first) first = rc;
+      if (!first) first = err;
     }
   }
   return first;
@@ -883,29 +895,16 @@ int batch_wait(spd_ctx *const *ctxs, int32_t n) {
 int spd_batch_generate(spd_ctx *const *ctxs, int32_t n, int32_t n_steps) {
   int rc = batch_enqueue(ctxs, n, n_steps);
   if (rc) return rc;
-  return batch_wait(ctxs, n);
+  std::vector<int32_t> rows;
+  return batch_wait(ctxs, n, rows);
 }
 
 int spd_batch_step(spd_ctx *const *ctxs, int32_t n, int32_t *out_ids, int32_t *out_parent, float *out_gamma) {
   int rc = batch_enqueue(ctxs, n, 1);
   if (rc) return rc;
-  // One copy and one wait for the whole batch: the tail kernel left every request's state words and new tokens in
-  // its row of the leading context's results.  (The products record a wait that ran out in the leading context's
-  // state, which is row 0's.)
-  spd_ctx *lead = ctxs[0];
   static_assert(SPD_MAX_K == spd::kMaxK, "the rows' lists are kMaxK apart");
-  std::vector<int32_t> rows((size_t)n * spd::kBtResultWords);
-  SPD_CUDA(cudaMemcpyAsync(rows.data(), lead->ws + lead->lay.bt_out, rows.size() * 4, cudaMemcpyDeviceToHost, lead->stream));
-  SPD_CUDA(cudaStreamSynchronize(lead->stream));
-  int first = SPD_OK;
-  for (int r = 0; r < n; ++r) {
-    const int32_t *row = rows.data() + (size_t)r * spd::kBtResultWords;
-    if (row[2]) {
-      ctxs[r]->prefilled = false;
-      if (!first) first = row[2];
-    }
-  }
-  if (first) return first;
+  std::vector<int32_t> rows;
+  if ((rc = batch_wait(ctxs, n, rows))) return rc;
   for (int r = 0; r < n; ++r) {
     const int32_t *row = rows.data() + (size_t)r * spd::kBtResultWords;
     const int k = ctxs[r]->cfg.k;

@@ -113,14 +113,19 @@ __device__ __forceinline__ int bt_pos(const KParams &p) { return p.pos0 + p.st->
 
 // grid (requests, column chunks): the superposed input of Eq. 3, h = sum_i gamma_i E[last token of draft i], stored as
 // the request's residual row; h * gain of the first layer's norm as three bf16 terms; the chunk's sum of squares.
+// begin: the first timestep of a call, which clears the requests' error words (a memset per request took the stream 0.1 ms for 64).
 __global__ void __launch_bounds__(kBtThreads) spd_batch_input_kernel(const KParams *kps, float *h, const __nv_bfloat16 *gain, uint16_t *X,
-                                                                     size_t term_stride, int d, float *ss) {
+                                                                     size_t term_stride, int d, float *ss, int begin) {
   dep_launch();
   const int c = blockIdx.y * kBtCols + threadIdx.x * 4;
   const float4 gq = bt_gain(gain, c, d);
   dep_wait();
   const KParams &p = kps[blockIdx.x];
   const State *st = p.st;
+  if (begin && blockIdx.y == 0 && threadIdx.x == 0) {
+    p.st->bar = p.st->stop = p.st->abort_flag = 0u;
+    p.st->err = p.st->err_info = 0;
+  }
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   if (c < d)
     for (int i = 0; i < p.k; ++i) {
@@ -557,7 +562,8 @@ constexpr size_t kBatchTailSmem = 20480;
 // Enqueues one batched timestep of n requests (kps: their parameters in device memory, in row order) on stream s.
 // job: the buffers of the context that lends its long-prefix workspace; y_logits: [128][V] floats.  *launches receives
 // the number of kernels enqueued.
-extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd::KParams *kps, int n, int V, const __nv_bfloat16 *final_norm,
+// begin: the call's first timestep.
+extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd::KParams *kps, int n, int begin, int V, const __nv_bfloat16 *final_norm,
                                                float *y_logits, int32_t *results, cudaStream_t s, int *launches) {
   const spd::TcJob &j = *job;
   const int d = j.d, f = j.f;
@@ -577,7 +583,7 @@ extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd:
   auto resid = [&](const __nv_bfloat16 *gain) {
     if (e == cudaSuccess) done(spd::launch_dep(spd::spd_batch_resid_kernel, dim3(n, nch), threads, 0, s, j.h, pr, gain, j.x, ts_d, d, j.ss));
   };
-  done(spd::launch_dep(spd::spd_batch_input_kernel, dim3(n, nch), threads, 0, s, kps, j.h, j.layers[0].attn_norm, j.x, ts_d, d, j.ss));
+  done(spd::launch_dep(spd::spd_batch_input_kernel, dim3(n, nch), threads, 0, s, kps, j.h, j.layers[0].attn_norm, j.x, ts_d, d, j.ss, begin));
   for (int l = 0; l < j.L && e == cudaSuccess; ++l) {
     product(0, 4 * l, 3 * d);
     if (e == cudaSuccess)

@@ -49,15 +49,15 @@ struct State {
   int32_t n_gen;            // tokens generated per draft so far
   int32_t win[kMaxK][kWin]; // right-aligned: win[i][kWin-1] is draft i's last token
   float logP[kMaxK], gamma[kMaxK];
-  // intermediates of the last step
+  // intermediates of the last step; up to here and with the next two, what a step's caller is told (StepResult)
   int32_t cand_tok[kMaxK];
+  int32_t sel[kMaxK];
   float cand_lp[kMaxK];
   float logP_in[kMaxK];
   int32_t win_in[kMaxK][kWin];
   float score[kMaxK * kMaxK], png[kMaxK * kMaxK];
   uint32_t cnt[kMaxK * kMaxK][kMaxTables];  // 0xffffffff: order skipped
   uint32_t tot[kMaxK][kMaxTables];
-  int32_t sel[kMaxK];
 };
 
 struct KParams {
