@@ -342,8 +342,8 @@ int spd_finished(const spd_ctx *ctx);
 int64_t spd_launch_count(const spd_ctx *ctx);
 
 /* Tuning knobs of the weight-streaming ring (bytes per stage, stages); 0 keeps the default.  Takes
- * effect from the next launch.  SPD_EINVAL if a matrix row does not fit a stage or shared memory
- * would overflow. */
+ * effect from the next launch.  SPD_EINVAL if a matrix row does not fit a stage, shared memory would
+ * overflow or, with fragment-order images, a stage is shorter than 32 columns of 8 rows (512 bytes). */
 int spd_set_ring(spd_ctx *ctx, int32_t stage_bytes, int32_t n_stages);
 
 /* The ring spd_create chooses for a model (host only, no device needed): bytes per stage and stages of the decode

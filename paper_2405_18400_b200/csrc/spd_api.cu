@@ -240,12 +240,35 @@ int pick_ring(const spd_config &c, int32_t stage_bytes, int32_t n_stages, size_t
     else if (maxrow > sb / 2) sb = align_up(maxrow, 1024);
   }
   if (sb % 128 || sb < maxrow) return SPD_EINVAL;
+  if (reserve && sb < (size_t)spd::kPairBytes) return SPD_EINVAL;  // fragment order: a stage takes at least 32 columns of a unit
   int ns = n_stages > 0 ? n_stages : (int)(avail / sb);
   if (ns > spd::kMaxStages) ns = spd::kMaxStages;
   if (ns < 2 || (size_t)ns * sb > avail) return SPD_EINVAL;
   *out_stage = (int32_t)sb;
   *out_n = ns;
   return SPD_OK;
+}
+
+// How the units of matrices in fragment order (d_model columns) pass through the ring.  Units that fill the fewest stages they fit
+// to a tenth keep these to themselves, and the ring is refilled at once (d_model 5120: 54, 54 and 52 of 54 pairs).  Others
+// would leave the ring that much emptier (4096: two stages of 64 pairs where 86 fit), so stages run on across units; then a full
+// ring is more than HBM needs at a time.  Two 32 KB copies per SM already bring 7.0 of the 7.3 TB/s that a bare stream
+// reaches, more requests only queue, the barriers' stores, counters and loads behind them: 112 KB under way at most, in whole
+// stages, two at least (7B shape: stages to themselves and no limit 2.495 ms per timestep; full stages and three under way
+// 2.478, two 2.460).  The 13B shape keeps its units apart without a limit: its steps run into the power cap, and full stages with
+// four under way, 4.50 against 4.55 ms on a cold GPU, took 4.80 against 4.68.
+void plan_units(const spd_config &c, bool images, spd::KParams &kp) {
+  kp.most_flying = kp.n_stages;
+  kp.img_span = 0;
+  kp.img_pairs = 1;
+  if (!images) return;
+  const int unit = c.d_model / 32, cap = kp.stage_bytes / spd::kPairBytes, parts = (unit + cap - 1) / cap, even = (unit + parts - 1) / parts;
+  kp.img_span = even * 10 < cap * 9;
+  kp.img_pairs = kp.img_span ? cap : even;
+  if (kp.img_span) {
+    const int flying = 112 * 1024 / kp.stage_bytes;
+    kp.most_flying = flying < 2 ? 2 : (flying < kp.n_stages ? flying : kp.n_stages);
+  }
 }
 
 // What a call tells its caller about the last step, as it lies in the state: one copy.  (A copy into pageable memory is a round
@@ -499,6 +522,7 @@ int spd_create(const spd_config *cfg, const spd_weights *w, const spd_ngram_tabl
     rc = pick_ring(*cfg, 0, 0, 0, &kp.stage_bytes, &kp.n_stages);
   }
   if (rc) return fail(rc);
+  plan_units(*cfg, img, kp);
   ctx->dyn_smem = (size_t)kp.stage_bytes * kp.n_stages + kPartBytes + (img ? frag_bytes(*cfg) : 0);
   int per_sm = 0;
   e = spd_internal_prepare(ctx->dyn_smem, &per_sm);
@@ -645,6 +669,7 @@ int spd_set_ring(spd_ctx *ctx, int32_t stage_bytes, int32_t n_stages) {
   if (per_sm < 1) return SPD_EINVAL;
   ctx->kp.stage_bytes = sb;
   ctx->kp.n_stages = ns;
+  plan_units(ctx->cfg, ctx->kp.lm_head_img != nullptr, ctx->kp);
   ctx->dyn_smem = dyn;
   return SPD_OK;
 }

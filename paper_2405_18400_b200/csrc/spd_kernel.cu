@@ -97,7 +97,26 @@ struct Producer {
   uint32_t stage, phase;
   uint32_t issued;  // chunks issued so far (saturating at n_stages for the drain)
   uint64_t policy;  // the weights' L2 policy
+  uint32_t landed, landed_phase;  // stage and phase of the oldest chunk that may still be under way
+  uint32_t flying;                // chunks issued from that one on
 };
+
+// A chunk of weights into the next stage, once that is free.
+__device__ __forceinline__ void issue_chunk(Blk &b, Producer &pr, const uint8_t *src, uint32_t bytes) {
+  const KParams &p = *b.p;
+  if (pr.flying == (uint32_t)p.most_flying) {
+    wait_mbar(b, &s_full[pr.landed], pr.landed_phase, 210);
+    if (++pr.landed == (uint32_t)p.n_stages) { pr.landed = 0; pr.landed_phase ^= 1u; }
+  } else {
+    ++pr.flying;
+  }
+  wait_mbar(b, &s_empty[pr.stage], pr.phase ^ 1u, 200);
+  if (s_dead) return;
+  mbar_expect_tx(&s_full[pr.stage], bytes);
+  bulk_load_policy(smem + (size_t)pr.stage * p.stage_bytes, src, bytes, &s_full[pr.stage], pr.policy);
+  if (pr.issued < (uint32_t)p.n_stages) ++pr.issued;
+  if (++pr.stage == (uint32_t)p.n_stages) { pr.stage = 0; pr.phase ^= 1u; }
+}
 
 __device__ __forceinline__ void produce_matrix(Blk &b, Producer &pr, const __nv_bfloat16 *W, int R, int C, int gran) {
   const KParams &p = *b.p;
@@ -109,54 +128,31 @@ __device__ __forceinline__ void produce_matrix(Blk &b, Producer &pr, const __nv_
     const int t1 = min(t0 + kTile, r1);
     for (int r = t0; r < t1; r += rpc) {
       const int n = min(rpc, t1 - r);
-      wait_mbar(b, &s_empty[pr.stage], pr.phase ^ 1u, 200);
+      issue_chunk(b, pr, (const uint8_t *)W + (size_t)r * rowbytes, (uint32_t)n * rowbytes);
       if (s_dead) return;
-      const uint32_t bytes = (uint32_t)n * rowbytes;
-      mbar_expect_tx(&s_full[pr.stage], bytes);
-      bulk_load_policy(smem + (size_t)pr.stage * p.stage_bytes, (const uint8_t *)W + (size_t)r * rowbytes, bytes, &s_full[pr.stage],
-                       pr.policy);
-      if (pr.issued < (uint32_t)p.n_stages) ++pr.issued;
-      if (++pr.stage == (uint32_t)p.n_stages) { pr.stage = 0; pr.phase ^= 1u; }
     }
   }
 }
 
-constexpr int kPairBytes = kUnitRows * 64;  // a unit's share of a pair of 16-column blocks: 4 lanes of 16 bytes per row
-// Bytes of a fragment-order unit of C columns that one ring stage takes: the unit in the fewest equal parts that fit
-// a stage, in whole pairs of 16-column blocks (the last part may be shorter).
-__device__ __forceinline__ uint32_t img_chunk(const KParams &p, int C) {
-  const uint32_t unit = (uint32_t)C * 2u * kUnitRows, cap = (uint32_t)p.stage_bytes / kPairBytes * kPairBytes;
-  const uint32_t parts = (unit + cap - 1) / cap;
-  const uint32_t pairs = ((uint32_t)C / 32 + parts - 1) / parts;
-  return pairs * kPairBytes;
-}
-
-// A matrix in fragment order (spd_pack_image): the units of this block, each unit in stages of img_chunk bytes and a
-// shorter last one.
+// A matrix in fragment order (spd_pack_image): the units of this block are one contiguous run.
 __device__ __forceinline__ void produce_image(Blk &b, Producer &pr, const __nv_bfloat16 *img, int R, int C) {
   const KParams &p = *b.p;
   int r0, r1;
   cta_rows(R, kUnitRows, r0, r1);
-  const uint32_t unit_bytes = (uint32_t)C * 2u * kUnitRows;
-  for (int r = r0; r < r1; r += kUnitRows) {
-    const uint8_t *src = reinterpret_cast<const uint8_t *>(img) + (size_t)(r / kUnitRows) * unit_bytes;
-    const uint32_t chunk = img_chunk(p, C);
-    for (uint32_t off = 0; off < unit_bytes; off += chunk) {
-      const uint32_t bytes = unit_bytes - off < chunk ? unit_bytes - off : chunk;
-      wait_mbar(b, &s_empty[pr.stage], pr.phase ^ 1u, 200);
+  const uint8_t *src = reinterpret_cast<const uint8_t *>(img) + (size_t)r0 * C * 2;
+  const int unit = C / 32, all = (r1 - r0) / kUnitRows * unit;
+  const int run = p.img_span ? all : unit;  // what a stage does not reach beyond
+  for (int at = 0; at < all; at += run)
+    for (int u = 0; u < run; u += p.img_pairs) {
+      issue_chunk(b, pr, src + (size_t)(at + u) * kPairBytes, (uint32_t)min(p.img_pairs, run - u) * kPairBytes);
       if (s_dead) return;
-      mbar_expect_tx(&s_full[pr.stage], bytes);
-      bulk_load_policy(smem + (size_t)pr.stage * p.stage_bytes, src + off, bytes, &s_full[pr.stage], pr.policy);
-      if (pr.issued < (uint32_t)p.n_stages) ++pr.issued;
-      if (++pr.stage == (uint32_t)p.n_stages) { pr.stage = 0; pr.phase ^= 1u; }
     }
-  }
 }
 
 template <bool kSampler, bool kImg>
 __device__ void producer_main(Blk &b) {
   const KParams &p = *b.p;
-  Producer pr{0u, 0u, 0u, evict_first_policy()};
+  Producer pr{0u, 0u, 0u, evict_first_policy(), 0u, 0u, 0u};
   // The layers' pointers sit in device memory that the weight stream has long pushed out of L2 when their turn
   // comes: each layer's are fetched while the layer before is streamed.
   LayerW lw = p.layers[0];
@@ -470,14 +466,17 @@ __device__ __forceinline__ void store_frags(const KParams &p, int C, const float
 }
 
 // Streams this block's units of one matrix in fragment order through the ring: per unit and 32 columns one 16-byte load of
-// weights, one 8-byte load of x and one instruction, the pairs of column blocks of a stage dealt to the warps in turn; a
-// row's sum is the sum of its six wanted columns of the accumulator.
+// weights, one 8-byte load of x and one instruction, a unit's pairs of column blocks dealt to the warps in turn; a row's
+// sum is the sum of its six wanted columns of the accumulator.
 __device__ __forceinline__ void consume_image(Blk &b, int R, int C, int kind, const EpiArgs &ea) {
   const KParams &p = *b.p;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int r0, r1;
   cta_rows(R, kUnitRows, r0, r1);
-  const int n_pairs = C / 32;
+  const int unit_pairs = C / 32;
+  int left = (r1 - r0) / kUnitRows * unit_pairs;  // pairs behind the stage at hand
+  int in_stage = 0, n = 0;                        // the stage's pairs used up, in all
+  const uint8_t *stage = smem;
   const uint2 *xf = reinterpret_cast<const uint2 *>(xfrag_base(p)) + min(lane, 23);
   float h_pre = 0.f;
   if (kind == kEpiAddH && r0 + (int)threadIdx.x < min(r0 + kTile, r1)) h_pre = __ldcg(p.h + r0 + threadIdx.x);
@@ -488,17 +487,26 @@ __device__ __forceinline__ void consume_image(Blk &b, int R, int C, int kind, co
     float *part = scratch_base(p) + (size_t)buf * kTile * kConsumerWarps;
     for (int r = t0; r < t1; r += kUnitRows) {
       float c[4] = {0.f, 0.f, 0.f, 0.f};
-      const int per_stage = (int)(img_chunk(p, C) / kPairBytes);
-      for (int pr0 = 0; pr0 < n_pairs; pr0 += per_stage) {  // one stage
-        wait_mbar(b, &s_full[b.c_stage], b.c_phase, 300);
-        const uint8_t *stage = smem + (size_t)b.c_stage * p.stage_bytes;
-        const int n = min(per_stage, n_pairs - pr0);
+      for (int u = 0; u < unit_pairs;) {  // the unit's pairs, stage by stage
+        if (in_stage == n) {
+          wait_mbar(b, &s_full[b.c_stage], b.c_phase, 300);
+          stage = smem + (size_t)b.c_stage * p.stage_bytes;
+          in_stage = 0;
+          n = min(p.img_pairs, p.img_span ? left : unit_pairs - u);
+          left -= n;
+        }
+        const int m = min(unit_pairs - u, n - in_stage);
+        const uint8_t *w = stage + ((size_t)in_stage * (4 * kUnitRows) + lane) * 16;
+        const uint2 *x = xf + (size_t)u * 24;
 #pragma unroll 1  // unrolled, the loop costs more registers than the kernel has
-        for (int j = warp; j < n; j += kConsumerWarps)
-          mma_terms(c, lds128(stage + ((size_t)j * (4 * kUnitRows) + lane) * 16), xf[(size_t)(pr0 + j) * 24]);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&s_empty[b.c_stage]);
-        if (++b.c_stage == (uint32_t)p.n_stages) { b.c_stage = 0; b.c_phase ^= 1u; }
+        for (int j = (warp - u) & (kConsumerWarps - 1); j < m; j += kConsumerWarps) mma_terms(c, lds128(w + (size_t)j * kPairBytes), x[(size_t)j * 24]);
+        u += m;
+        in_stage += m;
+        if (in_stage == n) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&s_empty[b.c_stage]);
+          if (++b.c_stage == (uint32_t)p.n_stages) { b.c_stage = 0; b.c_phase ^= 1u; }
+        }
       }
       // row g: columns 0 and 1 in lane 4 g; 2 and, of row 8 + g, 3 in lane 4 g + 1; 4 and 5 of row 8 + g in lane 4 g + 2
       const int t = lane & 3;

@@ -23,6 +23,7 @@ constexpr int kTensorMapBytes = 128; // size of one tensor map object (CUtensorM
 constexpr int kPfTokens = 16;       // prefix tokens one prefill launch takes
 constexpr int kUnitRows = 8;        // rows of a unit of a matrix in fragment order (the granularity of the blocks' shares; 4 was
                                     // measured too: the shares come out more even, but a 7B timestep took 4.16 ms against 2.65 ms)
+constexpr int kPairBytes = kUnitRows * 64; // a unit's share of a pair of 16-column blocks: 4 lanes of 16 bytes per row
 constexpr int kScratchBytes = 20480; // per-block scratch after the decode kernel's ring: row partials / attention merge / tail
 
 enum Mode { kModePrefill = 0, kModeDecode = 1, kModeScoreOnly = 2, kModeSample = 3, kModeNucleusOnly = 4 };
@@ -107,6 +108,9 @@ struct KParams {
   int32_t pf_stall;          // prefill kernel, test hook: block 0 withholds its arrival at the grid barriers
   int32_t eos_id;            // stop token (-1: none): decoding ends with the step in which the most probable draft emits it
   const __nv_bfloat16 *lm_head_img;  // the LM head in fragment order, or null
+  // how units in fragment order pass through the ring (plan_units): pairs of column blocks a stage takes, whether a stage may hold the
+  // end of a unit and the start of the next; stages of weights that a block has under way at most
+  int32_t img_pairs, img_span, most_flying;
 };
 
 }  // namespace spd
