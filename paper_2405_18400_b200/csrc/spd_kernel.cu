@@ -1083,7 +1083,7 @@ __global__ void __launch_bounds__(kThreads, 1) spd_sample_kernel(const __grid_co
 // units of them divide unevenly among the blocks and their fragments of x would take a third of the ring's memory
 // (measured: 2.96 ms per 7B timestep with it on the tensor cores too, against 2.64 ms).
 __global__ void __launch_bounds__(kThreads, 1) spd_decode_img_kernel(const __grid_constant__ KParams p) { kernel_body<false, true>(p); }
-// The sampling twin for such weights (7B shape: 2.72 ms per sampled token; the float32 loop for every matrix 2.99).
+// The sampling twin for such weights (7B shape: 2.63 ms per sampled token; the float32 loop for every matrix 2.99).
 __global__ void __launch_bounds__(kThreads, 1) spd_sample_img_kernel(const __grid_constant__ KParams p) { kernel_body<true, true>(p); }
 
 }  // namespace spd
