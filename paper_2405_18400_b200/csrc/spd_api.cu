@@ -366,6 +366,7 @@ spd::TcJob tc_job(spd_ctx *ctx) {
   job.ss = reinterpret_cast<float *>(ctx->ws + ctx->lay.bt_ss);
   job.ids = nullptr;
   job.pos0 = job.n_tok = 0;
+  job.short_chains = 0;
   return job;
 }
 
@@ -397,6 +398,7 @@ int prefill_tokens(spd_ctx *ctx, int first, int count) {
       job.ids = base + first + tc_done;
       job.pos0 = first + tc_done;
       job.n_tok = n;
+      job.short_chains = n > (kp.max_pos - 2) / spd::kTcTile * spd::kTcTile;
       int launched = 0;
       const cudaError_t e = spd_internal_tc_prefill(&job, tc_done + n == count ? &kp : nullptr, ctx->stream, &launched);
       ctx->launches += launched;

@@ -318,12 +318,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
         if (!tc_wait(sh, st, &sh.full[stage], phase, 410)) break;
         tc_fence_after();
         const uint32_t base = ring + stage * (uint32_t)S::kStageBytes, acc = tmem + (uint32_t)(a * S::kAccStride);
-        const uint32_t term0 = base + kTcWBytes + (S::kFused ? 0 : 2 * S::kTermBytes);  // (a stage's small terms before the large one)
+        const uint32_t term0 = base + kTcWBytes + (!S::kFused && pr.small_first ? 2 * S::kTermBytes : 0);
+        const int term_step = pr.small_first ? -S::kTermBytes : S::kTermBytes;
 #pragma unroll
         for (int j = 0; j < (S::kFused ? 1 : 3); ++j)
 #pragma unroll
           for (int kk = 0; kk < kTcKB / 16; ++kk)  // 16 columns = 32 bytes further into the swizzled rows
-            tc_pair_mma(acc, tc_desc(base + kk * 32), tc_desc(term0 - j * S::kTermBytes + kk * 32), idesc, (uint32_t)((in_seg | j | kk) != 0));
+            tc_pair_mma(acc, tc_desc(base + kk * 32), tc_desc(term0 + j * term_step + kk * 32), idesc, (uint32_t)((in_seg | j | kk) != 0));
         tc_pair_commit(&sh.empty[stage]);  // the stage is free in both blocks once these have read it
         if (++stage == (uint32_t)S::kStages) { stage = 0; phase ^= 1u; }
         ++kb;
@@ -815,7 +816,7 @@ extern "C" cudaError_t spd_internal_tc_prepare(void) {
 extern "C" cudaError_t spd_internal_product(const spd::TcJob *job, int n_tok, int wide, int which, float *Y, int N, spd::Product *out, cudaStream_t s) {
   const spd::TcJob &j = *job;
   const void *wmap = j.w_tmaps + (size_t)which * spd::kTensorMapBytes;
-  const spd::Product pr = spd::plan_product(n_tok, N, wide ? j.f : j.d, j.sm_count, Y, j.parts);
+  const spd::Product pr = spd::plan_product(n_tok, N, wide ? j.f : j.d, j.sm_count, Y, j.parts, j.short_chains != 0);
   *out = pr;
   switch (pr.shape) {
     case 16: return launch_product<16>(j, wide, wmap, Y, pr, n_tok, s, 0);

@@ -23,9 +23,10 @@ struct Product {
   int32_t N, nk, tile_tok, tok_tiles, total, pairs, shape;  // shape: 16, 32, 64, 128 or 256, the kernel's instance
   int32_t align;  // a cut lies a multiple of so many stages behind its tile's first (rounded down)
   int32_t seg;    // stages whose sums an accumulator takes before they move to registers
+  int32_t small_first;  // one instruction per term: a stage's small terms before the large one
 };
 
-inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *y, const float *parts) {
+inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *y, const float *parts, bool short_chains = false) {
   Product pr;
   pr.y = y;
   pr.parts = parts;
@@ -46,12 +47,14 @@ inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *
   // sum's own size).  4 stages cost nothing (2: 1 % at 15 tokens, 3 % at 64; 1: 2 % and 10 %).  Where the terms share one, C / 512
   // stages at most, as many additions as the 3 C / 128 that a warp of the 16-token kernel chains; two at least beyond 128 rows,
   // where the epilogue of one stage takes longer than its instructions (8 layers of 256 columns, 200 tokens: one stage 0.85 ms,
-  // two 0.77; error of the first timestep 4.0e-7 and 5.9e-7, the 16-token kernel's path 1.9e-6).  129 to 384 rows take no more
-  // than those two, so that a prefix of that length is no further from 64 bits in one job than in two shorter ones (7B shape,
-  // first timestep's logits, relative 2-norm: 200 tokens 5.5e-6, with four stages 1.1e-5; 300 tokens 6.8e-6, four 1.3e-5, 256 and
-  // 44 tokens apart 9.8e-6), for 1 % of the time; beyond, four (512 tokens 1.1e-5; with eight and the terms in order 2.9e-5).
-  const int least_seg = n_tok > 128 ? 2 : 1, most_seg = n_tok > 128 && n_tok <= 384 ? 2 : 4, wide = C / 512;
+  // two 0.77; error of the first timestep 4.0e-7 and 5.9e-7, the 16-token kernel's path 1.9e-6).  Uncut tiles of wide matrices
+  // take up to 8 stages, the terms in order: a bf16 cache behind a long prefix then holds the bits that it always has (with four,
+  // and two up to 384 rows, 28 of 60 requests chose another draft within nine timesteps behind 100 to 1900 tokens).  short_chains: a job that stands for two (TcJob), which is to be no further
+  // from 64 bits than these: two stages beyond 128 rows, for 1 % of the time (7B shape, first timestep's logits, relative 2-norm:
+  // 144 tokens 5.1e-6, as 128 and 16 7.1e-6, with four stages 1.1e-5; 300 tokens 6.8e-6, as 256 and 44 9.8e-6, with eight 3.1e-5).
+  const int least_seg = n_tok > 128 ? 2 : 1, most_seg = n_tok > 128 && short_chains ? 2 : (whole ? 8 : 4), wide = C / 512;
   pr.seg = pr.shape <= 64 ? 4 : (wide < least_seg ? least_seg : (wide < most_seg ? wide : most_seg));
+  pr.small_first = pr.seg < 8;
   // a pair takes a tile, two segments or four stages at least (small matrices: fewer parts to add)
   const int least = whole ? pr.nk : (pr.align > 1 ? 2 * pr.align : 4);
   const int most = sm_count / 2 < kTcMaxPairs ? sm_count / 2 : kTcMaxPairs, worth = pr.total / least;
@@ -126,6 +129,7 @@ struct TcJob {
   int32_t pos0, n_tok;               // first position; tokens (<= x_term_rows)
   State *st;
   int32_t sm_count;                  // SMs of the device
+  int32_t short_chains;              // the job is longer than the context's positions rounded down to a multiple of 128, so that it stands for two
   float *ss;                         // [128][32]: sums of squares of the residual rows per 512-column chunk
 };
 

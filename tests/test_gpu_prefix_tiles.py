@@ -40,18 +40,20 @@ def test_tokens_of_a_job(wide, max_pos, m, jobs):
     ctx.close()
 
 
-@pytest.mark.parametrize("m", [129, 200, 257, 300, 400, 512])
-def test_first_timestep_of_long_jobs(wide, m):
-    """Jobs of more than 128 rows: chains of 24 additions (up to 384 rows) or 24 at this width beyond (C / 512 stages of 12), the
-    small terms first.  The logits are below 8, a rounding of float32 there is 2.4e-7 at most; twenty of them are the bound
-    (chains of 96 additions: 1.6e-5 and more at 7B width)."""
+@pytest.mark.parametrize("m", [129, 200, 257, 300, 400])
+def test_a_job_that_stands_for_two_is_as_exact(wide, m):
+    """In a context of m + 65 positions these prefixes are one job, longer than the positions rounded down to a multiple of 128:
+    chains of 24 additions, the small terms first.  The logits are below 8, a rounding of float32 there is 2.4e-7 at most;
+    twenty of them are the bound (chains of 96 additions: 1.6e-5 and more at 7B width)."""
     import numpy as np
     shape, weights, tables = wide
-    ctx, orc = make_pair(shape, weights, tables, 3, (2, 3), LAM, 0.4, 0.2, 0.05, 768, "f32")
+    ctx, orc = make_pair(shape, weights, tables, 3, (2, 3), LAM, 0.4, 0.2, 0.05, m + 65, "f32")
     worst = []
     for seed in range(3):
         prefix = si.make_prefix("zipf", m, shape.vocab, 1.1, seed=115 + seed)
+        before = ctx.spd_launch_count()
         ctx.spd_prefill(prefix)
+        assert ctx.spd_launch_count() - before == 9 * shape.n_layers + 1
         orc.prefill(prefix)
         worst.append(float(np.abs(ctx.spd_debug_read("LOGITS").astype(np.float64) - orc.logits()).max()))
         assert np.abs(orc.logits()).max() < 8
