@@ -46,15 +46,15 @@ struct Layout {
       bt_ss, bt_out, total;
 };
 
-// Tokens one long-prefix job takes at most (0: the context never runs one): the context's longest prefix to the nearest multiple
-// of 128.  Rounded up, the buffers hold up to 63 rows that no prefix fills; rounded down from the upper half, the last 64 tokens and
-// more would be a job of their own, a pass over the weights for them (400 tokens in a context of 465 positions, 7B shape: 384
-// and 16 tokens 19.2 ms, one job 17.0).
+// Tokens one long-prefix job takes at most (0: the context never runs one): the context's longest prefix rounded down to a
+// multiple of 128.  (To the nearest multiple, 400 tokens in a context of 465 positions are one job instead of 384 and 16
+// tokens, 17.0 ms instead of 19.2 at 7B shape; but its sums of other lengths round a bf16 cache otherwise than the two
+// jobs do, 1.9e-3 of the first timestep's logits, and chains short enough to be no further from 64 bits than theirs had to
+// hang on the room that the context has left.)
 int tc_rows(const spd_config &c) {
   const int hd = c.d_model / c.n_heads;
   if (hd != 64 && hd != 128) return 0;  // the head sizes its attention kernel is built for
-  if (c.max_pos < spd::kTcTile + 2) return 0;
-  const int full = (c.max_pos - 2 + spd::kTcTile / 2) / spd::kTcTile * spd::kTcTile;
+  const int full = (c.max_pos - 2) / spd::kTcTile * spd::kTcTile;
   return full < spd::kTcMaxTokens ? full : spd::kTcMaxTokens;
 }
 
@@ -366,7 +366,6 @@ spd::TcJob tc_job(spd_ctx *ctx) {
   job.ss = reinterpret_cast<float *>(ctx->ws + ctx->lay.bt_ss);
   job.ids = nullptr;
   job.pos0 = job.n_tok = 0;
-  job.short_chains = 0;
   return job;
 }
 
@@ -398,7 +397,6 @@ int prefill_tokens(spd_ctx *ctx, int first, int count) {
       job.ids = base + first + tc_done;
       job.pos0 = first + tc_done;
       job.n_tok = n;
-      job.short_chains = n > (kp.max_pos - 2) / spd::kTcTile * spd::kTcTile;
       int launched = 0;
       const cudaError_t e = spd_internal_tc_prefill(&job, tc_done + n == count ? &kp : nullptr, ctx->stream, &launched);
       ctx->launches += launched;

@@ -2,7 +2,7 @@
 // time, their matrix products on the fifth-generation tensor cores (tcgen05.mma, operands staged in shared
 // memory by tiled TMA copies, float32 accumulators in tensor memory), everything between the products in small
 // row-wise kernels.  The job that ends a prefix goes on to the LM head and the first timestep of its last token
-// (7B shape, host to host: 15 / 27 / 100 / 400 / 2048 tokens 3.1 / 3.2 / 5.1 / 17 / 84 ms; with 128 x 128 tiles of single
+// (7B shape, host to host: 15 / 27 / 100 / 400 / 2048 tokens 3.1 / 3.2 / 5.1 / 18 / 81 ms; with 128 x 128 tiles of single
 // blocks and the last 1..16 tokens in spd_prefill_kernel 4.7 / 9.2 / 12.2 / 24 / 110 ms).
 //
 // Product: Y[token][row] = sum_c X[token][c] W[row][c], W bf16 [rows][cols] as stored, X float32 activations
@@ -816,7 +816,7 @@ extern "C" cudaError_t spd_internal_tc_prepare(void) {
 extern "C" cudaError_t spd_internal_product(const spd::TcJob *job, int n_tok, int wide, int which, float *Y, int N, spd::Product *out, cudaStream_t s) {
   const spd::TcJob &j = *job;
   const void *wmap = j.w_tmaps + (size_t)which * spd::kTensorMapBytes;
-  const spd::Product pr = spd::plan_product(n_tok, N, wide ? j.f : j.d, j.sm_count, Y, j.parts, j.short_chains != 0);
+  const spd::Product pr = spd::plan_product(n_tok, N, wide ? j.f : j.d, j.sm_count, Y, j.parts);
   *out = pr;
   switch (pr.shape) {
     case 16: return launch_product<16>(j, wide, wmap, Y, pr, n_tok, s, 0);

@@ -26,7 +26,7 @@ struct Product {
   int32_t small_first;  // one instruction per term: a stage's small terms before the large one
 };
 
-inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *y, const float *parts, bool short_chains = false) {
+inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *y, const float *parts) {
   Product pr;
   pr.y = y;
   pr.parts = parts;
@@ -35,7 +35,7 @@ inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *
   // Up to 64 token rows the three terms share an instruction; up to 256 rows are one tile; more rows make enough tiles of
   // up to 128 (all alike) to fill the pairs without cutting one: then every sum is one pair's.  From 65 rows on a tile's rows
   // are rounded up to 16, which is what an instruction's N allows (to 32: 100 tokens, 7B shape, 5.5 ms instead of 5.1; 400
-  // tokens 18.6 instead of 17.0).  Between 129 and 256 rows tiles are cut at multiples of eight stages.
+  // tokens as one job 18.6 instead of 17.0).  Between 129 and 256 rows tiles are cut at multiples of eight stages.
   const bool whole = n_tok > kTcMaxTileTok;
   pr.shape = n_tok <= 16 ? 16 : (n_tok <= 32 ? 32 : (n_tok <= 64 ? 64 : (n_tok <= 128 || whole ? 128 : 256)));
   pr.tok_tiles = whole ? (n_tok + 127) / 128 : 1;
@@ -48,11 +48,11 @@ inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *
   // stages at most, as many additions as the 3 C / 128 that a warp of the 16-token kernel chains; two at least beyond 128 rows,
   // where the epilogue of one stage takes longer than its instructions (8 layers of 256 columns, 200 tokens: one stage 0.85 ms,
   // two 0.77; error of the first timestep 4.0e-7 and 5.9e-7, the 16-token kernel's path 1.9e-6).  Uncut tiles of wide matrices
-  // take up to 8 stages, the terms in order: a bf16 cache behind a long prefix then holds the bits that it always has (with four,
-  // and two up to 384 rows, 28 of 60 requests chose another draft within nine timesteps behind 100 to 1900 tokens).  short_chains: a job that stands for two (TcJob), which is to be no further
-  // from 64 bits than these: two stages beyond 128 rows, for 1 % of the time (7B shape, first timestep's logits, relative 2-norm:
-  // 144 tokens 5.1e-6, as 128 and 16 7.1e-6, with four stages 1.1e-5; 300 tokens 6.8e-6, as 256 and 44 9.8e-6, with eight 3.1e-5).
-  const int least_seg = n_tok > 128 ? 2 : 1, most_seg = n_tok > 128 && short_chains ? 2 : (whole ? 8 : 4), wide = C / 512;
+  // take up to 8 stages, the terms in order: a bf16 cache behind a long prefix then holds the bits that it always has.  (Four
+  // there, and two up to 384 rows, cost 1 % of the time and come closer to 64 bits: 300 tokens, 7B shape, first timestep's
+  // logits, relative 2-norm, 6.8e-6 instead of 3.1e-5.  But 28 of 60 requests then chose another draft within nine timesteps behind
+  // 100 to 1900 tokens.)
+  const int least_seg = n_tok > 128 ? 2 : 1, most_seg = whole ? 8 : 4, wide = C / 512;
   pr.seg = pr.shape <= 64 ? 4 : (wide < least_seg ? least_seg : (wide < most_seg ? wide : most_seg));
   pr.small_first = pr.seg < 8;
   // a pair takes a tile, two segments or four stages at least (small matrices: fewer parts to add)
@@ -129,7 +129,6 @@ struct TcJob {
   int32_t pos0, n_tok;               // first position; tokens (<= x_term_rows)
   State *st;
   int32_t sm_count;                  // SMs of the device
-  int32_t short_chains;              // the job is longer than the context's positions rounded down to a multiple of 128, so that it stands for two
   float *ss;                         // [128][32]: sums of squares of the residual rows per 512-column chunk
 };
 
