@@ -705,6 +705,9 @@ __device__ __forceinline__ void unpack16(const uint4 &v, float (&x)[16 / sizeof(
     }
   }
 }
+// What scores are taken relative to: their maximum, or 0 while that is -inf, so that scores of -inf have the weight 0 (relative
+// to -inf they would be NaN, which no later weight of 0 takes out of a sum; a NaN score stays one).
+__device__ __forceinline__ float score_base(float largest) { return largest == -CUDART_INF_F ? 0.f : largest; }
 // The attention phase for head sizes 64 and 128: HD * sizeof(E) / 16 lanes take one position with 16-byte loads (a whole
 // warp for float32 of head size 128, half of one for bf16, a quarter for bf16 of 64), and each such group keeps four positions
 // in flight, which enter its running softmax together (one rescale per round instead of four dependent ones): the phase stands
@@ -757,13 +760,13 @@ __device__ void attention_rows(Blk &b, int layer, int pos) {
         mn = fmaxf(mn, sc[u]);
       }
       if (tb + grp < t1) {  // else no position of this round belongs to the group (a NaN score, which fmaxf passes over, has to reach the sums)
-        const float c = __expf(m - mn);
+        const float from = score_base(mn), c = __expf(m - from);
         l *= c;
 #pragma unroll
         for (int e = 0; e < EPL; ++e) acc[e] *= c;
 #pragma unroll
         for (int u = 0; u < F; ++u) {
-          const float pw = __expf(sc[u] - mn);
+          const float pw = __expf(sc[u] - from);
           l += pw;
           float vx[EPL];
           unpack16<E>(vq[u], vx);
@@ -854,8 +857,8 @@ __device__ void attention_phase(Blk &b, int layer, int pos) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
       const float s = dot * scale;
-      const float mn = fmaxf(m, s);
-      const float c = __expf(m - mn), pw = __expf(s - mn);
+      const float mn = fmaxf(m, s), from = score_base(mn);
+      const float c = __expf(m - from), pw = __expf(s - from);
       l = l * c + pw;
 #pragma unroll
       for (int e = 0; e < 8; ++e) acc[e] = acc[e] * c + pw * vv[e];

@@ -42,3 +42,33 @@ def test_nan_in_the_cache_reaches_the_logits(shapes):
         ctx.spd_step()
         assert np.isnan(ctx.spd_debug_read("LOGITS")).all()
         ctx.close()
+
+
+@pytest.mark.parametrize("kv_dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("hd", [32, 64, 128])
+def test_positions_that_score_minus_infinity_have_no_weight(hd, kv_dtype):
+    """The first 40 of 41 keys of a head infinite in one dimension: with the sign that makes their scores -inf they drop out of
+    the softmax, to the bit as with a score of -1e27 or so; with the other, scores of +inf, the head's output is NaN.  Most
+    groups of lanes meet nothing but -inf."""
+    import paper_2405_18400_b200 as P
+    import torch
+    shape = si.ModelShape("inf%d" % hd, 2, 2 * hd, 2, 256, 600)
+    packed = P.pack_weights(si.make_weights(shape, seed=105), "cuda:0")
+    ctx = P.SpdContext(shape, packed, [], 3, (2, 3), [0.0] * 8, 0.4, 0.2, 0.05, 64, kv_dtype)
+    prefix = si.make_prefix("zipf", 41, shape.vocab, 1.1, seed=106)
+    dtype, size = (torch.bfloat16, 2) if kv_dtype == "bf16" else (torch.float32, 4)
+
+    def step(value):
+        ctx.spd_prefill(prefix)
+        keys = ctx.workspace[: 64 * 2 * hd * size].view(dtype).view(64, 2 * hd)   # first layer [max_pos][d_model]
+        keys[:40, hd + 5] = value
+        ctx.spd_step()
+        return ctx.spd_debug_read("LOGITS")
+
+    large = {s: step(s * 1e30) for s in (1.0, -1.0)}
+    infinite = {s: step(s * float("inf")) for s in (1.0, -1.0)}
+    assert all(np.isfinite(z).all() for z in large.values())
+    sign = 1.0 if np.isnan(infinite[-1.0]).all() else -1.0
+    assert np.isnan(infinite[-sign]).all()
+    assert np.array_equal(infinite[sign], large[sign])
+    ctx.close()
