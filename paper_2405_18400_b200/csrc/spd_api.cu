@@ -304,6 +304,14 @@ int check_device_error(spd_ctx *ctx) {
   return rc ? rc : await_result(ctx, r);
 }
 
+// The same behind decode steps: a run that failed, or whose result did not arrive, leaves no drafts to go on from.
+int step_result(spd_ctx *ctx, StepResult &r) {
+  int rc = fetch_result(ctx, r);
+  if (!rc) rc = await_result(ctx, r);
+  if (rc) ctx->prefilled = false;
+  return rc;
+}
+
 // The way out of a call that fails: the copies from the caller's memory and from this call's have been made.
 int give_back(spd_ctx *ctx, int rc) {
   cudaStreamSynchronize(ctx->stream);
@@ -792,20 +800,15 @@ int spd_sync(spd_ctx *ctx) {
   if (!ctx) return SPD_EINVAL;
   int rc = set_device(ctx);
   if (rc) return rc;
-  rc = check_device_error(ctx);
-  if (rc) ctx->prefilled = false;
-  return rc;
+  StepResult r;
+  return step_result(ctx, r);
 }
 
 int spd_step(spd_ctx *ctx, int32_t *out_ids, int32_t *out_parent, float *out_gamma) {
   int rc = spd_generate_async(ctx, 1);
   if (rc) return rc;
   StepResult r;
-  if ((rc = fetch_result(ctx, r))) return rc;
-  if ((rc = await_result(ctx, r))) {
-    ctx->prefilled = false;
-    return rc;
-  }
+  if ((rc = step_result(ctx, r))) return rc;
   const int k = ctx->cfg.k;
   for (int i = 0; i < k; ++i) {  // option i * k + j: draft i continued with kept token j
     if (out_ids) out_ids[i] = r.cand_tok[r.sel[i] % k];
@@ -819,11 +822,7 @@ int spd_generate(spd_ctx *ctx, int32_t n_steps, int32_t *out_tokens, int32_t *ou
   int rc = spd_generate_async(ctx, n_steps);
   if (rc) return rc;
   StepResult r;
-  if ((rc = fetch_result(ctx, r))) return rc;
-  if ((rc = await_result(ctx, r))) {  // with a stop token the run may have ended early: n_gen is the device's from here on
-    ctx->prefilled = false;
-    return rc;
-  }
+  if ((rc = step_result(ctx, r))) return rc;  // with a stop token the run may have ended early: n_gen is the device's from here on
   const int k = ctx->cfg.k, len = ctx->n_gen;
   std::vector<int32_t> tok((size_t)len * k), par((size_t)len * k);
   SPD_CUDA(cudaMemcpyAsync(tok.data(), ctx->ws + ctx->lay.hist_tok, tok.size() * 4, cudaMemcpyDeviceToHost, ctx->stream));
@@ -848,6 +847,12 @@ int spd_generate(spd_ctx *ctx, int32_t n_steps, int32_t *out_tokens, int32_t *ou
 }
 
 namespace {
+
+// A batch that failed on its way: how far each request came is not known, so none has drafts to go on from.
+int batch_fail(spd_ctx *const *ctxs, int32_t n, cudaError_t e, const char *what) {
+  for (int r = 0; r < n; ++r) ctxs[r]->prefilled = false;
+  return cuda_fail(e, what);
+}
 
 // Checks a batch and enqueues n_steps timesteps of it; the requests' host-side counters move on.
 int batch_enqueue(spd_ctx *const *ctxs, int32_t n, int32_t n_steps) {
@@ -887,7 +892,7 @@ int batch_enqueue(spd_ctx *const *ctxs, int32_t n, int32_t n_steps) {
     const cudaError_t e = spd_internal_batch_step(&job, dkp, n, s == 0, c0.vocab, lead->kp.final_norm, reinterpret_cast<float *>(lead->ws + lead->lay.bt_y),
                                                   reinterpret_cast<int32_t *>(lead->ws + lead->lay.bt_out), lead->stream, &launched);
     lead->launches += launched;
-    if (e != cudaSuccess) return cuda_fail(e, "batched timestep");
+    if (e != cudaSuccess) return batch_fail(ctxs, n, e, "batched timestep");
   }
   for (int r = 0; r < n; ++r) {
     ctxs[r]->n_gen += n_steps;
@@ -902,8 +907,9 @@ int batch_enqueue(spd_ctx *const *ctxs, int32_t n, int32_t n_steps) {
 int batch_wait(spd_ctx *const *ctxs, int32_t n, std::vector<int32_t> &rows) {
   spd_ctx *lead = ctxs[0];
   rows.resize((size_t)n * spd::kBtResultWords);
-  SPD_CUDA(cudaMemcpyAsync(rows.data(), lead->ws + lead->lay.bt_out, rows.size() * 4, cudaMemcpyDeviceToHost, lead->stream));
-  SPD_CUDA(cudaStreamSynchronize(lead->stream));
+  cudaError_t e = cudaMemcpyAsync(rows.data(), lead->ws + lead->lay.bt_out, rows.size() * 4, cudaMemcpyDeviceToHost, lead->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(lead->stream);
+  if (e != cudaSuccess) return batch_fail(ctxs, n, e, "results of a batch");
   int first = SPD_OK;
   for (int r = 0; r < n; ++r) {
     const int32_t err = rows[(size_t)r * spd::kBtResultWords + 2];
