@@ -439,6 +439,14 @@ int set_device(const spd_ctx *ctx) {
   return SPD_OK;
 }
 
+// A call that waits for the stream cannot be captured.  Refused while nothing has changed, it leaves the context (and the
+// capture) as they were.
+int refuse_capture(const spd_ctx *ctx) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  SPD_CUDA(cudaStreamIsCapturing(ctx->stream, &status));
+  return status == cudaStreamCaptureStatusNone ? SPD_OK : cuda_fail(cudaErrorStreamCaptureUnsupported, "a call that waits for its stream");
+}
+
 int read_state(spd_ctx *ctx, size_t field_off, void *dst, size_t bytes) {
   SPD_CUDA(cudaMemcpyAsync(dst, ctx->ws + ctx->lay.state + field_off, bytes, cudaMemcpyDeviceToHost, ctx->stream));
   return SPD_OK;
@@ -690,6 +698,7 @@ int spd_prefill(spd_ctx *ctx, const int32_t *prefix_ids, int32_t m, int32_t *out
     if (prefix_ids[i] < 0 || prefix_ids[i] >= c.vocab) return SPD_ERANGE;
   int rc = set_device(ctx);
   if (rc) return rc;
+  if ((rc = refuse_capture(ctx))) return rc;
   // fresh draft state: every history window holds the end of the prefix
   spd::State st;
   std::memset(&st, 0, sizeof st);
@@ -758,6 +767,7 @@ int spd_sample(spd_ctx *ctx, int32_t n_new, float top_p, float temperature, cons
     if (!(uniforms[i] >= 0.f) || !(uniforms[i] < 1.f)) return SPD_ERANGE;
   int rc = set_device(ctx);
   if (rc) return rc;
+  if ((rc = refuse_capture(ctx))) return rc;
   SPD_CUDA(cudaMemcpyAsync(ctx->ws + ctx->lay.ns_u, uniforms, (size_t)n_new * 4, cudaMemcpyHostToDevice, ctx->stream));
   ctx->prefilled = false;
   ctx->decoding = false;
@@ -878,6 +888,7 @@ int batch_enqueue(spd_ctx *const *ctxs, int32_t n, int32_t n_steps) {
   }
   int rc = set_device(lead);
   if (rc) return rc;
+  if ((rc = refuse_capture(lead))) return rc;
   // the requests' parameters in row order; pos0 = m - 1, so that a request's next position is pos0 + n_gen on the device
   std::vector<spd::KParams> kps(n);
   for (int r = 0; r < n; ++r) {

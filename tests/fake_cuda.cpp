@@ -8,7 +8,7 @@
 #include "spd_prefill_tc.h"
 
 namespace {
-int copies_until_failure = -1, waits_until_failure = -1, enqueued = 0;
+int copies_until_failure = -1, waits_until_failure = -1, enqueued = 0, capturing = 0;
 bool due(int &left) { return left >= 0 && left-- == 0; }
 CUresult encode(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
                 const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill) {
@@ -28,6 +28,8 @@ void fake_fail(int copies, int waits) {
   waits_until_failure = waits;
 }
 int fake_enqueued() { return enqueued; }
+// Whether the stream is being captured; a wait for it fails then.
+void fake_capture(int on) { capturing = on; }
 
 cudaError_t cudaGetDevice(int *d) {
   *d = 0;
@@ -63,7 +65,14 @@ cudaError_t cudaMemsetAsync(void *dst, int v, size_t n, cudaStream_t) {
   std::memset(dst, v, n);
   return cudaSuccess;
 }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return due(waits_until_failure) ? cudaErrorLaunchFailure : cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) {
+  if (capturing) return cudaErrorStreamCaptureUnsupported;
+  return due(waits_until_failure) ? cudaErrorLaunchFailure : cudaSuccess;
+}
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s) {
+  *s = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+  return cudaSuccess;
+}
 
 cudaError_t spd_internal_prepare(size_t, int *per_sm) {
   *per_sm = 1;

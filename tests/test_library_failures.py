@@ -102,3 +102,17 @@ def test_steps_that_fail_leave_no_drafts_to_go_on_from(lib, pair, copies, waits,
     lib.fake_fail(-1, -1)
     assert ctx.step() == ESTATE
     assert ctx.prefill() == 0 and call(ctx) == 0 and ctx.step() == 0
+
+
+@pytest.mark.parametrize("call", ["prefill", "sample", "batch"])
+def test_calls_that_wait_are_refused_under_capture(lib, pair, call):
+    """Before anything has changed: nothing is enqueued, and the contexts go on from where they were."""
+    ctxs, handles = pair
+    calls = {"prefill": ctxs[0].prefill, "sample": ctxs[0].sample, "batch": lambda: lib.spd_batch_generate(handles, 2, 3)}
+    before = lib.fake_enqueued()
+    lib.fake_capture(1)
+    assert calls[call]() == ECUDA
+    lib.fake_capture(0)
+    assert lib.fake_enqueued() == before
+    assert calls["sample"]() == 0 and calls["batch"]() == 0       # sampling continues a prefix behind which no step was taken yet
+    assert ctxs[0].step() == 0
