@@ -159,3 +159,43 @@ def test_a_nan_in_the_cache_reaches_the_logits(heads, k, kv_dtype):
             assert ids.min() >= 0 and ids.max() < shape.vocab and par.min() >= 0 and par.max() < k
     for ctx in ctxs:
         ctx.close()
+
+
+def test_a_malformed_table_of_one_request_stops_only_that_request(tiny_inputs):
+    """A table image without an empty slot makes one request's probes run to their bound in the first of three timesteps: the
+    call reports it, that request has no drafts to go on from, the others are where a batch without it has them."""
+    import paper_2405_18400_b200 as P
+
+    wl, weights, tables, prefix = tiny_inputs
+    packed = P.pack_weights(weights, "cuda:0")
+    good = P.build_ngram_tables(tables, "cuda:0")
+    slots = 1 << 15
+    img = np.zeros((slots, 4), np.uint32)
+    img[:, 0] = np.arange(slots, dtype=np.uint32) | 0xfff00000          # keys no lookup asks for
+    img[:, 3] = 1
+    full = torch.from_numpy(img.view(np.uint8).reshape(-1)).to("cuda:0")
+    bad = [dict(t) for t in good]
+    bad[0] = {"n": 2, "ngram_slots": slots, "ctx_slots": slots, "ngram": full, "ctx": full}
+    mk = lambda tabs: P.SpdContext(wl.shape, packed, tabs, wl.k, wl.orders, wl.lambdas(), wl.alpha, wl.tau, wl.delta, 256, "f32")
+    for at in (0, 1, 2):                        # the leading context, whose workspace the batch borrows, among them
+        ctxs, sound = [mk(bad if r == at else good) for r in range(3)], [mk(good) for _ in range(3)]
+        for r in range(3):
+            for c in (ctxs[r], sound[r]):
+                c.spd_prefill(np.roll(prefix, r))
+        with pytest.raises(P.SpdError) as e:
+            P.spd_batch_generate(ctxs, 3)
+        assert e.value.status == -6
+        P.spd_batch_generate(sound, 3)
+        with pytest.raises(P.SpdError) as e:
+            ctxs[at].spd_step()
+        assert e.value.status == -2
+        others = [r for r in range(3) if r != at]
+        for _ in range(2):
+            for r in others:
+                for what in ("LOGITS", "LOGP", "SEL"):
+                    assert np.array_equal(ctxs[r].spd_debug_read(what), sound[r].spd_debug_read(what)), (at, r, what)
+            P.spd_batch_step([ctxs[r] for r in others])
+            P.spd_batch_step([sound[r] for r in others])
+        ctxs[at].spd_prefill(prefix)            # and the request itself can be taken up again, up to its table
+        for c in ctxs + sound:
+            c.close()
