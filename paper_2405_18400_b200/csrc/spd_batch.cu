@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(kBtThreads) spd_job_input_kernel(const int32_t
 }
 
 // grid (rows, column chunks): residual add h += y, h * gain of the next norm as terms, the chunk's sum of squares.
+template <int kFlight>
 __global__ void __launch_bounds__(kBtThreads) spd_batch_resid_kernel(float *h, const __grid_constant__ Product y, const __nv_bfloat16 *gain,
                                                                      uint16_t *X, size_t term_stride, int d, float *ss) {
   dep_launch();
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(kBtThreads) spd_batch_resid_kernel(float *h, c
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
   if (c < d) {
     v = *reinterpret_cast<const float4 *>(h + (size_t)blockIdx.x * d + c);
-    const float4 a = product_sum4(y, blockIdx.x, c);
+    const float4 a = product_sum4<kFlight>(y, blockIdx.x, c);
     v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
   }
   bt_store_row(h, gq, X, term_stride, blockIdx.x, d, c, v, ss);
@@ -172,6 +173,7 @@ __global__ void __launch_bounds__(kBtThreads) spd_batch_resid_kernel(float *h, c
 // and truncate the same way, as they always have for these lengths (a bf16 cache turns a difference in the sixth digit into
 // another rounding of one value in a hundred).  The row waits in shared memory between the sum of squares, taken a column
 // per thread, and the terms, four columns per thread (8-byte stores).
+template <int kFlight>
 __global__ void __launch_bounds__(256) spd_job_norm_kernel(float *h, const __grid_constant__ Product y, const int32_t *ids, const __nv_bfloat16 *emb,
                                                            const __nv_bfloat16 *gain, uint16_t *X, size_t term_stride, int d, float eps) {
   dep_launch();
@@ -185,7 +187,7 @@ __global__ void __launch_bounds__(256) spd_job_norm_kernel(float *h, const __gri
     if (ids) v = bt_load4(emb + (size_t)ids[t] * d + c);
     else {
       v = *reinterpret_cast<const float4 *>(hr + c);
-      const float4 a = product_sum4(y, t, c);
+      const float4 a = product_sum4<kFlight>(y, t, c);
       v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
     }
     *reinterpret_cast<float4 *>(hr + c) = v;
@@ -227,9 +229,10 @@ __device__ __forceinline__ void bt_store_kv(void *cache, int kv_bf16, size_t at,
 __device__ __forceinline__ float4 bt_angles(const float2 *rope, int hd, int pos, int c) {
   return *reinterpret_cast<const float4 *>(rope + (size_t)pos * (hd / 2) + (c % hd) / 2);
 }
+template <int kFlight>
 __device__ __forceinline__ void bt_rope_cache(const Product &y, float rs, float *Q, void *kcache, void *vcache, const float4 &cs, int max_pos,
                                               int kv_bf16, int d, int layer, int t, int pos, int c) {
-  const float4 q = product_sum4(y, t, c), k = product_sum4(y, t, d + c), v = product_sum4(y, t, 2 * d + c);
+  const float4 q = product_sum4<kFlight>(y, t, c), k = product_sum4<kFlight>(y, t, d + c), v = product_sum4<kFlight>(y, t, 2 * d + c);
   const size_t at = ((size_t)layer * max_pos + pos) * d + c;
   *reinterpret_cast<float4 *>(Q + (size_t)t * d + c) = bt_rotate(make_float4(q.x * rs, q.y * rs, q.z * rs, q.w * rs), cs);
   bt_store_kv(kcache, kv_bf16, at, bt_rotate(make_float4(k.x * rs, k.y * rs, k.z * rs, k.w * rs), cs));
@@ -237,6 +240,7 @@ __device__ __forceinline__ void bt_rope_cache(const Product &y, float rs, float 
 }
 
 // grid (requests, column chunks): each request at its own position, into its own cache.
+template <int kFlight>
 __global__ void __launch_bounds__(kBtThreads) spd_batch_rope_cache_kernel(const __grid_constant__ Product y, const float *ss, float eps, float *Q,
                                                                           const KParams *kps, int d, int hd, int layer) {
   dep_wait();
@@ -245,11 +249,12 @@ __global__ void __launch_bounds__(kBtThreads) spd_batch_rope_cache_kernel(const 
   const int c = blockIdx.y * kBtCols + threadIdx.x * 4;
   if (c >= d) return;
   const int pos = bt_pos(p);
-  bt_rope_cache(y, bt_rs(ss, blockIdx.x, d, eps), Q, p.kcache, p.vcache, bt_angles(p.rope, hd, pos, c), p.max_pos, p.kv_bf16, d, layer, blockIdx.x,
-                pos, c);
+  bt_rope_cache<kFlight>(y, bt_rs(ss, blockIdx.x, d, eps), Q, p.kcache, p.vcache, bt_angles(p.rope, hd, pos, c), p.max_pos, p.kv_bf16, d, layer,
+                         blockIdx.x, pos, c);
 }
 
 // The same for a job of prefix tokens of one request (token t at position pos0 + t, one cache).
+template <int kFlight>
 __global__ void __launch_bounds__(kBtThreads) spd_job_rope_cache_kernel(const __grid_constant__ Product y, const float *ss, float eps, float *Q,
                                                                         void *kcache, void *vcache, const float2 *rope, int max_pos, int kv_bf16,
                                                                         int d, int hd, int layer, int pos0) {
@@ -258,7 +263,7 @@ __global__ void __launch_bounds__(kBtThreads) spd_job_rope_cache_kernel(const __
   dep_wait();
   dep_launch();
   if (c >= d) return;
-  bt_rope_cache(y, bt_rs(ss, blockIdx.x, d, eps), Q, kcache, vcache, cs, max_pos, kv_bf16, d, layer, blockIdx.x, pos, c);
+  bt_rope_cache<kFlight>(y, bt_rs(ss, blockIdx.x, d, eps), Q, kcache, vcache, cs, max_pos, kv_bf16, d, layer, blockIdx.x, pos, c);
 }
 
 // grid (rows, chunks of the FFN): u = SiLU(gate) * up from the gate / up product's row times 1 / rms
@@ -267,6 +272,7 @@ __device__ __forceinline__ float bt_swiglu(float gate, float up, float rs) {
   const float g = gate * rs, u = up * rs;
   return g / (1.f + __expf(-g)) * u;
 }
+template <int kFlight>
 __global__ void __launch_bounds__(kBtThreads) spd_batch_swiglu_kernel(const __grid_constant__ Product y, const float *ss, float eps, int d, uint16_t *X,
                                                                       size_t term_stride, int f) {
   dep_launch();
@@ -274,7 +280,7 @@ __global__ void __launch_bounds__(kBtThreads) spd_batch_swiglu_kernel(const __gr
   const int t = blockIdx.x, j = blockIdx.y * kBtCols + threadIdx.x * 4;
   if (j >= f) return;
   const float rs = bt_rs(ss, t, d, eps);
-  const float4 a = product_sum4(y, t, 2 * j), b = product_sum4(y, t, 2 * j + 4);
+  const float4 a = product_sum4<kFlight>(y, t, 2 * j), b = product_sum4<kFlight>(y, t, 2 * j + 4);
   bt_put3x4(X, term_stride, (size_t)t * f + j,
             make_float4(bt_swiglu(a.x, a.y, rs), bt_swiglu(a.z, a.w, rs), bt_swiglu(b.x, b.y, rs), bt_swiglu(b.z, b.w, rs)));
 }
@@ -490,7 +496,7 @@ __global__ void __launch_bounds__(kConsumerThreads) spd_job_head_kernel(const __
   float sq = 0.f;
   for (int c = threadIdx.x * 4; c < p.d; c += kConsumerThreads * 4) {
     float4 v = *reinterpret_cast<const float4 *>(h + c);
-    const float4 a = product_sum4(y, 0, c);
+    const float4 a = product_sum4<kPartFlight>(y, 0, c);
     v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
     sq = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, sq))));
     *reinterpret_cast<float4 *>(jh_x + c) = bt_mul(v, bt_load4(p.final_norm + c));
@@ -570,6 +576,7 @@ extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd:
   const size_t ts_d = (size_t)j.x_term_rows * d, ts_f = (size_t)j.x_term_rows * f;
   const int nch = (d + spd::kBtCols - 1) / spd::kBtCols, nch_f = (f + spd::kBtCols - 1) / spd::kBtCols;
   const dim3 threads(spd::kBtThreads);
+  const bool few = n <= spd::kFewRows;
   int count = 0;
   cudaError_t e = cudaSuccess;
   spd::Product pr;  // where the last product's sums are
@@ -581,20 +588,25 @@ extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd:
     if (e == cudaSuccess) done(spd_internal_product(job, n, wide, which, j.y, N, &pr, s));
   };
   auto resid = [&](const __nv_bfloat16 *gain) {
-    if (e == cudaSuccess) done(spd::launch_dep(spd::spd_batch_resid_kernel, dim3(n, nch), threads, 0, s, j.h, pr, gain, j.x, ts_d, d, j.ss));
+    if (e == cudaSuccess)
+      done(spd::launch_dep(few ? spd::spd_batch_resid_kernel<spd::kPartFlight> : spd::spd_batch_resid_kernel<1>, dim3(n, nch), threads, 0, s, j.h, pr, gain,
+                           j.x, ts_d, d, j.ss));
   };
   done(spd::launch_dep(spd::spd_batch_input_kernel, dim3(n, nch), threads, 0, s, kps, j.h, j.layers[0].attn_norm, j.x, ts_d, d, j.ss, begin));
   for (int l = 0; l < j.L && e == cudaSuccess; ++l) {
     product(0, 4 * l, 3 * d);
     if (e == cudaSuccess)
-      done(spd::launch_dep(spd::spd_batch_rope_cache_kernel, dim3(n, nch), threads, 0, s, pr, j.ss, j.eps, j.q, kps, d, j.hd, l));
+      done(spd::launch_dep(few ? spd::spd_batch_rope_cache_kernel<spd::kPartFlight> : spd::spd_batch_rope_cache_kernel<1>, dim3(n, nch), threads, 0, s, pr, j.ss,
+                           j.eps, j.q, kps, d, j.hd, l));
     if (e == cudaSuccess)
       done(j.hd == 128 ? spd::launch_dep(spd::spd_batch_attn_kernel<128>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l)
                        : spd::launch_dep(spd::spd_batch_attn_kernel<64>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l));
     product(0, 4 * l + 1, d);
     resid(j.layers[l].ffn_norm);
     product(0, 4 * l + 2, 2 * f);
-    if (e == cudaSuccess) done(spd::launch_dep(spd::spd_batch_swiglu_kernel, dim3(n, nch_f), threads, 0, s, pr, j.ss, j.eps, d, j.x, ts_f, f));
+    if (e == cudaSuccess)
+      done(spd::launch_dep(few ? spd::spd_batch_swiglu_kernel<spd::kPartFlight> : spd::spd_batch_swiglu_kernel<1>, dim3(n, nch_f), threads, 0, s, pr, j.ss,
+                           j.eps, d, j.x, ts_f, f));
     product(1, 4 * l + 3, d);
     resid(l + 1 < j.L ? j.layers[l + 1].attn_norm : final_norm);
   }
@@ -613,22 +625,27 @@ extern "C" cudaError_t spd_internal_job_resid(const spd::TcJob *job, const spd::
   const dim3 grid(j.n_tok, (j.d + spd::kBtCols - 1) / spd::kBtCols);
   const size_t ts = (size_t)j.x_term_rows * j.d;
   if (!y) return spd::launch_dep(spd::spd_job_input_kernel, grid, dim3(spd::kBtThreads), 0, s, j.ids, j.tok_emb, j.h, gain, j.x, ts, j.d, j.ss);
-  return spd::launch_dep(spd::spd_batch_resid_kernel, grid, dim3(spd::kBtThreads), 0, s, j.h, *y, gain, j.x, ts, j.d, j.ss);
+  return spd::launch_dep(j.n_tok <= spd::kFewRows ? spd::spd_batch_resid_kernel<spd::kPartFlight> : spd::spd_batch_resid_kernel<1>, grid,
+                         dim3(spd::kBtThreads), 0, s, j.h, *y, gain, j.x, ts, j.d, j.ss);
 }
 extern "C" cudaError_t spd_internal_job_norm(const spd::TcJob *job, const spd::Product *y, const __nv_bfloat16 *gain, cudaStream_t s) {
   const spd::TcJob &j = *job;
   const spd::Product none = {};
-  return spd::launch_dep(spd::spd_job_norm_kernel, dim3(j.n_tok), dim3(256), (size_t)j.d * 4, s, j.h, y ? *y : none, y ? nullptr : j.ids, j.tok_emb, gain,
-                         j.x, (size_t)j.x_term_rows * j.d, j.d, j.eps);
+  return spd::launch_dep(spd::cuts_tiles(j.n_tok) ? spd::spd_job_norm_kernel<1> : spd::spd_job_norm_kernel<0>, dim3(j.n_tok), dim3(256),
+                         (size_t)j.d * 4, s, j.h, y ? *y : none, y ? nullptr : j.ids, j.tok_emb, gain, j.x, (size_t)j.x_term_rows * j.d, j.d, j.eps);
 }
 extern "C" cudaError_t spd_internal_job_rope_cache(const spd::TcJob *job, const spd::Product *y, int normed, int layer, cudaStream_t s) {
   const spd::TcJob &j = *job;
-  return spd::launch_dep(spd::spd_job_rope_cache_kernel, dim3(j.n_tok, (j.d + spd::kBtCols - 1) / spd::kBtCols), dim3(spd::kBtThreads), 0, s, *y,
+  return spd::launch_dep(j.n_tok <= spd::kFewRows ? spd::spd_job_rope_cache_kernel<spd::kPartFlight>
+                         : spd::cuts_tiles(j.n_tok) ? spd::spd_job_rope_cache_kernel<1> : spd::spd_job_rope_cache_kernel<0>,
+                         dim3(j.n_tok, (j.d + spd::kBtCols - 1) / spd::kBtCols), dim3(spd::kBtThreads), 0, s, *y,
                          normed ? nullptr : j.ss, j.eps, j.q, j.kcache, j.vcache, j.rope, j.max_pos, j.kv_bf16, j.d, j.hd, layer, j.pos0);
 }
 extern "C" cudaError_t spd_internal_job_swiglu(const spd::TcJob *job, const spd::Product *y, int normed, cudaStream_t s) {
   const spd::TcJob &j = *job;
-  return spd::launch_dep(spd::spd_batch_swiglu_kernel, dim3(j.n_tok, (j.f + spd::kBtCols - 1) / spd::kBtCols), dim3(spd::kBtThreads), 0, s, *y,
+  return spd::launch_dep(j.n_tok <= spd::kFewRows ? spd::spd_batch_swiglu_kernel<spd::kPartFlight>
+                         : spd::cuts_tiles(j.n_tok) ? spd::spd_batch_swiglu_kernel<1> : spd::spd_batch_swiglu_kernel<0>,
+                         dim3(j.n_tok, (j.f + spd::kBtCols - 1) / spd::kBtCols), dim3(spd::kBtThreads), 0, s, *y,
                          normed ? nullptr : j.ss, j.eps, j.d, j.x, (size_t)j.x_term_rows * j.f, j.f);
 }
 
@@ -638,7 +655,9 @@ extern "C" cudaError_t spd_internal_job_head(const spd::KParams *p, const float 
 
 // Kernel attributes of the current device: a row of up to 16384 float32 values in shared memory.
 extern "C" cudaError_t spd_internal_job_prepare(void) {
-  const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_job_norm_kernel), cudaFuncAttributeMaxDynamicSharedMemorySize, 65536);
+  cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_job_norm_kernel<0>), cudaFuncAttributeMaxDynamicSharedMemorySize, 65536);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_job_norm_kernel<1>), cudaFuncAttributeMaxDynamicSharedMemorySize, 65536);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_job_head_kernel), cudaFuncAttributeMaxDynamicSharedMemorySize, 65536);
 }

@@ -26,6 +26,9 @@ struct Product {
   int32_t small_first;  // one instruction per term: a stage's small terms before the large one
 };
 
+// Whether products of so many token rows may cut tiles.
+inline bool cuts_tiles(int n_tok) { return n_tok <= kTcMaxTileTok; }
+
 inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *y, const float *parts) {
   Product pr;
   pr.y = y;
@@ -36,7 +39,7 @@ inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *
   // up to 128 (all alike) to fill the pairs without cutting one: then every sum is one pair's.  From 65 rows on a tile's rows
   // are rounded up to 16, which is what an instruction's N allows (to 32: 100 tokens, 7B shape, 5.5 ms instead of 5.1; 400
   // tokens as one job 18.6 instead of 17.0).  Between 129 and 256 rows tiles are cut at multiples of eight stages.
-  const bool whole = n_tok > kTcMaxTileTok;
+  const bool whole = !cuts_tiles(n_tok);
   pr.shape = n_tok <= 16 ? 16 : (n_tok <= 32 ? 32 : (n_tok <= 64 ? 64 : (n_tok <= 128 || whole ? 128 : 256)));
   pr.tok_tiles = whole ? (n_tok + 127) / 128 : 1;
   pr.tile_tok = pr.shape <= 64 ? pr.shape : ((n_tok + pr.tok_tiles - 1) / pr.tok_tiles + 15) / 16 * 16;
@@ -87,24 +90,32 @@ __device__ __forceinline__ TileParts product_parts(const Product &pr, int t, int
   tp.at = (size_t)(t - tt * pr.tile_tok) * 256;
   return tp;
 }
-// Y[t][r .. r+3]; r and N multiples of 4.  The parts are asked for together and added in order: the row-wise kernels between
-// two products are little more than a chain of trips to L2, and a loop that adds as it loads makes one trip per part (7B shape,
-// up to 256 rows: five later parts of a tile in the attention-output and down
-// products).  With the gains and rotary angles asked for before dep_wait: 8 requests 3.13 -> 3.03 ms per timestep, 27 tokens 3.29 ->
-// 3.22 ms.
-constexpr int kPartFlight = 6;
+// Y[t][r .. r+3]; r and N multiples of 4.  kFlight parts are asked for together; they are added in order whatever it is.
+// Few token rows (up to kFewRows), 6: the row-wise kernels between two products are little more than a chain of trips to L2, and
+// a loop that adds as it loads makes one trip per part (7B shape: five later parts of a tile in the attention-output and
+// down products).  With the gains and rotary angles asked for before dep_wait, 8 requests 3.13 -> 3.03 ms per timestep, 27 tokens
+// 3.29 -> 3.22 ms.
+// More rows, 1: six parts take 56 to 72 registers instead of 42 to 54, so fewer blocks fit an SM, and the attention's blocks,
+// which come onto the SMs as these leave, lie less evenly.  One / six: 4096 columns, 8 layers, 15 tokens 0.859 / 0.842 ms, 27
+// 0.878 / 0.869, 64 1.012 / 1.043; 3072 columns, 4 layers, 128 tokens 0.500 / 0.558.
+// Rows whose products cut no tiles, 0: no parts, 28 to 32 registers.  None / one / six: 1024 columns, heads of 64, 8 layers,
+// 700 tokens 1.72 / 1.76 / 1.82 ms, 1500 3.09 / 3.27 / 3.38; 4096 columns, 8 layers, 512 tokens 4.39 / 4.44 / 4.42.
+constexpr int kFewRows = 32, kPartFlight = 6;
+template <int kFlight>
 __device__ __forceinline__ float4 product_sum4(const Product &pr, int t, int r) {
-  const TileParts tp = product_parts(pr, t, r >> 8);
   float4 v = *reinterpret_cast<const float4 *>(pr.y + (size_t)t * pr.N + r);
-  const float *part = pr.parts + tp.at + (r & 255);
-  for (int p = tp.first; p < tp.last; p += kPartFlight) {
-    float4 w[kPartFlight];
+  if constexpr (kFlight > 0) {
+    const TileParts tp = product_parts(pr, t, r >> 8);
+    const float *part = pr.parts + tp.at + (r & 255);
+    for (int p = tp.first; p < tp.last; p += kFlight) {
+      float4 w[kFlight];
 #pragma unroll
-    for (int u = 0; u < kPartFlight; ++u)
-      if (p + u < tp.last) w[u] = *reinterpret_cast<const float4 *>(part + (p + u) * tp.step);
+      for (int u = 0; u < kFlight; ++u)
+        if (p + u < tp.last) w[u] = *reinterpret_cast<const float4 *>(part + (p + u) * tp.step);
 #pragma unroll
-    for (int u = 0; u < kPartFlight; ++u)
-      if (p + u < tp.last) { v.x += w[u].x; v.y += w[u].y; v.z += w[u].z; v.w += w[u].w; }
+      for (int u = 0; u < kFlight; ++u)
+        if (p + u < tp.last) { v.x += w[u].x; v.y += w[u].y; v.z += w[u].z; v.w += w[u].w; }
+    }
   }
   return v;
 }
