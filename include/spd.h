@@ -35,7 +35,10 @@ enum {
   SPD_ESTATE = -2,   /* spd_step / spd_generate before spd_prefill                                   */
   SPD_ERANGE = -3,   /* prefix empty or too long, token id outside the vocabulary, out of positions  */
   SPD_ENOMEM = -4,   /* workspace (or a caller-provided buffer) too small                            */
-  SPD_ECUDA = -5,    /* a CUDA runtime call failed; spd_last_cuda_error() gives its text             */
+  SPD_ECUDA = -5,    /* a CUDA runtime call failed; spd_last_cuda_error() gives its text.  Calls that
+                        synchronise their stream return it while the stream is being captured;
+                        spd_prefill, spd_sample and the batched calls then leave the context as it was.
+                        Steps and batches that fail otherwise need a new spd_prefill.               */
   SPD_ETABLE = -6,   /* an n-gram table probe ran past its bound (malformed table)                   */
   SPD_ETIMEOUT = -7  /* a bounded wait inside the decode kernel expired                              */
 };

@@ -219,8 +219,8 @@ struct spd_ctx {
 
 namespace {
 
-// Shared memory behind the scratch area that the fragment-order multiply loop needs for the activation vector: 12
-// vectors of 16 bytes per 32 columns.
+// Shared memory behind the scratch area that the fragment-order multiply loop needs for the activation vector: 24
+// vectors of 8 bytes per 32 columns.
 size_t frag_bytes(const spd_config &c) { return (size_t)c.d_model / 32 * 192; }
 
 // reserve: bytes of shared memory kept back behind the ring and the scratch area.
@@ -251,12 +251,15 @@ int pick_ring(const spd_config &c, int32_t stage_bytes, int32_t n_stages, size_t
 
 // How the units of matrices in fragment order (d_model columns) pass through the ring.  Units that fill the fewest stages they fit
 // to a tenth keep these to themselves, and the ring is refilled at once (d_model 5120: 54, 54 and 52 of 54 pairs).  Others
-// would leave the ring that much emptier (4096: two stages of 64 pairs where 86 fit), so stages run on across units; then a full
-// ring is more than HBM needs at a time.  Two 32 KB copies per SM already bring 7.0 of the 7.3 TB/s that a bare stream
-// reaches, more requests only queue, the barriers' stores, counters and loads behind them: 112 KB under way at most, in whole
-// stages, two at least (7B shape: stages to themselves and no limit 2.495 ms per timestep; full stages and three under way
-// 2.478, two 2.460).  The 13B shape keeps its units apart without a limit: its steps run into the power cap, and full stages with
-// four under way, 4.50 against 4.55 ms on a cold GPU, took 4.80 against 4.68.
+// would leave the ring that much emptier (4096: two stages of 64 pairs where 86 fit), so stages run on across units, and then
+// at most as many stages are under way as 112 KB hold, two at least: two 32 KB copies per SM already bring 7.0 of the 7.3 TB/s
+// that a bare stream reaches, and more requests only queue, the barriers' stores, counters and loads behind them.
+// Both choices were measured together at ten widths, 1024 to 8192, and the rule's is within 1 % of the best everywhere.  ms per
+// timestep, whole models, units apart / apart with the limit / across / across with the limit (* the rule's):
+//   3072, 28 layers  1.536  1.550  1.492  1.504*     4096, 32 layers  2.527  2.610  2.531  2.519*
+//   5120, 40 layers  4.512*  4.543  4.537  4.553     6144, 16 layers  2.473*  2.461  2.474  2.456
+// Running on across units gains up to 5 % where stages would stay a tenth and more empty (2560, 20 layers: 0.953 and 0.901) and
+// costs 0.6 % at 5120; the limit behind it gains or costs up to 0.8 % depending on the width.
 void plan_units(const spd_config &c, bool images, spd::KParams &kp) {
   kp.most_flying = kp.n_stages;
   kp.img_span = 0;

@@ -223,9 +223,9 @@ __device__ __forceinline__ void pf_put(uint16_t *F, int t, int c, float v) {
   F[e + 256] = (uint16_t)(lo >> 16);
 }
 
-// Fragment producer (one thread): copies the K blocks of each phase's fragment buffer into shared memory, in the order the consumers take them.  A phase's fragments are complete once the consumers have
-// passed the grid barrier before it (they say so on `xgo`); a buffer is free again once all consumer warps
-// have taken their fragments of it into registers (`xempty`).
+// Fragment producer (one thread): copies the K blocks of each phase's fragment buffer into shared memory, in the order the
+// consumers take them.  A phase's fragments are complete once the consumers have passed the grid barrier before it (they say
+// so on `xgo`); a buffer is free again once all consumer warps have taken their fragments of it into registers (`xempty`).
 __device__ void pf_xproducer(PfBlk &b) {
   const KParams &p = *b.p;
   uint32_t n = 0;

@@ -153,10 +153,11 @@ __device__ __forceinline__ bool tc_wait(TcShared &sh, State *st, uint64_t *bar, 
 // Tile: 256 weight rows (tcgen05.mma.cta_group::2, M = 256, 128 rows in each block's shared and tensor memory) x the token
 // rows of a tile.  The weights are the wide operand whatever the number of tokens, the terms the narrow one:
 //   F = 16, 32, 64 (up to that many token rows): the three term tiles lie behind one another, so one instruction of
-//     N = 3 x rows per 16 columns multiplies all three (N = 64 for 16 rows: a multiple of 32 is wanted; the 16 columns
-//     left over hold nothing that is read); each term has its own accumulator columns, added in the epilogue's registers.
-//   128, 256 (that many rows at most, N = the tile's rows rounded up to 16): one instruction per term and 16 columns, all
-//     into the same columns.
+//     N = 3 x rows per 16 columns multiplies all three (N = 64 for 16 rows, whose 16 columns left over hold nothing that is
+//     read: N goes in steps of 16, so 48 would do, which was not measured); each term has its own accumulator columns, added
+//     in the epilogue's registers.
+//   128, 256 (that many rows at most, N = the tile's rows rounded up to 16, 80 to 256): one instruction per term and 16
+//     columns, all into the same columns.
 // Each block brings its 128 weight rows and half of the tile's tokens.
 //
 // What bounds it: with up to about 64 tokens the weight stream; beyond, the tensor pipe (N = 128: 89 cycles an

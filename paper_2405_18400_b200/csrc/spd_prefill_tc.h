@@ -58,7 +58,7 @@ inline Product plan_product(int n_tok, int N, int C, int sm_count, const float *
   const int least_seg = n_tok > 128 ? 2 : 1, most_seg = whole ? 8 : 4, wide = C / 512;
   pr.seg = pr.shape <= 64 ? 4 : (wide < least_seg ? least_seg : (wide < most_seg ? wide : most_seg));
   pr.small_first = pr.seg < 8;
-  // a pair takes a tile, two segments or four stages at least (small matrices: fewer parts to add)
+  // a pair takes a whole tile, two steps of the cuts (16 stages) or four stages at least (small matrices: fewer parts to add)
   const int least = whole ? pr.nk : (pr.align > 1 ? 2 * pr.align : 4);
   const int most = sm_count / 2 < kTcMaxPairs ? sm_count / 2 : kTcMaxPairs, worth = pr.total / least;
   pr.pairs = most < worth ? most : worth;
