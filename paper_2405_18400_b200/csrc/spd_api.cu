@@ -597,6 +597,8 @@ int spd_create(const spd_config *cfg, const spd_weights *w, const spd_ngram_tabl
   kp.pf_part = reinterpret_cast<float *>(ws + lay.pf_part); kp.pf_ml = reinterpret_cast<float2 *>(ws + lay.pf_ml);
   kp.pf_cnt = reinterpret_cast<unsigned int *>(ws + lay.pf_cnt);
   kp.eos_id = cfg->eos_id;
+  kp.hd_inverse = (uint32_t)((((uint64_t)1 << 32) + hd - 1) / hd);
+  kp.attn_most = ctx->grid / cfg->n_heads < 1 ? 1 : (ctx->grid / cfg->n_heads > spd::kMaxSplit ? spd::kMaxSplit : ctx->grid / cfg->n_heads);
 
   // rotary table: cos / sin of pos * theta^(-2i/hd), evaluated in double and rounded once
   std::vector<float2> rope((size_t)cfg->max_pos * (hd / 2));

@@ -38,6 +38,13 @@ __shared__ float2 s_rope[128];  // the current position's row of the rotary tabl
 constexpr int kGainSlots = 256;  // gain pointers kept in shared memory: models of up to 127 layers (deeper ones read them late)
 __shared__ const __nv_bfloat16 *s_gain_ptrs[kGainSlots];
 __shared__ int s_dead, s_quit;
+// The matrices of a layer in the order of their phases, then the LM head.
+enum Matrix { kMatQKV = 0, kMatO = 1, kMatGateUp = 2, kMatDown = 3, kMatHead = 4, kMatrices = 5 };
+// This block's rows [x, y) of each matrix and the whole rows of it that a stage takes.  They stay what they are for the whole
+// launch, and their divisions stood between a phase's first barrier and its first multiply: two of 64 bits, 0.5 us, four times a
+// layer (7B shape).
+__shared__ int2 s_rows[kMatrices];
+__shared__ int s_chunk_rows[kMatrices];
 
 __device__ __forceinline__ float *scratch_base(const KParams &p) { return reinterpret_cast<float *>(smem + (size_t)p.n_stages * p.stage_bytes); }
 
@@ -81,15 +88,16 @@ __device__ __forceinline__ bool grid_barrier(Blk &b) {
   return s_quit != 0;
 }
 
-__device__ __forceinline__ void cta_rows(int R, int gran, int &r0, int &r1) {
-  long long U = R / gran;
-  r0 = (int)(U * blockIdx.x / gridDim.x) * gran;
-  r1 = (int)(U * (blockIdx.x + 1) / gridDim.x) * gran;
-}
-
-__device__ __forceinline__ int rows_per_chunk(const KParams &p, int C) {
-  int rpc = p.stage_bytes / (C * 2);
-  return rpc > kMaxRowsPerChunk ? kMaxRowsPerChunk : rpc;
+// The rows are dealt in units: of kUnitRows in fragment order, of a pair where an epilogue needs both rows of one.
+template <bool kImg>
+__device__ __forceinline__ void share_rows(const KParams &p, int m) {
+  const int R = m == kMatQKV ? 3 * p.d : (m == kMatGateUp ? 2 * p.f : (m == kMatHead ? p.V : p.d));
+  const int C = m == kMatDown ? p.f : p.d;
+  const int gran = kImg && m != kMatDown ? kUnitRows : (m == kMatQKV || m == kMatGateUp ? 2 : 1);
+  const long long U = R / gran;
+  s_rows[m] = make_int2((int)(U * blockIdx.x / gridDim.x) * gran, (int)(U * (blockIdx.x + 1) / gridDim.x) * gran);
+  const int rpc = p.stage_bytes / (C * 2);
+  s_chunk_rows[m] = rpc > kMaxRowsPerChunk ? kMaxRowsPerChunk : rpc;
 }
 
 // ---------------------------------------------------------------- producer
@@ -118,11 +126,8 @@ __device__ __forceinline__ void issue_chunk(Blk &b, Producer &pr, const uint8_t 
   if (++pr.stage == (uint32_t)p.n_stages) { pr.stage = 0; pr.phase ^= 1u; }
 }
 
-__device__ __forceinline__ void produce_matrix(Blk &b, Producer &pr, const __nv_bfloat16 *W, int R, int C, int gran) {
-  const KParams &p = *b.p;
-  int r0, r1;
-  cta_rows(R, gran, r0, r1);
-  const int rpc = rows_per_chunk(p, C);
+__device__ __forceinline__ void produce_matrix(Blk &b, Producer &pr, const __nv_bfloat16 *W, int m, int C) {
+  const int r0 = s_rows[m].x, r1 = s_rows[m].y, rpc = s_chunk_rows[m];
   const uint32_t rowbytes = (uint32_t)C * 2u;
   for (int t0 = r0; t0 < r1; t0 += kTile) {
     const int t1 = min(t0 + kTile, r1);
@@ -135,10 +140,9 @@ __device__ __forceinline__ void produce_matrix(Blk &b, Producer &pr, const __nv_
 }
 
 // A matrix in fragment order (spd_pack_image): the units of this block are one contiguous run.
-__device__ __forceinline__ void produce_image(Blk &b, Producer &pr, const __nv_bfloat16 *img, int R, int C) {
+__device__ __forceinline__ void produce_image(Blk &b, Producer &pr, const __nv_bfloat16 *img, int m, int C) {
   const KParams &p = *b.p;
-  int r0, r1;
-  cta_rows(R, kUnitRows, r0, r1);
+  const int r0 = s_rows[m].x, r1 = s_rows[m].y;
   const uint8_t *src = reinterpret_cast<const uint8_t *>(img) + (size_t)r0 * C * 2;
   const int unit = C / 32, all = (r1 - r0) / kUnitRows * unit;
   const int run = p.img_span ? all : unit;  // what a stage does not reach beyond
@@ -160,21 +164,21 @@ __device__ void producer_main(Blk &b) {
     for (int l = 0; l < p.L && !s_dead; ++l) {
       const LayerW nxt = p.layers[l + 1 < p.L ? l + 1 : 0];
       if constexpr (kImg) {
-        produce_image(b, pr, lw.wqkv_img, 3 * p.d, p.d);
-        produce_image(b, pr, lw.wo_img, p.d, p.d);
-        produce_image(b, pr, lw.wgate_up_img, 2 * p.f, p.d);
+        produce_image(b, pr, lw.wqkv_img, kMatQKV, p.d);
+        produce_image(b, pr, lw.wo_img, kMatO, p.d);
+        produce_image(b, pr, lw.wgate_up_img, kMatGateUp, p.d);
       } else {
-        produce_matrix(b, pr, lw.wqkv, 3 * p.d, p.d, 2);
-        produce_matrix(b, pr, lw.wo, p.d, p.d, 1);
-        produce_matrix(b, pr, lw.wgate_up, 2 * p.f, p.d, 2);
+        produce_matrix(b, pr, lw.wqkv, kMatQKV, p.d);
+        produce_matrix(b, pr, lw.wo, kMatO, p.d);
+        produce_matrix(b, pr, lw.wgate_up, kMatGateUp, p.d);
       }
-      produce_matrix(b, pr, lw.wdown, p.d, p.f, 1);
+      produce_matrix(b, pr, lw.wdown, kMatDown, p.f);
       lw = nxt;
     }
     const bool head = kSampler ? p.mode != kModePrefill : p.mode == kModeDecode;
     if (head || it == p.n_iters - 1) {
-      if constexpr (kImg) produce_image(b, pr, p.lm_head_img, p.V, p.d);
-      else produce_matrix(b, pr, p.lm_head, p.V, p.d, 1);
+      if constexpr (kImg) produce_image(b, pr, p.lm_head_img, kMatHead, p.d);
+      else produce_matrix(b, pr, p.lm_head, kMatHead, p.d);
     }
   }
   if (s_dead) {
@@ -312,6 +316,9 @@ __device__ __forceinline__ void store_kv(const KParams &p, void *cache, size_t i
   else reinterpret_cast<float *>(cache)[idx] = v;
 }
 
+// The head that a column belongs to: col / hd for all columns there can be (hd_inverse is 2^32 / hd rounded up, hd at most 256).
+__device__ __forceinline__ int head_of(const KParams &p, int col) { return (int)__umulhi((uint32_t)col, p.hd_inverse); }
+
 // Finishes rows [t0, t1) of the current matrix from the warps' partial sums.
 // rs: the factor of the phase's RMSNorm, 1 / rms(h), which the prologue left out of x (1 for a phase without one).
 __device__ __forceinline__ void epilogue(Blk &b, int kind, const EpiArgs &ea, const float *part, int t0, int t1, bool have_h,
@@ -325,9 +332,9 @@ __device__ __forceinline__ void epilogue(Blk &b, int kind, const EpiArgs &ea, co
       const int r = t0 + tid * 2;
       float a = part_sum(part + (size_t)(tid * 2) * kConsumerWarps) * rs;
       float c = part_sum(part + (size_t)(tid * 2 + 1) * kConsumerWarps) * rs;
-      const int sec = r / p.d, col = r - sec * p.d;
+      const int sec = (r >= p.d) + (r >= 2 * p.d), col = r - sec * p.d;
       if (sec < 2) {
-        const float2 cs = s_rope[(col % p.hd) / 2];  // the position's row of the rotary table
+        const float2 cs = s_rope[(col - head_of(p, col) * p.hd) / 2];  // the position's row of the rotary table
         const float ra = a * cs.x - c * cs.y, rc = a * cs.y + c * cs.x;
         a = ra;
         c = rc;
@@ -363,13 +370,10 @@ __device__ __forceinline__ void epilogue(Blk &b, int kind, const EpiArgs &ea, co
 }
 
 // Streams this block's rows of one matrix through the ring against the register-resident x.
-__device__ __forceinline__ void consume_matrix(Blk &b, int R, int C, int gran, const float (&xr)[kMaxVec][8], int kind,
-                                               const EpiArgs &ea) {
+__device__ __forceinline__ void consume_matrix(Blk &b, int m, int C, const float (&xr)[kMaxVec][8], int kind, const EpiArgs &ea) {
   const KParams &p = *b.p;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int r0, r1;
-  cta_rows(R, gran, r0, r1);
-  const int rpc = rows_per_chunk(p, C);
+  const int r0 = s_rows[m].x, r1 = s_rows[m].y, rpc = s_chunk_rows[m];
   const int rowbytes = C * 2, nv = C / 8;
   // the residual rows this thread will update in the first tile are fetched now, off the critical path
   float h_pre = 0.f;
@@ -468,11 +472,10 @@ __device__ __forceinline__ void store_frags(const KParams &p, int C, const float
 // Streams this block's units of one matrix in fragment order through the ring: per unit and 32 columns one 16-byte load of
 // weights, one 8-byte load of x and one instruction, a unit's pairs of column blocks dealt to the warps in turn; a row's
 // sum is the sum of its six wanted columns of the accumulator.
-__device__ __forceinline__ void consume_image(Blk &b, int R, int C, int kind, const EpiArgs &ea) {
+__device__ __forceinline__ void consume_image(Blk &b, int m, int C, int kind, const EpiArgs &ea) {
   const KParams &p = *b.p;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int r0, r1;
-  cta_rows(R, kUnitRows, r0, r1);
+  const int r0 = s_rows[m].x, r1 = s_rows[m].y;
   const int unit_pairs = C / 32;
   int left = (r1 - r0) / kUnitRows * unit_pairs;  // pairs behind the stage at hand
   int in_stage = 0, n = 0;                        // the stage's pairs used up, in all
@@ -495,13 +498,13 @@ __device__ __forceinline__ void consume_image(Blk &b, int R, int C, int kind, co
           n = min(p.img_pairs, p.img_span ? left : unit_pairs - u);
           left -= n;
         }
-        const int m = min(unit_pairs - u, n - in_stage);
+        const int now = min(unit_pairs - u, n - in_stage);
         const uint8_t *w = stage + ((size_t)in_stage * (4 * kUnitRows) + lane) * 16;
         const uint2 *x = xf + (size_t)u * 24;
 #pragma unroll 1  // unrolled, the loop costs more registers than the kernel has
-        for (int j = (warp - u) & (kConsumerWarps - 1); j < m; j += kConsumerWarps) mma_terms(c, lds128(w + (size_t)j * kPairBytes), x[(size_t)j * 24]);
-        u += m;
-        in_stage += m;
+        for (int j = (warp - u) & (kConsumerWarps - 1); j < now; j += kConsumerWarps) mma_terms(c, lds128(w + (size_t)j * kPairBytes), x[(size_t)j * 24]);
+        u += now;
+        in_stage += now;
         if (in_stage == n) {
           __syncwarp();
           if (lane == 0) mbar_arrive(&s_empty[b.c_stage]);
@@ -619,11 +622,11 @@ __device__ __forceinline__ void prologue_plain(const float *src, int C, float (&
   }
 }
 
-__device__ __forceinline__ int attn_splits(const KParams &p, int T) {
-  int ms = (int)gridDim.x / p.H;
-  ms = ms < 1 ? 1 : (ms > kMaxSplit ? kMaxSplit : ms);
-  int ns = (T + 63) / 64;
-  return ns < 1 ? 1 : (ns > ms ? ms : ns);
+// Ranges that the T cached positions of a head are split into, and the first position of range sp (T * sp / ns).
+__device__ __forceinline__ int attn_splits(const KParams &p, int T) { return min((int)((unsigned)(T + 63) / 64u), p.attn_most); }
+__device__ __forceinline__ int attn_from(int T, int ns, int sp) {
+  const unsigned q = (unsigned)T / (unsigned)ns, r = (unsigned)T - q * (unsigned)ns;
+  return (int)(q * (unsigned)sp + r * (unsigned)sp / (unsigned)ns);
 }
 
 // x = attention output: merges the per-split partial sums of each head
@@ -633,7 +636,15 @@ __device__ __forceinline__ void prologue_attn(const KParams &p, int T, float (&x
   for (int i = 0; i < kMaxVec; ++i) {
     const int v = (int)threadIdx.x + i * kConsumerThreads;
     if (v < nv) {
-      const int col = v * 8, head = col / p.hd, c = col - head * p.hd;
+      const int col = v * 8, head = head_of(p, col), c = col - head * p.hd;
+      if (ns == 1) {  // nothing to merge (the sums below, with one split, come to the same)
+        float o[8];
+        load8(p.opart + col, o);
+        const float inv = 1.f / __ldcg(&p.oml[head]).y;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) xr[i][e] = o[e] * inv;
+        continue;
+      }
       // one pass with a running maximum, so that a split's (max, sum) and its partial output are asked for
       // together: one trip to L2 after the grid barrier instead of two
       float M = -CUDART_INF_F, den = 0.f, acc[8];
@@ -680,7 +691,7 @@ __device__ __forceinline__ void prefetch_kv(const KParams &p, int layer, int pos
   const int lpr = (p.hd * esz + 127) >> 7;  // 128-byte lines per cache row of a head
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
     const int head = item / ns, sp = item - head * ns;
-    const int t0 = (int)((long long)T * sp / ns), t1 = min((int)((long long)T * (sp + 1) / ns), pos);
+    const int t0 = attn_from(T, ns, sp), t1 = min(attn_from(T, ns, sp + 1), pos);
     const int n = (t1 - t0) * lpr;
     for (int i = threadIdx.x; i < n; i += kConsumerThreads) {
       const int t = t0 + i / lpr, c = i - (i / lpr) * lpr;
@@ -724,7 +735,7 @@ __device__ void attention_rows(Blk &b, int layer, int pos) {
   const E *kc = reinterpret_cast<const E *>(p.kcache), *vc = reinterpret_cast<const E *>(p.vcache);
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
     const int head = item / ns, sp = item - head * ns;
-    const int t0 = (int)((long long)T * sp / ns), t1 = (int)((long long)T * (sp + 1) / ns);
+    const int t0 = attn_from(T, ns, sp), t1 = attn_from(T, ns, sp + 1);
     float q[EPL], acc[EPL];
 #pragma unroll
     for (int e = 0; e < EPL; e += 4) {
@@ -834,7 +845,7 @@ __device__ void attention_phase(Blk &b, int layer, int pos) {
   float *s_l = s_m + kConsumerWarps;               // [warps]
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
     const int head = item / ns, sp = item - head * ns;
-    const int t0 = (int)((long long)T * sp / ns), t1 = (int)((long long)T * (sp + 1) / ns);
+    const int t0 = attn_from(T, ns, sp), t1 = attn_from(T, ns, sp + 1);
     float q[8], acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
@@ -976,9 +987,9 @@ __device__ void consumer_main(Blk &b) {
       if constexpr (kImg) {
         store_frags(p, p.d, xr);
         named_sync(1, kConsumerThreads);
-        consume_image(b, 3 * p.d, p.d, kEpiQKV, ea);
+        consume_image(b, kMatQKV, p.d, kEpiQKV, ea);
       } else {
-        consume_matrix(b, 3 * p.d, p.d, 2, xr, kEpiQKV, ea);
+        consume_matrix(b, kMatQKV, p.d, xr, kEpiQKV, ea);
       }
       if (grid_barrier(b)) return;
       attention_phase(b, l, pos);
@@ -988,24 +999,24 @@ __device__ void consumer_main(Blk &b) {
       if constexpr (kImg) {
         store_frags(p, p.d, xr);
         named_sync(1, kConsumerThreads);
-        consume_image(b, p.d, p.d, kEpiAddH, ea);
+        consume_image(b, kMatO, p.d, kEpiAddH, ea);
       } else {
-        consume_matrix(b, p.d, p.d, 1, xr, kEpiAddH, ea);
+        consume_matrix(b, kMatO, p.d, xr, kEpiAddH, ea);
       }
       if (grid_barrier(b)) return;
       prologue_norm(b, p.h, gq, 2 * l + 1, p.d, xr);
       if constexpr (kImg) {
         store_frags(p, p.d, xr);
         named_sync(1, kConsumerThreads);
-        consume_image(b, 2 * p.f, p.d, kEpiSwiGLU, ea);
+        consume_image(b, kMatGateUp, p.d, kEpiSwiGLU, ea);
       } else {
-        consume_matrix(b, 2 * p.f, p.d, 2, xr, kEpiSwiGLU, ea);
+        consume_matrix(b, kMatGateUp, p.d, xr, kEpiSwiGLU, ea);
       }
       if (grid_barrier(b)) return;
       prologue_plain(p.u, p.f, xr);
       fetch_gain(gain_ptr(b, l + 1 < p.L || head ? 2 * l + 2 : 0), p.d, gq);
       ea.which = 1;
-      consume_matrix(b, p.d, p.f, 1, xr, kEpiAddH, ea);
+      consume_matrix(b, kMatDown, p.f, xr, kEpiAddH, ea);
       if (grid_barrier(b)) return;
     }
     if (head) {
@@ -1015,14 +1026,12 @@ __device__ void consumer_main(Blk &b) {
       if constexpr (kImg) {
         store_frags(p, p.d, xr);
         named_sync(1, kConsumerThreads);
-        consume_image(b, p.V, p.d, kEpiLogits, ea);
+        consume_image(b, kMatHead, p.d, kEpiLogits, ea);
       } else {
-        consume_matrix(b, p.V, p.d, 1, xr, kEpiLogits, ea);
+        consume_matrix(b, kMatHead, p.d, xr, kEpiLogits, ea);
       }
       named_sync(1, kConsumerThreads);
-      int r0, r1;
-      cta_rows(p.V, kImg ? kUnitRows : 1, r0, r1);
-      if (threadIdx.x < 32) block_topk(p, r0, r1, blockIdx.x);
+      if (threadIdx.x < 32) block_topk(p, s_rows[kMatHead].x, s_rows[kMatHead].y, blockIdx.x);
       if (grid_barrier(b)) return;
       if (blockIdx.x == 0 && (!kSampler || p.mode != kModeSample || last)) {
         if (threadIdx.x < 32) tail_keep_topk(p, gridDim.x);
@@ -1043,6 +1052,7 @@ __device__ __forceinline__ void kernel_body(const KParams &p) {
   if (p.mode != kModeScoreOnly && p.mode != kModeNucleusOnly && 2 * p.L + 1 <= kGainSlots)
     for (int j = threadIdx.x; j <= 2 * p.L; j += kThreads)
       s_gain_ptrs[j] = j == 2 * p.L ? p.final_norm : ((j & 1) ? p.layers[j >> 1].ffn_norm : p.layers[j >> 1].attn_norm);
+  if (p.mode != kModeScoreOnly && p.mode != kModeNucleusOnly && threadIdx.x < kMatrices) share_rows<kImg>(p, threadIdx.x);
   b.dead = &s_dead;
   b.quit = &s_quit;
   b.bar_target = 0;

@@ -111,6 +111,8 @@ struct KParams {
   // how units in fragment order pass through the ring (plan_units): pairs of column blocks a stage takes, whether a stage may hold the
   // end of a unit and the start of the next; stages of weights that a block has under way at most
   int32_t img_pairs, img_span, most_flying;
+  uint32_t hd_inverse;       // 2^32 / hd, rounded up: columns become heads by a multiplication
+  int32_t attn_most;         // ranges that the cached positions of a head are split into at most: blocks per head, 1 to kMaxSplit
 };
 
 }  // namespace spd
