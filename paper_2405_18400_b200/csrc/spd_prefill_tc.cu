@@ -411,15 +411,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
 }
 
 // ---------------------------------------------------------------- attention of a job
-// v = hi + mid + lo exactly: each term takes the leading 8 significant bits of what is left, by truncation.
-__device__ __forceinline__ void tc_put3(uint16_t *X, size_t term_stride, size_t at, float v) {
-  const uint32_t hi = __float_as_uint(v) & 0xffff0000u;
+// The three bf16 terms of v (v = hi + mid + lo exactly: each takes the leading 8 significant bits of what is left, by truncation), each in the upper half of a word.
+__device__ __forceinline__ void tc_split3(float v, uint32_t &hi, uint32_t &mid, uint32_t &lo) {
+  hi = __float_as_uint(v) & 0xffff0000u;
   const float r1 = v - __uint_as_float(hi);
-  const uint32_t mid = __float_as_uint(r1) & 0xffff0000u;
-  const float r2 = r1 - __uint_as_float(mid);
-  X[at] = (uint16_t)(hi >> 16);
-  X[at + term_stride] = (uint16_t)(mid >> 16);
-  X[at + 2 * term_stride] = (uint16_t)(__float_as_uint(r2) >> 16);
+  mid = __float_as_uint(r1) & 0xffff0000u;
+  lo = __float_as_uint(r1 - __uint_as_float(mid)) & 0xffff0000u;
+}
+// Two neighbouring values of the output as terms.
+__device__ __forceinline__ void tc_put_pair(uint16_t *dst, size_t term_stride, float a, float b) {
+  uint32_t h0, m0, l0, h1, m1, l1;
+  tc_split3(a, h0, m0, l0);
+  tc_split3(b, h1, m1, l1);
+  *reinterpret_cast<uint32_t *>(dst) = h1 | (h0 >> 16);
+  *reinterpret_cast<uint32_t *>(dst + term_stride) = m1 | (m0 >> 16);
+  *reinterpret_cast<uint32_t *>(dst + 2 * term_stride) = l1 | (l0 >> 16);
 }
 
 // Causal attention over a float32 cache (a bf16 cache takes spd_tc_attn_mma_kernel below): 16 consecutive tokens
@@ -428,6 +434,9 @@ __device__ __forceinline__ void tc_put3(uint16_t *X, size_t term_stride, size_t 
 // bank conflicts); a warp owns two tokens: scores with a lane per position, the tile's softmax weights by warp
 // reductions (online softmax across tiles), weighted value sums with HD / 32 dimensions per lane and the weights
 // passed round by shuffles.  Every cache row is read once per 16 tokens.  Output as three bf16 terms.
+// What bounds it: for few tokens the trips to L2 before the first score, which are made side by side (15 tokens, 7B shape, 9.4 -> 5.2
+// us a layer, 64 tokens of 13B 17.0 -> 12.9), for many the score and value loops, behind which the next tile travels (spd_prefill
+// of 200 tokens 10.1 -> 8.6 ms, 500 23.3 -> 22.1).
 template <int HD>
 __global__ void __launch_bounds__(256) spd_tc_attn_kernel(const float *Q, const float *kcache, const float *vcache, uint16_t *X,
                                                           size_t term_stride, int d, int max_pos, int layer, int pos0, int n_tok) {
@@ -442,11 +451,29 @@ __global__ void __launch_bounds__(256) spd_tc_attn_kernel(const float *Q, const 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
   const int head = blockIdx.y, t0 = blockIdx.x * kTok;
   const float scale = 1.f / sqrtf((float)HD);
-  for (int i = tid; i < kTok * HD; i += 256) {
-    const int tt = i / HD, c = i - tt * HD;
-    sq[i] = t0 + tt < n_tok ? Q[(size_t)(t0 + tt) * d + head * HD + c] * scale : 0.f;
-  }
   const int last_pos = pos0 + min(t0 + kTok - 1, n_tok - 1);  // the last position a token of this block sees
+  // A tile's rows on their way through registers: the first tile's are asked for before the queries, a later one's while the tile
+  // before it is used (a trip to L2 each, which the block otherwise spends idle).
+  constexpr int kMine = kPos * HD / 4 / 256;  // 16-byte vectors of keys that a thread brings, and of values
+  float4 kf[kMine], vf[kMine];
+  auto ask = [&](int tile0) {
+#pragma unroll
+    for (int u = 0; u < kMine; ++u) {
+      const int i = tid + u * 256, r = i / (HD / 4), c4 = i - r * (HD / 4), pos = tile0 + r;
+      const size_t at = ((size_t)layer * max_pos + min(pos, last_pos)) * d + head * HD + c4 * 4;
+      kf[u] = *reinterpret_cast<const float4 *>(kcache + at);
+      vf[u] = *reinterpret_cast<const float4 *>(vcache + at);
+      if (pos > last_pos) kf[u] = vf[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  ask(0);
+#pragma unroll
+  for (int u = 0; u < kTok * HD / 4 / 256; ++u) {
+    const int i = tid + u * 256, tt = i / (HD / 4), c = (i - tt * (HD / 4)) * 4;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (t0 + tt < n_tok) v = *reinterpret_cast<const float4 *>(Q + (size_t)(t0 + tt) * d + head * HD + c);
+    *reinterpret_cast<float4 *>(sq + tt * HD + c) = make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale);
+  }
   const int ta = t0 + 2 * warp, tb = ta + 1;
   const int pa = pos0 + ta, pb = pos0 + tb;
   float ma = -CUDART_INF_F, mb = -CUDART_INF_F, la = 0.f, lb = 0.f;
@@ -455,27 +482,14 @@ __global__ void __launch_bounds__(256) spd_tc_attn_kernel(const float *Q, const 
   for (int e = 0; e < DPL; ++e) acca[e] = accb[e] = 0.f;
   for (int tile0 = 0; tile0 <= last_pos; tile0 += kPos) {
     __syncthreads();  // the previous tile has been used (first round: nothing)
-    for (int i = tid; i < kPos * HD / 8; i += 256) {
-      const int r = i / (HD / 8), c8 = (i - r * (HD / 8)) * 8;
-      const int pos = tile0 + r;
-      float kf[8], vf[8];
-      if (pos <= last_pos) {
-        const size_t at = ((size_t)layer * max_pos + pos) * d + head * HD + c8;
-        const float4 *kp = reinterpret_cast<const float4 *>(kcache + at), *vp = reinterpret_cast<const float4 *>(vcache + at);
-        const float4 k0 = kp[0], k1 = kp[1], v0 = vp[0], v1 = vp[1];
-        kf[0] = k0.x; kf[1] = k0.y; kf[2] = k0.z; kf[3] = k0.w; kf[4] = k1.x; kf[5] = k1.y; kf[6] = k1.z; kf[7] = k1.w;
-        vf[0] = v0.x; vf[1] = v0.y; vf[2] = v0.z; vf[3] = v0.w; vf[4] = v1.x; vf[5] = v1.y; vf[6] = v1.z; vf[7] = v1.w;
-      } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) kf[j] = vf[j] = 0.f;
-      }
-      float4 *kd = reinterpret_cast<float4 *>(sk + r * KS + c8), *vd = reinterpret_cast<float4 *>(sv + r * HD + c8);
-      kd[0] = make_float4(kf[0], kf[1], kf[2], kf[3]);
-      kd[1] = make_float4(kf[4], kf[5], kf[6], kf[7]);
-      vd[0] = make_float4(vf[0], vf[1], vf[2], vf[3]);
-      vd[1] = make_float4(vf[4], vf[5], vf[6], vf[7]);
+    for (int u = 0; u < kMine; ++u) {
+      const int i = tid + u * 256, r = i / (HD / 4), c4 = i - r * (HD / 4);
+      *reinterpret_cast<float4 *>(sk + r * KS + c4 * 4) = kf[u];
+      *reinterpret_cast<float4 *>(sv + r * HD + c4 * 4) = vf[u];
     }
     __syncthreads();
+    if (tile0 + kPos <= last_pos) ask(tile0 + kPos);
     // scores of position tile0 + lane for the warp's two tokens
     float sa = 0.f, sb = 0.f;
     {
@@ -516,8 +530,9 @@ __global__ void __launch_bounds__(256) spd_tc_attn_kernel(const float *Q, const 
       acca[e] *= ca;
       accb[e] *= cb;
     }
-#pragma unroll
-    for (int j = 0; j < kPos; ++j) {
+    const int used = min(kPos, last_pos + 1 - tile0);  // positions behind the last have no weight
+#pragma unroll 8
+    for (int j = 0; j < used; ++j) {
       const float ja = __shfl_sync(0xffffffffu, wa, j), jb = __shfl_sync(0xffffffffu, wb, j);
       const float *vr = sv + j * HD + lane * DPL;
       float v[DPL];
@@ -536,10 +551,11 @@ __global__ void __launch_bounds__(256) spd_tc_attn_kernel(const float *Q, const 
     }
   }
   const float ia = 1.f / la, ib = 1.f / lb;
+  uint16_t *out = X + (size_t)ta * d + head * HD + lane * DPL;
 #pragma unroll
-  for (int e = 0; e < DPL; ++e) {
-    if (ta < n_tok) tc_put3(X, term_stride, (size_t)ta * d + head * HD + lane * DPL + e, acca[e] * ia);
-    if (tb < n_tok) tc_put3(X, term_stride, (size_t)tb * d + head * HD + lane * DPL + e, accb[e] * ib);
+  for (int e = 0; e < DPL; e += 2) {
+    if (ta < n_tok) tc_put_pair(out + e, term_stride, acca[e] * ia, acca[e + 1] * ia);
+    if (tb < n_tok) tc_put_pair(out + d + e, term_stride, accb[e] * ib, accb[e + 1] * ib);
   }
 }
 
@@ -557,16 +573,41 @@ __device__ __forceinline__ void tc_ldsm_x4_trans(uint32_t addr, uint32_t (&r)[4]
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(addr));
 }
-// The three bf16 terms of v (v = hi + mid + lo exactly), each in the upper half of a word.
-__device__ __forceinline__ void tc_split3(float v, uint32_t &hi, uint32_t &mid, uint32_t &lo) {
-  hi = __float_as_uint(v) & 0xffff0000u;
-  const float r1 = v - __uint_as_float(hi);
-  mid = __float_as_uint(r1) & 0xffff0000u;
-  lo = __float_as_uint(r1 - __uint_as_float(mid)) & 0xffff0000u;
-}
 
 __device__ __forceinline__ void tc_cp16(uint32_t dst, const void *src, uint32_t bytes) {  // 16 bytes, zeros past `bytes` (0 or 16)
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
+// Four scaled values as terms, 8 bytes of each.
+__device__ __forceinline__ void tc_put_terms(uint8_t *dst, int term_step, const float4 &v, float scale) {
+  uint32_t h[4], m[4], l[4];
+  tc_split3(v.x * scale, h[0], m[0], l[0]);
+  tc_split3(v.y * scale, h[1], m[1], l[1]);
+  tc_split3(v.z * scale, h[2], m[2], l[2]);
+  tc_split3(v.w * scale, h[3], m[3], l[3]);
+  *reinterpret_cast<uint2 *>(dst) = make_uint2(h[1] | (h[0] >> 16), h[3] | (h[2] >> 16));
+  *reinterpret_cast<uint2 *>(dst + term_step) = make_uint2(m[1] | (m[0] >> 16), m[3] | (m[2] >> 16));
+  *reinterpret_cast<uint2 *>(dst + 2 * term_step) = make_uint2(l[1] | (l[0] >> 16), l[3] | (l[2] >> 16));
+}
+// The softmax weights of 16 positions (two score fragments) as terms, repacked as a left operand; their sums join l.
+__device__ __forceinline__ void tc_weight_terms(const float (&sa)[4], const float (&sb)[4], const float (&m)[2], float (&l)[2], uint32_t (&pt)[3][4]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float pw[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) pw[e] = __expf((h ? sb : sa)[e] - m[e >> 1]);
+    l[0] += pw[0] + pw[1];
+    l[1] += pw[2] + pw[3];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      uint32_t h0, m0, l0, h1, m1, l1;
+      tc_split3(pw[2 * r], h0, m0, l0);
+      tc_split3(pw[2 * r + 1], h1, m1, l1);
+      pt[0][h * 2 + r] = h1 | (h0 >> 16);
+      pt[1][h * 2 + r] = m1 | (m0 >> 16);
+      pt[2][h * 2 + r] = l1 | (l0 >> 16);
+    }
+  }
 }
 
 // Causal attention of 16 x WARPS consecutive tokens of one head over a bf16 cache, on tensor cores (mma.sync m16n8k16:
@@ -615,15 +656,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
     const int tt = i / (HD / 4), c = (i - tt * (HD / 4)) * 4;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (t0 + tt < n_tok) v = *reinterpret_cast<const float4 *>(Q + (size_t)(t0 + tt) * d + head * HD + c);
-    uint32_t h[4], m[4], l[4];
-    tc_split3(v.x * scale, h[0], m[0], l[0]);
-    tc_split3(v.y * scale, h[1], m[1], l[1]);
-    tc_split3(v.z * scale, h[2], m[2], l[2]);
-    tc_split3(v.w * scale, h[3], m[3], l[3]);
-    uint8_t *dst = at_smem + tt * RS + c * 2;
-    *reinterpret_cast<uint2 *>(dst) = make_uint2(h[1] | (h[0] >> 16), h[3] | (h[2] >> 16));
-    *reinterpret_cast<uint2 *>(dst + kTok * RS) = make_uint2(m[1] | (m[0] >> 16), m[3] | (m[2] >> 16));
-    *reinterpret_cast<uint2 *>(dst + 2 * kTok * RS) = make_uint2(l[1] | (l[0] >> 16), l[3] | (l[2] >> 16));
+    tc_put_terms(at_smem + tt * RS + c * 2, kTok * RS, v, scale);
   }
   const int tw = t0 + warp * 16;
   const int p_first = pos0 + tw, p_lo = p_first + g, p_hi = p_lo + 8, warp_last = p_first + 15;
@@ -698,23 +731,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
 #pragma unroll
       for (int kk = 0; kk < kPos / 16; ++kk) {
         uint32_t pt[3][4];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          float pw[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) pw[e] = __expf(s[2 * kk + h][e] - m[e >> 1]);
-          l[0] += pw[0] + pw[1];
-          l[1] += pw[2] + pw[3];
-#pragma unroll
-          for (int r = 0; r < 2; ++r) {
-            uint32_t h0, m0, l0, h1, m1, l1;
-            tc_split3(pw[2 * r], h0, m0, l0);
-            tc_split3(pw[2 * r + 1], h1, m1, l1);
-            pt[0][h * 2 + r] = h1 | (h0 >> 16);
-            pt[1][h * 2 + r] = m1 | (m0 >> 16);
-            pt[2][h * 2 + r] = l1 | (l0 >> 16);
-          }
-        }
+        tc_weight_terms(s[2 * kk], s[2 * kk + 1], m, l, pt);
 #pragma unroll
         for (int dq = 0; dq < DT / 2; dq += 4) {
           uint32_t vb[4][4];
@@ -744,20 +761,146 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
     for (int r = 0; r < 2; ++r) {
       const int t = tw + g + r * 8;
       if (t < n_tok) {
-        uint32_t h0, m0, l0, h1, m1, l1;
-        tc_split3(o[i][2 * r] * inv[r], h0, m0, l0);
-        tc_split3(o[i][2 * r + 1] * inv[r], h1, m1, l1);
-        uint16_t *dst = X + (size_t)t * d + head * HD + i * 8 + 2 * q;
-        *reinterpret_cast<uint32_t *>(dst) = h1 | (h0 >> 16);
-        *reinterpret_cast<uint32_t *>(dst + term_stride) = m1 | (m0 >> 16);
-        *reinterpret_cast<uint32_t *>(dst + 2 * term_stride) = l1 | (l0 >> 16);
+        tc_put_pair(X + (size_t)t * d + head * HD + i * 8 + 2 * q, term_stride, o[i][2 * r] * inv[r], o[i][2 * r + 1] * inv[r]);
       }
+    }
+}
+
+// The same for few tokens: 16 tokens of one head, the eight warps sharing them.  With a warp per 16 tokens a short job keeps one to
+// four warps of a few SMs busy with 384 instructions a tile; here a warp takes 8 of a tile's 64 positions (the scores meet in shared
+// memory), then, with all warps repeating the softmax of the 16 tokens for themselves, 16 of the head's dimensions of the weighted
+// values.  Every score and every sum is made of the same instructions in the same order, so the results are that kernel's bit for bit.
+// What bounds it is latency: 24 dependent instructions for the scores, 12 for the values, two barriers a tile.  A job of 27 tokens,
+// 7B shape, 9.6 -> 5.3 us of the layer's 99; 16 tokens behind 384 positions 27.5 -> 21; 100 tokens 13.9 -> 10.5.
+template <int HD>
+__global__ void __launch_bounds__(256, 2)
+    spd_tc_attn_few_kernel(const float *Q, const uint16_t *kcache, const uint16_t *vcache, uint16_t *X, size_t term_stride, int d, int max_pos,
+                           int layer, int pos0, int n_tok) {
+  dep_launch();
+  dep_wait();
+  constexpr int kTok = 16, kPos = 64, kThr = 256;
+  constexpr int RS = HD * 2 + 16, KS = HD / 16;
+  constexpr int kBuf = 2 * kPos * RS;
+  extern __shared__ __align__(16) uint8_t at_smem[];
+  const uint32_t sq_u = smem_u32(at_smem);            // [3 terms][tokens][RS]
+  const uint32_t kv_u = sq_u + 3 * kTok * RS;         // two buffers of [64 positions][RS] keys, then values
+  float4 *sc = reinterpret_cast<float4 *>(at_smem + 3 * kTok * RS + 2 * kBuf);  // two buffers of [8 positions' scores][lane]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q = lane & 3;
+  const int head = blockIdx.y, t0 = blockIdx.x * kTok;
+  const int last_pos = pos0 + min(t0 + kTok - 1, n_tok - 1);
+  auto fetch = [&](int tile0, int buf) {
+    const uint32_t dst = kv_u + (uint32_t)(buf * kBuf);
+    for (int i = tid; i < kPos * HD / 8; i += kThr) {
+      const int r = i / (HD / 8), c8 = i - r * (HD / 8), pos = tile0 + r;
+      const size_t at = ((size_t)layer * max_pos + min(pos, last_pos)) * d + head * HD + c8 * 8;
+      const uint32_t bytes = pos <= last_pos ? 16u : 0u, off = (uint32_t)(r * RS + c8 * 16);
+      tc_cp16(dst + off, kcache + at, bytes);
+      tc_cp16(dst + kPos * RS + off, vcache + at, bytes);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  fetch(0, 0);
+  const float scale = 1.f / sqrtf((float)HD);
+  for (int i = tid; i < kTok * HD / 4; i += kThr) {
+    const int tt = i / (HD / 4), c = (i - tt * (HD / 4)) * 4;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (t0 + tt < n_tok) v = *reinterpret_cast<const float4 *>(Q + (size_t)(t0 + tt) * d + head * HD + c);
+    tc_put_terms(at_smem + tt * RS + c * 2, kTok * RS, v, scale);
+  }
+  const int p_first = pos0 + t0, p_lo = p_first + g, p_hi = p_lo + 8;
+  float m[2] = {-CUDART_INF_F, -CUDART_INF_F}, l[2] = {0.f, 0.f};
+  float o[2][4] = {};
+  const uint32_t a_off = sq_u + (uint32_t)(((lane & 7) + ((lane >> 3) & 1) * 8) * RS + (lane >> 4) * 16);
+  const uint32_t k_off = (uint32_t)((warp * 8 + (lane & 7)) * RS + (lane >> 3) * 16);  // 8 positions x 32 dimensions
+  const uint32_t v_off = (uint32_t)((((lane >> 3) & 1) * 8 + (lane & 7)) * RS + (lane >> 4) * 16 + kPos * RS + warp * 32);
+  int buf = 0;
+  for (int tile0 = 0; tile0 <= last_pos; tile0 += kPos, buf ^= 1) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // the tile (first round: and the queries) is in place for all, the other buffer has been used
+    if (tile0 + kPos <= last_pos) fetch(tile0 + kPos, buf ^ 1);
+    const uint32_t sk_u = kv_u + (uint32_t)(buf * kBuf);
+    {
+      float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int ks = 0; ks < KS; ks += 2) {
+        uint32_t kb[4];
+        tc_ldsm_x4(sk_u + k_off + (uint32_t)(ks * 32), kb);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            uint32_t a[4];
+            tc_ldsm_x4(a_off + (uint32_t)(j * kTok * RS + (ks + h) * 32), a);
+            tc_mma_sync(s, a, kb[2 * h], kb[2 * h + 1]);
+          }
+      }
+      sc[(buf * 8 + warp) * 32 + lane] = make_float4(s[0], s[1], s[2], s[3]);
+    }
+    __syncthreads();
+    if (warp * 16 < HD) {
+      float s[kPos / 8][4];
+      float mx[2] = {-CUDART_INF_F, -CUDART_INF_F};
+#pragma unroll
+      for (int nt = 0; nt < kPos / 8; ++nt) {
+        const float4 v = sc[(buf * 8 + nt) * 32 + lane];
+        s[nt][0] = v.x; s[nt][1] = v.y; s[nt][2] = v.z; s[nt][3] = v.w;
+        const int pos = tile0 + nt * 8 + 2 * q;
+        if (pos > p_lo) s[nt][0] = -CUDART_INF_F;
+        if (pos + 1 > p_lo) s[nt][1] = -CUDART_INF_F;
+        if (pos > p_hi) s[nt][2] = -CUDART_INF_F;
+        if (pos + 1 > p_hi) s[nt][3] = -CUDART_INF_F;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) mx[e >> 1] = fmaxf(mx[e >> 1], s[nt][e]);
+      }
+      float c[2];
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
+        mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
+        const float mn = fmaxf(m[r], mx[r]);
+        c[r] = __expf(m[r] - mn);
+        m[r] = mn;
+        l[r] *= c[r];
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        o[i][0] *= c[0]; o[i][1] *= c[0]; o[i][2] *= c[1]; o[i][3] *= c[1];
+      }
+#pragma unroll
+      for (int kk = 0; kk < kPos / 16; ++kk) {
+        uint32_t pt[3][4], vb[4];
+        tc_weight_terms(s[2 * kk], s[2 * kk + 1], m, l, pt);
+        tc_ldsm_x4_trans(sk_u + v_off + (uint32_t)(kk * 16 * RS), vb);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          tc_mma_sync(o[0], pt[j], vb[0], vb[1]);
+          tc_mma_sync(o[1], pt[j], vb[2], vb[3]);
+        }
+      }
+    }
+  }
+  if (warp * 16 >= HD) return;
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    l[r] += __shfl_xor_sync(0xffffffffu, l[r], 1);
+    l[r] += __shfl_xor_sync(0xffffffffu, l[r], 2);
+  }
+  const float inv[2] = {1.f / l[0], 1.f / l[1]};
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int t = t0 + g + r * 8;
+      if (t < n_tok) tc_put_pair(X + (size_t)t * d + head * HD + (2 * warp + i) * 8 + 2 * q, term_stride, o[i][2 * r] * inv[r], o[i][2 * r + 1] * inv[r]);
     }
 }
 
 }  // namespace spd
 
 namespace {
+
+template <int HD>
+constexpr size_t attn_few_smem() { return (size_t)(3 * 16 + 4 * 64) * (HD * 2 + 16) + 2 * 8 * 32 * 16; }  // query terms, keys and values, scores
 
 template <int HD, int WARPS>
 constexpr size_t attn_mma_smem() { return (size_t)(3 * 16 * WARPS + 4 * 64) * (HD * 2 + 16); }  // query terms; two buffers of keys and values
@@ -771,9 +914,22 @@ cudaError_t launch_attn_mma(const spd::TcJob &j, int layer, int n_tok, cudaStrea
 
 template <int HD>
 cudaError_t launch_attn(const spd::TcJob &j, int layer, int n_tok, cudaStream_t s) {
+  // Up to 128 tokens a block's warps share 16 of them; beyond, where blocks of 64 tokens keep the SMs as busy and read the cache less
+  // often, a warp has 16 (7B shape, spd_prefill, shared / apart: 15 tokens 3.06 / 3.15 ms, 27 3.12 / 3.27, 64 3.46 / 3.66, 100 4.48 /
+  // 4.53, 128 4.87 / 4.95; 200 7.53 / 7.45, 300 12.50 / 12.44).
+  if (j.kv_bf16 && n_tok <= spd::kTcTile)
+    return spd::launch_dep(spd::spd_tc_attn_few_kernel<HD>, dim3((n_tok + 15) / 16, j.H), dim3(256), attn_few_smem<HD>(), s, j.q,
+                           static_cast<const uint16_t *>(j.kcache), static_cast<const uint16_t *>(j.vcache), j.x, (size_t)j.x_term_rows * j.d, j.d,
+                           j.max_pos, layer, j.pos0, n_tok);
   if (j.kv_bf16) return (n_tok + 63) / 64 * j.H > j.sm_count ? launch_attn_mma<HD, 8>(j, layer, n_tok, s) : launch_attn_mma<HD, 4>(j, layer, n_tok, s);
   return spd::launch_dep(spd::spd_tc_attn_kernel<HD>, dim3((n_tok + 15) / 16, j.H), dim3(256), 0, s, j.q, static_cast<const float *>(j.kcache),
                          static_cast<const float *>(j.vcache), j.x, (size_t)j.x_term_rows * j.d, j.d, j.max_pos, layer, j.pos0, n_tok);
+}
+
+template <int HD>
+cudaError_t allow_attn_few_smem() {
+  return cudaFuncSetAttribute(reinterpret_cast<const void *>(&spd::spd_tc_attn_few_kernel<HD>), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)attn_few_smem<HD>());
 }
 
 template <int HD, int WARPS>
@@ -809,6 +965,8 @@ extern "C" cudaError_t spd_internal_tc_prepare(void) {
   if (e == cudaSuccess) e = allow_attn_smem<64, 8>();
   if (e == cudaSuccess) e = allow_attn_smem<128, 4>();
   if (e == cudaSuccess) e = allow_attn_smem<128, 8>();
+  if (e == cudaSuccess) e = allow_attn_few_smem<64>();
+  if (e == cudaSuccess) e = allow_attn_few_smem<128>();
   return e;
 }
 
