@@ -17,7 +17,7 @@ extern "C" cudaError_t spd_internal_prepare(size_t dyn_smem, int *blocks_per_sm)
 extern "C" cudaError_t spd_internal_prefill_prepare(int *blocks_per_sm);
 extern "C" cudaError_t spd_internal_prefill_launch(const spd::KParams *p, int grid, cudaStream_t stream);
 extern "C" cudaError_t spd_internal_pack_image(const void *w, void *out, int rows, int cols, cudaStream_t stream);
-extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd::KParams *kps, int n, int begin, int V, const __nv_bfloat16 *final_norm,
+extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd::KParams *kps, int n, int step, int V, const __nv_bfloat16 *final_norm,
                                                float *y_logits, int32_t *results, cudaStream_t s, int *launches);
 
 namespace {
@@ -894,18 +894,18 @@ int batch_enqueue(spd_ctx *const *ctxs, int32_t n, int32_t n_steps) {
   int rc = set_device(lead);
   if (rc) return rc;
   if ((rc = refuse_capture(lead))) return rc;
-  // the requests' parameters in row order; pos0 = m - 1, so that a request's next position is pos0 + n_gen on the device
+  // the requests' parameters in row order, pos0 the position of the call's first input
   std::vector<spd::KParams> kps(n);
   for (int r = 0; r < n; ++r) {
     kps[r] = ctxs[r]->kp;
-    kps[r].pos0 = ctxs[r]->m - 1;
+    kps[r].pos0 = ctxs[r]->m + ctxs[r]->n_gen - 1;
   }
   spd::KParams *dkp = reinterpret_cast<spd::KParams *>(lead->ws + lead->lay.bt_kp);
   SPD_CUDA(cudaMemcpyAsync(dkp, kps.data(), kps.size() * sizeof(spd::KParams), cudaMemcpyHostToDevice, lead->stream));  // (pageable: read on return)
   const spd::TcJob job = tc_job(lead);
   for (int s = 0; s < n_steps; ++s) {
     int launched = 0;
-    const cudaError_t e = spd_internal_batch_step(&job, dkp, n, s == 0, c0.vocab, lead->kp.final_norm, reinterpret_cast<float *>(lead->ws + lead->lay.bt_y),
+    const cudaError_t e = spd_internal_batch_step(&job, dkp, n, s, c0.vocab, lead->kp.final_norm, reinterpret_cast<float *>(lead->ws + lead->lay.bt_y),
                                                   reinterpret_cast<int32_t *>(lead->ws + lead->lay.bt_out), lead->stream, &launched);
     lead->launches += launched;
     if (e != cudaSuccess) return batch_fail(ctxs, n, e, "batched timestep");

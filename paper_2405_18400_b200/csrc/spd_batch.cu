@@ -92,24 +92,30 @@ __device__ __forceinline__ void bt_store_row(float *h, const float4 &gain, uint1
   }
 }
 
-// (ss null: the product's terms were whole RMSNorms)
-__device__ __forceinline__ float bt_rs(const float *ss, int row, int d, float eps) {
-  if (!ss) return 1.f;
-  const int nch = (d + kBtCols - 1) / kBtCols;
-  float s = 0.f;
-  for (int c = 0; c < nch; c += 8) {  // (asked for together, added in order)
-    float a[8];
+// 1 / rms of a row from its chunks' sums of squares (ss null: the product's terms were whole RMSNorms).  The first eight are asked for
+// when the object is made, the product's sums by the caller behind that, and all are waited for together; they are added in order.
+struct RowScale {
+  static constexpr int kFirst = 8;
+  const float *ss;
+  int nch;
+  float a[kFirst];
+  __device__ __forceinline__ RowScale(const float *rows, int row, int d) : ss(rows ? rows + row * kBtMaxChunks : nullptr), nch((d + kBtCols - 1) / kBtCols) {
 #pragma unroll
-    for (int u = 0; u < 8; ++u) a[u] = c + u < nch ? ss[row * kBtMaxChunks + c + u] : 0.f;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) s += a[u];
+    for (int u = 0; u < kFirst; ++u) a[u] = ss && u < nch ? ss[u] : 0.f;
   }
-  return rsqrtf(s / (float)d + eps);
-}
+  __device__ __forceinline__ float value(int d, float eps) const {
+    if (!ss) return 1.f;
+    float s = 0.f;
+#pragma unroll
+    for (int u = 0; u < kFirst; ++u) s += a[u];
+    for (int c = kFirst; c < nch; ++c) s += ss[c];
+    return rsqrtf(s / (float)d + eps);
+  }
+};
 
-// Position of the request's next input: the prefix's m positions, then one per superposed input so far.  The
-// device copy of a request's parameters keeps m - 1 in pos0; n_gen counts the tokens generated per draft.
-__device__ __forceinline__ int bt_pos(const KParams &p) { return p.pos0 + p.st->n_gen; }
+// Position of the request's input in timestep `step` of the call: the device copy of a request's parameters keeps the first one's in
+// pos0.  (From the draft state, which the timestep before writes, it was two trips to L2 behind the kernels' wait.)
+__device__ __forceinline__ int bt_pos(const KParams &p, int step) { return p.pos0 + step; }
 
 // grid (requests, column chunks): the superposed input of Eq. 3, h = sum_i gamma_i E[last token of draft i], stored as
 // the request's residual row; h * gain of the first layer's norm as three bf16 terms; the chunk's sum of squares.
@@ -230,9 +236,11 @@ __device__ __forceinline__ float4 bt_angles(const float2 *rope, int hd, int pos,
   return *reinterpret_cast<const float4 *>(rope + (size_t)pos * (hd / 2) + (c % hd) / 2);
 }
 template <int kFlight>
-__device__ __forceinline__ void bt_rope_cache(const Product &y, float rs, float *Q, void *kcache, void *vcache, const float4 &cs, int max_pos,
+__device__ __forceinline__ void bt_rope_cache(const Product &y, const float *ss, float eps, float *Q, void *kcache, void *vcache, const float4 &cs, int max_pos,
                                               int kv_bf16, int d, int layer, int t, int pos, int c) {
+  const RowScale scale(ss, t, d);
   const float4 q = product_sum4<kFlight>(y, t, c), k = product_sum4<kFlight>(y, t, d + c), v = product_sum4<kFlight>(y, t, 2 * d + c);
+  const float rs = scale.value(d, eps);
   const size_t at = ((size_t)layer * max_pos + pos) * d + c;
   *reinterpret_cast<float4 *>(Q + (size_t)t * d + c) = bt_rotate(make_float4(q.x * rs, q.y * rs, q.z * rs, q.w * rs), cs);
   bt_store_kv(kcache, kv_bf16, at, bt_rotate(make_float4(k.x * rs, k.y * rs, k.z * rs, k.w * rs), cs));
@@ -242,15 +250,16 @@ __device__ __forceinline__ void bt_rope_cache(const Product &y, float rs, float 
 // grid (requests, column chunks): each request at its own position, into its own cache.
 template <int kFlight>
 __global__ void __launch_bounds__(kBtThreads) spd_batch_rope_cache_kernel(const __grid_constant__ Product y, const float *ss, float eps, float *Q,
-                                                                          const KParams *kps, int d, int hd, int layer) {
+                                                                          const KParams *kps, int d, int hd, int layer, int step) {
+  // what does not hang on the product: the request's parameters (as old as the call), its position's angles
+  const KParams &p = kps[blockIdx.x];
+  const int c = blockIdx.y * kBtCols + threadIdx.x * 4, pos = bt_pos(p, step), max_pos = p.max_pos, kv_bf16 = p.kv_bf16;
+  void *kcache = p.kcache, *vcache = p.vcache;
+  const float4 cs = c < d ? bt_angles(p.rope, hd, pos, c) : make_float4(0.f, 0.f, 0.f, 0.f);
   dep_wait();
   dep_launch();
-  const KParams &p = kps[blockIdx.x];
-  const int c = blockIdx.y * kBtCols + threadIdx.x * 4;
   if (c >= d) return;
-  const int pos = bt_pos(p);
-  bt_rope_cache<kFlight>(y, bt_rs(ss, blockIdx.x, d, eps), Q, p.kcache, p.vcache, bt_angles(p.rope, hd, pos, c), p.max_pos, p.kv_bf16, d, layer,
-                         blockIdx.x, pos, c);
+  bt_rope_cache<kFlight>(y, ss, eps, Q, kcache, vcache, cs, max_pos, kv_bf16, d, layer, blockIdx.x, pos, c);
 }
 
 // The same for a job of prefix tokens of one request (token t at position pos0 + t, one cache).
@@ -263,7 +272,7 @@ __global__ void __launch_bounds__(kBtThreads) spd_job_rope_cache_kernel(const __
   dep_wait();
   dep_launch();
   if (c >= d) return;
-  bt_rope_cache<kFlight>(y, bt_rs(ss, blockIdx.x, d, eps), Q, kcache, vcache, cs, max_pos, kv_bf16, d, layer, blockIdx.x, pos, c);
+  bt_rope_cache<kFlight>(y, ss, eps, Q, kcache, vcache, cs, max_pos, kv_bf16, d, layer, blockIdx.x, pos, c);
 }
 
 // grid (rows, chunks of the FFN): u = SiLU(gate) * up from the gate / up product's row times 1 / rms
@@ -279,8 +288,9 @@ __global__ void __launch_bounds__(kBtThreads) spd_batch_swiglu_kernel(const __gr
   dep_wait();
   const int t = blockIdx.x, j = blockIdx.y * kBtCols + threadIdx.x * 4;
   if (j >= f) return;
-  const float rs = bt_rs(ss, t, d, eps);
+  const RowScale scale(ss, t, d);
   const float4 a = product_sum4<kFlight>(y, t, 2 * j), b = product_sum4<kFlight>(y, t, 2 * j + 4);
+  const float rs = scale.value(d, eps);
   bt_put3x4(X, term_stride, (size_t)t * f + j,
             make_float4(bt_swiglu(a.x, a.y, rs), bt_swiglu(a.z, a.w, rs), bt_swiglu(b.x, b.y, rs), bt_swiglu(b.z, b.w, rs)));
 }
@@ -291,7 +301,9 @@ __global__ void __launch_bounds__(kBtThreads) spd_batch_swiglu_kernel(const __gr
 // group of lanes are in flight before the first is used; they enter the running softmax together (one rescale per round).
 // A round of the block is 32 (float32, head size 128) to 128 positions (bf16, 64).  The groups' states are merged in
 // shared memory in a fixed order; output as three bf16 terms.  7B shape, bf16 cache, whole timestep of 8 / 64 requests
-// behind 150 positions each: 4.58 / 7.99 ms (a warp per position, one in flight, element-wise loads), now 3.51 / 6.14 ms.
+// behind 150 positions each: 4.58 / 7.99 ms (a warp per position, one in flight, element-wise loads), now 3.51 / 6.14 ms; with the
+// request's position known before the wait, no trip to L2 for it, and the rows asked into L2 while the rotary kernel runs, three
+// timesteps of 8 / 64 requests behind 15 to 90 positions (float32 cache) 9.47 / 16.28 -> 9.31 / 15.58 ms.
 constexpr int kBaWarps = 8, kBaFlight = 4;
 
 template <typename E>
@@ -318,10 +330,12 @@ __device__ void ba_head(const float *q_row, const E *kc, const E *vc, int d, int
   const float scale = 1.f / sqrtf((float)HD);
   float q[EPL], acc[EPL];
 #pragma unroll
-  for (int e = 0; e < EPL; ++e) {
-    q[e] = q_row[at + e];
-    acc[e] = 0.f;
+  for (int e = 0; e < EPL; e += 4) {
+    const float4 v = *reinterpret_cast<const float4 *>(q_row + at + e);
+    q[e] = v.x; q[e + 1] = v.y; q[e + 2] = v.z; q[e + 3] = v.w;
   }
+#pragma unroll
+  for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
   float m = -CUDART_INF_F, l = 0.f;
   for (int tb = 0; tb < T; tb += G * kBaFlight) {  // all lanes of a warp go round together (the shuffles)
     uint4 kq[kBaFlight], vq[kBaFlight];
@@ -384,19 +398,29 @@ __device__ void ba_head(const float *q_row, const E *kc, const E *vc, int d, int
 
 template <int HD>
 __global__ void __launch_bounds__(kBaWarps * 32) spd_batch_attn_kernel(const float *Q, const KParams *kps, uint16_t *X, size_t term_stride, int d,
-                                                                       int layer) {
+                                                                       int layer, int step) {
   dep_launch();
-  dep_wait();
   constexpr int kGroups = kBaWarps * 32 / (HD / 8);  // bf16: the larger number of groups
   __shared__ float s_acc[kGroups * HD], s_m[kGroups], s_l[kGroups];
   const KParams &p = kps[blockIdx.x];
-  const int T = bt_pos(p) + 1;
+  const int T = bt_pos(p, step) + 1, kv_bf16 = p.kv_bf16;
+  const void *kcache = p.kcache, *vcache = p.vcache;
   const size_t x_at = (size_t)blockIdx.x * d + blockIdx.y * HD, base = (size_t)layer * p.max_pos * d + blockIdx.y * HD;
-  if (p.kv_bf16)
-    ba_head<HD>(Q + x_at, static_cast<const __nv_bfloat16 *>(p.kcache) + base, static_cast<const __nv_bfloat16 *>(p.vcache) + base, d, T, X,
+  // The cached rows are on their way to L2 while the kernel before this one still runs (a hint: they are read behind the wait).
+  {
+    const int lines = HD * (kv_bf16 ? 2 : 4) / 128, esz = kv_bf16 ? 2 : 4;
+    for (int i = threadIdx.x; i < (T - 1) * lines; i += kBaWarps * 32) {
+      const size_t off = (base + (size_t)(i / lines) * d) * esz + (size_t)(i % lines) * 128;
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const uint8_t *>(kcache) + off));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const uint8_t *>(vcache) + off));
+    }
+  }
+  dep_wait();
+  if (kv_bf16)
+    ba_head<HD>(Q + x_at, static_cast<const __nv_bfloat16 *>(kcache) + base, static_cast<const __nv_bfloat16 *>(vcache) + base, d, T, X,
                 term_stride, x_at, s_acc, s_m, s_l);
   else
-    ba_head<HD>(Q + x_at, static_cast<const float *>(p.kcache) + base, static_cast<const float *>(p.vcache) + base, d, T, X, term_stride, x_at,
+    ba_head<HD>(Q + x_at, static_cast<const float *>(kcache) + base, static_cast<const float *>(vcache) + base, d, T, X, term_stride, x_at,
                 s_acc, s_m, s_l);
 }
 
@@ -411,7 +435,7 @@ __global__ void __launch_bounds__(kConsumerThreads) spd_batch_tail_kernel(const 
   extern __shared__ __align__(16) uint8_t bt_smem[];
   __shared__ int s_dead, s_quit;
   const KParams &p = kps[blockIdx.x];
-  const float rs = bt_rs(ss, blockIdx.x, p.d, eps);
+  const float rs = RowScale(ss, blockIdx.x, p.d).value(p.d, eps);
   const float *row = y.y + (size_t)blockIdx.x * V;
   // a warp takes row tiles of the product (256 logits, alike in their parts) in turn
   for (int rt = threadIdx.x >> 5; rt * 256 < V; rt += kConsumerWarps) {
@@ -568,8 +592,8 @@ constexpr size_t kBatchTailSmem = 20480;
 // Enqueues one batched timestep of n requests (kps: their parameters in device memory, in row order) on stream s.
 // job: the buffers of the context that lends its long-prefix workspace; y_logits: [128][V] floats.  *launches receives
 // the number of kernels enqueued.
-// begin: the call's first timestep.
-extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd::KParams *kps, int n, int begin, int V, const __nv_bfloat16 *final_norm,
+// step: timesteps of the call before this one.
+extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd::KParams *kps, int n, int step, int V, const __nv_bfloat16 *final_norm,
                                                float *y_logits, int32_t *results, cudaStream_t s, int *launches) {
   const spd::TcJob &j = *job;
   const int d = j.d, f = j.f;
@@ -592,15 +616,15 @@ extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd:
       done(spd::launch_dep(few ? spd::spd_batch_resid_kernel<spd::kPartFlight> : spd::spd_batch_resid_kernel<1>, dim3(n, nch), threads, 0, s, j.h, pr, gain,
                            j.x, ts_d, d, j.ss));
   };
-  done(spd::launch_dep(spd::spd_batch_input_kernel, dim3(n, nch), threads, 0, s, kps, j.h, j.layers[0].attn_norm, j.x, ts_d, d, j.ss, begin));
+  done(spd::launch_dep(spd::spd_batch_input_kernel, dim3(n, nch), threads, 0, s, kps, j.h, j.layers[0].attn_norm, j.x, ts_d, d, j.ss, step == 0));
   for (int l = 0; l < j.L && e == cudaSuccess; ++l) {
     product(0, 4 * l, 3 * d);
     if (e == cudaSuccess)
       done(spd::launch_dep(few ? spd::spd_batch_rope_cache_kernel<spd::kPartFlight> : spd::spd_batch_rope_cache_kernel<1>, dim3(n, nch), threads, 0, s, pr, j.ss,
-                           j.eps, j.q, kps, d, j.hd, l));
+                           j.eps, j.q, kps, d, j.hd, l, step));
     if (e == cudaSuccess)
-      done(j.hd == 128 ? spd::launch_dep(spd::spd_batch_attn_kernel<128>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l)
-                       : spd::launch_dep(spd::spd_batch_attn_kernel<64>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l));
+      done(j.hd == 128 ? spd::launch_dep(spd::spd_batch_attn_kernel<128>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l, step)
+                       : spd::launch_dep(spd::spd_batch_attn_kernel<64>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l, step));
     product(0, 4 * l + 1, d);
     resid(j.layers[l].ffn_norm);
     product(0, 4 * l + 2, 2 * f);

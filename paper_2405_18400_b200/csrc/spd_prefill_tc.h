@@ -158,7 +158,8 @@ __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.laun
 // Launch with programmatic stream serialization: the kernel may be brought onto the SMs once every block of the one
 // before it in the stream has said so (dep_launch) or has ended, and waits there (dep_wait) until that one has completed.
 // Every block passes dep_wait before it ends, so a kernel that has completed stands for all before it and the kernels of a
-// chain may be set up several deep; before its dep_wait a block touches only weights and its own shared and tensor memory.
+// chain may be set up several deep; before its dep_wait a block touches only weights, what is as old as the call (a batch's request
+// parameters, rotary tables), its own shared and tensor memory, and L2 by prefetches.
 // No kernel waits for one that cannot start: a block comes onto an SM only when all blocks of the kernel before it have.
 // All kernels say so first thing, so that the next product's first weight copies are under way while the one before
 // drains (8 / 64 requests 3.29 / 4.38 -> 3.19 / 4.30 ms per 7B timestep), but for the rotary embedding: the attention's
