@@ -122,8 +122,8 @@ static __device__ void tail_score_select(Blk &b, bool first, int step) {
     if (tid < 32) {
       // the k best options, best first (Eq. 2); then the state moves to the new drafts
       const int lane = tid;
-      float pv = 0.f;
-      int pi = -1;
+      static_assert(kMaxK * kMaxK <= 32 * 32, "a bit per option of a lane");
+      uint32_t taken = 0u;
       int my_sel = -1;
       float my_score = 0.f;
       for (int r = 0; r < k; ++r) {
@@ -131,13 +131,11 @@ static __device__ void tail_score_select(Blk &b, bool first, int step) {
         int bi = -1;
         for (int c = lane; c < k * k; c += 32) {
           const float z = s_score[c];
-          if (r > 0 && !ranks_before(pv, pi, z, c)) continue;
-          if (bi < 0 || ranks_before(z, c, bv, bi)) { bv = z; bi = c; }
+          if (!(taken >> (c >> 5) & 1u) && (bi < 0 || z > bv)) { bv = z; bi = c; }
         }
         warp_best(bv, bi);
+        if ((bi & 31) == lane) taken |= 1u << (bi >> 5);
         if (lane == r) { my_sel = max(bi, 0); my_score = bv; }  // NaN scores can leave a round without a winner: keep the option valid
-        pv = bv;
-        pi = bi;
       }
       int w[kWin];
       float old_lp = 0.f;

@@ -13,13 +13,19 @@ namespace spd {
 // Ranking order everywhere: larger value first, then smaller index.
 __device__ __forceinline__ bool ranks_before(float v, int i, float w, int j) { return v > w || (v == w && i < j); }
 
+// Floats as words of the same order; 0 is below all of them, NaN the next, -0 and +0 are one value.
+__device__ __forceinline__ uint32_t order_key(float v) {
+  const uint32_t u = __float_as_uint(v + 0.f);
+  return v != v ? 1u : ((u & 0x80000000u) ? ~u : (u | 0x80000000u));
+}
+__device__ __forceinline__ float order_value(uint32_t key) { return __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key); }
+
+// The warp's best candidate (i < 0: a lane without one), to all lanes.  Two reductions of words: with five rounds of two shuffles and
+// the comparison a call took 0.2 us, and a timestep's tail makes 3 k of them while all blocks wait.
 __device__ __forceinline__ void warp_best(float &v, int &i) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float ov = __shfl_xor_sync(0xffffffffu, v, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, i, o);
-    if (oi >= 0 && (i < 0 || ranks_before(ov, oi, v, i))) { v = ov; i = oi; }
-  }
+  const uint32_t mine = i >= 0 ? order_key(v) : 0u, best = __reduce_max_sync(0xffffffffu, mine);
+  i = (int)__reduce_min_sync(0xffffffffu, mine == best && i >= 0 ? (uint32_t)i : 0xffffffffu);
+  if (best) v = order_value(best);
 }
 
 // One warp: the k best logits among rows [r0, r1) and (max, sum exp) of z / tau over them, into list `slot` of the
@@ -37,20 +43,30 @@ static __device__ void block_topk(const KParams &p, int r0, int r1, int slot) {
   fetch(r0 + lane);
   float pv = 0.f;
   int pi = -1;
+  uint32_t taken = 0u;  // of the lane's rows in registers
   float mx = -CUDART_INF_F;
   for (int j = 0; j < p.k; ++j) {
     float bv = 0.f;
     int bi = -1;
-    for (int r = r0 + lane; r < r1; r += 32 * kTopkFlight) {
-      if (!once) fetch(r);
+    if (once) {
 #pragma unroll
       for (int e = 0; e < kTopkFlight; ++e) {
-        const int id = r + 32 * e;
-        // (rows already taken, the previous winner among them, are passed over)
-        if (id < r1 && (j == 0 || ranks_before(pv, pi, z[e], id)) && (bi < 0 || ranks_before(z[e], id, bv, bi))) { bv = z[e]; bi = id; }
+        const int id = r0 + lane + 32 * e;
+        if (id < r1 && !(taken >> e & 1u) && (bi < 0 || z[e] > bv)) { bv = z[e]; bi = id; }
+      }
+    } else {
+      for (int r = r0 + lane; r < r1; r += 32 * kTopkFlight) {
+        fetch(r);
+#pragma unroll
+        for (int e = 0; e < kTopkFlight; ++e) {
+          const int id = r + 32 * e;
+          // (rows already taken, the previous winner among them, are passed over)
+          if (id < r1 && (j == 0 || ranks_before(pv, pi, z[e], id)) && (bi < 0 || ranks_before(z[e], id, bv, bi))) { bv = z[e]; bi = id; }
+        }
       }
     }
     warp_best(bv, bi);
+    if (once && bi >= 0 && ((bi - r0) & 31) == lane) taken |= 1u << ((bi - r0) >> 5);
     if (lane == 0) {
       p.pk_val[(size_t)slot * p.k + j] = bi >= 0 ? bv : -CUDART_INF_F;
       p.pk_id[(size_t)slot * p.k + j] = bi;
@@ -104,8 +120,7 @@ static __device__ void tail_keep_topk(const KParams &p, int n_lists) {
   float M = -CUDART_INF_F;
 #pragma unroll
   for (int i = 0; i < kMine; ++i) M = fmaxf(M, ms[i].x);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  M = order_value(__reduce_max_sync(0xffffffffu, order_key(M)));
   float S = 0.f;
 #pragma unroll
   for (int i = 0; i < kMine; ++i)

@@ -27,3 +27,33 @@ def test_keep_topk_lists(vocab, k, hot):
     compare_first_step(ctx, orc, si.make_prefix("zipf", 20, vocab, 1.1, seed=94))  # the end of a job
     compare_step(ctx, orc)
     ctx.close()
+
+
+@pytest.mark.parametrize("vocab,k", [(96, 16), (1504, 3), (1504, 16), (37888, 8), (40000, 16)])
+def test_equal_logits_are_kept_by_id(vocab, k):
+    """The kept tokens are the largest of the device's own logits, equal ones by ascending id: a row and its negative, eight times as
+    large as the others, in twelve places each make ties at the top, between lanes, between blocks and (k = 3, 8) between the last kept
+    and the first left out; rows of zeros make logits of zero."""
+    import numpy as np
+    import paper_2405_18400_b200 as P
+    shape = si.ModelShape("ties", 1, 128, 2, 128, vocab)
+    weights = si.make_weights(shape, seed=95)
+    head = weights["lm_head"]
+    step = vocab // 12
+    for r in range(12):
+        head[r * step + 1] = head[step + 3] * 8      # exact in bf16
+        head[r * step + 2] = head[step + 3] * -8
+        head[r * step] = 0
+    ctx = P.SpdContext(shape, P.pack_weights(weights, "cuda:0"), [], k, (2, 3), [0.0] * 8, 0.4, 0.2, 0.05, 192, "f32")
+    prefixes = [si.make_prefix("zipf", 20, vocab, 1.1, seed=s) for s in (96, 97, 98, 99)]
+    tied = 0
+    for prefix in prefixes:
+        ctx.spd_prefill(prefix)
+        for _ in range(3):
+            z = ctx.spd_debug_read("LOGITS")
+            order = np.lexsort((np.arange(vocab), -z.astype(np.float64)))
+            assert ctx.spd_debug_read("CAND_TOK").tolist() == order[:k].tolist()
+            tied += int(len(np.unique(z[order[:k + 1]])) < k + 1)
+            ctx.spd_step()
+    assert tied                                      # (a step whose hidden row is nearly at right angles to that row has none)
+    ctx.close()
