@@ -962,7 +962,8 @@ __device__ void consumer_main(Blk &b) {
     if (blockIdx.x == 0) {
       if (kSampler && p.mode == kModeSample) {
         // the next token is drawn from the logits of the pass before (Section 4.5: a nucleus-sampled prefix)
-        const int tok = ns_sample(p.logits, p.V, p.ns_inv_temp, p.ns_p, p.ns_u[it], reinterpret_cast<uint8_t *>(scratch_base(p)));
+        const int tok = ns_sample(p.logits, p.V, p.ns_inv_temp, p.ns_p, p.ns_u[it], reinterpret_cast<uint8_t *>(scratch_base(p)),
+                                  p.pk_val, gridDim.x, p.k);  // (the blocks' lists of the pass before begin with their largest logits)
         if (threadIdx.x == 0) p.prefix[it] = tok;
         named_sync(1, kConsumerThreads);
       }
@@ -1074,7 +1075,7 @@ __device__ __forceinline__ void kernel_body(const KParams &p) {
   }
   if (kSampler && p.mode == kModeNucleusOnly) {
     if (blockIdx.x == 0 && threadIdx.x < kConsumerThreads) {
-      const int tok = ns_sample(p.logits, p.V, p.ns_inv_temp, p.ns_p, p.ns_u[0], reinterpret_cast<uint8_t *>(scratch_base(p)));
+      const int tok = ns_sample(p.logits, p.V, p.ns_inv_temp, p.ns_p, p.ns_u[0], reinterpret_cast<uint8_t *>(scratch_base(p)), nullptr, 0, 0);
       if (threadIdx.x == 0) p.st->cand_tok[0] = tok;
     }
     return;

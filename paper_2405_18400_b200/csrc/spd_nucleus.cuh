@@ -6,9 +6,9 @@
 // nucleus is the shortest head of that order whose sum reaches p * sum_i e_i, and the draw u in [0, 1) picks
 // the first token whose running sum exceeds u * (mass of the nucleus).  All sums are taken in 64-bit fixed
 // point (e_i * 2^40, rounded down), so they are exact, independent of the order of summation, and every
-// comparison is an integer comparison.  Both thresholds are located by a radix search over the logits'
-// order-preserving 32-bit keys: six passes (6,6,6,6,6,2 bits), each a histogram of mass and count per digit
-// among the logits that share the digits fixed so far, scanned from the top digit down.
+// comparison is an integer comparison.  A nucleus of few tokens close to the best (ns_near) takes one pass over the logits.  Else both
+// thresholds are located by a radix search over the logits' order-preserving 32-bit keys: six passes (6,6,6,6,6,2 bits), each a
+// histogram of mass and count per digit among the logits that share the digits fixed so far, scanned from the top digit down.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -157,19 +157,140 @@ static __device__ void ns_search(NsShared &s, const float *logits, int V, float 
   }
 }
 
+// The draw when few tokens lie near the best.  Those at distances x = max - z / T below 8 are listed and fall into 32 bins a quarter
+// wide (in the order of the logits, for the distance is one rounding of a monotone function); what lies further off only adds to the
+// total.  When the list holds them all and the nucleus ends among them, the two tokens sought are found by the running sums of their
+// own bin: the same sums of the same whole numbers as in the search.  False: not such a case (a flat distribution, a nucleus of
+// hundreds of tokens, no mass at all), nothing decided; known as soon as the list is full.
+// One pass over the logits instead of fourteen, with four trips to L2 in it: 10 tokens drawn from 32000 logits at temperature 0.2,
+// 7B shape, 25.60 -> 24.17 ms, 0.143 ms a draw.
+constexpr int kNearBins = 32, kNearList = kConsumerThreads, kNearFlight = 16;
+struct NsNear {
+  unsigned int hi[kNearBins], lo[kNearBins];
+  unsigned long long tot[kNearBins], before[kNearBins];  // per bin: its mass, the mass of the bins before it
+  unsigned long long ord[kNearList], mass[kNearList];    // per listed token: place in the order (larger first), mass
+  unsigned char bin[kNearList];
+  unsigned long long far[kConsumerWarps];                // mass behind the bins, per warp
+  unsigned long long target, nucleus;
+  int listed, cut_bin, hit_bin, token;
+};
+static_assert(sizeof(NsNear) <= 20480, "nucleus scratch must fit the block's scratch area");
+
+static __device__ bool ns_near(NsNear &s, const float *logits, int V, float inv_t, float m, float top_p, float u, int &token) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid < kNearBins) s.hi[tid] = s.lo[tid] = 0u;
+  if (tid == 0) {
+    s.listed = 0;
+    s.cut_bin = s.hit_bin = -1;
+    s.token = 0;
+  }
+  named_sync(1, kConsumerThreads);
+  unsigned int far_hi = 0u, far_lo = 0u;  // at most 128 values (V is below 65536), halves below 2^20
+  for (int base = 0; base < V && *reinterpret_cast<volatile int *>(&s.listed) <= kNearList; base += kNearFlight * kConsumerThreads) {
+    float zb[kNearFlight];
+#pragma unroll
+    for (int e = 0; e < kNearFlight; ++e) {
+      const int r = base + e * kConsumerThreads + tid;
+      zb[e] = r < V ? __ldcg(logits + r) : -CUDART_INF_F;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int e = 0; e < kNearFlight; ++e) {
+      const float x = -fmaf(zb[e], inv_t, -m);
+      const bool near = x < 8.f;
+      unsigned int h = 0u, l = 0u;
+      if (x < 30.f) ns_mass(zb[e], inv_t, m, h, l);  // (e^-30 is below 2^-40: no mass)
+      const unsigned int votes = __ballot_sync(0xffffffffu, near);
+      if (votes) {
+        int at = 0;
+        if (lane == 0) at = atomicAdd(&s.listed, __popc(votes));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(votes & ((1u << lane) - 1u));
+        if (near && at < kNearList) {
+          const int b = max((int)(x * 4.f), 0);
+          atomicAdd(&s.hi[b], h);  // at most kNearList values of 2^20 in all
+          atomicAdd(&s.lo[b], l);
+          s.ord[at] = (unsigned long long)ns_key(zb[e]) << 32 | (0xffffffffu - (unsigned int)(base + e * kConsumerThreads + tid));
+          s.mass[at] = ((unsigned long long)h << 20) + l;
+          s.bin[at] = (unsigned char)b;
+        }
+      }
+      if (!near) {
+        far_hi += h;
+        far_lo += l;
+      }
+    }
+  }
+  unsigned long long far = ((unsigned long long)far_hi << 20) + far_lo;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) far += __shfl_xor_sync(0xffffffffu, far, o);
+  if (lane == 0) s.far[warp] = far;
+  named_sync(1, kConsumerThreads);
+  if (tid == 0 && s.listed <= kNearList) {
+    unsigned long long all = 0ull;
+    for (int b = 0; b < kNearBins; ++b) {
+      s.before[b] = all;
+      all += s.tot[b] = ((unsigned long long)s.hi[b] << 20) + s.lo[b];
+    }
+    for (int w = 0; w < kConsumerWarps; ++w) all += s.far[w];
+    unsigned long long t = __double2ull_ru((double)top_p * (double)all);
+    t = t < 1ull ? 1ull : (t > all ? all : t);
+    s.target = t;
+    for (int b = 0; b < kNearBins && s.cut_bin < 0; ++b)
+      if (all > 0ull && s.before[b] + s.tot[b] >= t) s.cut_bin = b;
+  }
+  named_sync(1, kConsumerThreads);
+  if (s.cut_bin < 0) return false;
+  const int n = s.listed;
+  const bool mine = tid < n;
+  const unsigned long long ord = mine ? s.ord[tid] : 0ull, mass = mine ? s.mass[tid] : 0ull;
+  const int bin = mine ? s.bin[tid] : -1;
+  // the running sum in front of the thread's token, for the tokens of one bin
+  auto sum_before = [&]() {
+    unsigned long long a = s.before[bin];
+    for (int j = 0; j < n; ++j)
+      if (s.bin[j] == bin && s.ord[j] > ord) a += s.mass[j];
+    return a;
+  };
+  if (bin == s.cut_bin) {
+    const unsigned long long a = sum_before();
+    if (a < s.target && a + mass >= s.target) s.nucleus = a + mass;  // the nucleus' last token
+  }
+  named_sync(1, kConsumerThreads);
+  const unsigned long long all = s.nucleus;
+  unsigned long long t = __double2ull_rd((double)u * (double)all);
+  if (t >= all) t = all - 1ull;
+  if (tid < kNearBins && s.before[tid] <= t && t < s.before[tid] + s.tot[tid]) s.hit_bin = tid;
+  named_sync(1, kConsumerThreads);
+  if (mine && bin == s.hit_bin) {
+    const unsigned long long a = sum_before();
+    if (a <= t && t < a + mass) s.token = (int)(0xffffffffu - (unsigned int)ord);
+  }
+  named_sync(1, kConsumerThreads);
+  token = s.token;
+  named_sync(1, kConsumerThreads);
+  return true;
+}
+
 // Draws one token from the nucleus of softmax(logits / T) with the uniform number u in [0, 1).  Every
 // consumer thread of the block calls it; all get the token.
-static __device__ __noinline__ int ns_sample(const float *logits, int V, float inv_t, float top_p, float u, uint8_t *scratch) {
+// heads: the largest logit of each of n_heads parts of the vocabulary, stride apart (null: looked for here).
+static __device__ __noinline__ int ns_sample(const float *logits, int V, float inv_t, float top_p, float u, uint8_t *scratch, const float *heads,
+                                             int n_heads, int stride) {
   NsShared &s = *reinterpret_cast<NsShared *>(scratch);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   named_sync(1, kConsumerThreads);
   // largest logit
-  float zm = -3.402823466e38f;
-  for (int r0 = tid; r0 < V; r0 += kNsBatch * kConsumerThreads) {
+  float zm = -3.402823466e38f, head = -CUDART_INF_F;
+  if (heads) {
+    if (tid < n_heads) head = __ldcg(heads + (size_t)tid * stride);
+    zm = fmaxf(zm, head);
+  } else {
+    for (int r0 = tid; r0 < V; r0 += kNsBatch * kConsumerThreads) {
 #pragma unroll
-    for (int e = 0; e < kNsBatch; ++e) {
-      const int r = r0 + e * kConsumerThreads;
-      if (r < V) zm = fmaxf(zm, __ldcg(logits + r));
+      for (int e = 0; e < kNsBatch; ++e) {
+        const int r = r0 + e * kConsumerThreads;
+        if (r < V) zm = fmaxf(zm, __ldcg(logits + r));
+      }
     }
   }
 #pragma unroll
@@ -187,6 +308,25 @@ static __device__ __noinline__ int ns_sample(const float *logits, int V, float i
   }
   named_sync(1, kConsumerThreads);
   const float m = s.zmax * inv_t;
+  // Not tried when fifteen in sixteen of the parts' largest logits are that near: with 148 parts of 216 some 400 tokens are then (an
+  // attempt in vain costs a draw 8 us).
+  const unsigned int near_votes = __ballot_sync(0xffffffffu, -fmaf(head, inv_t, -m) < 8.f);
+  if (lane == 0) s.warp_cnt[warp] = __popc(near_votes);
+  named_sync(1, kConsumerThreads);
+  int heads_near = 0;
+  for (int w = 0; w < kConsumerWarps; ++w) heads_near += s.warp_cnt[w];
+  if (16 * heads_near <= 15 * n_heads) {
+    named_sync(1, kConsumerThreads);  // (maximum and counts have been read: the scratch is laid out anew)
+    int token;
+    if (ns_near(*reinterpret_cast<NsNear *>(scratch), logits, V, inv_t, m, top_p, u, token)) return token;
+    named_sync(1, kConsumerThreads);
+    if (tid == 0) {
+      s.above = 0ull;
+      s.prefix = 0u;
+      s.target = 1ull;
+    }
+    named_sync(1, kConsumerThreads);
+  }
   // where the nucleus ends
   ns_search(s, logits, V, inv_t, m, top_p);
   if (tid == 0) {

@@ -80,6 +80,31 @@ def test_sampler_edge_cases(tiny_inputs):
     assert ctx.spd_debug_nucleus(z, 0.99, 1e-3, 0.7) == int(np.argmax(z))
 
 
+# Tokens at distances below 8 from the best: as many as the one-pass draw lists, one more, a nucleus that ends with the last of them,
+# at its first, beyond them; equal logits on both sides of the cut.  `rest`: the others' distance (30 and more have no mass).
+@pytest.mark.parametrize("near,rest,top_p", [(1, 40.0, 0.9), (511, 40.0, 1.0), (512, 40.0, 1.0), (512, 9.0, 0.9), (513, 40.0, 1.0), (513, 9.0, 0.5),
+                                             (40, 8.5, 0.97), (40, 8.0, 1.0), (300, 20.0, 1e-6)])
+@pytest.mark.parametrize("equal", [False, True])
+def test_few_tokens_near_the_best(tiny_inputs, near, rest, top_p, equal):
+    ctx, _ = make_tiny_pair(tiny_inputs)
+    v = ctx.shape.vocab
+    rng = np.random.default_rng(near + int(10 * rest))
+    temperature = 0.25                                # distances in steps of 1/16 are exact
+    x = np.full(v, rest)
+    at = rng.permutation(v)[:near]
+    x[at] = (rng.integers(0, 8 if equal else 127, near) / 16) * (15.5 / 16 if equal else 1.0)
+    x[at[0]] = 0.0
+    z = (3.0 - temperature * x).astype(np.float32)
+    exact = 0
+    for u in list(uniforms(12, near)) + [np.float32(0.0), np.float32(1.0 - 2.0 ** -24)]:
+        tok = ctx.spd_debug_nucleus(z, top_p, temperature, float(u))
+        want, ok = accepted(z, temperature, top_p, float(u))
+        assert tok in ok, (u, tok, want)
+        exact += tok == want
+    assert exact >= 11
+    ctx.close()
+
+
 def test_arguments_are_checked(tiny_inputs):
     ctx, _ = make_tiny_pair(tiny_inputs)
     _, _, _, prefix = tiny_inputs
