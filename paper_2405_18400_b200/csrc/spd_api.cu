@@ -275,7 +275,7 @@ void plan_units(const spd_config &c, bool images, spd::KParams &kp) {
 }
 
 // What a call tells its caller about the last step, as it lies in the state: one copy.  (A copy into pageable memory is a round
-// trip of its own: with four of them a step of the tiny model took 114 us, of which the device worked 54; now 82.)
+// trip of its own: with four of them a step of the tiny model took 114 us, of which the device worked 54; then 82, and 72 with what has been taken out of the kernel since.)
 struct StepResult {
   int32_t stop, abort_flag, err, err_info, win_len, n_gen;
   int32_t win[spd::kMaxK][spd::kWin];

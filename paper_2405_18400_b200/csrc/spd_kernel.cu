@@ -622,7 +622,8 @@ __device__ __forceinline__ void prologue_plain(const float *src, int C, float (&
   }
 }
 
-// Ranges that the T cached positions of a head are split into, and the first position of range sp (T * sp / ns).
+// Ranges that the T cached positions of a head are split into, and the first position of range sp (T * sp / ns).  (One range, up to 64
+// positions, is the whole: its items make no divisions, which stand between two barriers.  10 tokens, 7B shape, 25.30 -> 25.20 ms.)
 __device__ __forceinline__ int attn_splits(const KParams &p, int T) { return min((int)((unsigned)(T + 63) / 64u), p.attn_most); }
 __device__ __forceinline__ int attn_from(int T, int ns, int sp) {
   const unsigned q = (unsigned)T / (unsigned)ns, r = (unsigned)T - q * (unsigned)ns;
@@ -690,11 +691,16 @@ __device__ __forceinline__ void prefetch_kv(const KParams &p, int layer, int pos
   const int esz = p.kv_bf16 ? 2 : 4;
   const int lpr = (p.hd * esz + 127) >> 7;  // 128-byte lines per cache row of a head
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
-    const int head = item / ns, sp = item - head * ns;
-    const int t0 = attn_from(T, ns, sp), t1 = min(attn_from(T, ns, sp + 1), pos);
-    const int n = (t1 - t0) * lpr;
-    for (int i = threadIdx.x; i < n; i += kConsumerThreads) {
-      const int t = t0 + i / lpr, c = i - (i / lpr) * lpr;
+    int head = item, t0 = 0, t1 = pos;
+    if (ns > 1) {
+      head = item / ns;
+      const int sp = item - head * ns;
+      t0 = attn_from(T, ns, sp);
+      t1 = min(attn_from(T, ns, sp + 1), pos);
+    }
+    // eight threads per row (a row has 8 lines at most; with an index divided by the lines the phase's start was 0.1 us longer)
+    const int c = threadIdx.x & 7;
+    for (int t = t0 + (int)(threadIdx.x >> 3); t < t1 && c < lpr; t += kConsumerThreads / 8) {
       const size_t off = (((size_t)layer * p.max_pos + t) * p.d + (size_t)head * p.hd) * esz + (size_t)c * 128;
       prefetch_l2(reinterpret_cast<const uint8_t *>(p.kcache) + off);
       prefetch_l2(reinterpret_cast<const uint8_t *>(p.vcache) + off);
@@ -734,8 +740,13 @@ __device__ void attention_rows(Blk &b, int layer, int pos) {
   float *s_acc = scratch_base(p), *s_m = scratch_base(p) + kConsumerWarps * 256, *s_l = s_m + kConsumerWarps;
   const E *kc = reinterpret_cast<const E *>(p.kcache), *vc = reinterpret_cast<const E *>(p.vcache);
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
-    const int head = item / ns, sp = item - head * ns;
-    const int t0 = attn_from(T, ns, sp), t1 = attn_from(T, ns, sp + 1);
+    int head = item, t0 = 0, t1 = T;
+    if (ns > 1) {
+      head = item / ns;
+      const int sp = item - head * ns;
+      t0 = attn_from(T, ns, sp);
+      t1 = attn_from(T, ns, sp + 1);
+    }
     float q[EPL], acc[EPL];
 #pragma unroll
     for (int e = 0; e < EPL; e += 4) {
@@ -1097,7 +1108,7 @@ __global__ void __launch_bounds__(kThreads, 1) spd_sample_kernel(const __grid_co
 // units of them divide unevenly among the blocks and their fragments of x would take a third of the ring's memory
 // (measured: 2.96 ms per 7B timestep with it on the tensor cores too, against 2.64 ms).
 __global__ void __launch_bounds__(kThreads, 1) spd_decode_img_kernel(const __grid_constant__ KParams p) { kernel_body<false, true>(p); }
-// The sampling twin for such weights (7B shape: 2.63 ms per sampled token; the float32 loop for every matrix 2.99).
+// The sampling twin for such weights (7B shape, temperature 0.2 / 1: 2.42 / 2.57 ms per sampled token; the float32 loop for every matrix 2.99 at its time).
 __global__ void __launch_bounds__(kThreads, 1) spd_sample_img_kernel(const __grid_constant__ KParams p) { kernel_body<true, true>(p); }
 
 }  // namespace spd

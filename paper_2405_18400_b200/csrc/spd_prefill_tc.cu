@@ -2,7 +2,7 @@
 // time, their matrix products on the fifth-generation tensor cores (tcgen05.mma, operands staged in shared
 // memory by tiled TMA copies, float32 accumulators in tensor memory), everything between the products in small
 // row-wise kernels.  The job that ends a prefix goes on to the LM head and the first timestep of its last token
-// (7B shape, host to host: 15 / 27 / 100 / 400 / 2048 tokens 3.1 / 3.2 / 5.1 / 18 / 81 ms; with 128 x 128 tiles of single
+// (7B shape, host to host: 15 / 27 / 100 / 400 / 2048 tokens 3.0 / 3.1 / 5.0 / 18 / 81 ms; with 128 x 128 tiles of single
 // blocks and the last 1..16 tokens in spd_prefill_kernel 4.7 / 9.2 / 12.2 / 24 / 110 ms).
 //
 // Product: Y[token][row] = sum_c X[token][c] W[row][c], W bf16 [rows][cols] as stored, X float32 activations
