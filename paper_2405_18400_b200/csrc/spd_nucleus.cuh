@@ -186,7 +186,12 @@ static __device__ bool ns_near(NsNear &s, const float *logits, int V, float inv_
   }
   named_sync(1, kConsumerThreads);
   unsigned int far_hi = 0u, far_lo = 0u;  // at most 128 values (V is below 65536), halves below 2^20
-  for (int base = 0; base < V && *reinterpret_cast<volatile int *>(&s.listed) <= kNearList; base += kNearFlight * kConsumerThreads) {
+  for (int base = 0; base < V; base += kNearFlight * kConsumerThreads) {
+    // One lane looks whether the list is full and all follow it: other warps add to it meanwhile, and lanes that each looked for
+    // themselves could part in front of the votes below, which wait for the whole warp.  (Warps may leave in different rounds.)
+    int listed = 0;
+    if (lane == 0) listed = *reinterpret_cast<volatile int *>(&s.listed);
+    if (__shfl_sync(0xffffffffu, listed, 0) > kNearList) break;
     float zb[kNearFlight];
 #pragma unroll
     for (int e = 0; e < kNearFlight; ++e) {

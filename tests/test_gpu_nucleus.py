@@ -12,7 +12,7 @@ import torch
 
 import spd_inputs as si
 from oracle import spd_oracle as so
-from tests.gpu_common import LOGIT_TOL, compare_first_step, compare_step, make_tiny_pair
+from tests.gpu_common import LOGIT_TOL, compare_first_step, compare_step, make_pair, make_tiny_pair
 
 pytestmark = pytest.mark.gpu
 
@@ -102,6 +102,39 @@ def test_few_tokens_near_the_best(tiny_inputs, near, rest, top_p, equal):
         assert tok in ok, (u, tok, want)
         exact += tok == want
     assert exact >= 11
+    ctx.close()
+
+
+# A pass over the logits is 8192 of them a round.  The list of near tokens is full, or not, at the end of a round, in the middle of one
+# where some warps have left and some have not, in the last: by where the near tokens lie.
+@pytest.mark.parametrize("spans", [[(0, 8192, 512)], [(0, 8192, 513)], [(8000, 8400, 400), (30000, 40000, 112)], [(8000, 8400, 400), (39000, 40000, 113)],
+                                   [(0, 40000, 513)], [(0, 40000, 4000)], [(8192, 16384, 8192)], [(0, 40000, 40000)]])
+def test_a_list_that_fills_up_on_the_way(spans):
+    shape = si.ModelShape("wide", 1, 128, 2, 128, 40000)
+    ctx, _ = make_pair(shape, si.make_weights(shape, seed=107), [], 3, (2, 3), [0.0] * 8, 0.4, 0.2, 0.05, 64, "f32")
+    rng = np.random.default_rng(len(spans) + spans[0][2])
+    temperature, exact, n = 0.25, 0, 0
+    for seed in range(3):
+        x = np.full(shape.vocab, 12.0)
+        for lo, hi, near in spans:
+            x[lo + rng.permutation(hi - lo)[:near]] = rng.integers(0, 127, near) / 16
+        z = (3.0 - temperature * x).astype(np.float32)
+        for top_p in (0.3, 0.95, 1.0):
+            for u in uniforms(3, seed):
+                tok = ctx.spd_debug_nucleus(z, top_p, temperature, float(u))
+                want, ok = accepted(z, temperature, top_p, float(u))
+                assert tok in ok, (top_p, u, tok, want)
+                exact += tok == want
+                n += 1
+    if sum(near for _, _, near in spans) < 1000:     # (thousands of tokens: most draws are within EPS of a boundary)
+        assert exact >= n - 6
+    # and from a model's own logits, with their largest ones known by the blocks' lists: peaked to flat
+    ctx.spd_prefill(si.make_prefix("zipf", 9, shape.vocab, 1.1, seed=108))
+    for i, temperature in enumerate((0.005, 0.02, 0.05, 0.1, 1.0)):
+        z = ctx.spd_debug_read("LOGITS")
+        u = uniforms(5, 9)[i]
+        new, _, _ = ctx.spd_sample([u], 0.9, temperature)
+        assert int(new[0]) in accepted(z, temperature, 0.9, float(u))[1]
     ctx.close()
 
 
