@@ -31,6 +31,7 @@ __device__ __forceinline__ void warp_best(float &v, int &i) {
 // One warp: the k best logits among rows [r0, r1) and (max, sum exp) of z / tau over them, into list `slot` of the
 // partial lists (the decode and prefill kernels: warp 0 of each block, slot = the block), best first.  A lane asks for eight
 // rows at a time, and keeps them for all rounds when that is all there is (up to 256 rows: a block's share of the LM head).
+// A NaN ranks as -inf does (fmaxf passes over it): compared as it is, one in a lane's first row would hide the lane's other rows.
 constexpr int kTopkFlight = 8;
 static __device__ void block_topk(const KParams &p, int r0, int r1, int slot) {
   const int lane = threadIdx.x & 31;
@@ -52,7 +53,8 @@ static __device__ void block_topk(const KParams &p, int r0, int r1, int slot) {
 #pragma unroll
       for (int e = 0; e < kTopkFlight; ++e) {
         const int id = r0 + lane + 32 * e;
-        if (id < r1 && !(taken >> e & 1u) && (bi < 0 || z[e] > bv)) { bv = z[e]; bi = id; }
+        const float v = fmaxf(z[e], -CUDART_INF_F);
+        if (id < r1 && !(taken >> e & 1u) && (bi < 0 || v > bv)) { bv = v; bi = id; }
       }
     } else {
       for (int r = r0 + lane; r < r1; r += 32 * kTopkFlight) {
@@ -60,8 +62,9 @@ static __device__ void block_topk(const KParams &p, int r0, int r1, int slot) {
 #pragma unroll
         for (int e = 0; e < kTopkFlight; ++e) {
           const int id = r + 32 * e;
+          const float v = fmaxf(z[e], -CUDART_INF_F);
           // (rows already taken, the previous winner among them, are passed over)
-          if (id < r1 && (j == 0 || ranks_before(pv, pi, z[e], id)) && (bi < 0 || ranks_before(z[e], id, bv, bi))) { bv = z[e]; bi = id; }
+          if (id < r1 && (j == 0 || ranks_before(pv, pi, v, id)) && (bi < 0 || ranks_before(v, id, bv, bi))) { bv = v; bi = id; }
         }
       }
     }

@@ -138,6 +138,33 @@ def test_a_list_that_fills_up_on_the_way(spans):
     ctx.close()
 
 
+@pytest.mark.parametrize("vocab", [20000, 37888, 40000])
+def test_nan_logits_are_not_drawn(vocab):
+    """The draw behind a pass takes its maximum from the blocks' lists: a NaN beside the largest logit does not hide it."""
+    import paper_2405_18400_b200 as P
+
+    shape = si.ModelShape("nan", 1, 128, 2, 128, vocab)
+    weights = si.make_weights(shape, seed=111)
+    make = lambda: P.SpdContext(shape, P.pack_weights(weights, "cuda:0"), [], 8, (2, 3), [0.0] * 8, 0.4, 0.2, 0.05, 64, "f32")
+    prefix = si.make_prefix("zipf", 9, vocab, 1.1, seed=112)
+    sound = make()
+    sound.spd_prefill(prefix)
+    top = sound.spd_debug_read("CAND_TOK").tolist()
+    bad = [r for r in sorted({t + o for t in top for o in (-96, -64, -32, 32)} - set(top)) if 0 <= r < vocab]
+    weights["lm_head"][bad] = float("nan")
+    damaged = make()
+    for temperature in (0.01, 0.05, 1.0):
+        for u in uniforms(6, 113):
+            damaged.spd_prefill(prefix)
+            z = damaged.spd_debug_read("LOGITS")
+            assert np.isnan(z[bad]).all() and np.isnan(z).sum() == len(bad)
+            new, _, _ = damaged.spd_sample([u], 0.9, temperature)
+            z[bad] = -1e30
+            want, ok = accepted(z, temperature, 0.9, float(u))
+            assert int(new[0]) in ok, (temperature, u, new, want)
+    sound.close(); damaged.close()
+
+
 def test_arguments_are_checked(tiny_inputs):
     ctx, _ = make_tiny_pair(tiny_inputs)
     _, _, _, prefix = tiny_inputs

@@ -57,3 +57,41 @@ def test_equal_logits_are_kept_by_id(vocab, k):
             ctx.spd_step()
     assert tied                                      # (a step whose hidden row is nearly at right angles to that row has none)
     ctx.close()
+
+
+@pytest.mark.parametrize("vocab", [20000, 37888, 40000])     # 136 rows a block, 256 (the most that stay in registers), 272
+def test_nan_logits_are_passed_over(vocab):
+    """Logits that are NaN are left out of the kept tokens, wherever they lie beside them."""
+    import numpy as np
+    import paper_2405_18400_b200 as P
+    shape = si.ModelShape("nan", 1, 128, 2, 128, vocab)
+    weights = si.make_weights(shape, seed=109)
+    make = lambda: P.SpdContext(shape, P.pack_weights(weights, "cuda:0"), [], 8, (2, 3), [0.0] * 8, 0.4, 0.2, 0.05, 192, "f32")
+    prefixes = [si.make_prefix("zipf", m, vocab, 1.1, seed=110 + m) for m in (9, 40)]      # the 16-token kernel's end, a job's
+    sound = make()
+    top = set()
+    for prefix in prefixes:
+        top |= set(sound.spd_prefill(prefix)[0].tolist())
+    # rows of the kept tokens' lanes (a lane has every 32nd row of its block), none of the kept ones
+    bad = [r for r in sorted({t + o for t in top for o in (-96, -64, -32, 32)} - top) if 0 <= r < vocab]
+    weights["lm_head"][bad] = float("nan")
+    damaged = make()
+    for prefix in prefixes:
+        want = sound.spd_prefill(prefix)[0]
+        z = sound.spd_debug_read("LOGITS")
+        z[bad] = np.nan
+        got = damaged.spd_prefill(prefix)[0]
+        assert np.array_equal(damaged.spd_debug_read("LOGITS"), z, equal_nan=True)
+        assert got.tolist() == want.tolist()
+    # and with all but three rows lost, those three, then the lost ones by their ids
+    keep = sound.spd_debug_read("CAND_TOK")[:3].tolist()
+    weights["lm_head"][[r for r in range(vocab) if r not in keep]] = float("nan")
+    lost = make()
+    for prefix in prefixes:
+        lost.spd_prefill(prefix)
+        z = lost.spd_debug_read("LOGITS")
+        best = sorted(keep, key=lambda t: (-float(z[t]), t))
+        first = [r for r in range(11) if r not in keep][:5]
+        assert lost.spd_debug_read("CAND_TOK").tolist() == best + first
+    for c in (sound, damaged, lost):
+        c.close()
