@@ -131,11 +131,11 @@ static __device__ void tail_score_select(Blk &b, bool first, int step) {
         int bi = -1;
         for (int c = lane; c < k * k; c += 32) {
           const float z = s_score[c];
-          if (!(taken >> (c >> 5) & 1u) && (bi < 0 || z > bv)) { bv = z; bi = c; }
+          if (!(taken >> (c >> 5) & 1u) && (bi < 0 || z > bv || (bv != bv && z == z))) { bv = z; bi = c; }
         }
         warp_best(bv, bi);
         if ((bi & 31) == lane) taken |= 1u << (bi >> 5);
-        if (lane == r) { my_sel = max(bi, 0); my_score = bv; }  // NaN scores can leave a round without a winner: keep the option valid
+        if (lane == r) { my_sel = bi; my_score = bv; }  // (every round has a winner: k options at least, and NaN is one, behind all others)
       }
       int w[kWin];
       float old_lp = 0.f;

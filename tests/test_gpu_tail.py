@@ -95,3 +95,24 @@ def test_nan_logits_are_passed_over(vocab):
         assert lost.spd_debug_read("CAND_TOK").tolist() == best + first
     for c in (sound, damaged, lost):
         c.close()
+
+
+@pytest.mark.parametrize("k", [3, 6, 8, 16])                  # 9 to 256 options: one to eight of a lane
+def test_nan_scores_rank_last(k):
+    """Options whose score is NaN (a draft's or a kept token's log-probability is) are chosen when nothing else is left, by index."""
+    import numpy as np
+    import paper_2405_18400_b200 as P
+    shape = si.ModelShape("nan", 1, 128, 2, 128, 800)
+    ctx = P.SpdContext(shape, P.pack_weights(si.make_weights(shape, seed=114), "cuda:0"), [], k, (2, 3), [0.0] * 8, 0.4, 0.2, 0.05, 64, "f32")
+    rng = np.random.default_rng(k)
+    for lost_drafts, lost_tokens in ([0], []), ([], [0]), (list(range(k - 1)), []), (list(range(k - 1)), [0, k - 1]), (list(range(1, k)), [1]), ([], []):
+        logp, cand_lp = rng.normal(-8, 2, k).astype(np.float32), rng.normal(-3, 1, k).astype(np.float32)
+        logp[k // 2] = -1.0                                   # the best draft's options lie beside the first draft's in their lanes (k = 8)
+        logp[lost_drafts] = np.nan
+        cand_lp[lost_tokens] = np.nan
+        ctx.spd_debug_score(rng.integers(0, 800, (k, 2)), logp, rng.permutation(800)[:k].astype(np.int32), cand_lp)
+        score = ctx.spd_debug_read("SCORE").astype(np.float64).reshape(-1)
+        assert np.isnan(score).sum() == k * k - (k - len(lost_drafts)) * (k - len(lost_tokens))
+        order = np.lexsort((np.arange(k * k), -np.where(np.isnan(score), -np.inf, score), np.isnan(score)))
+        assert ctx.spd_debug_read("SEL").tolist() == order[:k].tolist(), (lost_drafts, lost_tokens)
+    ctx.close()
