@@ -306,7 +306,11 @@ __global__ void __launch_bounds__(kBtThreads) spd_batch_swiglu_kernel(const __gr
 // behind 150 positions each: 4.58 / 7.99 ms (a warp per position, one in flight, element-wise loads), now 3.51 / 6.14 ms; with the
 // request's position known before the wait, no trip to L2 for it, and the rows asked into L2 while the rotary kernel runs, three
 // timesteps of 8 / 64 requests behind 15 to 90 positions (float32 cache) 9.47 / 16.28 -> 9.31 / 15.58 ms.
-constexpr int kBaWarps = 8, kBaFlight = 4;
+// The blocks that are resident together ask for half of L2, their first rows.  All rows at once, where that is more than L2 holds, push
+// one another out before they are read.  8 layers of the 7B shape, ms per timestep, none / bounded / all: float32, 32 requests behind
+// 500 positions 1.66 / 1.63 / 1.89, behind 2000 3.75 / 3.76 / 5.11, 16 behind 1000 1.66 / 1.55 / 1.73, 1 behind 2000 1.40 / 1.28 / 1.27;
+// bf16, 32 behind 2000 2.54 / 2.46 / 2.93.  (32 to 96 MB, for all blocks or for the first to come only: alike.)
+constexpr int kBaWarps = 8, kBaFlight = 4, kBaPerSm = 5, kBaAhead = 64 << 20;
 
 template <typename E>
 __device__ __forceinline__ void ba_unpack(const uint4 &v, float (&x)[16 / sizeof(E)]) {
@@ -398,9 +402,10 @@ __device__ void ba_head(const float *q_row, const E *kc, const E *vc, int d, int
   }
 }
 
+// ahead: bytes of keys, and of values, that a block may ask for before its wait.
 template <int HD>
 __global__ void __launch_bounds__(kBaWarps * 32) spd_batch_attn_kernel(const float *Q, const KParams *kps, uint16_t *X, size_t term_stride, int d,
-                                                                       int layer, int step) {
+                                                                       int layer, int step, int ahead) {
   dep_launch();
   constexpr int kGroups = kBaWarps * 32 / (HD / 8);  // bf16: the larger number of groups
   __shared__ float s_acc[kGroups * HD], s_m[kGroups], s_l[kGroups];
@@ -408,11 +413,12 @@ __global__ void __launch_bounds__(kBaWarps * 32) spd_batch_attn_kernel(const flo
   const int T = bt_pos(p, step) + 1, kv_bf16 = p.kv_bf16;
   const void *kcache = p.kcache, *vcache = p.vcache;
   const size_t x_at = (size_t)blockIdx.x * d + blockIdx.y * HD, base = (size_t)layer * p.max_pos * d + blockIdx.y * HD;
-  // The cached rows are on their way to L2 while the kernel before this one still runs (a hint: they are read behind the wait).
+  // The first cached rows are on their way to L2 while the kernel before this one still runs (a hint: they are read behind the wait).
   {
-    const int lines = HD * (kv_bf16 ? 2 : 4) / 128, esz = kv_bf16 ? 2 : 4;
-    for (int i = threadIdx.x; i < (T - 1) * lines; i += kBaWarps * 32) {
-      const size_t off = (base + (size_t)(i / lines) * d) * esz + (size_t)(i % lines) * 128;
+    const int esz = kv_bf16 ? 2 : 4, shift = (HD == 128 ? 1 : 0) + (kv_bf16 ? 0 : 1);  // a row is 2^shift lines of 128 bytes
+    const int rows = min(T - 1, ahead >> (7 + shift));
+    for (int i = threadIdx.x; i < rows << shift; i += kBaWarps * 32) {
+      const size_t off = (base + (size_t)(i >> shift) * d) * esz + (size_t)(i & ((1 << shift) - 1)) * 128;
       asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const uint8_t *>(kcache) + off));
       asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const uint8_t *>(vcache) + off));
     }
@@ -603,6 +609,7 @@ extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd:
   const int nch = (d + spd::kBtCols - 1) / spd::kBtCols, nch_f = (f + spd::kBtCols - 1) / spd::kBtCols;
   const dim3 threads(spd::kBtThreads);
   const bool few = n <= spd::kFewRows;
+  const int blocks = n * j.H, resident = spd::kBaPerSm * j.sm_count, ahead = spd::kBaAhead / 2 / (blocks < resident ? blocks : resident);
   int count = 0;
   cudaError_t e = cudaSuccess;
   spd::Product pr;  // where the last product's sums are
@@ -625,8 +632,8 @@ extern "C" cudaError_t spd_internal_batch_step(const spd::TcJob *job, const spd:
       done(spd::launch_dep(few ? spd::spd_batch_rope_cache_kernel<spd::kPartFlight> : spd::spd_batch_rope_cache_kernel<1>, dim3(n, nch), threads, 0, s, pr, j.ss,
                            j.eps, j.q, kps, d, j.hd, l, step));
     if (e == cudaSuccess)
-      done(j.hd == 128 ? spd::launch_dep(spd::spd_batch_attn_kernel<128>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l, step)
-                       : spd::launch_dep(spd::spd_batch_attn_kernel<64>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l, step));
+      done(j.hd == 128 ? spd::launch_dep(spd::spd_batch_attn_kernel<128>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l, step, ahead)
+                       : spd::launch_dep(spd::spd_batch_attn_kernel<64>, dim3(n, j.H), dim3(spd::kBaWarps * 32), 0, s, j.q, kps, j.x, ts_d, d, l, step, ahead));
     product(0, 4 * l + 1, d);
     resid(j.layers[l].ffn_norm);
     product(0, 4 * l + 2, 2 * f);

@@ -199,3 +199,36 @@ def test_a_malformed_table_of_one_request_stops_only_that_request(tiny_inputs):
         ctxs[at].spd_prefill(prefix)            # and the request itself can be taken up again, up to its table
         for c in ctxs + sound:
             c.close()
+
+
+@pytest.mark.parametrize("heads", [16, 8])
+def test_batches_behind_long_prefixes(heads):
+    """24 requests behind 2 to 900 positions, float32 and bf16 caches among them: the attention asks for the first rows of a cache ahead,
+    as many as a block's share of L2 (341 float32, 682 bf16 here), so for all rows of some requests and a part of others'."""
+    import paper_2405_18400_b200 as P
+
+    shape = si.ModelShape("long%d" % heads, 1, 1024, heads, 512, 600)
+    weights = si.make_weights(shape, seed=121)
+    packed = P.pack_weights(weights, "cuda:0")
+    tables = si.make_ngram_tables(shape.vocab, 1.1, 20_000, (2, 3), 2000, seed=122)
+    dtabs = P.build_ngram_tables(tables, "cuda:0")
+    otabs = sorted(tables, key=lambda t: int(t["n"]))
+    lam = [0.3, 0.2] + [0.0] * 6
+    lengths = [2, 341, 342, 343, 682, 683, 900, 100] + [40 * (r + 1) for r in range(16)]
+    ctxs, orcs = [], {}
+    for r, m in enumerate(lengths):
+        kv_dtype = "bf16" if r % 2 else "f32"
+        ctx = P.SpdContext(shape, packed, dtabs, 3, (2, 3), lam, 0.4, 0.2, 0.05, 920, kv_dtype)
+        prefix = si.make_prefix("zipf", m, shape.vocab, 1.1, seed=123 + r)
+        if r in (0, 2, 4, 5, 6):
+            orcs[r] = so.Oracle(so.make_config(shape, 3, (2, 3), lam, 0.4, 0.2, 0.05, 920, kv_dtype), weights, otabs)
+            compare_first_step(ctx, orcs[r], prefix)
+        else:
+            ctx.spd_prefill(prefix)
+        ctxs.append(ctx)
+    for _ in range(2):
+        res = P.spd_batch_step(ctxs)
+        for r, orc in orcs.items():
+            compare_step(ctxs[r], orc, None, stepped=res[r], path="prefill")
+    for c in ctxs + list(orcs.values()):
+        c.close()
