@@ -348,8 +348,8 @@ class SpdContext:
         if what in ("KCACHE", "VCACHE"):
             shapes[what] = (np.float32, (c.n_layers, int(positions), c.d_model))
         dt, shp = shapes[what]
-        # All but the caches are written whole.  (Zeroed memory is fresh pages, which the copy then faults in one by one: 128 KB of
-        # logits 46 us instead of 26.)
+        # All but the caches are written whole.  (Zeroing 128 KB of logits first, an array that the caller drops at once takes 44 us
+        # instead of 27, 64 arrays read after a batch's three timesteps 16.4 ms with these instead of 15.5.)
         out = np.zeros(shp, dt) if what in ("KCACHE", "VCACHE") else np.empty(shp, dt)
         _check(self.lib.spd_debug_read(self.h, DBG[what], out.ctypes.data, out.nbytes), "spd_debug_read")
         if what in ("CNT", "TOT"):      # unsigned 32-bit on the device, 0xffffffff = order skipped: as int64 with -1

@@ -41,8 +41,8 @@ __shared__ int s_dead, s_quit;
 // The matrices of a layer in the order of their phases, then the LM head.
 enum Matrix { kMatQKV = 0, kMatO = 1, kMatGateUp = 2, kMatDown = 3, kMatHead = 4, kMatrices = 5 };
 // This block's rows [x, y) of each matrix and the whole rows of it that a stage takes.  They stay what they are for the whole
-// launch, and their divisions stood between a phase's first barrier and its first multiply: two of 64 bits, 0.5 us, four times a
-// layer (7B shape).
+// launch, and their divisions stood between a phase's first barrier and its first multiply: two of 64 bits, 0.25 us for both, four
+// times a layer (7B shape).
 __shared__ int2 s_rows[kMatrices];
 __shared__ int s_chunk_rows[kMatrices];
 

@@ -314,7 +314,8 @@ static __device__ __noinline__ int ns_sample(const float *logits, int V, float i
   named_sync(1, kConsumerThreads);
   const float m = s.zmax * inv_t;
   // Not tried when fifteen in sixteen of the parts' largest logits are that near: with 148 parts of 216 some 400 tokens are then (an
-  // attempt in vain costs a draw 8 us).
+  // attempt in vain costs a draw 8 us).  Vocabularies of 2000, 32000 and 50000, temperatures 0.05 to 2: 0.33 to 0.98 of the time of a
+  // search with its own pass for the maximum, at the flat end 0.92 to 0.98.
   const unsigned int near_votes = __ballot_sync(0xffffffffu, -fmaf(head, inv_t, -m) < 8.f);
   if (lane == 0) s.warp_cnt[warp] = __popc(near_votes);
   named_sync(1, kConsumerThreads);
